@@ -207,21 +207,6 @@ struct PointEval {
     double inv_sub;   // 1 / n_sub
     double gl[MAXQ];  // Gauss-Lobatto support points of the velocity element
 
-    __device__ void locate(const double s[3], int k[3], double xi[3]) const {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            int c = (int)floor(s[a]);
-            c = c < 0 ? 0 : (c > m.n - 1 ? m.n - 1 : c);
-            k[a] = c;
-            xi[a] = s[a] - c;
-        }
-    }
-    __device__ void phi_grad(const double s[3], double& val, double g[3]) const {
-        int k[3];
-        double xi[3];
-        locate(s, k, xi);
-        q1_at(phi, m.n, k[0], k[1], k[2], xi[0], xi[1], xi[2], m.inv_h, val, g);
-    }
     __device__ void velocity(const double s_ls[3], double out[3]) const {
         int k[3];
         double xi[3];
@@ -269,30 +254,54 @@ __device__ __forceinline__ double dist3(const double a[3], const double b[3]) {
     return sqrt(d0 * d0 + d1 * d1 + d2 * d2);
 }
 
+enum : int { TRIAL_RUN = 0, TRIAL_FAIL, TRIAL_OK, TRIAL_IDLE };  // a trial point's projection
+
 // Closest point of x on d(phi_h) = d_t with the backtracked tangential step (App. C), written as a state machine
 // in which every trip of the loop makes exactly one point evaluation of phi_h and grad phi_h: the projection of the
-// node (phase 0, at most CPP_NORMAL_STEPS normal steps), the tangential direction at y (phase 1), the projection of a
-// trial point y - omega t (phase 2, at most CPP_TRIAL_STEPS normal steps, omega = 1, 1/2, ..., 1/2^(CPP_BACKTRACK-1)).
-// Lanes of a warp run their own nodes but share the expensive part of every trip (the FP64 evaluation), and a lane
-// whose node is done takes the next band entry, so warps stay full.  The sequence of evaluations and updates of a
-// node is: project x (normal steps y <- y - (d(y) - d*) / |grad d(y)| n(y) until |d(y) - d*| <= tol h); then
-// repeat up to kmax times: tangential part t of y - x at y; for omega = 1, 1/2, ...: project y - omega t; accept
-// the first trial point that reached the isocontour and is strictly closer to x; stop when none is, when the accepted
-// step is <= tol or shortens |y - x| by <= CPP_STALL of it.  Not converged: the first projection failed or kmax
-// outer iterations ran without a stop.
+// node (phase 0, at most CPP_NORMAL_STEPS normal steps) and the projection of a trial point y - omega t (phase 2, at
+// most CPP_TRIAL_STEPS normal steps, omega = 1, 1/2, ..., 1/2^(CPP_BACKTRACK-1)); the tangential direction at a new y
+// takes the normal of the evaluation that ended the projection there.  The sequence of updates of a node is: project x
+// (normal steps y <- y - (d(y) - d*) / |grad d(y)| n(y) until |d(y) - d*| <= tol h); then repeat up to kmax times:
+// tangential part t of y - x at y; for omega = 1, 1/2, ...: project y - omega t; accept the first trial point that
+// reached the isocontour and is strictly closer to x; stop when none is, when the accepted step is <= tol or shortens
+// |y - x| by <= CPP_STALL of it.  Not converged: the first projection failed or kmax outer iterations ran without a
+// stop.
 struct CppLane {
     int b = -1;  // band entry, -1 none
-    int phase = 0, steps = 0, k = 0, bt = 0, trips = 0;
+    int phase = 0, steps = 0, k = 0, bt = 0, ev = 0, trips = 0;
+    int st = TRIAL_IDLE;
     double x[3], y[3], yn[3], tp[3];
-    double dist = 0.0, dist_prev = 0.0, omega = 1.0;
+    double nv[3], nrm = 0.0, dn = 0.0;  // of the trial point that ended last: unit normal, |grad phi|, distance to x
+    double dist = 0.0, dist_prev = 0.0;
 };
+
+// Cell and local coordinate of s in [0, n] (cell units, n <= 2^11): clamp(floor(s), 0, n - 1) and s - cell, with the
+// difference as the only FP64 instruction: the floor of a non-negative double is its bits with the fraction masked off, and its integer value
+// the leading mantissa bits.  (Any other s, a NaN for one, still gives a cell of the mesh.)
+__device__ __forceinline__ void locate_in_range(double s, int n, int& k, double& xi) {
+    const int hi = __double2hiint(s);
+    const int e = min((hi >> 20) - 1023, 20);
+    const bool frac = e < 0;  // s < 1
+    const int sh = frac ? 0 : e;
+    const int fl = frac ? 0 : (hi & ~(0xFFFFF >> sh));
+    const int c = frac ? 0 : (((hi & 0xFFFFF) | 0x100000) >> (20 - sh));
+    k = min(c, n - 1);
+    xi = s - (c > n - 1 ? (double)(n - 1) : __hiloint2double(fl, 0));
+}
+
+// v clamped to [0, hi]: in the interior the high words alone decide (hi > 0)
+__device__ __forceinline__ double clamp_range(double v, double hi) {
+    if ((unsigned)__double2hiint(v) < (unsigned)__double2hiint(hi)) return v;
+    return clampd(v, 0.0, hi);
+}
 
 // phi_h and grad phi_h (physical units) at s (cell units) by successive linear interpolation along x, y, z
 // (the trilinear Q1 interpolant of Sec. 2.5; fewer FP64 operations than the weighted sum over the 8 nodes).
 __device__ __forceinline__ void q1_lerp(const PointEval& e, const double s[3], double& val, double g[3]) {
     int k[3];
     double t[3];
-    e.locate(s, k, t);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) locate_in_range(s[a], e.m.n, k[a], t[a]);
     const int64_t m1 = e.m.n + 1;
     const double* f = e.phi + k[0] + m1 * (k[1] + m1 * k[2]);
     double ex[2][2], dx[2][2];
@@ -318,24 +327,33 @@ __device__ __forceinline__ void q1_lerp(const PointEval& e, const double s[3], d
     g[2] = dz * e.m.inv_h;
 }
 
-// Transport velocity at Q1 node `node` from the point y (cell units) whose velocity is extended:
-// u_Gamma = u(y) + mdot/rho_* n(x), n(x) the point-located normal at the node.
-__device__ void transport_finish(const PointEval& e, const double* __restrict__ mdot, int64_t node, const double y[3],
-                                 double rho_t, double* __restrict__ ug) {
+// Unit normal of phi_h at lattice node (i, j, k), point-located in the cell clamp(node, 0, n - 1): the point is a corner
+// of that cell, so the gradient is the difference along each of its three edges there (the trilinear formula with
+// weights 0 and 1, in which only these terms are nonzero); zero where |grad phi| h <= GRAD_TINY.
+__device__ __forceinline__ void node_normal(const PointEval& e, int i, int j, int k, double nx[3]) {
     const MeshArgs<double>& m = e.m;
-    const int m1 = m.n + 1;
-    const double sx[3] = {(double)(node % m1), (double)((node / m1) % m1), (double)(node / ((int64_t)m1 * m1))};
-    double ph, g[3];
-    e.phi_grad(sx, ph, g);
+    const int64_t m1 = m.n + 1;
+    const int ic = min(i, m.n - 1), jc = min(j, m.n - 1), kc = min(k, m.n - 1);
+    const double* f = e.phi;
+    const double g[3] = {(f[ic + 1 + m1 * (j + m1 * k)] - f[ic + m1 * (j + m1 * k)]) * m.inv_h,
+                         (f[i + m1 * (jc + 1 + m1 * k)] - f[i + m1 * (jc + m1 * k)]) * m.inv_h,
+                         (f[i + m1 * (j + m1 * (kc + 1))] - f[i + m1 * (j + m1 * kc)]) * m.inv_h};
     const double nrm = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
-    double nx[3] = {0.0, 0.0, 0.0};
+    nx[0] = nx[1] = nx[2] = 0.0;
     if (nrm * m.h > GRAD_TINY) { nx[0] = g[0] / nrm; nx[1] = g[1] / nrm; nx[2] = g[2] / nrm; }
-    double out[3];
-    e.velocity(y, out);
+}
+
+// Transport velocity at Q1 node (i, j, k) from the fluid velocity uv of the point it takes:
+// u_Gamma = uv + mdot/rho_* n(x), n(x) the point-located normal at the node.
+__device__ __forceinline__ void transport_store(const PointEval& e, const double* __restrict__ mdot, int64_t node, int i,
+                                                int j, int k, const double uv[3], double rho_t,
+                                                double* __restrict__ ug) {
+    double nx[3];
+    node_normal(e, i, j, k, nx);
     const double c = mdot[node] / rho_t;
-    ug[node] = out[0] + c * nx[0];
-    ug[m.Nphi + node] = out[1] + c * nx[1];
-    ug[2 * m.Nphi + node] = out[2] + c * nx[2];
+    ug[node] = uv[0] + c * nx[0];
+    ug[e.m.Nphi + node] = uv[1] + c * nx[1];
+    ug[2 * e.m.Nphi + node] = uv[2] + c * nx[2];
 }
 
 __device__ __forceinline__ bool in_projection_band(int variant, double phx) {
@@ -352,52 +370,52 @@ __global__ void k_transport_direct(PointEval e, const double* __restrict__ mdot,
     if (node >= m.Nphi) return;
     const double phx = e.phi[node];
     flags[node] = 0;
-    if (m.variant == 1) {
-        const int m1 = m.n + 1;
-        const int i = (int)(node % m1), j = (int)((node / m1) % m1), k = (int)(node / ((int64_t)m1 * m1));
-        const double sx[3] = {(double)i, (double)j, (double)k};
-        double ph, g[3];
-        e.phi_grad(sx, ph, g);
-        const double nrm = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
-        double nx[3] = {0.0, 0.0, 0.0};
-        if (nrm * m.h > GRAD_TINY) { nx[0] = g[0] / nrm; nx[1] = g[1] / nrm; nx[2] = g[2] / nrm; }
-        const Material mat = material(phx, 0.0, 0.0, 0.0, m);
-        double uv[3];
-        if (m.nsub == 1 || m.nsub == m.P) {  // the node is a velocity node
-            const int st = m.nsub == 1 ? m.P : 1;
-            const int64_t vn = (int64_t)(st * i) + (int64_t)m.M * ((int64_t)(st * j) + (int64_t)m.M * (st * k));
-            uv[0] = e.u[vn];
-            uv[1] = e.u[m.Nu + vn];
-            uv[2] = e.u[2 * m.Nu + vn];
-        } else {
-            e.velocity(sx, uv);
-        }
-        const double c = mdot[node] / mat.rho;
-        ug[node] = uv[0] + c * nx[0];
-        ug[m.Nphi + node] = uv[1] + c * nx[1];
-        ug[2 * m.Nphi + node] = uv[2] + c * nx[2];
-        return;
-    }
-    if (in_projection_band(m.variant, phx)) {
+    if (m.variant != 1 && in_projection_band(m.variant, phx)) {
         band[atomicAdd(band_count, 1)] = (int32_t)node;
         return;
     }
-    const int m1 = m.n + 1;
-    const double y[3] = {(double)(node % m1), (double)((node / m1) % m1), (double)(node / ((int64_t)m1 * m1))};
-    transport_finish(e, mdot, node, y, m.variant == 2 ? m.rho_l : m.rho_g, ug);
+    const unsigned m1 = (unsigned)m.n + 1u, nd = (unsigned)node, t = nd / m1;  // N_phi < 2^31 (band entries are int32)
+    const int i = (int)(nd - t * m1), k = (int)(t / m1), j = (int)(t - (unsigned)k * m1);
+    double uv[3];
+    if (m.nsub == 1 || m.nsub == m.P) {  // the node is a velocity node
+        const int st = m.nsub == 1 ? m.P : 1;
+        const int64_t vn = (int64_t)(st * i) + (int64_t)m.M * ((int64_t)(st * j) + (int64_t)m.M * (st * k));
+        uv[0] = e.u[vn];
+        uv[1] = e.u[m.Nu + vn];
+        uv[2] = e.u[2 * m.Nu + vn];
+    } else {
+        const double y[3] = {(double)i, (double)j, (double)k};
+        e.velocity(y, uv);
+    }
+    const double rho_t = m.variant == 1 ? material(phx, 0.0, 0.0, 0.0, m).rho : (m.variant == 2 ? m.rho_l : m.rho_g);
+    transport_store(e, mdot, node, i, j, k, uv, rho_t, ug);
 }
 
-// Pass 2, persistent: closest points of the band nodes on the liquid (variant 2) or gas (variant 3) end of the zone,
-// y of band entry b to band_y[3 b], the convergence flag to flags[node].  band_count[1] hands out the entries.
+// Pass 2, persistent, one warp per block: closest points of the band nodes on the liquid (variant 2) or gas (variant 3)
+// end of the zone, y of band entry b to band_y[3 b], the convergence flag to flags[node].  band_count[1] hands out the
+// entries.
+//
+// What bounds it: a warp's FP64 instruction occupies its scheduler's FP64 unit for 64 cycles however few lanes are
+// active, so the pass costs (trips of the slowest lane) x (~200 instructions) x 64 cycles on every scheduler, and a node
+// makes 20 to 500 trips (mean 97, on four drops at 64^3).  Hence (a) a lane whose node is done takes the next band
+// entry; (b) when the list is exhausted the warp's remaining nodes are spread over its idle lanes, G = 2, 4 or 8 lanes
+// per node, which project the trial points of the next G backtracking lengths at once: the first accepted one in
+// the order of the lengths is taken, so the points are the ones of the serial iteration bit for bit, and the longest
+// chains (many rejected lengths per outer iteration) shrink several times; (c) the tangential direction reuses the
+// evaluation that ended the projection; (d) point location and clamping run on the integer units.
+// The evaluations counted are those of the serial iteration (one per trip, one per tangential direction).
 __global__ void __launch_bounds__(32) k_transport_band(PointEval e, double tol, int kmax, const int32_t* __restrict__ band,
                                                        int32_t* band_count, double* __restrict__ band_y,
                                                        int32_t* __restrict__ flags, unsigned long long* flag_count,
                                                        unsigned long long* evals) {
     const MeshArgs<double>& m = e.m;
+    constexpr unsigned FULL = 0xffffffffu;
     const int count = band_count[0];
     const int m1 = m.n + 1;
     const double d_t = m.variant == 2 ? 3.0 * m.eps : -3.0 * m.eps;
     const double eps = m.eps, h = m.h, nn = (double)m.n;
+    const int lane = threadIdx.x;
+    int G = 1, sub = 0;  // lanes per node (warp-uniform), this lane's place in its group
     CppLane L;
     auto take = [&]() {
         L.b = atomicAdd(&band_count[1], 1);
@@ -413,102 +431,191 @@ __global__ void __launch_bounds__(32) k_transport_band(PointEval e, double tol, 
         L.phase = 0;
         L.steps = 0;
         L.trips = 0;
+        L.ev = 0;
     };
+    // the group's node is done (called by all of its lanes); lanes look for the next entry while they work alone
     auto finish = [&](bool converged) {
-        band_y[3 * (int64_t)L.b + 0] = L.y[0];
-        band_y[3 * (int64_t)L.b + 1] = L.y[1];
-        band_y[3 * (int64_t)L.b + 2] = L.y[2];
-        flags[band[L.b]] = converged ? 0 : 1;
-        if (!converged) atomicAdd(flag_count, 1ULL);
-        atomicAdd(evals, (unsigned long long)L.trips);
-        take();
+        if (sub == 0) {
+            band_y[3 * (int64_t)L.b + 0] = L.y[0];
+            band_y[3 * (int64_t)L.b + 1] = L.y[1];
+            band_y[3 * (int64_t)L.b + 2] = L.y[2];
+            flags[band[L.b]] = converged ? 0 : 1;
+            if (!converged) atomicAdd(flag_count, 1ULL);
+            atomicAdd(evals, (unsigned long long)L.trips);
+        }
+        L.b = -1;
+        if (G == 1) take();
     };
-    take();
+    // this lane's trial point y - 2^-bt t
+    auto start_trial = [&](int bt) {
+        L.bt = bt;
+        L.steps = 0;
+        L.ev = 0;
+        L.st = bt < CPP_BACKTRACK ? TRIAL_RUN : TRIAL_IDLE;
+        const double omega = __hiloint2double((1023 - bt) << 20, 0);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) L.yn[a] = clamp_range(L.y[a] - omega * L.tp[a], nn);
+    };
+    // the lanes of a warp that start with a node: all, or an even share of a short list
+    if (lane < (count + (int)gridDim.x - 1) / (int)gridDim.x) take();
     const double c_step = 1.0 / (2.0 * eps * h);  // step (cell units) = r / (|grad d| h), |grad d| = 2 eps |g| / (1 - ph^2)
-    while (__any_sync(0xffffffffu, L.b >= 0)) {
-        if (L.b < 0) continue;
-        ++L.trips;
-        // the trip's point evaluation and the quantities every phase needs (computed by all lanes alike)
+    const double tol_h = tol * h;
+    for (;;) {
+        const unsigned act = __ballot_sync(FULL, L.b >= 0);
+        if (!act) break;
+        if (act != FULL && G < 8) {  // the list is exhausted: more lanes per node as soon as the nodes left allow it
+            const unsigned leaders = G == 1 ? FULL : (G == 2 ? 0x55555555u : 0x11111111u);
+            const unsigned lead = act & leaders;
+            const int na = __popc(lead);
+            const int Gn = na <= 4 ? 8 : (na <= 8 ? 4 : (na <= 16 ? 2 : 1));
+            if (Gn > G) {  // node j -> lanes j Gn ... j Gn + Gn - 1; its running trials keep their places
+                const int j = lane / Gn, s2 = lane % Gn;
+                const bool has = j < na;
+                const int src = (has ? (int)__fns(lead, 0, j + 1) : lane) + (has && s2 < G ? s2 : 0);
+                CppLane N;
+                N.b = __shfl_sync(FULL, L.b, src);
+                N.phase = __shfl_sync(FULL, L.phase, src);
+                N.steps = __shfl_sync(FULL, L.steps, src);
+                N.k = __shfl_sync(FULL, L.k, src);
+                N.bt = __shfl_sync(FULL, L.bt, src);
+                N.ev = __shfl_sync(FULL, L.ev, src);
+                N.trips = __shfl_sync(FULL, L.trips, src);
+                N.st = __shfl_sync(FULL, L.st, src);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    N.x[a] = __shfl_sync(FULL, L.x[a], src);
+                    N.y[a] = __shfl_sync(FULL, L.y[a], src);
+                    N.yn[a] = __shfl_sync(FULL, L.yn[a], src);
+                    N.tp[a] = __shfl_sync(FULL, L.tp[a], src);
+                    N.nv[a] = __shfl_sync(FULL, L.nv[a], src);
+                }
+                N.dist = __shfl_sync(FULL, L.dist, src);
+                N.dist_prev = __shfl_sync(FULL, L.dist_prev, src);
+                N.dn = __shfl_sync(FULL, L.dn, src);
+                N.nrm = __shfl_sync(FULL, L.nrm, src);
+                L = N;
+                if (!has) L.b = -1;
+                if (has && s2 >= G && L.phase == 2) start_trial(L.bt + s2);  // src is the leader: its bt is the base
+                G = Gn;
+                sub = s2;
+            }
+        }
+        // one point evaluation per running lane, and its normal step
+        bool on = false, ended = false;
+        double nrm = 0.0, nv[3] = {0.0, 0.0, 0.0};
         const bool trial = L.phase == 2;
-        double p[3];
+        if (L.b >= 0 && (!trial || L.st == TRIAL_RUN)) {
+            ++L.ev;
+            double p[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) p[a] = trial ? L.yn[a] : L.y[a];
-        double ph, g[3];
-        q1_lerp(e, p, ph, g);
-        ph = clampd(ph, -PHI_CLAMP, PHI_CLAMP);
-        const double r = eps * log((1.0 + ph) / (1.0 - ph)) - d_t;
-        const double nrm = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
-        const double inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
-        const double nv[3] = {g[0] * inv, g[1] * inv, g[2] * inv};
-        const bool on = fabs(r) <= tol * h;
-        const int max_steps = trial ? CPP_TRIAL_STEPS : CPP_NORMAL_STEPS;
-        const bool can_step = !on && L.steps < max_steps && nrm > 0.0;
-        if (L.phase != 1 && can_step) {  // normal step of the point being projected
-            const double step = r * (1.0 - ph * ph) * inv * c_step;
+            for (int a = 0; a < 3; ++a) p[a] = trial ? L.yn[a] : L.y[a];
+            double ph, g[3];
+            q1_lerp(e, p, ph, g);
+            ph = clampd(ph, -PHI_CLAMP, PHI_CLAMP);
+            const double r = eps * log((1.0 + ph) / (1.0 - ph)) - d_t;
+            nrm = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
+            const double inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
 #pragma unroll
-            for (int a = 0; a < 3; ++a) p[a] = clampd(p[a] - step * nv[a], 0.0, nn);
-            ++L.steps;
+            for (int a = 0; a < 3; ++a) nv[a] = g[a] * inv;
+            on = fabs(r) <= tol_h;
+            if (!on && L.steps < (trial ? CPP_TRIAL_STEPS : CPP_NORMAL_STEPS) && nrm > 0.0) {
+                const double step = r * (1.0 - ph * ph) * inv * c_step;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    p[a] = clamp_range(p[a] - step * nv[a], nn);
+                    if (trial) L.yn[a] = p[a];
+                    else L.y[a] = p[a];
+                }
+                ++L.steps;
+            } else {
+                ended = true;
+            }
+        }
+        __syncwarp();
+        if (!__any_sync(FULL, ended)) continue;
+        // a projection ended in some lane: its distance and normal, kept until the group decides
+        bool tangent = false;
+        if (ended) {
+            L.nrm = nrm;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) L.nv[a] = nv[a];
+            if (trial) {
+                L.dn = dist3(L.yn, L.x);
+                L.st = on && L.dn < L.dist ? TRIAL_OK : TRIAL_FAIL;
+            }
+        }
+        // the group's trials in the order of their lengths: the first that did not fail decides
+        const int base = lane - sub;
+        const unsigned gm = (1u << G) - 1u;
+        const bool in2 = L.b >= 0 && trial;
+        const unsigned failed = (__ballot_sync(FULL, in2 && (L.st == TRIAL_FAIL || L.st == TRIAL_IDLE)) >> base) & gm;
+        const unsigned okay = (__ballot_sync(FULL, in2 && L.st == TRIAL_OK) >> base) & gm;
+        const int first = __ffs(~failed) - 1;
+        const bool accept = in2 && first < G && ((okay >> first) & 1u);
+        const bool none = in2 && first >= G;
+        if (G == 1) {
+            if (accept || none) L.trips += L.ev;
+        } else if (__any_sync(FULL, accept || none)) {
+            // the accepted point with its distance and normal to all lanes of the group; the evaluations up to it
+            int ev = (accept && sub <= first) || none ? L.ev : 0;
+            for (int o = 1; o < G; o <<= 1) ev += __shfl_xor_sync(FULL, ev, o);
+            const int src = accept ? base + first : lane;
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                if (trial) L.yn[a] = p[a];
-                else L.y[a] = p[a];
+                L.yn[a] = __shfl_sync(FULL, L.yn[a], src);
+                L.nv[a] = __shfl_sync(FULL, L.nv[a], src);
             }
-            continue;
+            L.dn = __shfl_sync(FULL, L.dn, src);
+            L.nrm = __shfl_sync(FULL, L.nrm, src);
+            if (accept || none) L.trips += ev;
         }
-        if (L.phase == 0) {  // projection of the node ended
+        if (ended && !trial) {  // projection of the node
+            L.trips += L.ev;
             if (on) {
                 L.dist = dist3(L.y, L.x);
                 L.k = 0;
                 if (kmax <= 0) finish(false);
-                else L.phase = 1;
+                else tangent = true;
             } else {
                 finish(false);
             }
-        } else if (L.phase == 1) {  // tangential part of y - x at y, first trial point
+        } else if (accept) {
+            L.dist = L.dn;
+            const double step = dist3(L.yn, L.y);
+            const double gain = L.dist_prev - L.dist;
+            L.y[0] = L.yn[0]; L.y[1] = L.yn[1]; L.y[2] = L.yn[2];
+            if (step <= tol || gain <= CPP_STALL * L.dist) finish(true);
+            else if (++L.k == kmax) finish(false);
+            else tangent = true;
+        } else if (none) {
+            if (L.bt - sub + G >= CPP_BACKTRACK) finish(true);  // no shorter point on the isocontour
+            else start_trial(L.bt + G);
+        }
+        if (tangent) {  // tangential part of y - x at y, first trial points
+            ++L.trips;
+            const double n0 = L.nv[0], n1 = L.nv[1], n2 = L.nv[2];
             L.tp[0] = L.tp[1] = L.tp[2] = 0.0;
-            if (nrm > 0.0) {
-                const bool alt = fabs(nv[0]) > 0.9;  // v = e_y instead of e_x
-                const double vn = alt ? nv[1] : nv[0];
-                double t0[3] = {(alt ? 0.0 : 1.0) - vn * nv[0], (alt ? 1.0 : 0.0) - vn * nv[1], -vn * nv[2]};
+            if (L.nrm > 0.0) {
+                const bool alt = fabs(n0) > 0.9;  // v = e_y instead of e_x
+                const double vn = alt ? n1 : n0;
+                double t0[3] = {(alt ? 0.0 : 1.0) - vn * n0, (alt ? 1.0 : 0.0) - vn * n1, -vn * n2};
                 const double t0n = sqrt(t0[0] * t0[0] + t0[1] * t0[1] + t0[2] * t0[2]);
                 if (t0n > 0.0) {
                     const double it = 1.0 / t0n;
                     t0[0] *= it; t0[1] *= it; t0[2] *= it;
                 }
-                const double t1[3] = {nv[1] * t0[2] - nv[2] * t0[1], nv[2] * t0[0] - nv[0] * t0[2],
-                                      nv[0] * t0[1] - nv[1] * t0[0]};
+                const double t1[3] = {n1 * t0[2] - n2 * t0[1], n2 * t0[0] - n0 * t0[2], n0 * t0[1] - n1 * t0[0]};
                 const double dl[3] = {L.y[0] - L.x[0], L.y[1] - L.x[1], L.y[2] - L.x[2]};
                 const double a0 = dl[0] * t0[0] + dl[1] * t0[1] + dl[2] * t0[2];
                 const double a1 = dl[0] * t1[0] + dl[1] * t1[1] + dl[2] * t1[2];
 #pragma unroll
                 for (int a = 0; a < 3; ++a) L.tp[a] = a0 * t0[a] + a1 * t1[a];
             }
-            L.omega = 1.0;
-            L.bt = 0;
             L.dist_prev = L.dist;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) L.yn[a] = clampd(L.y[a] - L.omega * L.tp[a], 0.0, nn);
-            L.steps = 0;
             L.phase = 2;
-        } else {  // projection of the trial point ended: on the isocontour (on) or failed
-            const double dn = dist3(L.yn, L.x);
-            if (on && dn < L.dist) {  // accepted
-                L.dist = dn;
-                const double step = dist3(L.yn, L.y);
-                const double gain = L.dist_prev - L.dist;
-                L.y[0] = L.yn[0]; L.y[1] = L.yn[1]; L.y[2] = L.yn[2];
-                if (step <= tol || gain <= CPP_STALL * L.dist) finish(true);
-                else if (++L.k == kmax) finish(false);
-                else L.phase = 1;
-            } else if (++L.bt == CPP_BACKTRACK) {  // no shorter point on the isocontour
-                finish(true);
-            } else {
-                L.omega *= 0.5;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) L.yn[a] = clampd(L.y[a] - L.omega * L.tp[a], 0.0, nn);
-                L.steps = 0;
-            }
+            start_trial(sub);
         }
+        __syncwarp();
     }
 }
 
@@ -520,7 +627,11 @@ __global__ void k_transport_band_finish(PointEval e, const double* __restrict__ 
     const double rho_t = e.m.variant == 2 ? e.m.rho_l : e.m.rho_g;
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < count; b += gridDim.x * blockDim.x) {
         const double y[3] = {band_y[3 * (int64_t)b], band_y[3 * (int64_t)b + 1], band_y[3 * (int64_t)b + 2]};
-        transport_finish(e, mdot, band[b], y, rho_t, ug);
+        const unsigned m1 = (unsigned)e.m.n + 1u, nd = (unsigned)band[b], t = nd / m1;
+        const int i = (int)(nd - t * m1), k = (int)(t / m1), j = (int)(t - (unsigned)k * m1);
+        double uv[3];
+        e.velocity(y, uv);
+        transport_store(e, mdot, band[b], i, j, k, uv, rho_t, ug);
     }
 }
 
@@ -557,6 +668,7 @@ int launch_closest_points(evap_mesh* h, double* y, cudaStream_t s) {
     return EVAP_OK;
 }
 
+constexpr int CPP_WARPS = 6 * 152;  // 6 one-warp blocks per SM
 int launch_transport_velocity(evap_mesh* h, cudaStream_t s, const double* phi) {
     PointEval e;
     e.phi = phi ? phi : h->phi;
@@ -578,14 +690,15 @@ int launch_transport_velocity(evap_mesh* h, cudaStream_t s, const double* phi) {
                                                                             h->band_list, h->band_count);
     EVAP_CHECK_LAUNCH("transport_direct");
     if (h->m.variant != 1) {
-        // Persistent pass sized to about 2 band nodes per lane (lanes that finish early take the remaining entries,
-        // so warps stay full until the tail), at most 8 warps per SM: the FP64 pipe, not occupancy, bounds it.
-        // Measured on the 64^3 four-sphere band (49 k nodes): 2 nodes per lane 3.9 ms, 4 nodes 5.0 ms, 1 node 4.3 ms;
-        // on the 128^3 deformed sphere (181 k nodes, capped at 8 warps per SM) 9.6 ms, and 10.6 ms at 16 warps.
+        // Persistent pass of at most 6 warps per SM, each with an even share of a shorter list.  Measured (us per
+        // transport pass; sphere 33^3 with 13 k band nodes / four drops 64^3, 41 k / slab 64^3, 38 k / deformed 128^3,
+        // 181 k / sphere 48^3 with n_sub = 2, 198 k): 3 warps 1256 / 2588 / 304 / 7958 / 9117; 4 1231 / 2152 / 260 /
+        // 6336 / 7253; 6 1047 / 1960 / 267 / 5523 / 6334; 8 1156 / 2003 / 245 / 5518 / 6301; 16 1472 / 2639 / 292 /
+        // 5801 / 6581.  Before the lane groups (one lane per node to the end): 2970 / 3559 / 477 / 9290 / 9139.
         int32_t count = 0;
         EVAP_CUDA(cudaMemcpyAsync(&count, h->band_count, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
         EVAP_CUDA(cudaStreamSynchronize(s));
-        const int grid = (int)std::min<int64_t>(std::max<int64_t>(((int64_t)count + 63) / 64, 1), 152 * 8);
+        const int grid = (int)std::min<int64_t>(std::max<int64_t>(count, 1), CPP_WARPS);
         k_transport_band<<<grid, 32, 0, s>>>(e, h->prm.cpp_tol, h->prm.cpp_kmax, h->band_list, h->band_count,
                                              h->band_y, h->cpp_flags, h->flag_count, h->cpp_evals);
         EVAP_CHECK_LAUNCH("transport_band");
