@@ -20,27 +20,30 @@
 #include <algorithm>
 
 #include "async_copy.cuh"
-#include "dfloat.cuh"
+#include "df_lines.cuh"
 #include "physics.cuh"
 
 namespace evap {
 
-__device__ __forceinline__ bool cons_node(int gx, int gy, int gz, int M, unsigned f) {
-    return ((f & 1u) && gx == 0) || ((f & 2u) && gx == M - 1) || ((f & 4u) && gy == 0) ||
-           ((f & 8u) && gy == M - 1) || ((f & 16u) && gz == 0) || ((f & 32u) && gz == M - 1);
-}
-
-__global__ void k_adjoint_init(int M, int64_t Nu, int64_t Np, unsigned faces, const double* __restrict__ w,
-                               double* gx, double* gu, double* gphi, double* gm) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 3 * Nu; i += stride) {
-        if (gx) {
-            const int64_t node = i % Nu;
-            const int a = (int)(node % M), b = (int)((node / M) % M), c = (int)(node / ((int64_t)M * M));
-            gx[i] = cons_node(a, b, c, M, faces) ? w[i] : 0.0;
+// g_x = w on the Dirichlet DoFs and 0 elsewhere, g_u0 = g_phi = g_mdot = 0: a warp walks whole x-lines of nodes, so the
+// line's position is split once per warp.
+__global__ void __launch_bounds__(256) k_adjoint_init(int M, int64_t Nu, int64_t Np, unsigned faces,
+                                                      const double* __restrict__ w, double* gx, double* gu,
+                                                      double* gphi, double* gm) {
+    const int lines = 3 * M * M;
+    const int wpb = blockDim.x / 32, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    for (int line = blockIdx.x * wpb + warp; line < lines; line += gridDim.x * wpb) {
+        const int c = line / (M * M), rem = line - c * M * M, gz = rem / M, gy = rem - gz * M;
+        const bool cyz = ((faces & 4u) && gy == 0) || ((faces & 8u) && gy == M - 1) || ((faces & 16u) && gz == 0) ||
+                         ((faces & 32u) && gz == M - 1);
+        const int64_t off = c * Nu + (int64_t)M * (gy + (int64_t)M * gz);
+        for (int i = lane; i < M; i += 32) {
+            if (gx)
+                gx[off + i] = cyz || ((faces & 1u) && i == 0) || ((faces & 2u) && i == M - 1) ? w[off + i] : 0.0;
+            if (gu) gu[off + i] = 0.0;
         }
-        if (gu) gu[i] = 0.0;
     }
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < Np; i += stride) {
         if (gphi) gphi[i] = 0.0;
         if (gm) gm[i] = 0.0;
@@ -51,71 +54,66 @@ __global__ void k_adjoint_init(int M, int64_t Nu, int64_t Np, unsigned faces, co
 // The interpolation of x and w, the value / gradient sensitivities and their testing run in double-float arithmetic
 // (dfloat.cuh) on the FP32 pipe, with the coefficients of the double-float cache (the pairs of the FP64 values the
 // forward apply uses); so do the material-law sensitivities of the interface-zone points, with the factors of the
-// adjoint table.  The level-set test sweeps run in FP64 (only table cells carry them: blocks without a table cell skip
-// the sweeps).
-// Block shape for Q2 on the velocity mesh's level set: CB cells per block, at least MINB blocks per SM (a register
-// cap).  Measured at 64^3 on GB300 (20 back-to-back adjoints, ms), with the zone sensitivities from the adjoint
-// table: CB 7 / MINB 3 (96 registers, some spills) 1.962; 8 / 2 2.126; 7 / 2 2.150; 6 / 3 2.241; 4 / 4 2.301; with
-// the cached coefficients copied into shared memory by cp.async during the interpolation sweeps, 7 / 3 1.853; with
-// the lazy normalization below, 7 / 3 1.836, 8 / 2 1.974, 7 / 2 1.978.
-// Before the table (zone work in FP64): 7 / 3 2.995; 8 / 2 3.158; 7 / 2 3.261; 4 / 4 3.403; 4 / 3 3.526.
-// Normalization as in the forward double-float apply: the gradients at the points, the value sensitivities that
-// start the test sums and the last transposed sweep (converted to FP64 next) are left unnormalized (0: normalize).
-// Measured at 64^3: 1.856 -> 1.831 ms, the smoke case's gradients still within 5e-15 of the oracle's.
-#ifndef EVAP_ADJ_LAZY
-#define EVAP_ADJ_LAZY 1
-#endif
-template <int Q>
-__device__ __forceinline__ dfl adj_dot_lazy(const dfl* c, const dfl* v, int stride) {
-#if EVAP_ADJ_LAZY
-    dfl s = df_prod(c[0], v[0]);
-#pragma unroll
-    for (int k = 1; k < Q; ++k) df_fma(s, c[k], v[k * stride]);
-    return s;
-#else
-    return df_dot<Q>(c, v, stride);
-#endif
-}
-
+// adjoint table.  The level-set test sweeps run in FP64, in the table cells only.
+// Layout: as the forward apply (momentum_df.cu), sweeps by lines (df_lines.cuh; the 6 Q^2 lines of the six fields x and
+// w, two rounds over a cell's Q^3 threads) and the sensitivities by one thread per quadrature point, which overwrites
+// its own point's values and gradients with them.  Only the threads of table cells run the interface-zone work and the
+// level-set sweeps.  At most 48 KB of shared memory per block, so no launch needs a function attribute.
+// Measured at 48^3 Q2 (us; one point per thread with Q-term dot products 775 to 800): cells per block / blocks per SM 4 / 5
+// 632 (96 registers); 7 / 3 631; 2 / 10 651; 4 / 6 655; 1 / 20 669; 5 / 4 671; 3 / 7 673; 4 / 4 684.
+// Normalization as in the forward apply: the gradients at the points, the value sensitivities that start the test sums
+// and the last transposed sweep (converted to FP64 next) are left unnormalized.
 #ifndef EVAP_ADJ_CB2
-#define EVAP_ADJ_CB2 7
+#define EVAP_ADJ_CB2 4
 #endif
 #ifndef EVAP_ADJ_MINB2
-#define EVAP_ADJ_MINB2 3
+#define EVAP_ADJ_MINB2 5
+#endif
+#ifndef EVAP_ADJ_CB3
+#define EVAP_ADJ_CB3 1
+#endif
+#ifndef EVAP_ADJ_MINB3
+#define EVAP_ADJ_MINB3 6
 #endif
 
-template <int P, int CB, int K, int MINB = 2>
+// slots of a cell in shared memory (pairs of Q^3 points): 0..5 X, Om (then the value sensitivities of x and u0), 6..23
+// the gradients 6 + 3 f + d of field f (then the gradient sensitivities of x and u0), 24..38 the cached coefficients
+// 0..13 and 17 (then the tests along y and z, 12 slots); then the level-set sensitivities, 5 doubles per point
+constexpr int ADJ_SLOTS = 24, ADJ_COEF = 15;
+template <int P, int CB>
+constexpr size_t adj_smem() {
+    return sizeof(float2) * CB * (ADJ_SLOTS + ADJ_COEF + 5) * (P + 1) * (P + 1) * (P + 1);
+}
+
+template <int P, int CB, int K, int MINB>
 __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
-    k_adjoint(MeshArgs<double> m, DfBasis dfb, Basis<double> bas, dfl rho_liq, dfl rho_gas,
+    k_adjoint(MeshArgs<double> m, Basis<double> bas, dfl rho_liq, dfl rho_gas, dfl kap,
               const int8_t* __restrict__ code, const int32_t* __restrict__ tindex, const float2* __restrict__ adjt,
               const float2* __restrict__ qcd, const double* __restrict__ w,
               const double* __restrict__ wp, const double* __restrict__ x, double* gx, double* gu, double* gphi,
               double* gm, int colour) {
-    constexpr int Q = P + 1, NQ = Q * Q * Q;
+    constexpr int Q = P + 1, NQ = Q * Q * Q, NL = Q * Q, TASKS = 6 * NL;
+    using Ln = DfLine<Q>;
     static_assert(K * Q * Q <= NQ && K * K * K <= NQ, "one thread per entry of each level-set test sweep");
-    __shared__ dfl sS[Q][Q], sDc[Q][Q];
     __shared__ double sNL[Q][K], sDL[Q][K];
-    __shared__ dfl buf[2][CB][12][NQ];
     __shared__ double q1a[CB][5][K * Q * Q], q1b[CB][5][K * K * Q];  // level-set test sweeps (FP64)
-    extern __shared__ float2 sqc[];  // [cell][QC_K][point]: this block's cached coefficients, copied during the sweeps
+    extern __shared__ float2 smem_adj[];
+    constexpr int CELL = (ADJ_SLOTS + ADJ_COEF + 5) * NQ;
     const int tid = threadIdx.x;
     const int lc = tid / NQ, t = tid % NQ;
-    int cx = 0, cy = 0, cz = 0;
-    const bool active = colour_cell((int64_t)blockIdx.x * CB + lc, m.n, colour, cx, cy, cz);
+    dfl* const cb = reinterpret_cast<dfl*>(smem_adj) + lc * CELL;
+    int cx, cy, cz;
+    const bool active = colour_cell32(blockIdx.x * CB + lc, m.n, colour, cx, cy, cz);
     const int64_t cell = cx + (int64_t)m.n * (cy + (int64_t)m.n * cz);
     const bool plain = colour >= 0;  // a colour pass: no other cell of the launch touches this cell's nodes
-    float2* myq = sqc + (int64_t)lc * QC_K * NQ + t;
-    if (active) {  // each thread fetches (and later reads) only its own point's coefficients: 0..3, 13, 17, newton 4..12
+    {  // each thread fetches (and later reads) only its own point's coefficients: 0..3, 13, 17, newton 4..12
+        dfl* myq = cb + ADJ_SLOTS * NQ + t;
         const float2* src = qcd + cell * QC_K * NQ + t;
 #pragma unroll
-        for (int k = 0; k < QC_K; ++k)
-            if (k < 4 || k == 13 || k == 17 || (m.newton && k <= 12)) cp_async8(myq + k * NQ, src + k * NQ);
+        for (int k = 0; k < ADJ_COEF; ++k)
+            if (k < 4 || k > 12 || m.newton) cp_async8(myq + k * NQ, src + (k == 14 ? 17 : k) * NQ);
     }
     cp_async_commit();
-    if (tid < Q * Q) {
-        sS[tid / Q][tid % Q] = dfb.S[tid / Q][tid % Q];
-        sDc[tid / Q][tid % Q] = dfb.Dc[tid / Q][tid % Q];
-    }
     if (tid < K * Q) {
         sNL[tid / K][tid % K] = bas.NL[tid / K][tid % K];
         sDL[tid / K][tid % K] = bas.DL[tid / K][tid % K];
@@ -124,81 +122,82 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
     const int n = m.n, M = m.M;
     const int64_t m1 = n + 1;     // pressure nodes per axis (w_p)
     const int64_t ml = m.nl + 1;  // level-set nodes per axis
-    int64_t gidx = 0;
-    bool cons = false, tcell = false;
-    if (active) {
-        const int gxi = P * cx + a, gyi = P * cy + b, gzi = P * cz + c;
-        gidx = gxi + (int64_t)M * (gyi + (int64_t)M * gzi);
-        cons = cons_node(gxi, gyi, gzi, M, m.faces);
-        tcell = code[cell] == CELL_TABLE;
+    const bool tcell = code[cell] == CELL_TABLE;
+    // z-line l of a cell: offset of its first node in a component, and which of its nodes are constrained (bit k)
+    const int64_t zst = (int64_t)M * M;
+    auto zline = [&](int l, unsigned& cons) -> int64_t {
+        const int gxi = P * cx + l % Q, gyi = P * cy + l / Q, gz0 = P * cz;
+        const unsigned fc = m.faces;
+        cons = ((fc & 1u) && gxi == 0) || ((fc & 2u) && gxi == M - 1) || ((fc & 4u) && gyi == 0) ||
+                       ((fc & 8u) && gyi == M - 1)
+                   ? (1u << Q) - 1u
+                   : 0u;
+        if ((fc & 16u) && gz0 == 0) cons |= 1u;
+        if ((fc & 32u) && gz0 + P == M - 1) cons |= 1u << P;
+        return gxi + (int64_t)M * gyi + zst * gz0;
+    };
+    // values at the points: the lines along z (from memory), y and x, then the derivatives along the three directions
+    for (int k0 = t; k0 < TASKS; k0 += NQ) {
+        const int f = k0 / NL, l = k0 % NL;
+        unsigned cons;
+        const double* src = (f < 3 ? x : w) + (f < 3 ? f : f - 3) * m.Nu + zline(l, cons);
+        dfl u[Q], v[Q];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            buf[0][lc][k][t] = cons ? dfl{0.f, 0.f} : df_from_double(x[k * m.Nu + gidx]);
-            buf[0][lc][3 + k][t] = cons ? dfl{0.f, 0.f} : df_from_double(w[k * m.Nu + gidx]);
-        }
-    }
-    // whether any cell of the block carries level-set sensitivities (a table cell)
-    const bool block_table = __syncthreads_or(tcell) != 0;
-    if (active) {
-        dfl Sa[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Sa[k] = sS[a][k];
-#pragma unroll
-        for (int f = 0; f < 6; ++f) buf[1][lc][f][t] = df_dot<Q>(Sa, &buf[0][lc][f][Q * (b + Q * c)], 1);
-    }
-    __syncthreads();
-    if (active) {
-        dfl Sb[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Sb[k] = sS[b][k];
-#pragma unroll
-        for (int f = 0; f < 6; ++f) buf[0][lc][f][t] = df_dot<Q>(Sb, &buf[1][lc][f][a + Q * Q * c], Q);
+        for (int k = 0; k < Q; ++k) u[k] = (cons >> k) & 1u ? dfl{0.f, 0.f} : df_from_double(src[k * zst]);
+        Ln::val(u, v);
+        st_line<Q, 2>(cb + (6 + f) * NQ, l, v);
     }
     __syncthreads();
-    if (active) {
-        dfl Sc[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Sc[k] = sS[c][k];
-#pragma unroll
-        for (int f = 0; f < 6; ++f) buf[1][lc][f][t] = df_dot<Q>(Sc, &buf[0][lc][f][a + Q * b], Q * Q);
+    for (int k0 = t; k0 < TASKS; k0 += NQ) {
+        const int f = k0 / NL, l = k0 % NL;
+        dfl u[Q], v[Q];
+        ld_line<Q, 1>(cb + (6 + f) * NQ, l, u);
+        Ln::val(u, v);
+        st_line<Q, 1>(cb + (12 + f) * NQ, l, v);
     }
     __syncthreads();
-    dfl gxv[3], guv[3], gxg[3][3], gug[3][3];
+    for (int k0 = t; k0 < TASKS; k0 += NQ) {
+        const int f = k0 / NL, l = k0 % NL;
+        dfl u[Q], v[Q];
+        ld_line<Q, 0>(cb + (12 + f) * NQ, l, u);
+        Ln::val(u, v);
+        st_line<Q, 0>(cb + f * NQ, l, v);
+    }
+    __syncthreads();
+    for (int k0 = t; k0 < TASKS; k0 += NQ) {
+        const int f = k0 / NL, l = k0 % NL;
+        dfl u[Q], v[Q];
+        ld_line<Q, 0>(cb + f * NQ, l, u);
+        Ln::der(u, v);
+        st_line<Q, 0>(cb + (6 + 3 * f) * NQ, l, v);
+        ld_line<Q, 1>(cb + f * NQ, l, u);
+        Ln::der(u, v);
+        st_line<Q, 1>(cb + (7 + 3 * f) * NQ, l, v);
+        ld_line<Q, 2>(cb + f * NQ, l, u);
+        Ln::der(u, v);
+        st_line<Q, 2>(cb + (8 + 3 * f) * NQ, l, v);
+    }
+    __syncthreads();
     double dphi = 0.0, dg[3] = {0, 0, 0}, dm = 0.0;
-    if (active) {
-        dfl V[6], Gr[6][3];
-        {
-            dfl Da[Q], Db[Q], Dz[Q];
-#pragma unroll
-            for (int k = 0; k < Q; ++k) {
-                Da[k] = sDc[a][k];
-                Db[k] = sDc[b][k];
-                Dz[k] = sDc[c][k];
-            }
-#pragma unroll
-            for (int f = 0; f < 6; ++f) {
-                V[f] = buf[1][lc][f][t];
-                Gr[f][0] = adj_dot_lazy<Q>(Da, &buf[1][lc][f][Q * (b + Q * c)], 1);
-                Gr[f][1] = adj_dot_lazy<Q>(Db, &buf[1][lc][f][a + Q * Q * c], Q);
-                Gr[f][2] = adj_dot_lazy<Q>(Dz, &buf[1][lc][f][a + Q * b], Q * Q);
-            }
-        }
-        const dfl* X = &V[0];
-        const dfl* Om = &V[3];
-        dfl (*G)[3] = &Gr[0];
-        dfl (*OmG)[3] = &Gr[3];
-        // cached coefficients (k_qp_coeffs): 0 W rho c_m, 1..3 W rho u0, 4..12 newton W rho grad u0, 13 2 W mu, 17 W
+    {
+        // values and gradients of x (X, G) and w (Om, OmG) at this thread's point, in units of kappa, read where they
+        // are used: the sensitivities are formed in an order that lets them replace their inputs
+        const dfl* pt = cb + t;
+        auto X = [pt](int k) { return pt[k * NQ]; };
+        auto Om = [pt](int k) { return pt[(3 + k) * NQ]; };
+        auto G = [pt](int k, int d) { return pt[(6 + 3 * k + d) * NQ]; };
+        auto OmG = [pt](int k, int d) { return pt[(15 + 3 * k + d) * NQ]; };
         cp_async_wait_all();
-        const float2* qp = myq;
-        const dfl W = ld_df(qp + 17 * NQ);
+        const dfl* qp = cb + ADJ_SLOTS * NQ + t;
+        const dfl W = qp[14 * NQ], Wk = df_mul(W, kap);
         // this point's entries of the adjoint table (table cells only; k_fill_table)
         const float2* ap = tcell ? adjt + (int64_t)tindex[cell] * ADJ_K * NQ + t : nullptr;
         const dfl rho = tcell ? ld_df(ap + ADJ_RHO * NQ) : (code[cell] == CELL_LIQUID ? rho_liq : rho_gas);
-        const dfl wr = df_mul(W, rho);  // the W rho of the forward apply
-        // w_p (pressure space, Q1 on the cell) and the level set (its own mesh; only in table cells) at the point
-        const double tx = bas.t[a], ty = bas.t[b], tz = bas.t[c];
+        const dfl wr = df_mul(Wk, rho);
+        // w_p (pressure space, Q1 on the cell) at the point
         double pi = 0;
         if (wp) {  // trilinear interpolation by successive linear interpolation (14 FP64 operations, not 40)
+            const double tx = bas.t[a], ty = bas.t[b], tz = bas.t[c];
             const double* w0 = wp + cx + m1 * (cy + m1 * cz);
             double e[2][2];
 #pragma unroll
@@ -214,44 +213,22 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         // the phi / mdot sensitivities and the normal are needed only in the interface zone (or with the correction
         // applied everywhere), which lies in table cells; elsewhere H is 0 or 1 and its derivatives vanish
         const bool full = tcell && (ap[ADJ_ZONE * NQ].x != 0.f || (m.stress != 0 && m.corr_zone != 0));
-        const dfl wm = ld_df(qp + 13 * NQ);
-        const dfl hwm = df_scale2(wm, 0.5f);
-        const dfl Wpi = df_mul(W, df_from_double(pi));
-        // value / gradient sensitivities of the velocity block and of B^T w_p (the correction term added below)
-        const dfl c0 = ld_df(qp);
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            dfl v = df_prod(c0, Om[d]);
-            if (m.newton) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) df_fma(v, Om[k], ld_df(qp + (4 + 3 * k + d) * NQ));
-            }
-            gxv[d] = EVAP_ADJ_LAZY ? v : df_norm(v);
-            dfl u = df_prod(Om[0], G[0][d]);
-            df_fma(u, Om[1], G[1][d]);
-            df_fma(u, Om[2], G[2][d]);
-            guv[d] = df_mul(wr, df_norm(u));
-#pragma unroll
-            for (int e = 0; e < 3; ++e) {
-                dfl g = df_prod(Om[d], ld_df(qp + (1 + e) * NQ));
-                df_fma(g, hwm, df_add(OmG[d][e], OmG[e][d]));
-                gxg[d][e] = d == e ? df_add(df_norm(g), Wpi) : df_norm(g);
-                gug[d][e] = m.newton ? df_mul(wr, df_mul(Om[d], X[e])) : dfl{0.f, 0.f};
-            }
-        }
+        const dfl wm = qp[13 * NQ];
+        const dfl pid = df_from_double(pi), Wkpi = df_mul(Wk, pid);
+        dfl corr{0.f, 0.f};
         if (full) {  // material-law sensitivities (interface-zone points only), double-float arithmetic
             const dfl nv[3] = {ld_df(ap + (ADJ_N + 0) * NQ), ld_df(ap + (ADJ_N + 1) * NQ), ld_df(ap + (ADJ_N + 2) * NQ)};
             const bool zg = ap[ADJ_ZG * NQ].x != 0.f;
-            const dfl tr = df_add(df_add(G[0][0], G[1][1]), G[2][2]);
+            const dfl tr = df_add(df_add(G(0, 0), G(1, 1)), G(2, 2));
             // OmG n, OmG^T n and n . OmG n
             dfl on[3], otn[3];
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                dfl u = df_prod(OmG[i][0], nv[0]), v = df_prod(OmG[0][i], nv[0]);
+                dfl u = df_prod(OmG(i, 0), nv[0]), v = df_prod(OmG(0, i), nv[0]);
 #pragma unroll
                 for (int j = 1; j < 3; ++j) {
-                    df_fma(u, OmG[i][j], nv[j]);
-                    df_fma(v, OmG[j][i], nv[j]);
+                    df_fma(u, OmG(i, j), nv[j]);
+                    df_fma(v, OmG(j, i), nv[j]);
                 }
                 on[i] = df_norm(u);
                 otn[i] = df_norm(v);
@@ -260,40 +237,35 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
             df_fma(nOn, nv[1], on[1]);
             df_fma(nOn, nv[2], on[2]);
             nOn = df_norm(nOn);
-            if (zg) {  // the corrected strain's term of g_x
-                const dfl corr = df_mul(wm, nOn);
-#pragma unroll
-                for (int d = 0; d < 3; ++d) gxg[d][d] = df_sub(gxg[d][d], corr);
-            }
+            if (zg) corr = df_mul(wm, nOn);  // the corrected strain's term of g_x
             // dL/drho = W Om . (c_m X + G u0 + newton grad u0 X) = (1/rho) sum_k Om_k (cached W rho terms)_k
-            const dfl U[3] = {ld_df(qp + 1 * NQ), ld_df(qp + 2 * NQ), ld_df(qp + 3 * NQ)};
             dfl sr{0.f, 0.f};
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                dfl f = df_prod(c0, X[k]);
+                dfl f = df_prod(qp[0], X(k));
 #pragma unroll
-                for (int b2 = 0; b2 < 3; ++b2) df_fma(f, U[b2], G[k][b2]);
+                for (int b2 = 0; b2 < 3; ++b2) df_fma(f, qp[(1 + b2) * NQ], G(k, b2));
                 if (m.newton) {
 #pragma unroll
-                    for (int d = 0; d < 3; ++d) df_fma(f, ld_df(qp + (4 + 3 * k + d) * NQ), X[d]);
+                    for (int d = 0; d < 3; ++d) df_fma(f, qp[(4 + 3 * k + d) * NQ], X(d));
                 }
                 if (k == 0)
-                    sr = df_prod(Om[0], df_norm(f));
+                    sr = df_prod(Om(0), df_norm(f));
                 else
-                    df_fma(sr, Om[k], df_norm(f));
+                    df_fma(sr, Om(k), df_norm(f));
             }
             const dfl dL_drho = df_mul(ld_df(ap + ADJ_IRHO * NQ), df_norm(sr));
             // dL/dmu = 2 W (OmG : sym G - z tr(G) n . OmG n)
-            dfl smu = df_prod(OmG[0][0], G[0][0]);
-            df_fma(smu, OmG[1][1], G[1][1]);
-            df_fma(smu, OmG[2][2], G[2][2]);
+            dfl smu = df_prod(OmG(0, 0), G(0, 0));
+            df_fma(smu, OmG(1, 1), G(1, 1));
+            df_fma(smu, OmG(2, 2), G(2, 2));
 #pragma unroll
             for (int k = 0; k < 3; ++k)
 #pragma unroll
                 for (int l = k + 1; l < 3; ++l)
-                    df_fma(smu, df_add(OmG[k][l], OmG[l][k]), df_scale2(df_add(G[k][l], G[l][k]), 0.5f));
+                    df_fma(smu, df_add(OmG(k, l), OmG(l, k)), df_scale2(df_add(G(k, l), G(l, k)), 0.5f));
             if (zg) df_fma(smu, df_neg(tr), nOn);
-            const dfl dL_dmu = df_mul(df_scale2(W, 2.0f), df_norm(smu));
+            const dfl dL_dmu = df_mul(df_mul(df_scale2(Wk, 2.0f), kap), df_norm(smu));
             // dL/dn = -2 W mu z tr(G) (OmG + OmG^T) n; its part normal to n drops out (dn/dgrad phi)
             dfl dLdn[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
             if (zg) {
@@ -316,7 +288,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
                 dgv[i] = df_mul(df_norm(u), ign);
             }
             if (wp) {  // through v_dil = mdot c_1 delta (Eq. evaporDil), dL/dv_dil = -W pi
-                const dfl dLdv = df_neg(Wpi);
+                const dfl dLdv = df_neg(df_mul(W, pid));
                 dm = df_to_double(df_mul(dLdv, ld_df(ap + ADJ_KD1 * NQ)));
                 df_fma(dp, dLdv, ld_df(ap + ADJ_KD2 * NQ));
                 const dfl k3 = df_mul(dLdv, ld_df(ap + ADJ_KD3 * NQ));
@@ -327,83 +299,107 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
 #pragma unroll
             for (int i = 0; i < 3; ++i) dg[i] = df_to_double(dgv[i]);
         }
-    }
-    __syncthreads();
-    // level-set sensitivities (FP64) in the slots 6..10 of buf[1], stored as doubles (8 bytes like a dfl)
-    auto lsv = [&](int f, int pt) -> double& { return *reinterpret_cast<double*>(&buf[1][lc][6 + f][pt]); };
-    if (active) {
-        for (int s = 0; s < 9; ++s) buf[0][lc][s][t] = gxg[s / 3][s % 3];
-        for (int s = 0; s < 3; ++s) buf[0][lc][9 + s][t] = gug[0][s];
-        for (int s = 0; s < 6; ++s) buf[1][lc][s][t] = gug[1 + s / 3][s % 3];
-        lsv(0, t) = dphi;
-        lsv(1, t) = dg[0];
-        lsv(2, t) = dg[1];
-        lsv(3, t) = dg[2];
-        lsv(4, t) = dm;
-    }
-    __syncthreads();
-    dfl tx3[3], tu3[3];
-    if (active) {
-        dfl Ea[Q], Eb[Q], Ec[Q];
+        // value / gradient sensitivities of the velocity block and of B^T w_p, over the point's own entries: with X and
+        // Om in registers, those of u0 from G (3..5), of x (0..2), the gradients of x from OmG (over G), then of u0
+        const dfl xq[3] = {X(0), X(1), X(2)}, om[3] = {Om(0), Om(1), Om(2)};
+        dfl* const out = cb + t;
 #pragma unroll
-        for (int k = 0; k < Q; ++k) {
-            Ea[k] = sDc[k][a];
-            Eb[k] = sDc[k][b];
-            Ec[k] = sDc[k][c];
+        for (int d = 0; d < 3; ++d) {
+            dfl u = df_prod(om[0], G(0, d));
+            df_fma(u, om[1], G(1, d));
+            df_fma(u, om[2], G(2, d));
+            out[(3 + d) * NQ] = df_mul(wr, df_norm(u));
+            dfl v = df_prod(qp[0], om[d]);
+            if (m.newton) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) df_fma(v, om[k], qp[(4 + 3 * k + d) * NQ]);
+            }
+            out[d * NQ] = v;
         }
+        const dfl hwm = df_scale2(wm, 0.5f);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int ib = 3 * k;      // gxg[k][*] slots in buf[0]
-            const int iu = 9 + 3 * k;  // gug[k][*] slots: 9..17 over buf[0][9..11], buf[1][0..5]
-            dfl s = gxv[k], u = guv[k];
+        for (int d = 0; d < 3; ++d)
 #pragma unroll
-            for (int r = 0; r < Q; ++r) {
-                const int p0 = r + Q * (b + Q * c), p1 = a + Q * (r + Q * c), p2 = a + Q * (b + Q * r);
-                df_fma(s, Ea[r], buf[0][lc][ib + 0][p0]);
-                df_fma(s, Eb[r], buf[0][lc][ib + 1][p1]);
-                df_fma(s, Ec[r], buf[0][lc][ib + 2][p2]);
-                if (m.newton) {
-                    const int j0 = iu + 0, j1 = iu + 1, j2 = iu + 2;
-                    df_fma(u, Ea[r], j0 < 12 ? buf[0][lc][j0][p0] : buf[1][lc][j0 - 12][p0]);
-                    df_fma(u, Eb[r], j1 < 12 ? buf[0][lc][j1][p1] : buf[1][lc][j1 - 12][p1]);
-                    df_fma(u, Ec[r], j2 < 12 ? buf[0][lc][j2][p2] : buf[1][lc][j2 - 12][p2]);
+            for (int e = 0; e < 3; ++e) {
+                dfl g = df_prod(om[d], qp[(1 + e) * NQ]);
+                df_fma(g, hwm, df_add(OmG(d, e), OmG(e, d)));
+                dfl r = df_norm(g);
+                if (d == e) {
+                    r = df_add(r, Wkpi);
+                    if (full) r = df_sub(r, corr);
                 }
+                out[(6 + 3 * d + e) * NQ] = r;
             }
-            tx3[k] = df_norm(s);
-            tu3[k] = df_norm(u);
+        if (m.newton) {
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+#pragma unroll
+                for (int e = 0; e < 3; ++e) out[(15 + 3 * d + e) * NQ] = df_mul(wr, df_mul(om[d], xq[e]));
         }
-        // level-set sensitivities: g_phi[j] = sum_q N_j dL/dphi + grad N_j . dL/dgrad phi, g_mdot[j] = sum_q N_j
-        // dL/dmdot with the level-set shape functions N_j of the cell (K per direction), by three sweeps; field f:
-        // 0 dL/dphi, 1..3 dL/dgrad phi (x, y, z), 4 dL/dmdot.  Along direction d the 1D factor is the reference
-        // derivative DL for field 1 + d, NL otherwise.  x-sweep: [jx][qy][qz].
-        if (block_table && t < K * Q * Q) {
-            const int jx = t % K, qy = (t / K) % Q, qz = (t / K) / Q;
+    }
+    double* const lsv = reinterpret_cast<double*>(cb + (ADJ_SLOTS + ADJ_COEF) * NQ);  // [5][point]
+    if (tcell) {
+        lsv[t] = dphi;
+        lsv[NQ + t] = dg[0];
+        lsv[2 * NQ + t] = dg[1];
+        lsv[3 * NQ + t] = dg[2];
+        lsv[4 * NQ + t] = dm;
+    }
+    __syncthreads();
+    // test with gradients: the lines along y and z into the coefficients' slots (u0: only with the Newton term)
+    const int gtasks = m.newton ? TASKS : TASKS / 2;
+    for (int k0 = t; k0 < gtasks; k0 += NQ) {
+        const int f = k0 / NL, l = k0 % NL;
+        dfl u[Q], v[Q];
+        ld_line<Q, 1>(cb + (7 + 3 * f) * NQ, l, u);
+        Ln::derT(u, v);
+        st_line<Q, 1>(cb + (ADJ_SLOTS + f) * NQ, l, v);
+        ld_line<Q, 2>(cb + (8 + 3 * f) * NQ, l, u);
+        Ln::derT(u, v);
+        st_line<Q, 2>(cb + (ADJ_SLOTS + 6 + f) * NQ, l, v);
+    }
+    // level-set sensitivities: g_phi[j] = sum_q N_j dL/dphi + grad N_j . dL/dgrad phi, g_mdot[j] = sum_q N_j
+    // dL/dmdot with the level-set shape functions N_j of the cell (K per direction), by three sweeps; field f:
+    // 0 dL/dphi, 1..3 dL/dgrad phi (x, y, z), 4 dL/dmdot.  Along direction d the 1D factor is the reference
+    // derivative DL for field 1 + d, NL otherwise.  x-sweep: [jx][qy][qz].
+    if (tcell && t < K * Q * Q) {
+        const int jx = t % K, qy = (t / K) % Q, qz = (t / K) / Q;
 #pragma unroll
-            for (int f = 0; f < 5; ++f) {
-                double sacc = 0.0;
+        for (int f = 0; f < 5; ++f) {
+            double sacc = 0.0;
 #pragma unroll
-                for (int q = 0; q < Q; ++q) sacc += (f == 1 ? sDL[q][jx] : sNL[q][jx]) * lsv(f, q + Q * (qy + Q * qz));
-                q1a[lc][f][t] = sacc;
-            }
+            for (int q = 0; q < Q; ++q)
+                sacc += (f == 1 ? sDL[q][jx] : sNL[q][jx]) * lsv[f * NQ + q + Q * (qy + Q * qz)];
+            q1a[lc][f][t] = sacc;
         }
     }
     __syncthreads();
-    if (active) {
+    for (int k0 = t; k0 < TASKS; k0 += NQ) {  // x: values + the three tests, and their value sweep
+        const int f = k0 / NL, l = k0 % NL;
+        dfl u[Q], v[Q], s[Q];
+        ld_line<Q, 0>(cb + f * NQ, l, s);
+        if (f < 3 || m.newton) {
+            ld_line<Q, 0>(cb + (6 + 3 * f) * NQ, l, u);
+            Ln::derT(u, v);
+            ld_line<Q, 0>(cb + (ADJ_SLOTS + f) * NQ, l, u);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            buf[0][lc][k][t] = tx3[k];
-            buf[0][lc][3 + k][t] = tu3[k];
+            for (int k = 0; k < Q; ++k) s[k] = df_addl(df_addl(s[k], v[k]), u[k]);
+            ld_line<Q, 0>(cb + (ADJ_SLOTS + 6 + f) * NQ, l, u);
+#pragma unroll
+            for (int k = 0; k < Q; ++k) s[k] = df_add(s[k], u[k]);
         }
-        if (block_table && t < K * K * Q) {  // y-sweep: [jx][jy][qz]
-            const int jx = t % K, jy = (t / K) % K, qz = t / (K * K);
+        Ln::template valT<false>(s, v);
+        st_line<Q, 0>(cb + f * NQ, l, v);
+    }
+    if (tcell && t < K * K * Q) {  // y-sweep: [jx][jy][qz]
+        const int jx = t % K, jy = (t / K) % K, qz = t / (K * K);
 #pragma unroll
-            for (int f = 0; f < 5; ++f) {
-                double sacc = 0.0;
+        for (int f = 0; f < 5; ++f) {
+            double sacc = 0.0;
 #pragma unroll
-                for (int q = 0; q < Q; ++q)
-                    sacc += (f == 2 ? sDL[q][jy] : sNL[q][jy]) * q1a[lc][f][jx + K * (q + Q * qz)];
-                q1b[lc][f][t] = sacc;
-            }
+            for (int q = 0; q < Q; ++q)
+                sacc += (f == 2 ? sDL[q][jy] : sNL[q][jy]) * q1a[lc][f][jx + K * (q + Q * qz)];
+            q1b[lc][f][t] = sacc;
         }
     }
     __syncthreads();
@@ -422,70 +418,60 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         if (gphi) acc_add(&gphi[nd], r[0] + m.inv_h * (r[1] + r[2] + r[3]), plain);
         if (gm) acc_add(&gm[nd], r[4], plain);
     }
-    // transposed sweeps S^T of the 6 value fields (g_x, g_u0): z, y, x
-    if (active) {
-        dfl Tc[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Tc[k] = sS[k][c];
-#pragma unroll
-        for (int f = 0; f < 6; ++f) buf[1][lc][f][t] = df_dot<Q>(Tc, &buf[0][lc][f][a + Q * b], Q * Q);
+    for (int k0 = t; k0 < TASKS; k0 += NQ) {
+        const int f = k0 / NL, l = k0 % NL;
+        dfl u[Q], v[Q];
+        ld_line<Q, 1>(cb + f * NQ, l, u);
+        Ln::template valT<false>(u, v);
+        st_line<Q, 1>(cb + f * NQ, l, v);
     }
     __syncthreads();
-    if (active) {
-        dfl Tb[Q];
+    if (!active) return;
+    for (int k0 = t; k0 < TASKS; k0 += NQ) {  // z, and the scatter
+        const int f = k0 / NL, l = k0 % NL;
+        double* const out = f < 3 ? gx : gu;
+        if (!out) continue;
+        unsigned cons;
+        double* dst = out + (f < 3 ? f : f - 3) * m.Nu + zline(l, cons);
+        if (f >= 3) cons = 0u;
+        dfl u[Q], v[Q];
+        ld_line<Q, 2>(cb + f * NQ, l, u);
+        Ln::template valT<true>(u, v);
 #pragma unroll
-        for (int k = 0; k < Q; ++k) Tb[k] = sS[k][b];
-#pragma unroll
-        for (int f = 0; f < 6; ++f) buf[0][lc][f][t] = df_dot<Q>(Tb, &buf[1][lc][f][a + Q * Q * c], Q);
-    }
-    __syncthreads();
-    if (active) {
-        dfl Ta[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Ta[k] = sS[k][a];
-#pragma unroll
-        for (int f = 0; f < 6; ++f) {
-            const double s = df_to_double(adj_dot_lazy<Q>(Ta, &buf[0][lc][f][Q * (b + Q * c)], 1));
-            if (f < 3) {
-                if (gx && !cons) acc_add(&gx[f * m.Nu + gidx], s, plain);
-            } else if (gu) {
-                acc_add(&gu[(f - 3) * m.Nu + gidx], s, plain);
-            }
-        }
+        for (int k = 0; k < Q; ++k)
+            if (!((cons >> k) & 1u)) acc_add(&dst[k * zst], df_to_double(v[k]), plain);
     }
 }
 
 int launch_adjoint(evap_mesh* h, const double* w, const double* wp, const double* x, double* gx, double* gu,
                    double* gphi, double* gm, cudaStream_t s) {
     const MeshArgs<double>& m = h->m;
-    k_adjoint_init<<<blocks_for(3 * m.Nu, 256), 256, 0, s>>>(m.M, m.Nu, m.Nphi, m.faces, w, gx, gu, gphi, gm);  // level set
+    const unsigned gi = (unsigned)std::min<int64_t>((3 * (int64_t)m.M * m.M + 7) / 8, 152 * 16);
+    k_adjoint_init<<<gi, 256, 0, s>>>(m.M, m.Nu, m.Nphi, m.faces, w, gx, gu, gphi, gm);
     EVAP_CHECK_LAUNCH("adjoint_init");
-    const DfBasis dfb = make_df_basis(h->b, m.inv_h);
+    const dfl kap = df_from_double(df_kappa(m));
     const float2* qcd = reinterpret_cast<const float2*>(h->qcdf);
     const dfl rho_liq = df_from_double(m.rho_H1), rho_gas = df_from_double(m.rho_H0);  // rho outside table cells
     const int c0 = h->deterministic ? 0 : -1, c1 = h->deterministic ? 8 : 0;  // colour passes, or one atomic pass
-    auto run = [&](auto kern, int CB, int threads) -> int {
-        const size_t dyn = sizeof(float2) * QC_K * threads;  // the block's cached coefficients (threads = CB NQ)
-        EVAP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
-        EVAP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                       (int)cudaSharedmemCarveoutMaxShared));
+    auto run = [&](auto kern, int CB, int threads, size_t dyn) -> int {
         for (int colour = c0; colour < std::max(c1, c0 + 1); ++colour) {
             const int64_t cells = colour_cells(m.n, colour);
             if (cells == 0) continue;
-            kern<<<(unsigned)((cells + CB - 1) / CB), threads, dyn, s>>>(m, dfb, h->b, rho_liq, rho_gas, h->cell_code,
+            kern<<<(unsigned)((cells + CB - 1) / CB), threads, dyn, s>>>(m, h->b, rho_liq, rho_gas, kap, h->cell_code,
                                                                        h->table_index, h->adj_table, qcd, w, wp, x,
                                                                        gx, gu, gphi, gm, colour);
             EVAP_CHECK_LAUNCH("adjoint");
         }
         return EVAP_OK;
     };
-    constexpr int CA = EVAP_ADJ_CB2, MA = EVAP_ADJ_MINB2;
-    if (m.P == 2 && m.nsub == 1)  // 7 cells: 189 threads, 98 % of the lanes of 6 warps
-        return run(k_adjoint<2, CA, 2, MA>, CA, CA * 27);
-    if (m.P == 2)  // the subdivided level set's larger test-sweep buffers (static shared memory <= 48 KB)
-        return run(k_adjoint<2, 6, 3>, 6, 6 * 27);
-    if (m.nsub == 1) return run(k_adjoint<3, 2, 2>, 2, 2 * 64);
-    return run(k_adjoint<3, 2, 3>, 2, 2 * 64);
+    if (m.P == 2) {
+        constexpr int CB = EVAP_ADJ_CB2, MB = EVAP_ADJ_MINB2;
+        return m.nsub == 1 ? run(k_adjoint<2, CB, 2, MB>, CB, CB * 27, adj_smem<2, CB>())
+                           : run(k_adjoint<2, CB, 3, MB>, CB, CB * 27, adj_smem<2, CB>());
+    }
+    constexpr int CB = EVAP_ADJ_CB3, MB = EVAP_ADJ_MINB3;
+    return m.nsub == 1 ? run(k_adjoint<3, CB, 2, MB>, CB, CB * 64, adj_smem<3, CB>())
+                       : run(k_adjoint<3, CB, 3, MB>, CB, CB * 64, adj_smem<3, CB>());
 }
 
 }  // namespace evap

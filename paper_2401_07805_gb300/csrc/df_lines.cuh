@@ -1,0 +1,177 @@
+// Sweeps of the double-float operators along one line of Q = P + 1 points, in double-float arithmetic (dfloat.cuh).
+//
+// Support points (Gauss-Lobatto) and quadrature points (Gauss-Legendre) are symmetric about 1/2, so a line's even and
+// odd parts are transformed apart (the even-odd decomposition of tensor-product elements), and for Q = 3 the
+// interpolation of a quadratic c(t) = c_1 + (t - 1/2) dm + 2 (t - 1/2)^2 C with dm = c_2 - c_0, C = c_0 - 2 c_1 + c_2
+// needs only two multiplications: by tau = sqrt(3/20), the distance of the outer Gauss points from 1/2, and by
+// 2 tau^2 = 3/10.  FP32 instructions per line of 3 results: 80 (values), 60 (derivatives), against 93 for three
+// 3-term dot products each (df_dot), with a third of their shared-memory loads, since one thread forms a whole line.
+//
+//   val   y_q = sum_a S[q][a] u_a           valT  o_a = sum_q S[q][a] f_q
+//   der   d_q = sum_r D[q][r] y_r           derT  o_r = sum_q D[q][r] t_q,   D = (collocation derivative) / DSCALE:
+// the derivative at the Gauss points up to the factor DSCALE (1 / (2 tau) for Q = 3, where D holds the integers
+// -3, 4, -1 / -1, 0, 1 / 1, -4, 3; 1 for Q = 4); the factor and 1/h are part of the cached coefficients.
+#pragma once
+
+#include "dfloat.cuh"
+
+namespace evap {
+
+constexpr float dfk_hi(double v) { return (float)v; }
+constexpr float dfk_lo(double v) { return (float)(v - (double)(float)v); }
+#define EVAP_DFK(v) (dfl{dfk_hi(v), dfk_lo(v)})
+
+// a + b without the closing normalization (|lo| may reach a few ulp(hi)): for sums that are added further
+__device__ __forceinline__ dfl df_addl(dfl a, dfl b) {
+    dfl s = two_sum(a.hi, b.hi);
+    s.lo = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
+    return s;
+}
+__device__ __forceinline__ dfl df_twice(dfl a) { return {a.hi + a.hi, a.lo + a.lo}; }
+__device__ __forceinline__ dfl df_half(dfl a) { return {0.5f * a.hi, 0.5f * a.lo}; }
+
+// Which sums are normalized: results stored for the next sweep (df_addo) and sums multiplied next (df_addi); sums that are
+// added further are not.  Measured at 64^3 Q2 (us per apply, error against 64 bits; 1.12e-14 with Q-term dot products):
+// both 552, 1.10e-14; only the multiplied ones 540, 1.14e-14; only the stored ones 540, 1.11e-14 (5.25e-15 at 8^3, 5.21e-15
+// before); none 529, 1.17e-14.  Both are, so that no case loses accuracy.
+__device__ __forceinline__ dfl df_addo(dfl a, dfl b) { return df_add(a, b); }
+__device__ __forceinline__ dfl df_addi(dfl a, dfl b) { return df_add(a, b); }
+
+template <int Q>
+struct DfLine;
+
+template <>
+struct DfLine<3> {
+    static constexpr double TAU = 0.5 * 0.7745966692414833770358531;  // sqrt(3/5) / 2
+    static constexpr double DSCALE = 1.0 / (2.0 * TAU);
+    static __device__ __forceinline__ void val(const dfl u[3], dfl y[3]) {
+        const dfl dm = df_addi(u[2], df_neg(u[0]));
+        const dfl C = df_addi(df_addl(u[0], u[2]), df_neg(df_twice(u[1])));
+        const dfl base = df_addl(u[1], df_mul(C, EVAP_DFK(0.3)));
+        const dfl m = df_mul(dm, EVAP_DFK(TAU));
+        y[0] = df_addo(base, df_neg(m));
+        y[1] = u[1];
+        y[2] = df_addo(base, m);
+    }
+    template <bool FINAL>  // FINAL: the results are converted next
+    static __device__ __forceinline__ void valT(const dfl f[3], dfl o[3]) {
+        const dfl s = df_addi(f[0], f[2]), d = df_addi(f[0], df_neg(f[2]));
+        const dfl p = df_mul(s, EVAP_DFK(0.3)), r = df_mul(d, EVAP_DFK(TAU));
+        const dfl s1 = df_addl(s, f[1]), p2 = df_neg(df_twice(p));
+        o[0] = FINAL ? df_addl(p, r) : df_addo(p, r);
+        o[1] = FINAL ? df_addl(s1, p2) : df_addo(s1, p2);
+        o[2] = FINAL ? df_addl(p, df_neg(r)) : df_addo(p, df_neg(r));
+    }
+    static __device__ __forceinline__ void der(const dfl y[3], dfl d[3]) {
+        const dfl A = df_addl(y[1], df_neg(y[0])), B = df_addl(y[2], df_neg(y[1]));
+        const dfl D = df_addl(A, df_neg(B));
+        d[0] = df_addl(D, df_twice(A));
+        d[1] = df_addl(A, B);
+        d[2] = df_addl(df_twice(B), df_neg(D));
+    }
+    static __device__ __forceinline__ void derT(const dfl t[3], dfl o[3]) {
+        const dfl a = df_addl(t[0], df_neg(t[2]));
+        o[0] = df_neg(df_addl(df_addl(t[1], df_twice(t[0])), a));
+        o[1] = df_twice(df_twice(a));
+        o[2] = df_addl(df_addl(t[1], df_twice(t[2])), df_neg(a));
+    }
+};
+
+template <>
+struct DfLine<4> {
+    static constexpr double DSCALE = 1.0;
+    // even parts: sum over a pair of symmetric points; odd parts: difference.  A row q of S acts on the even part
+    // (e0, e1) as e1 / 2 + al (e0 - e1) (its entries sum to 1) and on the odd part (o0, o1) by (ga, de).
+    static constexpr CtBasis<3> B = make_ct_basis<3>();
+    static constexpr double al(int q) { return 0.5 * (B.S[q][0] + B.S[q][3]); }
+    static constexpr double ga(int q) { return 0.5 * (B.S[q][0] - B.S[q][3]); }
+    static constexpr double de(int q) { return 0.5 * (B.S[q][1] - B.S[q][2]); }
+    // a row q of the derivative: eta (e0 - e1) from the even part (its entries sum to 0), (xa, xb) on the odd part
+    static constexpr double eta(int q) { return 0.5 * (B.Dc[q][0] + B.Dc[q][3]); }
+    static constexpr double xa(int q) { return 0.5 * (B.Dc[q][0] - B.Dc[q][3]); }
+    static constexpr double xb(int q) { return 0.5 * (B.Dc[q][1] - B.Dc[q][2]); }
+    static __device__ __forceinline__ dfl dot2(dfl c0, dfl v0, dfl c1, dfl v1) {
+        dfl s = df_prod(c0, v0);
+        df_fma(s, c1, v1);
+        return s;
+    }
+    template <int q>
+    static __device__ __forceinline__ void val_pair(dfl e1h, dfl f, dfl o0, dfl o1, dfl y[4]) {
+        constexpr double a_ = al(q), g_ = ga(q), d_ = de(q);
+        dfl E = e1h;
+        df_fma(E, EVAP_DFK(a_), f);
+        const dfl O = dot2(EVAP_DFK(g_), o0, EVAP_DFK(d_), o1);
+        y[q] = df_addo(E, O);
+        y[3 - q] = df_addo(E, df_neg(O));
+    }
+    static __device__ __forceinline__ void val(const dfl u[4], dfl y[4]) {
+        const dfl e0 = df_addl(u[0], u[3]), e1 = df_addl(u[1], u[2]);
+        const dfl o0 = df_addi(u[0], df_neg(u[3])), o1 = df_addi(u[1], df_neg(u[2]));
+        const dfl f = df_addi(e0, df_neg(e1));
+        val_pair<0>(df_half(e1), f, o0, o1, y);
+        val_pair<1>(df_half(e1), f, o0, o1, y);
+    }
+    template <bool FINAL>
+    static __device__ __forceinline__ void valT(const dfl t[4], dfl o[4]) {
+        const dfl s0 = df_addi(t[0], t[3]), s1 = df_addi(t[1], t[2]);
+        const dfl d0 = df_addi(t[0], df_neg(t[3])), d1 = df_addi(t[1], df_neg(t[2]));
+        constexpr double a0 = al(0), a1 = al(1), g0 = ga(0), g1 = ga(1), e0 = de(0), e1 = de(1);
+        const dfl ev = dot2(EVAP_DFK(a0), s0, EVAP_DFK(a1), s1);               // even result of the outer pair
+        const dfl ei = df_addl(df_half(df_addl(s0, s1)), df_neg(ev));           // and of the inner one
+        const dfl od = dot2(EVAP_DFK(g0), d0, EVAP_DFK(g1), d1), oi = dot2(EVAP_DFK(e0), d0, EVAP_DFK(e1), d1);
+        o[0] = FINAL ? df_addl(ev, od) : df_addo(ev, od);
+        o[3] = FINAL ? df_addl(ev, df_neg(od)) : df_addo(ev, df_neg(od));
+        o[1] = FINAL ? df_addl(ei, oi) : df_addo(ei, oi);
+        o[2] = FINAL ? df_addl(ei, df_neg(oi)) : df_addo(ei, df_neg(oi));
+    }
+    static __device__ __forceinline__ void der(const dfl y[4], dfl d[4]) {
+        const dfl o0 = df_addi(y[0], df_neg(y[3])), o1 = df_addi(y[1], df_neg(y[2]));
+        const dfl f = df_addi(df_addl(y[0], y[3]), df_neg(df_addl(y[1], y[2])));
+        constexpr double h0 = eta(0), h1 = eta(1), a0 = xa(0), a1 = xa(1), b0 = xb(0), b1 = xb(1);
+        const dfl v0 = df_mul(EVAP_DFK(h0), f), v1 = df_mul(EVAP_DFK(h1), f);
+        const dfl w0 = dot2(EVAP_DFK(a0), o0, EVAP_DFK(b0), o1), w1 = dot2(EVAP_DFK(a1), o0, EVAP_DFK(b1), o1);
+        d[0] = df_addl(w0, v0);
+        d[3] = df_addl(w0, df_neg(v0));
+        d[1] = df_addl(w1, v1);
+        d[2] = df_addl(w1, df_neg(v1));
+    }
+    static __device__ __forceinline__ void derT(const dfl t[4], dfl o[4]) {
+        const dfl s0 = df_addi(t[0], t[3]), s1 = df_addi(t[1], t[2]);  // act on the odd part
+        const dfl d0 = df_addi(t[0], df_neg(t[3])), d1 = df_addi(t[1], df_neg(t[2]));
+        constexpr double h0 = eta(0), h1 = eta(1), a0 = xa(0), a1 = xa(1), b0 = xb(0), b1 = xb(1);
+        const dfl ev = dot2(EVAP_DFK(h0), d0, EVAP_DFK(h1), d1);  // even result, + on the outer and - on the inner pair
+        const dfl oo = dot2(EVAP_DFK(a0), s0, EVAP_DFK(a1), s1), oi = dot2(EVAP_DFK(b0), s0, EVAP_DFK(b1), s1);
+        o[0] = df_addl(ev, oo);
+        o[3] = df_addl(ev, df_neg(oo));
+        o[1] = df_addl(df_neg(ev), oi);
+        o[2] = df_neg(df_addl(ev, oi));
+    }
+};
+
+// kappa = DSCALE / h: physical gradient = kappa (D y)
+inline double df_kappa(const MeshArgs<double>& m) {
+    return (m.P == 2 ? DfLine<3>::DSCALE : DfLine<4>::DSCALE) * m.inv_h;
+}
+
+// Line `l` (of Q^2) of direction DIR (0 x, 1 y, 2 z) in a cell's Q^3 points, x fastest: first point and stride.
+template <int Q, int DIR>
+struct LineAt {
+    static constexpr int stride = DIR == 0 ? 1 : (DIR == 1 ? Q : Q * Q);
+    static __device__ __forceinline__ int first(int l) {
+        return DIR == 0 ? Q * l : (DIR == 1 ? l % Q + Q * Q * (l / Q) : l);
+    }
+};
+template <int Q, int DIR>
+__device__ __forceinline__ void ld_line(const dfl* cell, int l, dfl v[Q]) {
+    const int p0 = LineAt<Q, DIR>::first(l);
+#pragma unroll
+    for (int k = 0; k < Q; ++k) v[k] = cell[p0 + k * LineAt<Q, DIR>::stride];
+}
+template <int Q, int DIR>
+__device__ __forceinline__ void st_line(dfl* cell, int l, const dfl v[Q]) {
+    const int p0 = LineAt<Q, DIR>::first(l);
+#pragma unroll
+    for (int k = 0; k < Q; ++k) cell[p0 + k * LineAt<Q, DIR>::stride] = v[k];
+}
+
+}  // namespace evap

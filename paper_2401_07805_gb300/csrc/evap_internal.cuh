@@ -86,6 +86,20 @@ __device__ __forceinline__ bool colour_cell(int64_t idx, int n, int colour, int&
     cz = 2 * (int)(idx / ((int64_t)hx * hy)) + pz;
     return true;
 }
+// The same with 32-bit arithmetic (a mesh has at most 1024^3 cells), for kernels whose blocks take whole groups of
+// cells: an index past the end gives the last cell and false, so that its threads can run along without branches.
+__device__ __forceinline__ bool colour_cell32(unsigned idx, int n, int colour, int& cx, int& cy, int& cz) {
+    const unsigned px = colour < 0 ? 0u : (unsigned)colour & 1u, py = colour < 0 ? 0u : ((unsigned)colour >> 1) & 1u,
+                   pz = colour < 0 ? 0u : (unsigned)colour >> 2, sh = colour < 0 ? 0u : 1u;
+    const unsigned hx = ((unsigned)n - px + sh) >> sh, hy = ((unsigned)n - py + sh) >> sh, hz = ((unsigned)n - pz + sh) >> sh;
+    const unsigned total = hx * hy * hz;
+    const bool in = idx < total;
+    const unsigned i = in ? idx : total - 1u, r = i / hx, k = r / hy;
+    cx = (int)(((i - r * hx) << sh) + px);
+    cy = (int)(((r - k * hy) << sh) + py);
+    cz = (int)((k << sh) + pz);
+    return in;
+}
 // y += v: a plain read-modify-write inside a colour pass, else an atomic add
 template <typename T>
 __device__ __forceinline__ void acc_add(T* y, T v, bool plain) {

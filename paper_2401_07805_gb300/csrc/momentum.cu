@@ -9,7 +9,7 @@
 //                     arithmetic, not HBM, bounds these operators, and the material law and the u0 interpolation
 //                     would otherwise be recomputed by every apply
 //   launch_momentum   dispatch: FP64 -> double-float kernel, FP32 -> line kernel; the lifting variant (all columns)
-#include "dfloat.cuh"
+#include "df_lines.cuh"
 #include "physics.cuh"
 
 namespace evap {
@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256) k_momentum_init(int M, int64_t Nu, unsign
 // double-float results are the pairs of the apply's cache as they stand; the FP64 copy is their sum (within 2^-48).
 template <int P, int CB>
 __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
-    k_qp_coeffs(MeshArgs<double> m, Basis<double> bas, DfBasis dfb, dfl cm_df, dfl invh_df,
+    k_qp_coeffs(MeshArgs<double> m, Basis<double> bas, DfBasis dfb, dfl cm_df, dfl invh_df, dfl kap, dfl kap2,
                 const int8_t* __restrict__ code, const int32_t* __restrict__ tindex, const double* __restrict__ table,
                 const double* __restrict__ u0, double* __restrict__ qc, float2* __restrict__ qcdf,
                 float* __restrict__ qc32) {
@@ -150,7 +150,8 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
 #pragma unroll
     for (int k = 0; k < QC_K; ++k) {
         qc[base + (int64_t)k * NQ] = df_to_double(v[k]);
-        qcdf[base + (int64_t)k * NQ] = make_float2(v[k].hi, v[k].lo);
+        const dfl w = k >= 1 && k <= 3 ? df_mul(v[k], kap) : (k == 13 ? df_mul(v[k], kap2) : v[k]);
+        qcdf[base + (int64_t)k * NQ] = make_float2(w.hi, w.lo);
     }
     const int64_t row = cell / n;
     const int cx = (int)(cell - row * n);
@@ -188,14 +189,16 @@ int launch_qp_coeffs(evap_mesh* h, cudaStream_t s) {
     }
     const DfBasis dfb = make_df_basis(h->b, m.inv_h);
     const dfl cm = df_from_double(m.c_mass), ih = df_from_double(m.inv_h);
+    const double kd = df_kappa(m);
+    const dfl kap = df_from_double(kd), kap2 = df_from_double(kd * kd);
     if (m.P == 2) {
         constexpr int CB = 8;
         k_qp_coeffs<2, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 27, 0, s>>>(
-            m, h->b, dfb, cm, ih, h->cell_code, h->table_index, h->table, h->u, h->qc, (float2*)h->qcdf, h->qc32);
+            m, h->b, dfb, cm, ih, kap, kap2, h->cell_code, h->table_index, h->table, h->u, h->qc, (float2*)h->qcdf, h->qc32);
     } else {
         constexpr int CB = 4;
         k_qp_coeffs<3, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 64, 0, s>>>(
-            m, h->b, dfb, cm, ih, h->cell_code, h->table_index, h->table, h->u, h->qc, (float2*)h->qcdf, h->qc32);
+            m, h->b, dfb, cm, ih, kap, kap2, h->cell_code, h->table_index, h->table, h->u, h->qc, (float2*)h->qcdf, h->qc32);
     }
     EVAP_CHECK_LAUNCH("qp_coeffs");
     return EVAP_OK;

@@ -15,157 +15,156 @@
 // the same Gauss sums at ~48-bit precision (relative rounding ~4e-15 per operation, below the 1e-12 parity bar by
 // two orders of magnitude) leave the FP64 pipe with only the conversions of the nodal values (x in, y out).
 //
-// Layout: one thread per quadrature point, CB cells per block, sweeps through shared
-// memory; the thread keeps its rows of the 1D matrices (S, the physical collocation derivative Dc/h, their
-// transposes) in registers as double-float constants.  The quadrature-point coefficients are the FP64 values of
-// k_qp_coeffs split into double-float pairs (qcdf, [cell][QC_K][nq] float2, written by the same kernel), 8 bytes per
-// coefficient as in FP64; each thread copies its point's coefficients into shared memory with cp.async at the start,
-// so that their HBM latency is hidden behind the interpolation sweeps (without it, waits on these loads were the top
-// stall).  The correction term is skipped at points where its
-// gate z n is zero (outside the interface zone), and the Newton terms on Picard meshes.
+// Layout: CB cells per block with Q^3 threads each.  In a sweep a thread owns one line of Q points of one component
+// (Q^2 lines x 3 components: every thread for Q = 3, 48 of 64 for Q = 4) and forms its Q results in registers with the
+// even-odd line transforms of df_lines.cuh, so a sweep costs Q shared loads and Q stores per thread; the fluxes are
+// formed by one thread per quadrature point.  The first sweep (z) gathers its lines from memory and the last one (z)
+// scatters its own, both as rows of x-consecutive nodes.  The lines of the test along y and z overlay the coefficient
+// slots, which the fluxes have read by then.
+// What bounds it: FP32 issue (the additions of the error-free transformations).
+//
+// The quadrature-point coefficients are the pairs of k_qp_coeffs (qcdf, [cell][QC_K][nq] float2), 8 bytes per
+// coefficient as in FP64, with the factor kappa = DSCALE / h of the derivative in the slots that multiply one (1..3)
+// and kappa^2 in the viscous one (13).  Each thread copies its point's coefficients into shared memory with
+// cp.async at the start, so that their HBM latency is hidden behind the interpolation sweeps.  The correction term is
+// skipped at points where its gate z n is zero (outside the interface zone), and the Newton terms on Picard meshes.
 #include <algorithm>
 
 #include "async_copy.cuh"
-#include "dfloat.cuh"
+#include "df_lines.cuh"
 #include "physics.cuh"
 
 namespace evap {
 
+// slots of a cell in shared memory (pairs of Q^3 points): 0..2 X (then F), 3..11 G_kd at 3 + 3 k + d (then the six
+// stress entries at 3.., the divergence row at 9), 12.. the coefficients (then the tests along y and z, 6 slots)
+constexpr int DF_SLOTS = 12;
 template <int P, int CB>
-constexpr size_t df_coeff_smem() {
-    return sizeof(float2) * CB * QC_K * (P + 1) * (P + 1) * (P + 1);
+constexpr size_t df_smem() {
+    return sizeof(float2) * CB * (DF_SLOTS + QC_K) * (P + 1) * (P + 1) * (P + 1);
+}
+// slot of the symmetric stress entry (k, l)
+__device__ __forceinline__ constexpr int t_slot(int k, int l) {
+    return 3 + (k <= l ? (k * (5 - k)) / 2 + l : (l * (5 - l)) / 2 + k);
 }
 
-// Block shape for Q2: CB cells per block (one thread per point), at least MINB blocks per SM (which caps the
-// registers).  Measured at 64^3 on GB300, 100 back-to-back applies with the divergence row (ms per apply):
-// CB 4 / MINB 8 (64 registers) 0.685; CB 4 / 6 0.699; CB 8 / 4 0.700; CB 8 without a minimum (72 registers) 0.691;
-// CB 8 / 3 0.722; CB 4 / 1 (89 registers) 0.738; CB 8 / 1 0.848; CB 12 / 1 1.207.  Single- and two-warp blocks,
-// on another box against CB 4 / 8 at 0.691 there: CB 1 / 28 (72 registers) 0.695, CB 1 / 20 0.728, CB 2 / 14 0.709,
-// CB 3 / 10 0.720.
+// Cells per block and blocks per SM (a register cap).  Measured at 64^3 Q2 with the divergence row (us per apply; one
+// point per thread with Q-term dot products: 673): CB 1 / 28 blocks 503 (a block is one warp, so that the barriers of
+// the sweeps cost nothing); 2 / 16 526; 4 / 8 510; 5 / 6 552; 7 / 4 592; 8 / 4 581; 13 / 2 757.  Q3 at 45^3 (701
+// before): 2 and 4 cells 576.  ncu at 64^3, CB 4: 1842 warp instructions per cell (1064 FADD, 194 FMUL and FFMA, 142
+// shared accesses), issue 77 % active, FP64 pipe 59 % (conversions).
 #ifndef EVAP_DF_CB2
-#define EVAP_DF_CB2 4
+#define EVAP_DF_CB2 1
 #endif
 #ifndef EVAP_DF_MINB2
-#define EVAP_DF_MINB2 8
+#define EVAP_DF_MINB2 28
 #endif
-#ifndef EVAP_DF_MINB2_PRES
-#define EVAP_DF_MINB2_PRES 8
+#ifndef EVAP_DF_CB3
+#define EVAP_DF_CB3 2
 #endif
-
-// Normalization of the sweep results (the closing Fast2Sum of each dot product).  A result that is converted to FP64
-// next (the last transposed sweep) or that only starts a new accumulation (the value flux F, whose hi and lo enter
-// the test sum through TwoSum) loses nothing when left unnormalized (hi + lo stays exact).  A result that is then
-// multiplied carries its larger lo part into the rounded cross terms.  EVAP_DF_LAZY: 0 normalize all; 3 skip only the
-// free cases; 2 also the gradients; 1 every sweep result.  Measured at 64^3 (ms per apply; relative error of the
-// smoke case against the oracle): 0 0.6925, 4.8e-15; 3 0.6812, 5.7e-15; 2 0.6767, 5.7e-15; 1 0.6639, 8.9e-15, and
-// with 1 the coupled step's velocity-pressure solve no longer reaches its 1e-10 (its rounding floor rises to 1.2e-10).
-#ifndef EVAP_DF_LAZY
-#define EVAP_DF_LAZY 2
+#ifndef EVAP_DF_MINB3
+#define EVAP_DF_MINB3 4
 #endif
-template <int Q, bool LAZY>
-__device__ __forceinline__ dfl df_dot_lz(const dfl* c, const dfl* v, int stride) {
-    if constexpr (LAZY) {
-        dfl s = df_prod(c[0], v[0]);
-#pragma unroll
-        for (int k = 1; k < Q; ++k) df_fma(s, c[k], v[k * stride]);
-        return s;
-    } else {
-        return df_dot<Q>(c, v, stride);
-    }
-}
-constexpr bool LZ_SWEEP = EVAP_DF_LAZY == 1;                    // interpolation and transposed sweeps, w
-constexpr bool LZ_GRAD = EVAP_DF_LAZY == 1 || EVAP_DF_LAZY == 2;  // gradients at the points
-constexpr bool LZ_FREE = EVAP_DF_LAZY != 0;                      // the last sweep, the value flux
 
 template <int P, int CB, bool PRES, int MINB, bool DET>
 __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
-    k_momentum_df(MeshArgs<double> m, DfBasis bas, const float2* __restrict__ qc, const double* __restrict__ x,
+    k_momentum_df(MeshArgs<double> m, DfBasis bas, dfl kap, const float2* __restrict__ qc,
+                  const double* __restrict__ x,
                   double* __restrict__ y, double* __restrict__ yp, const double* __restrict__ pin, int colour) {
-    constexpr int Q = P + 1, NQ = Q * Q * Q;
-    __shared__ dfl sS[Q][Q], sDc[Q][Q], sN1[Q][2];
-    __shared__ dfl buf[2][6][CB][NQ];  // [half][slot][cell][point]
+    constexpr int Q = P + 1, NQ = Q * Q * Q, NL = Q * Q, TASKS = 3 * NL;
+    using Ln = DfLine<Q>;
+    __shared__ dfl sN1[Q][2];
     __shared__ dfl q1a[CB][2 * Q * Q], q1b[CB][4 * Q];
-    extern __shared__ float2 sqc[];  // [cell][QC_K][point]: this block's coefficients, copied while the sweeps run
+    extern __shared__ float2 smem_df[];
+    dfl* const sb = reinterpret_cast<dfl*>(smem_df);  // [cell][slot][point]
+    constexpr int CELL = (DF_SLOTS + QC_K) * NQ;
     const int tid = threadIdx.x;
-    const int lc = tid / NQ, t = tid % NQ;
-    int cx = 0, cy = 0, cz = 0;
-    const bool active = colour_cell((int64_t)blockIdx.x * CB + lc, m.n, DET ? colour : -1, cx, cy, cz);
-    const int64_t cell = cx + (int64_t)m.n * (cy + (int64_t)m.n * cz);
+    const int n = m.n, M = m.M;
+    const unsigned cell0 = blockIdx.x * CB;
     constexpr bool plain = DET;  // a colour pass: no other cell of the launch touches this cell's nodes
-    float2* myq = sqc + (int64_t)lc * QC_K * NQ + t;
-    if (active) {  // each thread fetches (and later reads) only its own point's coefficients
+    // ---- point view: cell lc, point t = (a, b, c)
+    const int lc = tid / NQ, t = tid % NQ;
+    int cx, cy, cz;
+    const bool active = colour_cell32(cell0 + lc, n, DET ? colour : -1, cx, cy, cz);
+    dfl* const cb = sb + lc * CELL;
+    {
+        const int64_t cell = cx + (int64_t)n * (cy + (int64_t)n * cz);
+        float2* myq = reinterpret_cast<float2*>(cb + DF_SLOTS * NQ + t);
+        // each thread fetches (and later reads) only its own point's coefficients
         const float2* src = qc + cell * QC_K * NQ + t;
 #pragma unroll
         for (int k = 0; k < QC_K; ++k)
             if (m.newton || k < 4 || k > 12) cp_async8(myq + k * NQ, src + k * NQ);
-    }
-    cp_async_commit();
-    if (tid < Q * Q) {
-        sS[tid / Q][tid % Q] = bas.S[tid / Q][tid % Q];
-        sDc[tid / Q][tid % Q] = bas.Dc[tid / Q][tid % Q];
+        cp_async_commit();
     }
     if (tid < 2 * Q) sN1[tid / 2][tid % 2] = bas.N1[tid / 2][tid % 2];
-    const int a = t % Q, b = (t / Q) % Q, c = t / (Q * Q);
-    const int n = m.n, M = m.M;
-    int64_t gidx = 0;
-    bool cons = false;
-    if (active) {
-        const int gx = P * cx + a, gy = P * cy + b, gz = P * cz + c;
-        gidx = gx + (int64_t)M * (gy + (int64_t)M * gz);
-        cons = constrained_node(gx, gy, gz, M, m.faces);
+    // ---- line view: cell ll, component f, line l
+    const int ll = Q == 3 ? lc : tid / TASKS, task = Q == 3 ? t : tid % TASKS;
+    const int f = task / NL, l = task % NL;
+    int lx = cx, ly = cy, lz = cz;
+    bool lact = active;  // the line's cell exists (a block's missing cells repeat the last one and scatter nothing)
+    if (Q != 3) lact = colour_cell32(cell0 + ll, n, DET ? colour : -1, lx, ly, lz);
+    const bool line = Q == 3 || ll < CB;  // this thread owns a line
+    dfl* const lb = sb + (line ? ll : 0) * CELL;
+    // the z-line of nodes this thread gathers and scatters, and which of them are free
+    const int gx = P * lx + l % Q, gy = P * ly + l / Q, gz0 = P * lz;
+    const int64_t zst = (int64_t)M * M;
+    const int64_t gidx = (int64_t)f * m.Nu + gx + (int64_t)M * gy + zst * gz0;
+    unsigned cons = 0;  // bit k: node k is constrained
+    if (line) {
+        const unsigned fc = m.faces;
+        const bool cxy = ((fc & 1u) && gx == 0) || ((fc & 2u) && gx == M - 1) || ((fc & 4u) && gy == 0) ||
+                         ((fc & 8u) && gy == M - 1);
+        cons = cxy ? (1u << Q) - 1u : 0u;
+        if ((fc & 16u) && gz0 == 0) cons |= 1u;
+        if ((fc & 32u) && gz0 + P == M - 1) cons |= 1u << P;
+        dfl u[Q], v[Q];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) buf[0][k][lc][t] = cons ? dfl{0.f, 0.f} : df_from_double(x[k * m.Nu + gidx]);
+        for (int k = 0; k < Q; ++k) u[k] = (cons >> k) & 1u ? dfl{0.f, 0.f} : df_from_double(x[gidx + k * zst]);
+        Ln::val(u, v);
+        st_line<Q, 2>(lb + (3 + f) * NQ, l, v);
     }
     __syncthreads();
-    // values at the Gauss points: x-, y-, z-sweeps of S
-    if (active) {
-        dfl Sa[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Sa[k] = sS[a][k];
-#pragma unroll
-        for (int f = 0; f < 3; ++f) buf[1][f][lc][t] = df_dot_lz<Q, LZ_SWEEP>(Sa, &buf[0][f][lc][Q * (b + Q * c)], 1);
+    if (line) {
+        dfl u[Q], v[Q];
+        ld_line<Q, 1>(lb + (3 + f) * NQ, l, u);
+        Ln::val(u, v);
+        st_line<Q, 1>(lb + (6 + f) * NQ, l, v);
     }
     __syncthreads();
-    if (active) {
-        dfl Sb[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Sb[k] = sS[b][k];
-#pragma unroll
-        for (int f = 0; f < 3; ++f) buf[0][f][lc][t] = df_dot_lz<Q, LZ_SWEEP>(Sb, &buf[1][f][lc][a + Q * Q * c], Q);
+    if (line) {  // x: the values at the points, and their derivative along x
+        dfl u[Q], v[Q];
+        ld_line<Q, 0>(lb + (6 + f) * NQ, l, u);
+        Ln::val(u, v);
+        st_line<Q, 0>(lb + f * NQ, l, v);
     }
     __syncthreads();
-    if (active) {
-        dfl Sc[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Sc[k] = sS[c][k];
-#pragma unroll
-        for (int f = 0; f < 3; ++f) buf[1][f][lc][t] = df_dot_lz<Q, LZ_SWEEP>(Sc, &buf[0][f][lc][a + Q * b], Q * Q);
+    if (line) {
+        dfl u[Q], v[Q];
+        ld_line<Q, 0>(lb + f * NQ, l, u);
+        Ln::der(u, v);
+        st_line<Q, 0>(lb + (3 + 3 * f) * NQ, l, v);
+        ld_line<Q, 1>(lb + f * NQ, l, u);
+        Ln::der(u, v);
+        st_line<Q, 1>(lb + (4 + 3 * f) * NQ, l, v);
+        ld_line<Q, 2>(lb + f * NQ, l, u);
+        Ln::der(u, v);
+        st_line<Q, 2>(lb + (5 + 3 * f) * NQ, l, v);
     }
     __syncthreads();
-    // quadrature-point fluxes from the cached coefficients
-    dfl F[3], Tf[3][3], rdiv{0.f, 0.f};
-    if (active) {
+    // quadrature-point fluxes from the cached coefficients; a thread reads and overwrites its own point's entries only
+    {
         dfl X[3], G[3][3];
-        {
-            dfl Da[Q], Db[Q], Dz[Q];
 #pragma unroll
-            for (int k = 0; k < Q; ++k) {
-                Da[k] = sDc[a][k];
-                Db[k] = sDc[b][k];
-                Dz[k] = sDc[c][k];
-            }
+        for (int k = 0; k < 3; ++k) {
+            X[k] = cb[k * NQ + t];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                X[k] = buf[1][k][lc][t];
-                G[k][0] = df_dot_lz<Q, LZ_GRAD>(Da, &buf[1][k][lc][Q * (b + Q * c)], 1);
-                G[k][1] = df_dot_lz<Q, LZ_GRAD>(Db, &buf[1][k][lc][a + Q * Q * c], Q);
-                G[k][2] = df_dot_lz<Q, LZ_GRAD>(Dz, &buf[1][k][lc][a + Q * b], Q * Q);
-            }
+            for (int d = 0; d < 3; ++d) G[k][d] = cb[(3 + 3 * k + d) * NQ + t];
         }
         cp_async_wait_all();
-        const float2* q = myq;
-        const dfl c0 = ld_df(q);
-        const dfl cu[3] = {ld_df(q + NQ), ld_df(q + 2 * NQ), ld_df(q + 3 * NQ)};
+        const dfl* q = cb + DF_SLOTS * NQ + t;
+        const dfl c0 = q[0];
+        const dfl cu[3] = {q[NQ], q[2 * NQ], q[3 * NQ]};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             dfl v = df_prod(c0, X[k]);
@@ -173,41 +172,22 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
             for (int d = 0; d < 3; ++d) df_fma(v, cu[d], G[k][d]);
             if (m.newton) {
 #pragma unroll
-                for (int d = 0; d < 3; ++d) df_fma(v, ld_df(q + (4 + 3 * k + d) * NQ), X[d]);
+                for (int d = 0; d < 3; ++d) df_fma(v, q[(4 + 3 * k + d) * NQ], X[d]);
             }
-            F[k] = LZ_FREE ? v : df_norm(v);
+            cb[k * NQ + t] = v;  // only starts a new accumulation: left unnormalized
         }
-        const dfl c13 = ld_df(q + 13 * NQ);
+        const dfl c13 = q[13 * NQ];
         const dfl tr = df_add(df_add(G[0][0], G[1][1]), G[2][2]);
         const dfl hm = df_scale2(c13, 0.5f);
-        const dfl nz[3] = {ld_df(q + 14 * NQ), ld_df(q + 15 * NQ), ld_df(q + 16 * NQ)};
+        const dfl nz[3] = {q[14 * NQ], q[15 * NQ], q[16 * NQ]};
         const bool corr = (nz[0].hi != 0.f) || (nz[1].hi != 0.f) || (nz[2].hi != 0.f);
         const dfl sm = corr ? df_mul(c13, tr) : dfl{0.f, 0.f};
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-#pragma unroll
-            for (int l = k; l < 3; ++l) {  // symmetric: 6 distinct entries
-                dfl v = k == l ? df_mul(c13, G[k][k]) : df_mul(hm, df_add(G[k][l], G[l][k]));
-                if (corr) {
-                    dfl w = v;
-                    df_fma(w, df_neg(sm), df_mul(nz[k], nz[l]));
-                    v = df_norm(w);
-                }
-                Tf[k][l] = v;
-                Tf[l][k] = v;
-            }
-        {
-            dfl r = df_prod(ld_df(q + 17 * NQ), tr);
-            const dfl src = ld_df(q + 18 * NQ);
-            const dfl s2 = two_sum(r.hi, -src.hi);
-            r.hi = s2.hi;
-            r.lo = __fadd_rn(r.lo, __fsub_rn(s2.lo, src.lo));
-            rdiv = df_norm(r);
-        }
+        const dfl rw = PRES || yp ? df_mul(q[17 * NQ], kap) : dfl{0.f, 0.f};  // kappa W
+        dfl wp{0.f, 0.f};
         if constexpr (PRES) {  // p at the point: trilinear interpolation by successive linear ones, in FP64
             const int64_t m1 = n + 1;
             const double* p0 = pin + cx + m1 * (cy + m1 * cz);
-            const double tx = bas.t[a], ty = bas.t[b], tz = bas.t[c];
+            const double tx = bas.t[t % Q], ty = bas.t[(t / Q) % Q], tz = bas.t[t / (Q * Q)];
             double e[2][2];
 #pragma unroll
             for (int jc = 0; jc < 2; ++jc)
@@ -217,94 +197,98 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
                     e[jc][jb] = fma(tx, r[1] - r[0], r[0]);
                 }
             const double f0 = fma(ty, e[0][1] - e[0][0], e[0][0]), f1 = fma(ty, e[1][1] - e[1][0], e[1][0]);
-            const dfl wp = df_mul(ld_df(q + 17 * NQ), df_from_double(fma(tz, f1 - f0, f0)));
-#pragma unroll
-            for (int k = 0; k < 3; ++k) Tf[k][k] = df_sub(Tf[k][k], wp);
+            wp = df_mul(rw, df_from_double(fma(tz, f1 - f0, f0)));
         }
-    }
-    __syncthreads();
-    if (active) {
-#pragma unroll
-        for (int s = 0; s < 9; ++s) buf[s / 6][s % 6][lc][t] = Tf[s / 3][s % 3];
-        buf[1][3][lc][t] = rdiv;
-    }
-    __syncthreads();
-    // test with gradients: w_c = F_c + sum_b Dc^T T_cb
-    dfl wv[3];
-    if (active) {
-        dfl Ea[Q], Eb[Q], Ec[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) {
-            Ea[k] = sDc[k][a];
-            Eb[k] = sDc[k][b];
-            Ec[k] = sDc[k][c];
-        }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int i0 = 3 * k + 0, i1 = 3 * k + 1, i2 = 3 * k + 2;
-            dfl s = F[k];
-#pragma unroll
-            for (int r = 0; r < Q; ++r) {
-                df_fma(s, Ea[r], buf[i0 / 6][i0 % 6][lc][r + Q * (b + Q * c)]);
-                df_fma(s, Eb[r], buf[i1 / 6][i1 % 6][lc][a + Q * (r + Q * c)]);
-                df_fma(s, Ec[r], buf[i2 / 6][i2 % 6][lc][a + Q * (b + Q * r)]);
-            }
-            wv[k] = LZ_SWEEP ? s : df_norm(s);
-        }
-        // divergence row, Q1 test functions: sum_q N1_j(q) r_q by three sweeps; x-sweep here: [jx][qy][qz]
-        if (yp && t < 2 * Q * Q) {
-            const int jx = t & 1, qy = (t >> 1) % Q, qz = (t >> 1) / Q;
-            dfl s = df_prod(sN1[0][jx], buf[1][3][lc][Q * (qy + Q * qz)]);
-#pragma unroll
-            for (int qq = 1; qq < Q; ++qq) df_fma(s, sN1[qq][jx], buf[1][3][lc][qq + Q * (qy + Q * qz)]);
-            q1a[lc][t] = df_norm(s);
-        }
-    }
-    __syncthreads();
-    if (active) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) buf[0][k][lc][t] = wv[k];
-        if (yp && t < 4 * Q) {  // y-sweep: [jx][jy][qz]
-            const int jx = t & 1, jy = (t >> 1) & 1, qz = t >> 2;
-            dfl s = df_prod(sN1[0][jy], q1a[lc][jx + 2 * (0 + Q * qz)]);
-#pragma unroll
-            for (int qq = 1; qq < Q; ++qq) df_fma(s, sN1[qq][jy], q1a[lc][jx + 2 * (qq + Q * qz)]);
-            q1b[lc][t] = df_norm(s);
-        }
-    }
-    __syncthreads();
-    // transposed sweeps S^T: z, y, x
-    if (active) {
-        dfl Tc[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Tc[k] = sS[k][c];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) buf[1][k][lc][t] = df_dot_lz<Q, LZ_SWEEP>(Tc, &buf[0][k][lc][a + Q * b], Q * Q);
-        if (yp && t < 8) {  // z-sweep: Q1 node (jx, jy, jz)
-            const int jx = t & 1, jy = (t >> 1) & 1, jz = t >> 2;
-            dfl s = df_prod(sN1[0][jz], q1b[lc][jx + 2 * (jy + 2 * 0)]);
-#pragma unroll
-            for (int qq = 1; qq < Q; ++qq) df_fma(s, sN1[qq][jz], q1b[lc][jx + 2 * (jy + 2 * qq)]);
-            const int64_t m1 = n + 1;
-            acc_add(&yp[(cx + jx) + m1 * ((cy + jy) + m1 * (cz + jz))], df_to_double(df_norm(s)), plain);
-        }
-    }
-    __syncthreads();
-    if (active) {
-        dfl Tb[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Tb[k] = sS[k][b];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) buf[0][k][lc][t] = df_dot_lz<Q, LZ_SWEEP>(Tb, &buf[1][k][lc][a + Q * Q * c], Q);
-    }
-    __syncthreads();
-    if (active && !cons) {
-        dfl Ta[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Ta[k] = sS[k][a];
 #pragma unroll
         for (int k = 0; k < 3; ++k)
-            acc_add(&y[k * m.Nu + gidx], df_to_double(df_dot_lz<Q, LZ_FREE>(Ta, &buf[0][k][lc][Q * (b + Q * c)], 1)), plain);
+#pragma unroll
+            for (int e = k; e < 3; ++e) {  // symmetric: 6 distinct entries
+                dfl v = k == e ? df_mul(c13, G[k][k]) : df_mul(hm, df_add(G[k][e], G[e][k]));
+                if (corr) {
+                    dfl w = v;
+                    df_fma(w, df_neg(sm), df_mul(nz[k], nz[e]));
+                    v = df_norm(w);
+                }
+                if (PRES && k == e) v = df_sub(v, wp);
+                cb[t_slot(k, e) * NQ + t] = v;
+            }
+        if (yp) {
+            dfl r = df_prod(rw, tr);
+            const dfl src = q[18 * NQ];
+            const dfl s2 = two_sum(r.hi, -src.hi);
+            r.hi = s2.hi;
+            r.lo = __fadd_rn(r.lo, __fsub_rn(s2.lo, src.lo));
+            cb[9 * NQ + t] = df_norm(r);
+        }
+    }
+    __syncthreads();
+    // test with gradients: the lines along y and z into the coefficients' slots
+    if (line) {
+        dfl u[Q], v[Q];
+        ld_line<Q, 1>(lb + t_slot(f, 1) * NQ, l, u);
+        Ln::derT(u, v);
+        st_line<Q, 1>(lb + (DF_SLOTS + f) * NQ, l, v);
+        ld_line<Q, 2>(lb + t_slot(f, 2) * NQ, l, u);
+        Ln::derT(u, v);
+        st_line<Q, 2>(lb + (DF_SLOTS + 3 + f) * NQ, l, v);
+    }
+    // divergence row, Q1 test functions: sum_q N1_j(q) r_q by three sweeps, whose outputs fill the first warps
+    if (yp && tid < CB * 2 * Q * Q) {  // x-sweep: [jx][qy][qz]
+        const int c2 = tid / (2 * Q * Q), o = tid % (2 * Q * Q);
+        const dfl* r = sb + c2 * CELL + 9 * NQ + Q * (o >> 1);
+        dfl s = df_prod(sN1[0][o & 1], r[0]);
+#pragma unroll
+        for (int qq = 1; qq < Q; ++qq) df_fma(s, sN1[qq][o & 1], r[qq]);
+        q1a[c2][o] = df_norm(s);
+    }
+    __syncthreads();
+    if (line) {  // x: F + the three tests, and its value sweep
+        dfl u[Q], v[Q], w[Q];
+        ld_line<Q, 0>(lb + t_slot(f, 0) * NQ, l, u);
+        Ln::derT(u, v);
+        ld_line<Q, 0>(lb + f * NQ, l, w);
+        ld_line<Q, 0>(lb + (DF_SLOTS + f) * NQ, l, u);
+#pragma unroll
+        for (int k = 0; k < Q; ++k) w[k] = df_addl(df_addl(w[k], v[k]), u[k]);
+        ld_line<Q, 0>(lb + (DF_SLOTS + 3 + f) * NQ, l, u);
+#pragma unroll
+        for (int k = 0; k < Q; ++k) w[k] = df_add(w[k], u[k]);
+        Ln::template valT<false>(w, v);
+        st_line<Q, 0>(lb + f * NQ, l, v);
+    }
+    if (yp && tid < CB * 4 * Q) {  // y-sweep: [jx][jy][qz]
+        const int c2 = tid / (4 * Q), o = tid % (4 * Q), jx = o & 1, jy = (o >> 1) & 1, qz = o >> 2;
+        dfl s = df_prod(sN1[0][jy], q1a[c2][jx + 2 * (0 + Q * qz)]);
+#pragma unroll
+        for (int qq = 1; qq < Q; ++qq) df_fma(s, sN1[qq][jy], q1a[c2][jx + 2 * (qq + Q * qz)]);
+        q1b[c2][o] = df_norm(s);
+    }
+    __syncthreads();
+    if (line) {
+        dfl u[Q], v[Q];
+        ld_line<Q, 1>(lb + f * NQ, l, u);
+        Ln::template valT<false>(u, v);
+        st_line<Q, 1>(lb + f * NQ, l, v);
+    }
+    if (yp && tid < CB * 8) {  // z-sweep: Q1 node (jx, jy, jz)
+        const int c2 = tid / 8, o = tid % 8, jx = o & 1, jy = (o >> 1) & 1, jz = o >> 2;
+        int ex, ey, ez;
+        if (colour_cell32(cell0 + c2, n, DET ? colour : -1, ex, ey, ez)) {
+            dfl s = df_prod(sN1[0][jz], q1b[c2][jx + 2 * (jy + 2 * 0)]);
+#pragma unroll
+            for (int qq = 1; qq < Q; ++qq) df_fma(s, sN1[qq][jz], q1b[c2][jx + 2 * (jy + 2 * qq)]);
+            const int64_t m1 = n + 1;
+            acc_add(&yp[(ex + jx) + m1 * ((ey + jy) + m1 * (ez + jz))], df_to_double(df_norm(s)), plain);
+        }
+    }
+    __syncthreads();
+    if (line && lact) {  // z, and the scatter of the line's free nodes
+        dfl u[Q], v[Q];
+        ld_line<Q, 2>(lb + f * NQ, l, u);
+        Ln::template valT<true>(u, v);
+#pragma unroll
+        for (int k = 0; k < Q; ++k)
+            if (!((cons >> k) & 1u)) acc_add(&y[gidx + k * zst], df_to_double(v[k]), plain);
     }
 }
 
@@ -327,38 +311,35 @@ DfBasis make_df_basis(const Basis<double>& b, double inv_h) {
 int launch_momentum_df(evap_mesh* h, const MeshArgs<double>& m, const double* x, double* y, double* yp,
                        const double* p, cudaStream_t s) {
     const DfBasis b = make_df_basis(h->b, m.inv_h);
+    const dfl kap = df_from_double(df_kappa(m));
     const float2* qc = reinterpret_cast<const float2*>(h->qcdf);
     const int c0 = h->deterministic ? 0 : -1, c1 = h->deterministic ? 8 : 0;  // colour passes, or one atomic pass
+    // at most 48 KB of shared memory per block, so no launch needs a function attribute
     auto run = [&](auto kern, int CB, int threads, size_t dyn) -> int {
-        EVAP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
         for (int colour = c0; colour < std::max(c1, c0 + 1); ++colour) {
             const int64_t cells = colour_cells(m.n, colour);
             if (cells == 0) continue;
             const unsigned grid = (unsigned)((cells + CB - 1) / CB);
-            kern<<<grid, threads, dyn, s>>>(m, b, qc, x, y, yp, p, colour);
+            kern<<<grid, threads, dyn, s>>>(m, b, kap, qc, x, y, yp, p, colour);
             EVAP_CHECK_LAUNCH("momentum_df");
         }
         return EVAP_OK;
     };
-    int rc;
+    const bool det = h->deterministic;
     if (m.P == 2) {
-        constexpr int CB = EVAP_DF_CB2, MINB = EVAP_DF_MINB2, MINBP = EVAP_DF_MINB2_PRES;
-        constexpr size_t dyn = df_coeff_smem<2, CB>();
-        const bool det = h->deterministic;
-        rc = p ? run(det ? k_momentum_df<2, CB, true, MINBP, true> : k_momentum_df<2, CB, true, MINBP, false>, CB,
-                     CB * 27, dyn)
-               : run(det ? k_momentum_df<2, CB, false, MINB, true> : k_momentum_df<2, CB, false, MINB, false>, CB,
-                     CB * 27, dyn);
-    } else {
-        constexpr int CB = 4;
-        constexpr size_t dyn = df_coeff_smem<3, CB>();
-        const bool det = h->deterministic;
-        rc = p ? run(det ? k_momentum_df<3, CB, true, 1, true> : k_momentum_df<3, CB, true, 1, false>, CB, CB * 64,
-                     dyn)
-               : run(det ? k_momentum_df<3, CB, false, 1, true> : k_momentum_df<3, CB, false, 1, false>, CB, CB * 64,
-                     dyn);
+        constexpr int CB = EVAP_DF_CB2, MINB = EVAP_DF_MINB2;
+        constexpr size_t dyn = df_smem<2, CB>();
+        return p ? run(det ? k_momentum_df<2, CB, true, MINB, true> : k_momentum_df<2, CB, true, MINB, false>, CB,
+                       CB * 27, dyn)
+                 : run(det ? k_momentum_df<2, CB, false, MINB, true> : k_momentum_df<2, CB, false, MINB, false>, CB,
+                       CB * 27, dyn);
     }
-    return rc;
+    constexpr int CB = EVAP_DF_CB3, MINB = EVAP_DF_MINB3;
+    constexpr size_t dyn = df_smem<3, CB>();
+    return p ? run(det ? k_momentum_df<3, CB, true, MINB, true> : k_momentum_df<3, CB, true, MINB, false>, CB, CB * 64,
+                   dyn)
+             : run(det ? k_momentum_df<3, CB, false, MINB, true> : k_momentum_df<3, CB, false, MINB, false>, CB,
+                   CB * 64, dyn);
 }
 
 }  // namespace evap
