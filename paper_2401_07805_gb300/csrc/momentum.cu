@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(256) k_momentum_init(int M, int64_t Nu, unsign
 // W = w_qx w_qy w_qz h^3.  One thread per quadrature point, CB cells per block (u0 interpolated by sum factorization).
 // Slots 1..12 are also stored in FP32 for the FP32 apply (slots 1..3 divided by h: that kernel takes reference
 // gradients), in its 32-cell block layout
-// qc32[((blk * QC32_K + k) * NQ + pt) * 32 + lane], cell (32 xb + lane, row) in block blk = xb + ceil(n / 32) row.
+// qc32[((blk * QC32_K + k) * NQ + pt) * 32 + lane], cell 32 blk + lane (lexicographic).
 // The interpolation of u0 and every product run in double-float arithmetic (dfloat.cuh) on the FP32 pipe: the FP64
 // pipe keeps the conversions (u0 in, the FP64 copy of each coefficient out) and the few scalar factors.  The
 // double-float results are the pairs of the apply's cache as they stand; the FP64 copy is their sum (within 2^-48).
@@ -153,10 +153,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
         const dfl w = k >= 1 && k <= 3 ? df_mul(v[k], kap) : (k == 13 ? df_mul(v[k], kap2) : v[k]);
         qcdf[base + (int64_t)k * NQ] = make_float2(w.hi, w.lo);
     }
-    const int64_t row = cell / n;
-    const int cx = (int)(cell - row * n);
-    const int64_t blk = cx / 32 + (int64_t)((n + 31) / 32) * row;
-    float* dst = qc32 + (blk * QC32_K * NQ + t) * 32 + (cx % 32);
+    float* dst = qc32 + ((cell >> 5) * QC32_K * NQ + t) * 32 + (cell & 31);
 #pragma unroll
     for (int k = 0; k < QC32_K; ++k) dst[(int64_t)k * NQ * 32] = k < 3 ? df_mul(v[1 + k], invh_df).hi : v[1 + k].hi;
 }
@@ -179,7 +176,7 @@ int launch_qp_coeffs(evap_mesh* h, cudaStream_t s) {
         EVAP_CUDA(cudaMalloc(&h->qcdf, 2 * need * sizeof(float)));
         h->qcdf_len = 2 * need;
     }
-    const int64_t need32 = (int64_t)((m.n + 31) / 32) * m.n * m.n * QC32_K * nq * 32;
+    const int64_t need32 = (m.ncell + 31) / 32 * QC32_K * nq * 32;
     if (h->qc32_len < need32) {
         if (h->qc32) cudaFree(h->qc32);
         h->qc32 = nullptr;

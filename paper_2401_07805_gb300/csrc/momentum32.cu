@@ -4,8 +4,8 @@
 // of Eq. modified_viscous_stress, divergence row of Eq. continuity), evaluated in FP32 with the material law from the
 // FP32 copy of the FP64 interface table.  The FP32 pipe is 60x faster than FP64 on GB300, so here the limit is the
 // load/store unit, not arithmetic; the kernel is laid out to move few operands through shared memory:
-//   * (P+1)^2 threads per cell, each owning one line of points; the 1D matrices are kernel parameters indexed at
-//     compile time (constant-bank operands, no loads);
+//   * (P+1)^2 threads per cell, each owning one line of points; the 1D matrices are compile-time constants, for Q = 3 in
+//     factored form (Line32);
 //   * the cell index is the fastest thread index (a warp holds the same line of 32 consecutive cells) and shared
 //     memory is laid out [slot][cell], so every shared access of a warp touches consecutive words (no bank
 //     conflicts), the gather and the scatter of a warp walk along x, and the cell codes load coalesced;
@@ -30,8 +30,84 @@ struct Scale32 {
 };
 
 
-// blocks per SM for Q2 (a register cap): measured at 64^3 (100 applies, ms) 3 blocks (72 registers) 0.145, 2 (90)
-// 0.171, 4 (56, spills) 0.222
+// Sweeps along one line in FP32: val y = S u, valder (y, d) = (S u, D u), tv o = S^T F, tvd o = S^T F + D^T T, D the
+// reference derivative.  Q = 3: with dm = u_2 - u_0 and C = u_0 - 2 u_1 + u_2 a quadratic and its derivative at the
+// Gauss points 1/2 -+ tau, 1/2 (tau = sqrt(3/20)) are u_1 + 2 tau^2 C -+ tau dm, u_1 and dm -+ 4 tau C, dm: 8
+// operations for both where the 3 x 3 matrices take 18, and the transposes by the same factorization 12.  Q = 4: the
+// matrices (their even-odd form saves nothing there).
+template <int Q>
+struct Line32 {
+    static __device__ __forceinline__ void val(const float (&u)[Q], float (&y)[Q]) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            y[q] = 0.f;
+#pragma unroll
+            for (int k = 0; k < Q; ++k) y[q] += (float)kCtBasis<Q - 1>.S[q][k] * u[k];
+        }
+    }
+    static __device__ __forceinline__ void valder(const float (&u)[Q], float (&y)[Q], float (&d)[Q]) {
+        val(u, y);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            d[q] = 0.f;
+#pragma unroll
+            for (int k = 0; k < Q; ++k) d[q] += (float)kCtBasis<Q - 1>.D[q][k] * u[k];
+        }
+    }
+    static __device__ __forceinline__ void tv(const float (&F)[Q], float (&o)[Q]) {
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            o[k] = 0.f;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) o[k] += (float)kCtBasis<Q - 1>.S[q][k] * F[q];
+        }
+    }
+    static __device__ __forceinline__ void tvd(const float (&F)[Q], const float (&T)[Q], float (&o)[Q]) {
+        tv(F, o);
+#pragma unroll
+        for (int k = 0; k < Q; ++k)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) o[k] += (float)kCtBasis<Q - 1>.D[q][k] * T[q];
+    }
+};
+template <>
+struct Line32<3> {
+    static constexpr float TAU = 0.3872983346207416885179265f, G = 0.3f;  // sqrt(3/20), 2 tau^2
+    static __device__ __forceinline__ void val(const float (&u)[3], float (&y)[3]) {
+        const float dm = u[2] - u[0], C = fmaf(-2.f, u[1], u[0] + u[2]), b = fmaf(G, C, u[1]);
+        y[0] = fmaf(-TAU, dm, b);
+        y[1] = u[1];
+        y[2] = fmaf(TAU, dm, b);
+    }
+    static __device__ __forceinline__ void valder(const float (&u)[3], float (&y)[3], float (&d)[3]) {
+        const float dm = u[2] - u[0], C = fmaf(-2.f, u[1], u[0] + u[2]), b = fmaf(G, C, u[1]);
+        y[0] = fmaf(-TAU, dm, b);
+        y[1] = u[1];
+        y[2] = fmaf(TAU, dm, b);
+        d[0] = fmaf(-4.f * TAU, C, dm);
+        d[1] = dm;
+        d[2] = fmaf(4.f * TAU, C, dm);
+    }
+    static __device__ __forceinline__ void tv(const float (&F)[3], float (&o)[3]) {
+        const float s = F[0] + F[2], be = TAU * (F[2] - F[0]), ga = G * s;
+        o[0] = ga - be;
+        o[1] = fmaf(-2.f, ga, s + F[1]);
+        o[2] = ga + be;
+    }
+    static __device__ __forceinline__ void tvd(const float (&F)[3], const float (&T)[3], float (&o)[3]) {
+        const float s = F[0] + F[2], be = fmaf(TAU, F[2] - F[0], T[0] + T[1] + T[2]);
+        const float ga = fmaf(4.f * TAU, T[2] - T[0], G * s);
+        o[0] = ga - be;
+        o[1] = fmaf(-2.f, ga, s + F[1]);
+        o[2] = ga + be;
+    }
+};
+
+// Blocks per SM for Q2 (a register cap).  What bounds the kernel is the latency of the streamed coefficients against the
+// 27 warps that 35 KB of shared memory per block leave on an SM, then issue.  Measured at 75^3 Q2 (us per apply): 273
+// with dense 3 x 3 sweeps and blocks of 32 cells of one x-row (96 lanes for 75 cells); 225 with the factored sweeps
+// and cells taken 32 at a time across rows; 203 with the 36 coefficients of a thread loaded before the y sweeps, 202
+// at the kernel's start (72 registers); 2 blocks per SM 244 to 252, 4 (56 registers) 223 without the early loads.
 #ifndef EVAP_M32_MINB2
 #define EVAP_M32_MINB2 3
 #endif
@@ -50,22 +126,23 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1), MINB)
     const int tid = threadIdx.x;
     const int lc = tid % CB, l = tid / CB;
     const int n = m.n, M = m.M;
-    // A block holds CB consecutive cells of one x-row: (cx, cy, cz) = (CB * xb + lc, row % n, row / n).  In a colour
-    // pass (DET, colour = pb + 2 py + 4 pz) the blocks with xb = pb mod 2 of the rows with cy = py, cz = pz mod 2:
-    // two such blocks share no node, and inside a block the even cells scatter before the odd ones.  The atomic
-    // variant (DET false) is compiled apart: it ignores colour and adds each result as soon as it is formed.
-    const int nxc = (n + CB - 1) / CB;
+    // A block holds CB consecutive cells (lexicographic, rows run on).  In a colour pass (DET, colour = pb + 2 py + 4 pz)
+    // it holds CB consecutive cells of one x-row, (cx, cy, cz) = (CB xb + lc, row), the blocks with xb = pb mod 2 of
+    // the rows with cy = py, cz = pz mod 2: two such blocks share no node, and inside a block the even cells scatter
+    // before the odd ones.  The atomic variant (DET false) is compiled apart: it ignores colour and adds each result as
+    // soon as it is formed.
     int cx, cy, cz;
-    int64_t cell;
+    unsigned cell;
     bool active;
     if constexpr (!DET) {
-        const int row = (int)(blockIdx.x / (unsigned)nxc);
-        cx = ((int)blockIdx.x - row * nxc) * CB + lc;
-        cy = row % n;
-        cz = row / n;
-        cell = cx + (int64_t)n * row;
-        active = cx < n;
+        cell = blockIdx.x * CB + lc;
+        const unsigned row = cell / (unsigned)n;
+        cx = (int)(cell - row * (unsigned)n);
+        cz = (int)(row / (unsigned)n);
+        cy = (int)(row - (unsigned)cz * (unsigned)n);
+        active = cell < (unsigned)m.ncell;
     } else {
+        const int nxc = (n + CB - 1) / CB;
         const int pb = colour & 1, py = (colour >> 1) & 1, pz = colour >> 2;
         const int hy = (n - py + 1) >> 1, hxb = (nxc - pb + 1) >> 1;
         const int rowc = (int)(blockIdx.x / (unsigned)hxb);
@@ -73,7 +150,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1), MINB)
         cx = xb * CB + lc;
         cy = 2 * (rowc % hy) + py;
         cz = 2 * (rowc / hy) + pz;
-        cell = cx + (int64_t)n * (cy + (int64_t)n * cz);
+        cell = (unsigned)cx + (unsigned)n * ((unsigned)cy + (unsigned)n * (unsigned)cz);
         active = cx < n;
     }
     float* cs = sm + lc;
@@ -94,6 +171,18 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1), MINB)
             keep[k] = !(cxy || ((fc & 16u) && gz0 + k == 0) || ((fc & 32u) && gz0 + k == M - 1));
         zbase = gx + (int64_t)M * gy + MM * gz0;
     }
+    // the cached coefficients of this thread's x-line (lane = cell: one 128-byte line per warp and coefficient), loaded
+    // ahead of the sweeps that precede their use
+    const float* cq = qc32 + (int64_t)(cell >> 5) * QC32_K * NQ * 32 + (cell & 31u);
+    float cf[Q][QC32_K];
+    auto load_coeffs = [&]() {
+        if (active)
+#pragma unroll
+            for (int qx = 0; qx < Q; ++qx)
+#pragma unroll
+                for (int k = 0; k < QC32_K; ++k) cf[qx][k] = __ldg(cq + (k * NQ + l * Q + qx) * 32);
+    };
+    if (P == 2) load_coeffs();
     // ---------------------------------------------------------------- z-lines: gather, S and D along z
     {
         const int i = l % Q, j = l / Q;
@@ -104,21 +193,18 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1), MINB)
                 const float* src = x + f * m.Nu + zbase;
 #pragma unroll
                 for (int k = 0; k < Q; ++k) v[k] = keep[k] ? src[k * MM] : 0.f;
+                float a[Q], d[Q];
+                Line32<Q>::valder(v, a, d);
 #pragma unroll
                 for (int q = 0; q < Q; ++q) {
-                    float a = 0.f, d = 0.f;
-#pragma unroll
-                    for (int k = 0; k < Q; ++k) {
-                        a += (float)B.S[q][k] * v[k];
-                        d += (float)B.D[q][k] * v[k];
-                    }
-                    S_(f * NQ + at(q, j, i)) = a;
-                    S_(OFF_Z + f * NQ + at(q, j, i)) = d;
+                    S_(f * NQ + at(q, j, i)) = a[q];
+                    S_(OFF_Z + f * NQ + at(q, j, i)) = d[q];
                 }
             }
         }
     }
     __syncthreads();
+    if (P == 3) load_coeffs();
     // ---------------------------------------------------------------- y-lines: S, D on A; S on Az
     {
         const int i = l % Q, qz = l / Q;
@@ -131,18 +217,14 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1), MINB)
                     a[jj] = S_(f * NQ + at(qz, jj, i));
                     az[jj] = S_(OFF_Z + f * NQ + at(qz, jj, i));
                 }
+                float bs[Q], bd[Q], bz[Q];
+                Line32<Q>::valder(a, bs, bd);
+                Line32<Q>::val(az, bz);
 #pragma unroll
                 for (int q = 0; q < Q; ++q) {
-                    float bs = 0.f, bd = 0.f, bz = 0.f;
-#pragma unroll
-                    for (int jj = 0; jj < Q; ++jj) {
-                        bs += (float)B.S[q][jj] * a[jj];
-                        bd += (float)B.D[q][jj] * a[jj];
-                        bz += (float)B.S[q][jj] * az[jj];
-                    }
-                    S_(f * NQ + at(qz, q, i)) = bs;
-                    S_(OFF_Y + f * NQ + at(qz, q, i)) = bd;
-                    S_(OFF_Z + f * NQ + at(qz, q, i)) = bz;
+                    S_(f * NQ + at(qz, q, i)) = bs[q];
+                    S_(OFF_Y + f * NQ + at(qz, q, i)) = bd[q];
+                    S_(OFF_Z + f * NQ + at(qz, q, i)) = bz[q];
                 }
             }
         }
@@ -152,42 +234,31 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1), MINB)
     {
         const int qy = l % Q, qz = l / Q;
         if (active) {
-            float bs[3][Q], by[3][Q], bz[3][Q];
+            // values and gradients at the line's points (X at q, G[.][0..2] in gx, gy, gz), replaced point by point by
+            // the fluxes (F, T[.][0..2])
+            float xv[3][Q], gx[3][Q], gy[3][Q], gz[3][Q];
 #pragma unroll
-            for (int f = 0; f < 3; ++f)
+            for (int f = 0; f < 3; ++f) {
+                float u[Q];
 #pragma unroll
-                for (int ii = 0; ii < Q; ++ii) {
-                    bs[f][ii] = S_(f * NQ + at(qz, qy, ii));
-                    by[f][ii] = S_(OFF_Y + f * NQ + at(qz, qy, ii));
-                    bz[f][ii] = S_(OFF_Z + f * NQ + at(qz, qy, ii));
-                }
+                for (int ii = 0; ii < Q; ++ii) u[ii] = S_(f * NQ + at(qz, qy, ii));
+                Line32<Q>::valder(u, xv[f], gx[f]);
+#pragma unroll
+                for (int ii = 0; ii < Q; ++ii) u[ii] = S_(OFF_Y + f * NQ + at(qz, qy, ii));
+                Line32<Q>::val(u, gy[f]);
+#pragma unroll
+                for (int ii = 0; ii < Q; ++ii) u[ii] = S_(OFF_Z + f * NQ + at(qz, qy, ii));
+                Line32<Q>::val(u, gz[f]);
+            }
             const int8_t cc = code[cell];
             const float* tb = cc == CELL_TABLE ? table + (int64_t)tindex[cell] * TAB_K * NQ : nullptr;
-            // the cache's block of 32 x-consecutive cells holding this cell, and its place in it
-            const int64_t cblk = DET ? (int64_t)(cy + n * cz) * nxc + cx / CB : (int64_t)blockIdx.x;
-            const float* cq = qc32 + cblk * QC32_K * NQ * 32 + (DET ? cx % CB : lc);
             const float wyz = B.wf[qy] * B.wf[qz];
-            float Pv[3][Q], Py[3][Q], Pz[3][Q], Pd[2];
-#pragma unroll
-            for (int c = 0; c < 3; ++c)
-#pragma unroll
-                for (int ii = 0; ii < Q; ++ii) Pv[c][ii] = Py[c][ii] = Pz[c][ii] = 0.f;
-            Pd[0] = Pd[1] = 0.f;
+            float Pd[2] = {0.f, 0.f};
 #pragma unroll
             for (int qx = 0; qx < Q; ++qx) {
-                float X[3], G[3][3];
-#pragma unroll
-                for (int f = 0; f < 3; ++f) {
-                    float v = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
-#pragma unroll
-                    for (int ii = 0; ii < Q; ++ii) {
-                        v += (float)B.S[qx][ii] * bs[f][ii];
-                        gx += (float)B.D[qx][ii] * bs[f][ii];
-                        gy += (float)B.S[qx][ii] * by[f][ii];
-                        gz += (float)B.S[qx][ii] * bz[f][ii];
-                    }
-                    X[f] = v; G[f][0] = gx; G[f][1] = gy; G[f][2] = gz;
-                }
+                const float X[3] = {xv[0][qx], xv[1][qx], xv[2][qx]};
+                const float G[3][3] = {{gx[0][qx], gy[0][qx], gz[0][qx]}, {gx[1][qx], gy[1][qx], gz[1][qx]},
+                                       {gx[2][qx], gy[2][qx], gz[2][qx]}};
                 float rho, mu, nz[3], vd;
                 const int qi = at(qz, qy, qx);
                 if (tb) {
@@ -204,38 +275,40 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1), MINB)
                 const float wr = Wr * rho * hs.hcm;  // W rho c_m
                 const float wm = Wr * mu * hs.c2h;   // 2 W mu / h^2
                 const float tr = G[0][0] + G[1][1] + G[2][2];
-                float cf[QC32_K];
-#pragma unroll
-                for (int k = 0; k < QC32_K; ++k) cf[k] = cq[(k * NQ + qi) * 32];
-                float F[3], T[3][3];
 #pragma unroll
                 for (int c = 0; c < 3; ++c)
-                    F[c] = wr * X[c] + cf[0] * G[c][0] + cf[1] * G[c][1] + cf[2] * G[c][2] +
-                           cf[3 + 3 * c] * X[0] + cf[4 + 3 * c] * X[1] + cf[5 + 3 * c] * X[2];
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) T[c][b] = wm * (0.5f * (G[c][b] + G[b][c]) - tr * nz[c] * nz[b]);
+                    xv[c][qx] = wr * X[c] + cf[qx][0] * G[c][0] + cf[qx][1] * G[c][1] + cf[qx][2] * G[c][2] +
+                                cf[qx][3 + 3 * c] * X[0] + cf[qx][4 + 3 * c] * X[1] + cf[qx][5 + 3 * c] * X[2];
+                const float hm = 0.5f * wm, sm_ = wm * tr;
+                const float t01 = hm * (G[0][1] + G[1][0]) - sm_ * nz[0] * nz[1];
+                const float t02 = hm * (G[0][2] + G[2][0]) - sm_ * nz[0] * nz[2];
+                const float t12 = hm * (G[1][2] + G[2][1]) - sm_ * nz[1] * nz[2];
+                gx[0][qx] = wm * G[0][0] - sm_ * nz[0] * nz[0];
+                gy[0][qx] = t01;
+                gz[0][qx] = t02;
+                gx[1][qx] = t01;
+                gy[1][qx] = wm * G[1][1] - sm_ * nz[1] * nz[1];
+                gz[1][qx] = t12;
+                gx[2][qx] = t02;
+                gy[2][qx] = t12;
+                gz[2][qx] = wm * G[2][2] - sm_ * nz[2] * nz[2];
                 const float rdiv = Wr * (hs.h2 * tr - hs.h3 * vd);
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-#pragma unroll
-                    for (int ii = 0; ii < Q; ++ii) {
-                        Pv[c][ii] += (float)B.S[qx][ii] * F[c] + (float)B.D[qx][ii] * T[c][0];
-                        Py[c][ii] += (float)B.S[qx][ii] * T[c][1];
-                        Pz[c][ii] += (float)B.S[qx][ii] * T[c][2];
-                    }
                 Pd[0] += (float)B.N1[qx][0] * rdiv;
                 Pd[1] += (float)B.N1[qx][1] * rdiv;
             }
 #pragma unroll
-            for (int c = 0; c < 3; ++c)
+            for (int c = 0; c < 3; ++c) {
+                float o[Q];
+                Line32<Q>::tvd(xv[c], gx[c], o);
 #pragma unroll
-                for (int ii = 0; ii < Q; ++ii) {
-                    S_(c * NQ + at(qz, qy, ii)) = Pv[c][ii];
-                    S_(OFF_Y + c * NQ + at(qz, qy, ii)) = Py[c][ii];
-                    S_(OFF_Z + c * NQ + at(qz, qy, ii)) = Pz[c][ii];
-                }
+                for (int ii = 0; ii < Q; ++ii) S_(c * NQ + at(qz, qy, ii)) = o[ii];
+                Line32<Q>::tv(gy[c], o);
+#pragma unroll
+                for (int ii = 0; ii < Q; ++ii) S_(OFF_Y + c * NQ + at(qz, qy, ii)) = o[ii];
+                Line32<Q>::tv(gz[c], o);
+#pragma unroll
+                for (int ii = 0; ii < Q; ++ii) S_(OFF_Z + c * NQ + at(qz, qy, ii)) = o[ii];
+            }
             S_(OFF_PD + 0 * L + qy + Q * qz) = Pd[0];
             S_(OFF_PD + 1 * L + qy + Q * qz) = Pd[1];
         }
@@ -254,16 +327,13 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1), MINB)
                     py[q] = S_(OFF_Y + c * NQ + at(qz, q, i));
                     pz[q] = S_(OFF_Z + c * NQ + at(qz, q, i));
                 }
+                float r[Q], rz[Q];
+                Line32<Q>::tvd(pv, py, r);
+                Line32<Q>::tv(pz, rz);
 #pragma unroll
                 for (int jj = 0; jj < Q; ++jj) {
-                    float r = 0.f, rz = 0.f;
-#pragma unroll
-                    for (int q = 0; q < Q; ++q) {
-                        r += (float)B.S[q][jj] * pv[q] + (float)B.D[q][jj] * py[q];
-                        rz += (float)B.S[q][jj] * pz[q];
-                    }
-                    S_(c * NQ + at(qz, jj, i)) = r;
-                    S_(OFF_Z + c * NQ + at(qz, jj, i)) = rz;
+                    S_(c * NQ + at(qz, jj, i)) = r[jj];
+                    S_(OFF_Z + c * NQ + at(qz, jj, i)) = rz[jj];
                 }
             }
             if (yp && l < 2 * Q) {  // divergence row: y-sweep [jx][jy][qz]
@@ -293,13 +363,11 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1), MINB)
                     r[q] = S_(c * NQ + at(q, j, i));
                     rz[q] = S_(OFF_Z + c * NQ + at(q, j, i));
                 }
+                float o[Q];
+                Line32<Q>::tvd(r, rz, o);
 #pragma unroll
-                for (int k = 0; k < Q; ++k) {
-                    float o = 0.f;
-#pragma unroll
-                    for (int q = 0; q < Q; ++q) o += (float)B.S[q][k] * r[q] + (float)B.D[q][k] * rz[q];
-                    if (keep[k]) atomicAdd(&y[c * m.Nu + zbase + k * MM], o);
-                }
+                for (int k = 0; k < Q; ++k)
+                    if (keep[k]) atomicAdd(&y[c * m.Nu + zbase + k * MM], o[k]);
             }
             if (yp && l < 4) {  // divergence row: z-sweep, Q1 node (jx, jy, jz)
                 const int jx = l % 2, jy = l / 2;
@@ -329,13 +397,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1), MINB)
                     r[q] = S_(c * NQ + at(q, j, i));
                     rz[q] = S_(OFF_Z + c * NQ + at(q, j, i));
                 }
-#pragma unroll
-                for (int k = 0; k < Q; ++k) {
-                    float v = 0.f;
-#pragma unroll
-                    for (int q = 0; q < Q; ++q) v += (float)B.S[q][k] * r[q] + (float)B.D[q][k] * rz[q];
-                    o[c][k] = v;
-                }
+                Line32<Q>::tvd(r, rz, o[c]);
             }
             if (div) {
 #pragma unroll
@@ -373,7 +435,7 @@ static int launch32(const evap_mesh* h, const MeshArgs<float>& m, const Scale32&
     constexpr int CB = 32;                // one warp per line: 288 / 512 threads
     constexpr int MINB = P == 2 ? EVAP_M32_MINB2 : 1;  // 35 KB / 80 KB of shared memory per block
     if (!h->deterministic) {
-        const unsigned grid = (unsigned)(((m.n + CB - 1) / CB) * (int64_t)m.n * m.n);
+        const unsigned grid = (unsigned)((m.ncell + CB - 1) / CB);
         k_momentum32<P, CB, MINB, false><<<grid, CB * L, 0, s>>>(m, hs, h->cell_code, h->table_index, h->table32, h->qc32, x,
                                                            y, yp, -1);
         EVAP_CHECK_LAUNCH("momentum32");
