@@ -47,7 +47,7 @@ struct MeshArgs {
 };
 
 enum CellCode : int8_t { CELL_GAS = 0, CELL_LIQUID = 1, CELL_TABLE = 2 };
-constexpr int TAB_K = 6;  // table entries per quadrature point: rho, mu, z n_x, z n_y, z n_z, v_dil
+constexpr int TAB_K = 7;  // table entries per quadrature point: rho, mu, z n_x, z n_y, z n_z, v_dil, delta
 constexpr int QC_K = 19;  // cached momentum coefficients per quadrature point (see k_qp_coeffs)
 constexpr int QC32_K = 12;  // of which the u0 terms, in FP32 for the FP32 apply (slots 1..12)
 

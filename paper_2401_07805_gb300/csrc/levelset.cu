@@ -2,20 +2,21 @@
 //   EVAP_ADVECT      y_i = sum_q W [ N_i x + theta dt N_i (u_Gamma . grad x) ]            Eq. (weakFormLevelSet), CN
 //   EVAP_REINIT      y_i = sum_q W [ N_i x / dtau + eps (grad N_i . n)(grad x . n) ]      Eq. (reinitialization)
 //   EVAP_REINIT_RHS  y_i = sum_q W [ N_i x / dtau + (grad N_i . n) (1 - x^2) / 2 ]        explicit compressive flux
+// The FP64 pipe bounds the FP64 reinitialization operators, so they run by sum factorization (q1_points.cuh).  Measured at
+// 64^3 (us): operator 454 -> 208, explicit side 413 -> 180 (direct sums over nodes and points before).
 // with n the frozen normal at the quadrature point: grad phi / |grad phi| of the level set (Eq. normal_vector), or,
 // when a nodal normal field is set (e.g. the projected normal of Eq. normal_vector_regularized), its normalized
-// interpolant (ls_frozen_normal).  The FP64 advection runs in double-float arithmetic (the FP64 pipe bounds the FP64
-// version), sum-factorized (k_levelset_advect_sf; k_levelset_advect_df evaluates the same sums directly); the
-// reinitialization operators stay in FP64.
+// interpolant (frozen_normals).  The FP64 advection runs in double-float arithmetic (the FP64 pipe bounds the FP64
+// version), sum-factorized (k_levelset_advect_sf); the reinitialization operators stay in FP64.
 #include <type_traits>
 
 #include "dfloat.cuh"
-#include "physics.cuh"
+#include "q1_points.cuh"
 
 namespace evap {
 
 template <typename T, int MODE, bool DET>
-__global__ void __launch_bounds__(128) k_levelset(MeshArgs<T> m, Basis<T> bas, const T* __restrict__ phi,
+__global__ void __launch_bounds__(128) k_levelset(MeshArgs<T> m, const T* __restrict__ phi,
                                                   const T* __restrict__ nf, const T* __restrict__ ug,
                                                   const T* __restrict__ x, T* __restrict__ y, int colour) {
     int cx, cy, cz;
@@ -45,131 +46,44 @@ __global__ void __launch_bounds__(128) k_levelset(MeshArgs<T> m, Basis<T> bas, c
             pv[j] = phi[node[j]];
         }
     }
-    T out[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) out[j] = 0;
+    T out[8], X[8], gx[4], gy[4], gz[4];  // values and reference gradient (physical gradient = reference / h)
     const T ih = m.inv_h;
     const T W = T(0.125) * m.vol_w;  // 2-point Gauss weights 1/2 in each direction
+    q1_points(xv, X, gx, gy, gz);
+    if (MODE == EVAP_ADVECT) {
+        T U[3][8], F[8], d0[4], d1[4], d2[4];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        // shape values and reference derivatives at the point: compile-time constants once the loops are unrolled
-        const int qx = q & 1, qy = (q >> 1) & 1, qz = q >> 2;
-        const T tx = T(g2_point(qx)), ty = T(g2_point(qy)), tz = T(g2_point(qz));
-        const T Nx[2] = {T(1) - tx, tx}, Ny[2] = {T(1) - ty, ty}, Nz[2] = {T(1) - tz, tz};
-        const T Dd[2] = {T(-1), T(1)};
-        T N[8], dR[8][3];
+        for (int k = 0; k < 3; ++k) q1_points(uv[k], U[k], d0, d1, d2);
+        const T c = m.theta * m.dt * ih;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int ja = j & 1, jb = (j >> 1) & 1, jc = j >> 2;
-            N[j] = Nx[ja] * Ny[jb] * Nz[jc];
-            dR[j][0] = Dd[ja] * Ny[jb] * Nz[jc];
-            dR[j][1] = Nx[ja] * Dd[jb] * Nz[jc];
-            dR[j][2] = Nx[ja] * Ny[jb] * Dd[jc];
+        for (int q = 0; q < 8; ++q) {
+            const int qx = q & 1, qy = (q >> 1) & 1, qz = q >> 2;
+            F[q] = W * (X[q] + c * (U[0][q] * gx[qy + 2 * qz] + U[1][q] * gy[qx + 2 * qz] + U[2][q] * gz[qx + 2 * qy]));
         }
-        T X = 0, GX[3] = {0, 0, 0};  // value and reference gradient (physical gradient = GX / h)
+        q1_test<false>(F, F, F, F, out);
+    } else {
+        T nv[8][3], F[8], G0[8], G1[8], G2[8];  // G: flux tested with the reference gradients (physical flux / h)
+        frozen_normals<T>(nf != nullptr, uv, pv, nv);
+        const T wm = W / m.dtau, wd = MODE == EVAP_REINIT ? W * m.eps * ih * ih : W * T(0.5) * ih;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            X += N[j] * xv[j];
-#pragma unroll
-            for (int d = 0; d < 3; ++d) GX[d] += dR[j][d] * xv[j];
+        for (int q = 0; q < 8; ++q) {
+            const int qx = q & 1, qy = (q >> 1) & 1, qz = q >> 2;
+            F[q] = wm * X[q];
+            const T s = MODE == EVAP_REINIT
+                            ? wd * (gx[qy + 2 * qz] * nv[q][0] + gy[qx + 2 * qz] * nv[q][1] + gz[qx + 2 * qy] * nv[q][2])
+                            : wd * (T(1) - X[q] * X[q]);
+            G0[q] = s * nv[q][0];
+            G1[q] = s * nv[q][1];
+            G2[q] = s * nv[q][2];
         }
-        T Fv, Gf[3] = {0, 0, 0};  // Gf: flux tested with the reference gradients (physical flux / h)
-        if (MODE == EVAP_ADVECT) {
-            T U[3] = {0, 0, 0};
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) U[k] += N[j] * uv[k][j];
-            Fv = W * (X + m.theta * m.dt * ih * (U[0] * GX[0] + U[1] * GX[1] + U[2] * GX[2]));
-        } else {
-            T nv[3];
-            ls_frozen_normal<T>(nf ? uv : nullptr, pv, N, dR, T(1), nv);  // |grad_ref phi| = |grad phi| h
-            Fv = W * X / m.dtau;
-            const T s = (MODE == EVAP_REINIT) ? W * m.eps * ih * ih * (GX[0] * nv[0] + GX[1] * nv[1] + GX[2] * nv[2])
-                                              : W * T(0.5) * ih * (T(1) - X * X);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) Gf[d] = s * nv[d];
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) out[j] += N[j] * Fv + dR[j][0] * Gf[0] + dR[j][1] * Gf[1] + dR[j][2] * Gf[2];
+        q1_test<true>(F, G0, G1, G2, out);
     }
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc_add(&y[node[j]], out[j], DET);
 }
 
-// EVAP_ADVECT for the FP64 applies in double-float arithmetic (dfloat.cuh): the same sums with x converted per node,
-// u_Gamma read from its double-float copy, every product and sum on hi + lo FP32 pairs, the scatter in FP64.  The
-// shape values at the Gauss points are compile-time doubles split into pairs.
-template <bool DET>
-__global__ void __launch_bounds__(128) k_levelset_advect_df(MeshArgs<double> m, dfl W, dfl thdt_ih,
-                                                            const float2* __restrict__ ug, const double* __restrict__ x,
-                                                            double* __restrict__ y, int colour) {
-    int cx, cy, cz;
-    if constexpr (DET) {
-        if (!colour_cell(blockIdx.x * (int64_t)blockDim.x + threadIdx.x, m.n, colour, cx, cy, cz)) return;
-    } else {  // written out: the shared helper's form of this test cost the atomic variant 100 registers
-        const int64_t cell = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-        if (cell >= m.ncell) return;
-        cx = (int)(cell % m.n), cy = (int)((cell / m.n) % m.n), cz = (int)(cell / ((int64_t)m.n * m.n));
-    }
-    const int n = m.n;
-    const int64_t m1 = n + 1;
-    int64_t node[8];
-    dfl xv[8], uv[3][8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        node[j] = (cx + (j & 1)) + m1 * ((cy + ((j >> 1) & 1)) + m1 * (cz + (j >> 2)));
-        xv[j] = df_from_double(x[node[j]]);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) uv[k][j] = ld_df(ug + k * m.Nphi + node[j]);
-    }
-    dfl out[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) out[j] = dfl{0.f, 0.f};
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int qx = q & 1, qy = (q >> 1) & 1, qz = q >> 2;
-        const double tx = g2_point(qx), ty = g2_point(qy), tz = g2_point(qz);
-        const double Nx[2] = {1.0 - tx, tx}, Ny[2] = {1.0 - ty, ty}, Nz[2] = {1.0 - tz, tz};
-        dfl N[8], dR[8][3];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int ja = j & 1, jb = (j >> 1) & 1, jc = j >> 2;
-            const double sx = ja ? 1.0 : -1.0, sy = jb ? 1.0 : -1.0, sz = jc ? 1.0 : -1.0;
-            N[j] = df_from_double(Nx[ja] * Ny[jb] * Nz[jc]);
-            dR[j][0] = df_from_double(sx * Ny[jb] * Nz[jc]);
-            dR[j][1] = df_from_double(Nx[ja] * sy * Nz[jc]);
-            dR[j][2] = df_from_double(Nx[ja] * Ny[jb] * sz);
-        }
-        dfl X = df_prod(N[0], xv[0]), GX[3], U[3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            GX[d] = df_prod(dR[0][d], xv[0]);
-            U[d] = df_prod(N[0], uv[d][0]);
-        }
-#pragma unroll
-        for (int j = 1; j < 8; ++j) {
-            df_fma(X, N[j], xv[j]);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                df_fma(GX[d], dR[j][d], xv[j]);
-                df_fma(U[d], N[j], uv[d][j]);
-            }
-        }
-        dfl ug_gx = df_prod(df_norm(U[0]), df_norm(GX[0]));
-        df_fma(ug_gx, df_norm(U[1]), df_norm(GX[1]));
-        df_fma(ug_gx, df_norm(U[2]), df_norm(GX[2]));
-        dfl v = df_norm(X);
-        df_fma(v, thdt_ih, df_norm(ug_gx));
-        const dfl Fv = df_mul(W, df_norm(v));
-#pragma unroll
-        for (int j = 0; j < 8; ++j) df_fma(out[j], N[j], Fv);
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc_add(&y[node[j]], df_to_double(df_norm(out[j])), DET);
-}
-
-// The same operator by sum factorization: the trilinear interpolation of x and u_Gamma to the 2^3 Gauss points and
+// EVAP_ADVECT for the FP64 applies in double-float arithmetic (dfloat.cuh) with x converted per node, u_Gamma read from its
+// double-float copy and the scatter in FP64, by sum factorization: the trilinear interpolation of x and u_Gamma to the 2^3 Gauss points and
 // the testing with the shape functions as three 1D sweeps of the 2 x 2 matrix N[q][j] (N_0 = 1 - t, N_1 = t at the
 // Gauss points t), the reference gradient of x as differences along its own direction interpolated along the other
 // two: 132 two-term double-float dot products per cell in place of the direct sums' 8 x 7 eight-term ones.
@@ -300,16 +214,10 @@ __global__ void __launch_bounds__(128) k_levelset_advect_sf(MeshArgs<double> m, 
         }
 }
 
-// Level-set advection kernel: 1 the sum-factorized k_levelset_advect_sf, 0 the direct sums of k_levelset_advect_df.
-// Measured at 64^3 (275 k DoFs, 100 back-to-back applies): 45.2 against 57.8 us per apply.
-#ifndef EVAP_LS_SF
-#define EVAP_LS_SF 1
-#endif
-
+// (The sum-factorized advection took 45.2 us per apply at 64^3, 275 k DoFs, where direct 8-point sums took 57.8.)
 template <typename T>
 int launch_levelset(evap_mesh* h, int mode, const T* x, T* y, cudaStream_t s) {
     const MeshArgs<T> m = ls_args<T>(h);  // Q1 on the level-set mesh
-    const Basis<T> b = cast_basis<T>(h->b);
     const bool dbl = sizeof(T) == 8;
     const T* phi = dbl ? (const T*)h->phi : (const T*)h->phi32;
     const T* ug = dbl ? (const T*)h->ugamma : (const T*)h->ugamma32;
@@ -329,19 +237,18 @@ int launch_levelset(evap_mesh* h, int mode, const T* x, T* y, cudaStream_t s) {
                 if (mode == EVAP_ADVECT) {  // FP64-accurate advection in double-float arithmetic
                     const dfl W = df_from_double(0.125 * (double)m.vol_w);  // 2-point Gauss weights 1/2 per direction
                     const dfl thdt_ih = df_from_double((double)m.theta * (double)m.dt * (double)m.inv_h);
-                    (EVAP_LS_SF ? k_levelset_advect_sf<DET> : k_levelset_advect_df<DET>)<<<grid, threads, 0, s>>>(
-                        m, W, thdt_ih, (const float2*)h->ugammadf,
+                    k_levelset_advect_sf<DET><<<grid, threads, 0, s>>>(m, W, thdt_ih, (const float2*)h->ugammadf,
                                                                        (const double*)x, (double*)y, colour);
                     done = true;
                 }
             }
             if (done) {
             } else if (mode == EVAP_ADVECT) {
-                k_levelset<T, EVAP_ADVECT, DET><<<grid, threads, 0, s>>>(m, b, phi, nullptr, ug, x, y, colour);
+                k_levelset<T, EVAP_ADVECT, DET><<<grid, threads, 0, s>>>(m, phi, nullptr, ug, x, y, colour);
             } else if (mode == EVAP_REINIT) {
-                k_levelset<T, EVAP_REINIT, DET><<<grid, threads, 0, s>>>(m, b, phi, nf, ug, x, y, colour);
+                k_levelset<T, EVAP_REINIT, DET><<<grid, threads, 0, s>>>(m, phi, nf, ug, x, y, colour);
             } else {
-                k_levelset<T, EVAP_REINIT_RHS, DET><<<grid, threads, 0, s>>>(m, b, phi, nf, ug, x, y, colour);
+                k_levelset<T, EVAP_REINIT_RHS, DET><<<grid, threads, 0, s>>>(m, phi, nf, ug, x, y, colour);
             }
             EVAP_CHECK_LAUNCH("levelset");
         }

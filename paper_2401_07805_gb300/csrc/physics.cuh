@@ -59,37 +59,8 @@ __device__ __forceinline__ Material material(double phi, double gx, double gy, d
     return r;
 }
 
-// Frozen normal of the reinitialization operators at a Q1 quadrature point (Eq. reinitialization): with a nodal
-// field nf (nf[c][j] at the cell's 8 nodes) the normalized interpolant n_h / |n_h| (zero where |n_h| <= 1e-4), else the
-// unit normal grad phi / |grad phi| (zero where |grad phi| h <= GRAD_TINY).  N[j], G[j][d]: Q1 values and
-// physical gradients at the point; pv[j]: phi at the nodes.
+// A nodal normal field interpolated to a point is normalized there, and read as 0 where |n_h| <= NODAL_NORMAL_TINY.
 constexpr double NODAL_NORMAL_TINY = 1e-4;
-template <typename T>
-__device__ __forceinline__ void ls_frozen_normal(const T (*nf)[8], const T pv[8], const T N[8], const T (*G)[3], T h,
-                                                 T nv[3]) {
-    T g[3] = {T(0), T(0), T(0)};
-    if (nf) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-#pragma unroll
-            for (int d = 0; d < 3; ++d) g[d] += N[j] * nf[d][j];
-    } else {
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-#pragma unroll
-            for (int d = 0; d < 3; ++d) g[d] += G[j][d] * pv[j];
-    }
-    const T gn = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
-    const bool ok = nf ? gn > T(NODAL_NORMAL_TINY) : gn * h > T(GRAD_TINY);
-    nv[0] = nv[1] = nv[2] = T(0);
-    if (ok) {
-        const T ig = T(1) / gn;
-        nv[0] = g[0] * ig;
-        nv[1] = g[1] * ig;
-        nv[2] = g[2] * ig;
-    }
-}
-
 // c_1 = 1/rho_g - 1/rho_l, the factor of mdot delta in the dilation rate v = div u (Eq. evaporDil).  Sign: the
 // printed Eq. (evaporDil) has the bracket reversed with respect to the paper's 1D solution (App. A,
 // Eq. stefan_diffuse_velocity: div u = mdot (1/rho_g - 1/rho_l) delta) and to the c_1 of the variant-1 derivation;

@@ -98,7 +98,7 @@ __global__ void k_classify(MeshArgs<double> m, Basis<double> b, const double* __
 }
 
 // Table entries at one quadrature point of a table cell: rho, mu, z n (z = correction gate), v_dil (Eq. evaporDil
-// with the sign of App. A, dilation_coefficient).
+// with the sign of App. A, dilation_coefficient), delta.
 __global__ void k_fill_table(MeshArgs<double> m, Basis<double> b, const double* __restrict__ phi,
                              const double* __restrict__ mdot, const int8_t* __restrict__ code,
                              const int32_t* __restrict__ tindex, double* table, float* table32, float2* adj) {
@@ -116,7 +116,7 @@ __global__ void k_fill_table(MeshArgs<double> m, Basis<double> b, const double* 
     const Material mat = material(ph, g[0], g[1], g[2], m);
     const double z = correction_on(m, mat.zone) ? 1.0 : 0.0;
     const double vals[TAB_K] = {mat.rho, mat.mu, z * mat.n[0], z * mat.n[1], z * mat.n[2],
-                                md * dilation_coefficient(m) * mat.delta};
+                                md * dilation_coefficient(m) * mat.delta, mat.delta};
     const int64_t base = (int64_t)tindex[cell] * TAB_K * nq + q;
 #pragma unroll
     for (int k = 0; k < TAB_K; ++k) {
