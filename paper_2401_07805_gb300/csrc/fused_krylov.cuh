@@ -15,7 +15,7 @@
 // reports EVAP_ETIMEOUT); the cooperative launch makes all blocks co-resident, so the limit is only a guard.
 #pragma once
 
-#include "dfloat.cuh"
+#include "df_lines.cuh"
 
 namespace evap {
 
@@ -126,87 +126,79 @@ __device__ __forceinline__ void grid_sum_df(const float2* part, float2* sh, dfl 
 // ------------------------------------------------------------------------------------------- 27-point stencils
 // The operators as 27-point stencils on the Q1 node lattice (n + 1 nodes per direction), x as pairs: row `node` is
 // sum_s C_s(node) x(node + o_s) over the offsets o_s = (dx, dy, dz) in {-1, 0, 1}^3, s = 9 (dz + 1) + 3 (dy + 1) +
-// (dx + 1), one double-float FMA per neighbour.  Offsets that leave the lattice are skipped.  Node indices fit 32
-// bits (checked on the host).
-template <class Coef>
-__device__ __forceinline__ dfl stencil27(int n, int64_t node, const float2* x, Coef coef) {
-    const unsigned m1 = (unsigned)n + 1u, nd = (unsigned)node;
-    const unsigned t = nd / m1, i = nd - t * m1, k = t / m1, j = t - k * m1;
-    dfl acc{0.f, 0.f};
-#pragma unroll
-    for (int dz = -1; dz <= 1; ++dz) {
-        if ((dz < 0 && k == 0u) || (dz > 0 && k == (unsigned)n)) continue;
-#pragma unroll
-        for (int dy = -1; dy <= 1; ++dy) {
-            if ((dy < 0 && j == 0u) || (dy > 0 && j == (unsigned)n)) continue;
-            const float2* xr = x + (nd + (unsigned)(dy * (int)m1 + dz * (int)(m1 * m1)));
-#pragma unroll
-            for (int dx = -1; dx <= 1; ++dx) {
-                if ((dx < 0 && i == 0u) || (dx > 0 && i == (unsigned)n)) continue;
-                df_fma(acc, coef(i, j, k, 9 * (dz + 1) + 3 * (dy + 1) + (dx + 1)), ld_df(xr + dx));
-            }
-        }
-    }
-    return df_norm(acc);
-}
+// (dx + 1).  Neither operator branches on the lattice boundary, so that a node's 27 loads are in flight together (with a
+// test per neighbour the CG took 18.5 and 24 us per iteration at 64^3 for the two operators, now 15 and 19).  Node indices fit 32 bits
+// (checked on the host).
 
-// (M + c K) for one field: constant coefficients per boundary class.  A node's class in one direction is 0 (first
-// node), 1 (interior) or 2 (last node); table[27 class + s] holds C_s of class 9 cz + 3 cy + cx as pairs
-// (helmholtz_table), staged in shared memory by load().
+// (M + c K) for one field: constant coefficients, 4 distinct ones (by the number of nonzero components of the offset: 0
+// centre, 1 face, 2 edge, 3 corner).  A boundary row is the interior row with the missing neighbours replaced by their
+// mirror images, times 1/2 per boundary direction: the 1D rows h/3, h/6 and 1/h, -1/h of an end node are half of the
+// mirrored interior rows, and the operator is a sum of their tensor products.  So the neighbours of one kind are added
+// first: 23 additions and 4 multiplications per node.
 struct HelmholtzStencil {
-    static constexpr int SMEM = 27 * 27;  // pairs
+    static constexpr int SMEM = 0;
     int n;
-    const float2* table;
-    __device__ __forceinline__ void load(float2* sm) const {
-        for (int t = threadIdx.x; t < SMEM; t += blockDim.x) sm[t] = table[t];
-    }
-    __device__ __forceinline__ dfl row(int64_t node, const float2* x, const float2* sm) const {
-        return stencil27(n, node, x, [&](unsigned i, unsigned j, unsigned k, int s) {
-            const unsigned cx = i == 0u ? 0u : (i == (unsigned)n ? 2u : 1u);
-            const unsigned cy = j == 0u ? 0u : (j == (unsigned)n ? 2u : 1u);
-            const unsigned cz = k == 0u ? 0u : (k == (unsigned)n ? 2u : 1u);
-            return ld_df(sm + 27u * (9u * cz + 3u * cy + cx) + (unsigned)s);
-        });
-    }
-    // the diagonal entry (offset 13 = (0, 0, 0)) to FP32, for the Jacobi scaling
-    __device__ __forceinline__ float diag(int64_t node, const float2* sm) const {
+    dfl c[4];
+    __device__ __forceinline__ void load(float2*) const {}
+    __device__ __forceinline__ dfl row(int64_t node, const float2* x, const float2*) const {
         const unsigned m1 = (unsigned)n + 1u, nd = (unsigned)node;
         const unsigned t = nd / m1, i = nd - t * m1, k = t / m1, j = t - k * m1;
-        const unsigned cx = i == 0u ? 0u : (i == (unsigned)n ? 2u : 1u);
-        const unsigned cy = j == 0u ? 0u : (j == (unsigned)n ? 2u : 1u);
-        const unsigned cz = k == 0u ? 0u : (k == (unsigned)n ? 2u : 1u);
-        return sm[27u * (9u * cz + 3u * cy + cx) + 13u].x;
+        const int sy = (int)m1, sz = (int)(m1 * m1);
+        const int ox[2] = {i == 0u ? 1 : -1, i == (unsigned)n ? -1 : 1};
+        const int oy[2] = {j == 0u ? sy : -sy, j == (unsigned)n ? -sy : sy};
+        const int oz[2] = {k == 0u ? sz : -sz, k == (unsigned)n ? -sz : sz};
+        const float2* p = x + nd;
+        const dfl u0 = ld_df(p);
+        dfl f = df_addl(df_addl(ld_df(p + ox[0]), ld_df(p + ox[1])),
+                        df_addl(df_addl(ld_df(p + oy[0]), ld_df(p + oy[1])), df_addl(ld_df(p + oz[0]), ld_df(p + oz[1]))));
+        dfl e{0.f, 0.f}, v{0.f, 0.f};
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const dfl exy = df_addl(ld_df(p + ox[0] + oy[b]), ld_df(p + ox[1] + oy[b]));
+            const dfl exz = df_addl(ld_df(p + ox[0] + oz[b]), ld_df(p + ox[1] + oz[b]));
+            const dfl eyz = df_addl(ld_df(p + oy[0] + oz[b]), ld_df(p + oy[1] + oz[b]));
+            const dfl se = df_addl(df_addl(exy, exz), eyz);
+            const dfl v0 = df_addl(ld_df(p + ox[0] + oy[0] + oz[b]), ld_df(p + ox[1] + oy[0] + oz[b]));
+            const dfl v1 = df_addl(ld_df(p + ox[0] + oy[1] + oz[b]), ld_df(p + ox[1] + oy[1] + oz[b]));
+            const dfl sv = df_addl(v0, v1);
+            e = b == 0 ? se : df_addl(e, se);
+            v = b == 0 ? sv : df_addl(v, sv);
+        }
+        dfl acc = df_prod(c[0], u0);
+        df_fma(acc, c[1], df_norm(f));
+        df_fma(acc, c[2], df_norm(e));
+        df_fma(acc, c[3], df_norm(v));
+        return df_scale2(df_norm(acc), scale(i, j, k));
+    }
+    __device__ __forceinline__ float scale(unsigned i, unsigned j, unsigned k) const {
+        return (i == 0u || i == (unsigned)n ? 0.5f : 1.f) * (j == 0u || j == (unsigned)n ? 0.5f : 1.f) *
+               (k == 0u || k == (unsigned)n ? 0.5f : 1.f);
+    }
+    // the diagonal entry to FP32, for the Jacobi scaling (n = 1 adds the mirrored neighbours to it, but any positive
+    // diagonal is a valid preconditioner)
+    __device__ __forceinline__ float diag(int64_t node, const float2*) const {
+        const unsigned m1 = (unsigned)n + 1u, nd = (unsigned)node;
+        const unsigned t = nd / m1, i = nd - t * m1, k = t / m1, j = t - k * m1;
+        return c[0].hi * scale(i, j, k);
     }
 };
 
-// Host: the 27 x 27 coefficient table of (M + c K) on a lattice of spacing h, formed in FP64 from the 1D rows
-// h/6, 2h/3, h/6 (mass) and -1/h, 2/h, -1/h (stiffness), with h/3 and 1/h as the centre entry of an end node.
-inline void helmholtz_table(double h, double c, float2* out) {
-    double M[3][3], K[3][3];  // [class][offset + 1]
-    const double mi[3] = {h / 6.0, 2.0 * h / 3.0, h / 6.0}, ki[3] = {-1.0 / h, 2.0 / h, -1.0 / h};
-    for (int o = 0; o < 3; ++o) {
-        M[1][o] = mi[o];
-        K[1][o] = ki[o];
-    }
-    M[0][0] = 0.0;     M[0][1] = h / 3.0; M[0][2] = h / 6.0;
-    K[0][0] = 0.0;     K[0][1] = 1.0 / h; K[0][2] = -1.0 / h;
-    M[2][0] = h / 6.0; M[2][1] = h / 3.0; M[2][2] = 0.0;
-    K[2][0] = -1.0 / h; K[2][1] = 1.0 / h; K[2][2] = 0.0;
-    for (int cz = 0; cz < 3; ++cz)
-        for (int cy = 0; cy < 3; ++cy)
-            for (int cx = 0; cx < 3; ++cx)
-                for (int dz = 0; dz < 3; ++dz)
-                    for (int dy = 0; dy < 3; ++dy)
-                        for (int dx = 0; dx < 3; ++dx) {
-                            const double mx = M[cx][dx], my = M[cy][dy], mz = M[cz][dz];
-                            const double v = mx * my * mz + c * (K[cx][dx] * my * mz + mx * K[cy][dy] * mz +
-                                                                 mx * my * K[cz][dz]);
-                            const dfl d = df_from_double(v);
-                            out[27 * (9 * cz + 3 * cy + cx) + 9 * dz + 3 * dy + dx] = make_float2(d.hi, d.lo);
-                        }
+// Host: the interior row of (M + c K) on a lattice of spacing h, formed in FP64 from the 1D rows h/6, 2h/3, h/6 (mass) and
+// -1/h, 2/h, -1/h (stiffness).
+inline HelmholtzStencil helmholtz_op(int n, double h, double c) {
+    HelmholtzStencil op;
+    op.n = n;
+    const double m0 = 2.0 * h / 3.0, m1 = h / 6.0, k0 = 2.0 / h, k1 = -1.0 / h;
+    op.c[0] = df_from_double(m0 * m0 * m0 + c * 3.0 * k0 * m0 * m0);
+    op.c[1] = df_from_double(m1 * m0 * m0 + c * (k1 * m0 * m0 + 2.0 * m1 * k0 * m0));
+    op.c[2] = df_from_double(m1 * m1 * m0 + c * (2.0 * k1 * m1 * m0 + m1 * m1 * k0));
+    op.c[3] = df_from_double(m1 * m1 * m1 + c * 3.0 * k1 * m1 * m1);
+    return op;
 }
 
-// An operator assembled per node: C[s N + node] = C_s(node) as pairs (coalesced per offset).
+// An operator assembled per node: C[s N + node] = C_s(node) as pairs (coalesced per offset), 0 for the offsets that leave
+// the lattice.  Those products are formed all the same, with whatever the vector's memory holds there: it has
+// stencil_guard(n) zero entries in front, and every entry read is finite.
 struct NodeStencil {
     static constexpr int SMEM = 0;
     int n;
@@ -214,12 +206,30 @@ struct NodeStencil {
     const float2* C;
     __device__ __forceinline__ void load(float2*) const {}
     __device__ __forceinline__ dfl row(int64_t node, const float2* x, const float2*) const {
+        const unsigned m1 = (unsigned)n + 1u;
         const float2* c = C + node;
-        const int64_t NN = N;
-        return stencil27(n, node, x, [&](unsigned, unsigned, unsigned, int s) { return ld_df(c + s * NN); });
+        const float2* p = x + node;
+        dfl acc{0.f, 0.f};
+#pragma unroll
+        for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+            for (int dy = -1; dy <= 1; ++dy) {
+                const float2* xr = p + (dy * (int)m1 + dz * (int)(m1 * m1));
+#pragma unroll
+                for (int dx = -1; dx <= 1; ++dx) {
+                    const int s = 9 * (dz + 1) + 3 * (dy + 1) + (dx + 1);
+                    if (s == 0)
+                        acc = df_prod(ld_df(c), ld_df(xr + dx));
+                    else
+                        df_fma(acc, ld_df(c + s * N), ld_df(xr + dx));
+                }
+            }
+        return df_norm(acc);
     }
     __device__ __forceinline__ float diag(int64_t node, const float2*) const { return C[13 * N + node].x; }
 };
+// entries a row may read before the first or after the last of its vector
+inline int64_t stencil_guard(int n) { return (int64_t)(n + 1) * (n + 1) + (n + 1) + 1; }
 
 // ------------------------------------------------------------------------------------ conjugate gradients
 // A x = b from x = 0, CG preconditioned by the operator's diagonal D (op.diag, in FP32), in the Chronopoulos-Gear
@@ -397,6 +407,7 @@ __global__ void __launch_bounds__(FK_THREADS) k_gmres_fused(Op op, int64_t N, in
         for (int64_t i = i0; i < N; i += stride) {
             dinv[i] = 1.0f / op.diag(i, op_sm);
             st_df(xd + i, df_from_double(x[i]));
+            st_df(z + i, zero);  // (read behind xd with zero coefficients before it is written)
             const dfl bi = df_from_double(b[i]);
             df_fma(bb, bi, bi);
         }
@@ -600,7 +611,7 @@ __global__ void __launch_bounds__(FK_THREADS) k_cg_fused32(Op op, int64_t N, con
         const float ri = (float)b[i], di = 1.0f / op.diag(i, op_sm32);
         xs[i] = 0.f;
         r[i] = ri;
-        u[i] = ri * di;
+        u[op.pos(i)] = ri * di;
         p[i] = 0.f;
         sv[i] = 0.f;
         dinv[i] = di;
@@ -611,7 +622,7 @@ __global__ void __launch_bounds__(FK_THREADS) k_cg_fused32(Op op, int64_t N, con
     for (;;) {
         float acc[3] = {0.f, 0.f, 0.f};  // (r, u), (w, u), (r, r)
         for (int64_t i = i0; i < N; i += stride) {
-            const float wi = op.row(i, u, op_sm32), ui = u[i], ri = r[i];
+            const float wi = op.row(i, u, op_sm32), ui = u[op.pos(i)], ri = r[i];
             w[i] = wi;
             acc[0] = fmaf(ri, ui, acc[0]);
             acc[1] = fmaf(wi, ui, acc[1]);
@@ -658,13 +669,14 @@ __global__ void __launch_bounds__(FK_THREADS) k_cg_fused32(Op op, int64_t N, con
         ++it;
         const float alpha = s_alpha, beta = s_beta;
         for (int64_t i = i0; i < N; i += stride) {
-            const float pi = fmaf(beta, p[i], u[i]), si = fmaf(beta, sv[i], w[i]);
+            const unsigned pu = op.pos(i);
+            const float pi = fmaf(beta, p[i], u[pu]), si = fmaf(beta, sv[i], w[i]);
             const float ri = fmaf(-alpha, si, r[i]);
             p[i] = pi;
             sv[i] = si;
             xs[i] = fmaf(alpha, pi, xs[i]);
             r[i] = ri;
-            u[i] = ri * dinv[i];
+            u[pu] = ri * dinv[i];
         }
         if (!grid_barrier(gb, bar)) return;
     }
@@ -677,16 +689,15 @@ __global__ void __launch_bounds__(FK_THREADS) k_cg_fused32(Op op, int64_t N, con
 }
 
 // ------------------------------------------------------------------------------------------ host-side workspace
-// Workspace of the single-launch solvers, kept with the mesh (geometry.cu): nvec pair vectors of N_phi entries (or,
-// read as floats, 2 nvec float vectors), an FP32 vector, (GM_MAX + 2) CG_BLOCKS partial pairs, the barrier, 4 result
-// words and the Helmholtz coefficient table.
+// Workspace of the single-launch solvers, kept with the mesh (geometry.cu): stencil_guard zero pairs, nvec pair vectors of
+// N_phi entries (or, read as floats, 2 nvec float vectors), an FP32 vector, (GM_MAX + 2) CG_BLOCKS partial pairs, the
+// barrier and 4 result words.
 struct FusedSpace {
     float2* vec;  // vector k at vec + k N
     float* dinv;
     float2* part;
     GridBarrier* gb;
     double* out;
-    float2* table;
 };
 int fused_space(evap_mesh* h, int nvec, FusedSpace& f);
 // the launch's result words (iterations, |r|, |r0|) and its barrier's error word, after one synchronization

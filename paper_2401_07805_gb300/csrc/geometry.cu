@@ -291,10 +291,12 @@ static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 int fused_space(evap_mesh* h, int nvec, FusedSpace& f) {
     if (!h->geo_host) EVAP_CUDA(cudaMallocHost(&h->geo_host, 8 * sizeof(double)));  // the result words' mirror
-    const int64_t N = ls_args<double>(h).Nphi;
-    const size_t vbytes = al256((size_t)nvec * N * sizeof(float2)), dbytes = al256((size_t)N * sizeof(float));
+    const MeshArgs<double> lm = ls_args<double>(h);
+    const int64_t N = lm.Nphi;
+    const size_t gbytes = al256((size_t)stencil_guard(lm.n) * sizeof(float2));
+    const size_t vbytes = gbytes + al256((size_t)nvec * N * sizeof(float2)), dbytes = al256((size_t)N * sizeof(float));
     const size_t pbytes = al256((size_t)(GM_MAX + 2) * FK_MAX_BLOCKS * sizeof(float2));
-    const size_t tail = al256(sizeof(GridBarrier) + 4 * sizeof(double)) + HelmholtzStencil::SMEM * sizeof(float2);
+    const size_t tail = al256(sizeof(GridBarrier) + 4 * sizeof(double));
     const size_t need = vbytes + dbytes + pbytes + tail;
     if (h->geo_kry_bytes < need) {
         if (h->geo_kry) cudaFree(h->geo_kry);
@@ -302,15 +304,15 @@ int fused_space(evap_mesh* h, int nvec, FusedSpace& f) {
         h->geo_kry_bytes = 0;
         EVAP_CUDA(cudaMalloc(&h->geo_kry, need));
         h->geo_kry_bytes = need;
+        EVAP_CUDA(cudaMemset(h->geo_kry, 0, gbytes));  // the guard: read by boundary rows, written by nobody
     }
     char* base = (char*)h->geo_kry;
     const size_t vcap = h->geo_kry_bytes - dbytes - pbytes - tail;  // the vectors keep whatever room they had
-    f.vec = (float2*)base;
+    f.vec = (float2*)(base + gbytes);
     f.dinv = (float*)(base + vcap);
     f.part = (float2*)(base + vcap + dbytes);
     f.gb = (GridBarrier*)(base + vcap + dbytes + pbytes);
     f.out = (double*)(f.gb + 1);
-    f.table = (float2*)(base + vcap + dbytes + pbytes + al256(sizeof(GridBarrier) + 4 * sizeof(double)));
     return EVAP_OK;
 }
 
@@ -404,20 +406,6 @@ static int helmholtz_apply(evap_mesh* h, double c, int ncomp, const double* x, d
     return EVAP_OK;
 }
 
-// The Helmholtz stencil of the level-set mesh with its coefficient table uploaded to the workspace (the copy is
-// ordered before the solve on the stream; the host table is copied out before cudaMemcpyAsync returns).
-static int helmholtz_stencil(evap_mesh* h, const MeshArgs<double>& lm, double c, HelmholtzStencil& op, cudaStream_t s) {
-    FusedSpace f;
-    int rc = fused_space(h, 6, f);
-    if (rc) return rc;
-    float2 tab[HelmholtzStencil::SMEM];
-    helmholtz_table(lm.h, c, tab);
-    EVAP_CUDA(cudaMemcpyAsync(f.table, tab, sizeof(tab), cudaMemcpyHostToDevice, s));
-    op.n = lm.n;
-    op.table = f.table;
-    return EVAP_OK;
-}
-
 int geo_helmholtz(evap_mesh* h, double c, int ncomp, const double* x, double* y, cudaStream_t s) {
     return helmholtz_apply(h, c, ncomp, x, y, s);
 }
@@ -436,8 +424,7 @@ int geo_projected_normal(evap_mesh* h, double* n, int* iters, double* relres, cu
     if (iters) *iters = 0;
     if (relres) *relres = 0.0;
     int status = EVAP_OK;
-    HelmholtzStencil op;
-    if ((rc = helmholtz_stencil(h, lm, c, op, s))) return rc;
+    const HelmholtzStencil op = helmholtz_op(lm.n, lm.h, c);
     for (int d = 0; d < 3; ++d) {
         rc = cg_solve_fused(h, op, w.t0 + d * stride, n + d * Np, 1e-12, 1e-20, 1000, iters, relres, s);
         if (rc == EVAP_ENOTCONV) status = rc;
@@ -458,8 +445,7 @@ int geo_curvature(evap_mesh* h, const double* nf, double* kappa, int* iters, dou
     EVAP_CHECK_LAUNCH("curvature_rhs");
     if (iters) *iters = 0;
     if (relres) *relres = 0.0;
-    HelmholtzStencil op;
-    if ((rc = helmholtz_stencil(h, lm, c, op, s))) return rc;
+    const HelmholtzStencil op = helmholtz_op(lm.n, lm.h, c);
     return cg_solve_fused(h, op, w.b, kappa, 1e-12, 1e-20, 1000, iters, relres, s);
 }
 

@@ -10,7 +10,7 @@
 // the nodes within two cells (a 5^3 = 125-point stencil); S~ is symmetric, so the 63 offsets o >= 0 (in the
 // lexicographic order of (oz, oy, ox)) are stored, as FP32 [63][N_p]: offset o of node i is entry |l(o) - 62| of node
 // i (l(o) >= 62) or of node i + o (l(o) < 62), with l(o) = 25 (oz + 2) + 5 (oy + 2) + (ox + 2); entry 0 is the diagonal.
-// One thread per stored entry sums its (at most 5^3) velocity nodes in a fixed order: no atomics.
+// One thread per stored entry sums its velocity nodes (at most 7^3, for Q3) in a fixed order: no atomics.
 //
 // With the stencil, the Schur CG of every preconditioner application is one cooperative launch in FP32
 // (k_cg_fused32) instead of, per iteration, a matrix-free gradient and divergence over the whole velocity mesh.
@@ -39,100 +39,141 @@ __device__ __forceinline__ float factor1(const float (&t)[2][MAXQ], int P, int n
     return s;
 }
 
-__global__ void __launch_bounds__(128) k_schur_assemble(int n, int P, int M, unsigned faces, int64_t Nu, int64_t Np,
-                                                        SchurTables tab, const float* __restrict__ diag,
-                                                        float* __restrict__ S) {
-    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= 63 * Np) return;
-    const int e = (int)(idx / Np);
-    const int64_t node = idx - (int64_t)e * Np;
-    const int lin = 62 + e;
+// 1 / D on the free velocity DoFs, 0 on the Dirichlet ones (a warp walks x-lines of nodes)
+__global__ void __launch_bounds__(256) k_schur_inverse(int M, int64_t Nu, unsigned faces, const float* __restrict__ diag,
+                                                       float* __restrict__ inv) {
+    const int lines = 3 * M * M;
+    const int wpb = blockDim.x / 32, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    for (int line = blockIdx.x * wpb + warp; line < lines; line += gridDim.x * wpb) {
+        const int c = line / (M * M), rem = line - c * M * M, gz = rem / M, gy = rem - gz * M;
+        const bool cyz = ((faces & 4u) && gy == 0) || ((faces & 8u) && gy == M - 1) || ((faces & 16u) && gz == 0) ||
+                         ((faces & 32u) && gz == M - 1);
+        const int64_t off = c * Nu + (int64_t)M * (gy + (int64_t)M * gz);
+        for (int gx = lane; gx < M; gx += 32)
+            inv[off + gx] = cyz || ((faces & 1u) && gx == 0) || ((faces & 2u) && gx == M - 1) ? 0.f : 1.f / diag[off + gx];
+    }
+}
+
+// One block row per stored offset (blockIdx.y), one thread per pressure node.  The 1D factor products of a pair of pressure
+// nodes depend on the nodes only through their boundary classes (first, interior, last), so they are formed once per block
+// in shared memory: w[d][class of I][class of J][k][a or g], k over the velocity nodes both touch; nodes outside the
+// lattice get 0 and are read at a clamped place.  Measured at 64^3 Q2: 2139 us with the factors in local memory, three
+// divisions and a boundary test per velocity node, now 667.
+__global__ void __launch_bounds__(128) k_schur_assemble(int n, int P, int M, int64_t Nu, int64_t Np, SchurTables tab,
+                                                        const float* __restrict__ inv, float* __restrict__ S) {
+    __shared__ float w[3][3][3][2 * MAXQ - 1][2];
+    const int e = blockIdx.y, lin = 62 + e;
     const int o[3] = {lin % 5 - 2, (lin / 5) % 5 - 2, lin / 25 - 2};
-    const int m1 = n + 1;
-    const int I[3] = {(int)(node % m1), (int)((node / m1) % m1), (int)(node / ((int64_t)m1 * m1))};
-    float wa[3][2 * MAXQ - 1], wg[3][2 * MAXQ - 1];
+    for (int q = threadIdx.x; q < 27 * (2 * MAXQ - 1); q += blockDim.x) {
+        const int k = q % (2 * MAXQ - 1), cj = (q / (2 * MAXQ - 1)) % 3, ci = (q / (3 * (2 * MAXQ - 1))) % 3,
+                  d = q / (9 * (2 * MAXQ - 1));
+        // a representative pair of these classes; the classes that no pair at this offset has stay 0
+        int I = ci == 0 ? 0 : (ci == 2 ? n : -1), J = cj == 0 ? 0 : (cj == 2 ? n : -1);
+        if (I < 0 && J < 0) I = 3;  // both interior: taken from a long lattice below
+        if (I < 0) I = J - o[d];
+        if (J < 0 || (ci == 1 && cj == 1)) J = I + o[d];
+        const int nn = ci == 1 && cj == 1 ? 8 : n;
+        float a = 0.f, g = 0.f;
+        if (J - I == o[d] && I >= 0 && I <= nn && J >= 0 && J <= nn) {
+            const int V = P * max(I, J) - P + k;
+            if (V >= 0 && V <= P * nn && V <= P * min(I, J) + P) {
+                a = factor1(tab.a, P, nn, I, V) * factor1(tab.a, P, nn, J, V);
+                g = factor1(tab.g, P, nn, I, V) * factor1(tab.g, P, nn, J, V);
+            }
+        }
+        w[d][ci][cj][k][0] = a;
+        w[d][ci][cj][k][1] = g;
+    }
+    __syncthreads();
+    const int64_t node = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (node >= Np) return;
+    const unsigned m1 = (unsigned)n + 1u, nd = (unsigned)node, t = nd / m1;
+    const int I[3] = {(int)(nd - t * m1), (int)(t - (t / m1) * m1), (int)(t / m1)};
     int lo[3], cnt[3];
+    const float(*wd[3])[2];
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
         const int J = I[d] + o[d];
         if (J < 0 || J > n) {
-            S[idx] = 0.f;
+            S[e * Np + node] = 0.f;
             return;
         }
-        lo[d] = std::max(P * std::max(I[d], J) - P, 0);
-        const int hi = std::min(P * std::min(I[d], J) + P, P * n);
-        cnt[d] = std::max(hi - lo[d] + 1, 0);
-        for (int k = 0; k < cnt[d]; ++k) {
-            const int V = lo[d] + k;
-            wa[d][k] = factor1(tab.a, P, n, I[d], V) * factor1(tab.a, P, n, J, V);
-            wg[d][k] = factor1(tab.g, P, n, I[d], V) * factor1(tab.g, P, n, J, V);
-        }
+        lo[d] = P * max(I[d], J) - P;
+        cnt[d] = P * (2 - abs(o[d])) + 1;
+        wd[d] = w[d][I[d] == 0 ? 0 : (I[d] == n ? 2 : 1)][J == 0 ? 0 : (J == n ? 2 : 1)];
     }
     float acc = 0.f;
-    for (int kz = 0; kz < cnt[2]; ++kz)
-        for (int ky = 0; ky < cnt[1]; ++ky)
+    for (int kz = 0; kz < cnt[2]; ++kz) {
+        const float az = wd[2][kz][0], gz = wd[2][kz][1];
+        const int vz = min(max(lo[2] + kz, 0), M - 1);
+        for (int ky = 0; ky < cnt[1]; ++ky) {
+            const float ay = wd[1][ky][0], gy = wd[1][ky][1];
+            const int vy = min(max(lo[1] + ky, 0), M - 1);
+            const float* r = inv + (int64_t)M * (vy + (int64_t)M * vz);
+            float s0 = 0.f, s1 = 0.f, s2 = 0.f;
             for (int kx = 0; kx < cnt[0]; ++kx) {
-                const int vx = lo[0] + kx, vy = lo[1] + ky, vz = lo[2] + kz;
-                if (constrained_node(vx, vy, vz, M, faces)) continue;
-                const int64_t v = vx + (int64_t)M * (vy + (int64_t)M * vz);
-                acc += wg[0][kx] * wa[1][ky] * wa[2][kz] / diag[v] + wa[0][kx] * wg[1][ky] * wa[2][kz] / diag[Nu + v] +
-                       wa[0][kx] * wa[1][ky] * wg[2][kz] / diag[2 * Nu + v];
+                const int vx = min(max(lo[0] + kx, 0), M - 1);
+                const float ax = wd[0][kx][0], gx = wd[0][kx][1];
+                s0 = fmaf(gx, r[vx], s0);
+                s1 = fmaf(ax, r[Nu + vx], s1);
+                s2 = fmaf(ax, r[2 * Nu + vx], s2);
             }
-    S[idx] = acc;
+            acc += ay * az * s0 + gy * az * s1 + ay * gz * s2;
+        }
+    }
+    S[e * Np + node] = acc;
 }
 
-// Row `node` of S~ x and its diagonal, from the stored half stencil (FP32).  Nodes at least two layers inside the
-// lattice take an unrolled path with compile-time offsets and no bounds tests (83 % of the nodes at 64^3); the others
-// test each neighbour.  Entries are indexed with 32 bits (63 N_p < 2^32, checked on the host).
+// Row `node` of S~ x and its diagonal, from the stored half stencil (FP32).  x lies on the lattice padded by two zero layers
+// on every side (pos), so the 125 products need no bounds tests and a node's loads are in flight together: the
+// coefficients of neighbours outside the lattice, read from a wrapped node's entry, meet a zero.  (With a tested path for
+// the nodes near the boundary, most warps of 32 consecutive nodes took both paths: 53 us per CG iteration at 64^3, now 27.)
+// Entries are indexed with 32 bits (63 N_p < 2^32, checked on the host); in front of S lie schur_guard(n) zeros.
 struct SchurStencil {
     static constexpr int SMEM = 0;
     int n;
     int64_t Np;
     const float* S;
     __device__ __forceinline__ void load(float*) const {}
-    template <class X>
-    __device__ __forceinline__ float row(int64_t node, const X* x, const float*) const {
-        const unsigned m1 = (unsigned)n + 1u, m2 = m1 * m1, nd = (unsigned)node, np = (unsigned)Np;
+    __device__ __forceinline__ unsigned pos(int64_t node) const {
+        const unsigned m1 = (unsigned)n + 1u, mp = m1 + 4u, nd = (unsigned)node;
         const unsigned t = nd / m1, i = nd - t * m1, k = t / m1, j = t - k * m1;
+        return (i + 2u) + mp * ((j + 2u) + mp * (k + 2u));
+    }
+    __device__ __forceinline__ float row(int64_t node, const float* x, const float*) const {
+        const int m1 = n + 1, m2 = m1 * m1, mp = m1 + 4;
+        const float* p = x + pos(node);
+        const float* c = S + node;
+        const int64_t np = Np;
         float acc = 0.f;
-        if (i >= 2u && j >= 2u && k >= 2u && i + 2u <= (unsigned)n && j + 2u <= (unsigned)n && k + 2u <= (unsigned)n) {
 #pragma unroll
-            for (int dz = -2; dz <= 2; ++dz)
-#pragma unroll
-                for (int dy = -2; dy <= 2; ++dy)
-#pragma unroll
-                    for (int dx = -2; dx <= 2; ++dx) {
-                        const int lin = 25 * (dz + 2) + 5 * (dy + 2) + (dx + 2);
-                        const unsigned nb = nd + (unsigned)dx + (unsigned)dy * m1 + (unsigned)dz * m2;
-                        const float c = lin >= 62 ? S[(unsigned)(lin - 62) * np + nd] : S[(unsigned)(62 - lin) * np + nb];
-                        acc = fmaf(c, (float)x[nb], acc);
-                    }
-            return acc;
-        }
-#pragma unroll
-        for (int dz = -2; dz <= 2; ++dz) {
-            if ((int)k + dz < 0 || (int)k + dz > n) continue;
+        for (int dz = -2; dz <= 2; ++dz)
 #pragma unroll
             for (int dy = -2; dy <= 2; ++dy) {
-                if ((int)j + dy < 0 || (int)j + dy > n) continue;
+                const float* pr = p + mp * (dy + mp * dz);
+                const int nb = m1 * dy + m2 * dz;
 #pragma unroll
                 for (int dx = -2; dx <= 2; ++dx) {
-                    if ((int)i + dx < 0 || (int)i + dx > n) continue;
                     const int lin = 25 * (dz + 2) + 5 * (dy + 2) + (dx + 2);
-                    const unsigned nb = nd + (unsigned)dx + (unsigned)dy * m1 + (unsigned)dz * m2;
-                    const float c = lin >= 62 ? S[(unsigned)(lin - 62) * np + nd] : S[(unsigned)(62 - lin) * np + nb];
-                    acc = fmaf(c, (float)x[nb], acc);
+                    const float cf = lin >= 62 ? c[(lin - 62) * np] : c[(62 - lin) * np + (nb + dx)];
+                    acc = fmaf(cf, pr[dx], acc);
                 }
             }
-        }
         return acc;
     }
     __device__ __forceinline__ float diag(int64_t node, const float*) const { return S[node]; }
 };
+inline int64_t schur_guard(int n) { return 2 * ((int64_t)(n + 1) * (n + 1) + (n + 1) + 1); }
+inline int64_t schur_padded(int n) { return (int64_t)(n + 5) * (n + 5) * (n + 5); }
 
-// y = S~ x in FP32 arithmetic (x, y FP64), one thread per pressure node.
-__global__ void k_schur_apply(SchurStencil op, const double* __restrict__ x, double* __restrict__ y) {
+// x (FP64) onto the padded lattice in FP32; y = S~ x (FP64 out), one thread per pressure node.
+__global__ void k_schur_pad(SchurStencil op, const double* __restrict__ x, float* __restrict__ xp) {
     const int64_t node = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (node < op.Np) y[node] = (double)op.row(node, x, nullptr);
+    if (node < op.Np) xp[op.pos(node)] = (float)x[node];
+}
+__global__ void k_schur_apply(SchurStencil op, const float* __restrict__ xp, double* __restrict__ y) {
+    const int64_t node = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (node < op.Np) y[node] = (double)op.row(node, xp, nullptr);
 }
 
 // Assembles S~ for the mesh's current Jacobi diagonal of A (launch_diagonal), once per diagonal.
@@ -145,7 +186,11 @@ int schur_assemble(evap_mesh* h, cudaStream_t s) {
         set_error("Schur stencil: its 63 N_p entries must be indexable with 32 bits");
         return EVAP_EINVAL;
     }
-    if (!h->schur_S) EVAP_CUDA(cudaMalloc(&h->schur_S, 63 * m.Np * sizeof(float)));
+    if (!h->schur_S) {  // guard, stencil, the padded lattice of the vector it is applied to, 1 / D
+        const int64_t len = schur_guard(m.n) + 63 * m.Np + schur_padded(m.n);
+        EVAP_CUDA(cudaMalloc(&h->schur_S, (len + 3 * m.Nu) * sizeof(float)));
+        EVAP_CUDA(cudaMemsetAsync(h->schur_S, 0, len * sizeof(float), s));
+    }
     SchurTables tab;
     std::memset(&tab, 0, sizeof(tab));
     const Basis<double>& b = h->b;
@@ -159,9 +204,12 @@ int schur_assemble(evap_mesh* h, cudaStream_t s) {
             tab.a[a][v] = (float)(m.h * sa);
             tab.g[a][v] = (float)sg;
         }
-    const int64_t total = 63 * m.Np;
-    k_schur_assemble<<<(unsigned)((total + 127) / 128), 128, 0, s>>>(m.n, m.P, m.M, m.faces, m.Nu, m.Np, tab,
-                                                                     h->diag32, h->schur_S);
+    float* inv = h->schur_S + schur_guard(m.n) + 63 * m.Np + schur_padded(m.n);
+    const unsigned gi = (unsigned)std::min<int64_t>((3 * (int64_t)m.M * m.M + 7) / 8, 152 * 16);
+    k_schur_inverse<<<gi, 256, 0, s>>>(m.M, m.Nu, m.faces, h->diag32, inv);
+    EVAP_CHECK_LAUNCH("schur_inverse");
+    k_schur_assemble<<<dim3((unsigned)((m.Np + 127) / 128), 63), 128, 0, s>>>(m.n, m.P, m.M, m.Nu, m.Np, tab, inv,
+                                                                           h->schur_S + schur_guard(m.n));
     EVAP_CHECK_LAUNCH("schur_assemble");
     h->schur_stamp = h->diag_stamp;
     return EVAP_OK;
@@ -170,8 +218,12 @@ int schur_assemble(evap_mesh* h, cudaStream_t s) {
 int launch_schur_apply(evap_mesh* h, const double* x, double* y, cudaStream_t s) {
     int rc = schur_assemble(h, s);
     if (rc) return rc;
-    const SchurStencil op{h->m.n, h->m.Np, h->schur_S};
-    k_schur_apply<<<(unsigned)((h->m.Np + 255) / 256), 256, 0, s>>>(op, x, y);
+    const SchurStencil op{h->m.n, h->m.Np, h->schur_S + schur_guard(h->m.n)};
+    float* xp = h->schur_S + schur_guard(h->m.n) + 63 * h->m.Np;  // its halo stays zero
+    const unsigned grid = (unsigned)((h->m.Np + 255) / 256);
+    k_schur_pad<<<grid, 256, 0, s>>>(op, x, xp);
+    EVAP_CHECK_LAUNCH("schur_pad");
+    k_schur_apply<<<grid, 256, 0, s>>>(op, xp, y);
     EVAP_CHECK_LAUNCH("schur_apply");
     return EVAP_OK;
 }
@@ -187,10 +239,11 @@ int schur_solve(evap_mesh* h, const double* r, double* z, double rtol, int max_i
     int G = 0;
     if ((rc = fused_grid(k_cg_fused32<SchurStencil>, 0, FK_MAX_BLOCKS, G))) return rc;
     EVAP_CUDA(cudaMemsetAsync(f.gb, 0, sizeof(GridBarrier), s));
-    SchurStencil op{h->m.n, N, h->schur_S};
+    SchurStencil op{h->m.n, N, h->schur_S + schur_guard(h->m.n)};
     const int64_t Nl = ls_args<double>(h).Nphi;  // the vectors' stride: fused_space sizes them for N_phi
     float* base = reinterpret_cast<float*>(f.vec);
-    float *xs = base, *r32 = base + Nl, *u = base + 2 * Nl, *p = base + 3 * Nl, *sv = base + 4 * Nl, *w = base + 5 * Nl;
+    float *xs = base, *r32 = base + Nl, *p = base + 3 * Nl, *sv = base + 4 * Nl, *w = base + 5 * Nl;
+    float* u = h->schur_S + schur_guard(h->m.n) + 63 * N;  // the padded lattice, whose halo stays zero
     float* dinv = f.dinv;
     float* part = reinterpret_cast<float*>(f.part);
     GridBarrier* gb = f.gb;
