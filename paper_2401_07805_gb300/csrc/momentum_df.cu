@@ -75,6 +75,14 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
     using Ln = DfLine<Q>;
     __shared__ dfl sN1[Q][2];
     __shared__ dfl q1a[CB][2 * Q * Q], q1b[CB][4 * Q];
+    // the pressure at the cell's corners, then interpolated along x and y (z: by the point's thread), in double-float
+    // arithmetic: 14 FP64 operations and a conversion per point had made the FP64 pipe the bound (672 -> 531 us at 64^3)
+    __shared__ dfl p0[PRES ? CB : 1][8], px[PRES ? CB : 1][4 * Q], py[PRES ? CB : 1][2 * Q * Q];
+    auto lerp = [&](dfl u, dfl v, int q) -> dfl {  // at Gauss point q, in double-float arithmetic
+        dfl r = u;
+        df_fma(r, sN1[q][1], df_add(v, df_neg(u)));
+        return df_norm(r);
+    };
     extern __shared__ float2 smem_df[];
     dfl* const sb = reinterpret_cast<dfl*>(smem_df);  // [cell][slot][point]
     constexpr int CELL = (DF_SLOTS + QC_K) * NQ;
@@ -124,7 +132,18 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         Ln::val(u, v);
         st_line<Q, 2>(lb + (3 + f) * NQ, l, v);
     }
+    if (PRES && tid < CB * 8) {
+        const int c2 = tid / 8, o = tid % 8;
+        int ex, ey, ez;
+        colour_cell32(cell0 + c2, n, DET ? colour : -1, ex, ey, ez);
+        const int64_t m1 = n + 1;
+        p0[c2][o] = df_from_double(pin[(ex + (o & 1)) + m1 * ((ey + ((o >> 1) & 1)) + m1 * (ez + (o >> 2)))]);
+    }
     __syncthreads();
+    if (PRES && tid < CB * 4 * Q) {  // [qx][jb][jc]
+        const int c2 = tid / (4 * Q), o = tid % (4 * Q), q = o % Q, r = o / Q;
+        px[c2][o] = lerp(p0[c2][2 * r], p0[c2][2 * r + 1], q);
+    }
     if (line) {
         dfl u[Q], v[Q];
         ld_line<Q, 1>(lb + (3 + f) * NQ, l, u);
@@ -132,6 +151,10 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         st_line<Q, 1>(lb + (6 + f) * NQ, l, v);
     }
     __syncthreads();
+    if (PRES && tid < CB * 2 * Q * Q) {  // [qx][qy][jc]
+        const int c2 = tid / (2 * Q * Q), o = tid % (2 * Q * Q), q = o % Q, r = (o / Q) % Q, jc = o / (Q * Q);
+        py[c2][o] = lerp(px[c2][q + Q * (2 * jc)], px[c2][q + Q * (2 * jc + 1)], r);
+    }
     if (line) {  // x: the values at the points, and their derivative along x
         dfl u[Q], v[Q];
         ld_line<Q, 0>(lb + (6 + f) * NQ, l, u);
@@ -184,21 +207,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         const dfl sm = corr ? df_mul(c13, tr) : dfl{0.f, 0.f};
         const dfl rw = PRES || yp ? df_mul(q[17 * NQ], kap) : dfl{0.f, 0.f};  // kappa W
         dfl wp{0.f, 0.f};
-        if constexpr (PRES) {  // p at the point: trilinear interpolation by successive linear ones, in FP64
-            const int64_t m1 = n + 1;
-            const double* p0 = pin + cx + m1 * (cy + m1 * cz);
-            const double tx = bas.t[t % Q], ty = bas.t[(t / Q) % Q], tz = bas.t[t / (Q * Q)];
-            double e[2][2];
-#pragma unroll
-            for (int jc = 0; jc < 2; ++jc)
-#pragma unroll
-                for (int jb = 0; jb < 2; ++jb) {
-                    const double* r = p0 + m1 * (jb + m1 * jc);
-                    e[jc][jb] = fma(tx, r[1] - r[0], r[0]);
-                }
-            const double f0 = fma(ty, e[0][1] - e[0][0], e[0][0]), f1 = fma(ty, e[1][1] - e[1][0], e[1][0]);
-            wp = df_mul(rw, df_from_double(fma(tz, f1 - f0, f0)));
-        }
+        if constexpr (PRES) wp = df_mul(rw, lerp(py[lc][t % NL], py[lc][t % NL + NL], t / NL));
 #pragma unroll
         for (int k = 0; k < 3; ++k)
 #pragma unroll
