@@ -12,7 +12,7 @@
 //
 // The free DoFs of a face-constrained box form a tensor product of per-axis ranges, so M^(-1) on them is three
 // sweeps of banded 1D solves (bandwidth p): one block per tile of 32 lines, staged through shared memory so that
-// global loads and stores stay coalesced for every axis (eight warps keep the loads in flight); each lane of the
+// global loads and stores stay coalesced for every axis; each lane of the
 // first warp solves one line with the LU factors of its axis (factorized once on the host in FP64, no pivoting: the
 // 1D mass matrix is symmetric positive definite).
 #include <cmath>
@@ -23,154 +23,198 @@
 namespace evap {
 
 constexpr int TP_LANES = 32;     // lines per tile (one solving warp)
-constexpr int TP_THREADS = 256;  // threads of a block: all load and store the tile, the first warp solves
+constexpr int TP_THREADS = 128;  // threads of a block: all load and store the tile, the first warp solves
+constexpr int TP_STEP = 8;       // line entries per step of the recurrences
 
-// Factor layout per axis (floats, Mf = hi - lo + 1 free nodes): rows k = 0..P-1 hold L[i][i-1-k], rows P..2P-1 hold
-// U[i][i+1+(k-P)], row 2P holds 1 / U[i][i].
+// Factors of one free node i in shared memory: f[0..P-1] = L[i][i-1-k], then b[0..P-1] = U[i][i+1+k] / U[i][i] and
+// b[P] = 1 / U[i][i], each padded to a vector.
+template <int P>
+struct TpShape {
+    static constexpr int FW = P == 2 ? 2 : 4, BW = 4;  // entries per node, forward and backward
+};
+template <typename T, int N>
+struct alignas(sizeof(T) * N <= 16 ? sizeof(T) * N : 16) TpVec {
+    T v[N];
+};
 template <typename T, int P>
-__device__ __forceinline__ void tp_solve_line(const T* __restrict__ fac, int Mf, T* __restrict__ col, int stride) {
-    // The last P values of each recurrence stay in registers (win[0] the nearest), so a step waits on FMAs only; the
-    // factor rows are zero where a neighbour falls outside the line, so no step needs a branch.
+__device__ __forceinline__ void tp_solve_line(const T* __restrict__ ff, const T* __restrict__ fb, int Mf,
+                                              T* __restrict__ col, int stride) {
+    using FV = TpVec<T, TpShape<P>::FW>;
+    using BV = TpVec<T, TpShape<P>::BW>;
+    // The last P values of each recurrence stay in registers (win[0] the nearest) and enter last, so that a step waits on
+    // one FMA only (the backward factors are scaled by the pivot for this); TP_STEP entries and their factors are loaded
+    // together, as vectors, ahead of the step's chain: 9 instructions per entry both ways.  The factors are zero where a
+    // neighbour falls outside the line.
     T win[P];
+    auto chain = [&](const T* f, T v) -> T {
 #pragma unroll
-    for (int k = 0; k < P; ++k) win[k] = T(0);
-    // forward: L y = d (unit lower)
-#pragma unroll 4
-    for (int i = 0; i < Mf; ++i) {
-        T v = col[i * stride];
-#pragma unroll
-        for (int k = 0; k < P; ++k) v -= fac[k * Mf + i] * win[k];
-        col[i * stride] = v;
+        for (int k = P - 1; k >= 0; --k) v -= f[k] * win[k];
 #pragma unroll
         for (int k = P - 1; k > 0; --k) win[k] = win[k - 1];
         win[0] = v;
-    }
-    // backward: U x = y
+        return v;
+    };
 #pragma unroll
     for (int k = 0; k < P; ++k) win[k] = T(0);
-#pragma unroll 4
-    for (int i = Mf - 1; i >= 0; --i) {
-        T v = col[i * stride];
+    const FV* f = reinterpret_cast<const FV*>(ff);
+    T* c = col;
+    int left = Mf;
+    for (; left >= TP_STEP; left -= TP_STEP, f += TP_STEP, c += TP_STEP * stride) {  // forward: L y = d (unit lower)
+        T v[TP_STEP];
+        FV w[TP_STEP];
 #pragma unroll
-        for (int k = 0; k < P; ++k) v -= fac[(P + k) * Mf + i] * win[k];
-        v *= fac[2 * P * Mf + i];
-        col[i * stride] = v;
+        for (int e = 0; e < TP_STEP; ++e) {
+            v[e] = c[e * stride];
+            w[e] = f[e];
+        }
 #pragma unroll
-        for (int k = P - 1; k > 0; --k) win[k] = win[k - 1];
-        win[0] = v;
+        for (int e = 0; e < TP_STEP; ++e) c[e * stride] = chain(w[e].v, v[e]);
     }
+    for (; left > 0; --left, ++f, c += stride) *c = chain(f->v, *c);
+#pragma unroll
+    for (int k = 0; k < P; ++k) win[k] = T(0);
+    const BV* g = reinterpret_cast<const BV*>(fb) + (Mf - 1);
+    c = col + (Mf - 1) * stride;
+    left = Mf;
+    for (; left >= TP_STEP; left -= TP_STEP, g -= TP_STEP, c -= TP_STEP * stride) {  // backward: U x = y
+        T v[TP_STEP];
+        BV w[TP_STEP];
+#pragma unroll
+        for (int e = 0; e < TP_STEP; ++e) {
+            w[e] = g[-e];
+            v[e] = c[-e * stride] * w[e].v[P];
+        }
+#pragma unroll
+        for (int e = 0; e < TP_STEP; ++e) c[-e * stride] = chain(w[e].v, v[e]);
+    }
+    for (; left > 0; --left, --g, c -= stride) *c = chain(g->v, *c * g->v[P]);
 }
 
 // One sweep along AXIS for all three components (v enters scaled by sc).  MODE 0: t = M_axis^(-1) (Sigma sc v);
 // MODE 1: t = M_axis^(-1) t; MODE 2: z = Sigma M_axis^(-1) t on the free DoFs, z = sc v on the Dirichlet ones, and
 // w = (Dirichlet ? z : 0) (the initialization of the operator apply that follows).  One block per tile of TP_LANES
 // lines; lines whose transverse position is constrained are all-Dirichlet and are solved only as a copy in MODE 2.
+// A tile of x-lines is one contiguous run of memory; a tile of y- or z-lines is rows of 32 neighbouring lines.  What
+// bounds the sweep is memory once enough loads are in flight: every thread issues LD independent ones at a time, and
+// blocks of 128 threads let all tiles of a 64^3 sweep be resident at once.  Measured at 64^3 Q2 FP32 (us, x / y / z
+// sweep, ncu): 68 / 28 / 35 with 256 threads and one load in flight per thread, the chain of a step two and three
+// operations long.
 template <typename T, int P, int AXIS, int MODE>
 __global__ void __launch_bounds__(TP_THREADS) k_tp_sweep(int M, int64_t Nu, unsigned faces, const T* __restrict__ fac_all,
                                                      int lo, int hi, const T* __restrict__ sigma,
                                                      const T* __restrict__ v, T sc, T* __restrict__ t,
                                                      T* __restrict__ z, T* __restrict__ w) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* smem = reinterpret_cast<T*>(smem_raw);
+    constexpr int FW = TpShape<P>::FW, BW = TpShape<P>::BW, LD = 8, TS = TP_LANES + 1;
     const int Mf = hi - lo + 1;
-    T* fac = smem;                     // (2P + 1) Mf
-    T* tile = smem + (2 * P + 1) * Mf;  // [M][TP_LANES + 1]
+    T* const fb = reinterpret_cast<T*>(smem_raw);  // [Mf][BW], first: its rows and those of ff are aligned vectors
+    T* const ff = fb + Mf * BW;                     // [Mf][FW]
+    T* const tile = ff + Mf * FW;                   // [M][TS]
     const int tid = threadIdx.x;
-    for (int i = tid; i < (2 * P + 1) * Mf; i += TP_THREADS) fac[i] = fac_all[i];
+    for (int i = tid; i < Mf; i += TP_THREADS) {
+#pragma unroll
+        for (int k = 0; k < P; ++k) {
+            ff[i * FW + k] = fac_all[k * Mf + i];
+            fb[i * BW + k] = fac_all[(P + k) * Mf + i];
+        }
+        fb[i * BW + P] = fac_all[2 * P * Mf + i];
+    }
     // tile -> (component, first line); line l of the tile has transverse coordinates (ta, tb) and base address
-    const int64_t M2 = (int64_t)M * M;
-    int comp;
-    int64_t first;  // first line index within the component
-    int nlines;     // lines in this tile
-    if (AXIS == 1) {  // y-lines: 32 consecutive x at fixed (z, component)
-        const int tiles_x = (M + TP_LANES - 1) / TP_LANES;
-        const int64_t b = blockIdx.x;
-        comp = (int)(b / ((int64_t)tiles_x * M));
-        const int64_t r = b - (int64_t)comp * tiles_x * M;
-        const int zz = (int)(r / tiles_x), tx = (int)(r % tiles_x);
-        first = (int64_t)zz * M + tx * TP_LANES;  // line id x + M z
+    const int M2 = M * M;
+    int comp, first, nlines;  // first line id of the tile within the component, its lines
+    if (AXIS == 1) {  // y-lines (id x + M z): 32 consecutive x at fixed (z, component)
+        const int tiles_x = (M + TP_LANES - 1) / TP_LANES, b = (int)blockIdx.x;
+        comp = b / (tiles_x * M);
+        const int r = b - comp * tiles_x * M, zz = r / tiles_x, tx = r - zz * tiles_x;
+        first = zz * M + tx * TP_LANES;
         nlines = min(TP_LANES, M - tx * TP_LANES);
     } else {  // x-lines (id y + M z) or z-lines (id x + M y): 32 consecutive ids per component
-        const int tiles = (int)((M2 + TP_LANES - 1) / TP_LANES);
-        comp = blockIdx.x / tiles;
-        first = (int64_t)(blockIdx.x % tiles) * TP_LANES;
-        nlines = (int)min((int64_t)TP_LANES, M2 - first);
+        const int tiles = (M2 + TP_LANES - 1) / TP_LANES;
+        comp = (int)blockIdx.x / tiles;
+        first = ((int)blockIdx.x - comp * tiles) * TP_LANES;
+        nlines = min(TP_LANES, M2 - first);
     }
-    const int64_t cbase = (int64_t)comp * Nu;
-    // per-lane line: base address, element stride, transverse constraint
-    auto line_base = [&](int l, bool& cons) -> int64_t {
-        const int64_t id = first + l;
-        int ta, tb;  // transverse node coordinates
-        int64_t base;
-        if (AXIS == 0) {  // id = y + M z
-            ta = (int)(id % M); tb = (int)(id / M);
-            base = id * M;
-            cons = constrained_node(1, ta, tb, M, faces & ~3u);
-        } else if (AXIS == 1) {  // id = x + M z
-            ta = (int)(id % M); tb = (int)(id / M);
-            base = ta + M2 * tb;
-            cons = constrained_node(ta, 1, tb, M, faces & ~12u);
-        } else {  // id = x + M y
-            ta = (int)(id % M); tb = (int)(id / M);
-            base = id;
-            cons = constrained_node(ta, tb, 1, M, faces & ~48u);
-        }
-        return cbase + base;
-    };
-    const int64_t es = AXIS == 0 ? 1 : (AXIS == 1 ? M : M2);  // element stride along the line
-    // per-line base address and constraint flag, once per tile (the element loops below divide nothing)
-    __shared__ int64_t s_base[TP_LANES];
+    // per-line constraint flag (lines on a Dirichlet face of a transverse direction)
     __shared__ int s_cons[TP_LANES];
-    if (tid < nlines) {
-        bool cons;
-        s_base[tid] = line_base(tid, cons);
-        s_cons[tid] = cons ? 1 : 0;
+    if (tid < TP_LANES) {
+        const int id = first + tid, tb = id / M, ta = id - tb * M;
+        s_cons[tid] = AXIS == 0 ? constrained_node(1, ta, tb, M, faces & ~3u)
+                                : (AXIS == 1 ? constrained_node(ta, 1, tb, M, faces & ~12u)
+                                             : constrained_node(ta, tb, 1, M, faces & ~48u));
     }
     __syncthreads();
-    // element loops: x-lines are contiguous, so each line is read by consecutive threads; for y- and z-lines a warp
-    // reads one element of 32 neighbouring lines (contiguous in memory) and the eight warps take every eighth element
-    constexpr int ROWS = TP_THREADS / TP_LANES;
-    const int lane = tid % TP_LANES, row = tid / TP_LANES;
-    auto load = [&](int64_t a) -> T { return MODE == 0 ? sc * v[a] * sigma[a] : t[a]; };
-    if (AXIS == 0) {
-        for (int l = 0; l < nlines; ++l) {
-            if (s_cons[l]) continue;
-            const int64_t b = s_base[l] + lo;
-            for (int e = tid; e < Mf; e += TP_THREADS) tile[e * (TP_LANES + 1) + l] = load(b + e);
-        }
-    } else if (lane < nlines && !s_cons[lane]) {
-        const int64_t b = s_base[lane] + (int64_t)lo * es;
-        for (int e = row; e < Mf; e += ROWS) tile[e * (TP_LANES + 1) + lane] = load(b + (int64_t)e * es);
-    }
-    __syncthreads();
-    if (tid < nlines && !s_cons[tid]) tp_solve_line<T, P>(fac, Mf, tile + tid, TP_LANES + 1);
-    __syncthreads();
-    if (MODE < 2) {
-        if (AXIS == 0) {
-            for (int l = 0; l < nlines; ++l) {
-                if (s_cons[l]) continue;
-                const int64_t b = s_base[l] + lo;
-                for (int e = tid; e < Mf; e += TP_THREADS) t[b + e] = tile[e * (TP_LANES + 1) + l];
+    // Addresses: line l of a tile of x-lines starts at base + l M, line `lane` of a tile of y-lines at x + M^2 z = (first +
+    // lane) + (M^2 - M) z and of z-lines at x + M y.  Loads past a range are clamped into it, not skipped, so that LD of
+    // them are in flight per thread.
+    const int lane = tid % 32, warp = tid / 32;
+    constexpr int WARPS = TP_THREADS / 32;
+    const int ln = AXIS == 0 ? 0 : min(lane, nlines - 1);
+    const int64_t base = (int64_t)comp * Nu + (AXIS == 0 ? (int64_t)first * M
+                                                         : first + ln + (AXIS == 1 ? (int64_t)(first / M) * (M2 - M) : 0));
+    const int64_t es = AXIS == 1 ? M : M2;
+    if (AXIS == 0) {  // a warp loads 2 lines, 4 entries per lane of each
+        for (int l0 = 2 * warp; l0 < nlines; l0 += 2 * WARPS)
+            for (int e0 = lane; e0 < Mf; e0 += 128) {
+                T x[2][4], g[2][4];
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int64_t a = base + min(l0 + q, nlines - 1) * M + lo + min(e0 + 32 * k, Mf - 1);
+                        x[q][k] = MODE == 0 ? v[a] : t[a];
+                        g[q][k] = MODE == 0 ? sigma[a] : T(1);
+                    }
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (e0 + 32 * k < Mf && l0 + q < nlines)
+                            tile[(e0 + 32 * k) * TS + l0 + q] = MODE == 0 ? sc * x[q][k] * g[q][k] : x[q][k];
             }
-        } else if (lane < nlines && !s_cons[lane]) {
-            const int64_t b = s_base[lane] + (int64_t)lo * es;
-            for (int e = row; e < Mf; e += ROWS) t[b + (int64_t)e * es] = tile[e * (TP_LANES + 1) + lane];
+    } else {
+        const T* src = t + base + lo * es;
+        for (int e0 = warp; e0 < Mf; e0 += LD * WARPS) {
+            T x[LD];
+#pragma unroll
+            for (int k = 0; k < LD; ++k) x[k] = src[min(e0 + k * WARPS, Mf - 1) * es];
+#pragma unroll
+            for (int k = 0; k < LD; ++k)
+                if (e0 + k * WARPS < Mf) tile[(e0 + k * WARPS) * TS + lane] = x[k];
+        }
+    }
+    __syncthreads();
+    if (tid < nlines && !s_cons[tid]) tp_solve_line<T, P>(ff, fb, Mf, tile + tid, TP_LANES + 1);
+    __syncthreads();
+    if (AXIS == 0) {
+        for (int l = warp; l < nlines; l += WARPS) {
+            if (s_cons[l]) continue;
+            T* dst = t + base + (int64_t)l * M + lo;
+            for (int e = lane; e < Mf; e += 32) dst[e] = tile[e * TS + l];
+        }
+    } else if (MODE < 2) {
+        if (lane < nlines && !s_cons[lane]) {
+            T* dst = t + base + lo * es;
+#pragma unroll 4
+            for (int e = warp; e < Mf; e += WARPS) dst[e * es] = tile[e * TS + lane];
         }
     } else {  // every node of the tile's lines: free -> Sigma t, Dirichlet -> sc v; w = Dirichlet ? z : 0
-        auto put = [&](int l, int e, int64_t a) {
-            const bool dir = s_cons[l] || e < lo || e > hi;
-            const T zz = dir ? sc * v[a] : sigma[a] * tile[(e - lo) * (TP_LANES + 1) + l];
-            z[a] = zz;
-            if (w) w[a] = dir ? zz : T(0);
-        };
-        if (AXIS == 0) {
-            for (int l = 0; l < nlines; ++l) {
-                const int64_t b = s_base[l];
-                for (int e = tid; e < M; e += TP_THREADS) put(l, e, b + e);
+        const bool cl = s_cons[ln] != 0;
+        for (int e0 = warp; e0 < M; e0 += LD * WARPS) {
+            T sv[LD];
+#pragma unroll
+            for (int k = 0; k < LD; ++k) {
+                const int e = min(e0 + k * WARPS, M - 1);
+                sv[k] = (cl || e < lo || e > hi ? v : sigma)[base + e * es];
             }
-        } else if (lane < nlines) {
-            const int64_t b = s_base[lane];
-            for (int e = row; e < M; e += ROWS) put(lane, e, b + (int64_t)e * es);
+#pragma unroll
+            for (int k = 0; k < LD; ++k) {
+                const int e = e0 + k * WARPS;
+                if (e >= M || lane >= nlines) continue;
+                const bool dir = cl || e < lo || e > hi;
+                const T zz = dir ? sc * sv[k] : sv[k] * tile[(e - lo) * TS + lane];
+                z[base + e * es] = zz;
+                if (w) w[base + e * es] = dir ? zz : T(0);
+            }
         }
     }
 }
@@ -216,7 +260,7 @@ static void factor_band(const std::vector<double>& Mg, int M, int P, int lo, int
     for (int i = 0; i < Mf; ++i) {
         for (int k = 0; k < P; ++k) {
             if (i - 1 - k >= 0) out[(size_t)k * Mf + i] = A[(size_t)i * Mf + (i - 1 - k)];
-            if (i + 1 + k < Mf) out[(size_t)(P + k) * Mf + i] = A[(size_t)i * Mf + (i + 1 + k)];
+            if (i + 1 + k < Mf) out[(size_t)(P + k) * Mf + i] = A[(size_t)i * Mf + (i + 1 + k)] / A[(size_t)i * Mf + i];
         }
         out[(size_t)2 * P * Mf + i] = 1.0 / A[(size_t)i * Mf + i];
     }
@@ -277,7 +321,7 @@ static int tp_launch(evap_mesh* h, const T* v, T sc, T* t, T* z, T* w, cudaStrea
     const MeshArgs<double>& m = h->m;
     const int M = m.M;
     const int lo = h->tp_lo[AXIS], hi = h->tp_hi[AXIS], Mf = hi - lo + 1;
-    const size_t smem = ((size_t)(2 * P + 1) * Mf + (size_t)M * (TP_LANES + 1)) * sizeof(T);
+    const size_t smem = ((size_t)(TpShape<P>::FW + TpShape<P>::BW) * Mf + (size_t)M * (TP_LANES + 1)) * sizeof(T);
     if (smem > 48 * 1024)
         EVAP_CUDA(cudaFuncSetAttribute(k_tp_sweep<T, P, AXIS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem));
