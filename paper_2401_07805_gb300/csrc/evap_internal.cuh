@@ -290,8 +290,8 @@ int geo_advect_levelset(evap_mesh* h, double* phi, int max_iters, double tol, in
                         double* last_change, cudaStream_t s);
 // Jacobi diagonal (in the geometry workspace, valid until the next geometry call) for CG on the pressure Schur
 // velocity-pressure coupling (saddle.cu)
-template <typename T>
-int launch_pressure_gradient(evap_mesh* h, const T* p, T scale, T* y, cudaStream_t s);
+// t = v + B^T p on the velocity vector (the gradient in FP32; Dirichlet rows of B^T p are 0)
+int launch_add_gradient(evap_mesh* h, const float* p, const double* v, double* t, cudaStream_t s);
 int continuity_rhs(evap_mesh* h, const double** g, cudaStream_t s);
 // [y; y_p] = K [x; p]; lifted: the system K_D of non-homogeneous Dirichlet data, whose free rows keep the columns of
 // the Dirichlet DoFs (y = A_full x - B^T p on free rows, x on constrained rows; y_p = B_full x)
@@ -305,10 +305,6 @@ int set_fields_flow(evap_mesh* h, const double* phi, const double* u, const doub
 int time_step(evap_mesh* h, double* phi, double* u, double* p, const double* mdot, const double* u_prev,
               const double g[3], double alpha, int picard_iters, double picard_atol, int fp_iters, int reinit_steps,
               double ns_rtol, int* ns_iters, double* ns_relres, double* picard_res, cudaStream_t s);
-// y_p += B D^(-1) x (the divergence row without its source; Dirichlet entries of x read as 0; D = diag, or the
-// identity when diag is null)
-template <typename T>
-int launch_divergence(evap_mesh* h, const T* x, const T* diag, T* yp, cudaStream_t s);
 // z = S~^(-1) r by at most cg_iters CG iterations on S~ = B diag(A)^(-1) B^T (applied in FP32) with the Jacobi
 // The assembled Schur approximation S~ = B diag(A)^-1 B^T (schur.cu): assembly for the current diagonal of A, y = S~ x,
 // and z ~ S~^-1 r by the FP32 single-launch CG (at most max_iter iterations or |r| <= rtol |r0|).

@@ -21,8 +21,8 @@ namespace evap {
 // in FP32 from the quadrature-point cache of set_fields (k_qp_coeffs); one thread per (cell, local node).
 template <int P, int CB>
 __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
-    k_diagonal(MeshArgs<float> m, Basis<float> bas, const double* __restrict__ qc, float* __restrict__ diag,
-               int colour) {
+    k_diagonal(MeshArgs<float> m, Basis<float> bas, const double* __restrict__ qc,
+               float* __restrict__ diag, int colour) {
     constexpr int Q = P + 1, NQ = Q * Q * Q;
     __shared__ float sS[Q][Q], sD[Q][Q];
     __shared__ float qd[CB][11][NQ];  // per point: W rho c_m, W rho U(3), newton W rho d_c u0_c (3), 2 W mu, z n(3)
@@ -359,17 +359,38 @@ __global__ void k_residual(const T* __restrict__ b, const T* __restrict__ Ax, T*
         r[k] = b[k] - Ax[k];
 }
 
+// 1 / sqrt(*nrm2) or sqrt(*nrm2), formed by one thread per block: on the FP64 pipe a square root and a division per thread
+// of a two-element grid-stride loop cost several times the scaling itself (85 us against 27 for k_scaled_to_float at
+// 64^3 Q2).
+template <bool INV>
+__device__ __forceinline__ double block_scale(const double* nrm2) {
+    __shared__ double v;
+    if (threadIdx.x == 0) v = INV ? 1.0 / sqrt(*nrm2) : sqrt(*nrm2);
+    __syncthreads();
+    return v;
+}
+
+static int scale_grid(int64_t N) { return blocks_for(N, 256, 152 * 8); }  // one wave
+
 __global__ void k_scaled_to_float(const double* __restrict__ r, const double* __restrict__ nrm2, float* __restrict__ out,
                                   int64_t N) {
-    const double inv = 1.0 / sqrt(*nrm2);
+    const double inv = block_scale<true>(nrm2);
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
         out[k] = (float)(r[k] * inv);
 }
 
 __global__ void k_refine(double* x, const float* __restrict__ d, const double* __restrict__ nrm2, int64_t N) {
-    const double s = sqrt(*nrm2);
+    const double s = block_scale<false>(nrm2);
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
         x[k] += s * (double)d[k];
+}
+
+// x = |r| d
+__global__ void k_scaled_to_double(double* __restrict__ x, const float* __restrict__ d, const double* __restrict__ nrm2,
+                                   int64_t N) {
+    const double s = block_scale<false>(nrm2);
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
+        x[k] = s * (double)d[k];
 }
 
 // ---------------------------------------------------------------------------------------------- GMRES core
@@ -380,6 +401,11 @@ __global__ void k_refine(double* x, const float* __restrict__ d, const double* _
 // the outer FP64 residual is checked regardless).
 constexpr double REORTH64 = 0.5;
 constexpr double REORTH32 = 1e-2;
+// The velocity-pressure solve: its preconditioned operator is close to the identity, so the DGKS test fired on almost
+// every step as well, and on GB300 a second pass over the FP64 basis costs as much as the operator (FP64-pipe bound).
+// With 1e-2 in place of 1/2 the solves and steps at 20^3 to 64^3 kept their application counts to within one in 28; the
+// true residual decides as before.  A step at 64^3: 105 -> 92 ms.
+constexpr double REORTH_SADDLE = 1e-2;
 // the operator of a solve (the momentum system; the level-set solves run in fused_krylov.cuh)
 enum { OP_MOMENTUM = 0 };
 struct Ctx {
@@ -452,11 +478,12 @@ static int set_scale(Ctx& c, int i, double sc) {
 // GMRES(m) on A x = b with right preconditioner diag^{-1}; x updated in place.  x_zero: x is known to be 0 on entry
 // (the first residual is b, no apply).  The Krylov basis is kept unnormalized (v_i = sc_i V_i): the operator writes
 // A z straight into the next basis slot and the scales enter the Gram-Schmidt coefficients, so no vector pass is
-// spent on normalization.  Classical Gram-Schmidt with a second pass only under REORTH64 / REORTH32.  Stops when the
+// spent on normalization.  one_cycle: a single cycle without the check of its true residual (an inexact solve inside a
+// flexible method, which would only discard it).  Classical Gram-Schmidt with a second pass only under REORTH64 / REORTH32.  Stops when the
 // Arnoldi residual estimate is <= tol_abs (then the true residual is recomputed) or after maxit applications.
 template <typename T>
 static int gmres(Ctx& c, int m, const T* b, T* x, bool x_zero, const T* diag, T* V, T* w, T* z, double tol_abs,
-                 int maxit, int* its, double* res_out) {
+                 int maxit, int* its, double* res_out, bool one_cycle = false) {
     const int64_t N = c.N;
     const int G = blocks_for(N, 256);
     std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m), sc(m + 1);
@@ -563,6 +590,7 @@ static int gmres(Ctx& c, int m, const T* b, T* x, bool x_zero, const T* diag, T*
             EVAP_CHECK_LAUNCH("update");
         }
         EVAP_CUDA(cudaStreamSynchronize(c.s));  // c.hcol is reused by the next fetch
+        if (one_cycle) break;  // (the residual estimate of the cycle stands)
     }
     *its = used;
     return EVAP_OK;
@@ -672,7 +700,7 @@ int solve_gmres(evap_mesh* h, const double* f, double* x, int mixed, int m, doub
             }
             x_zero = false;
             if (res <= rtol * fn || used >= max_iter) break;
-            k_scaled_to_float<<<G, 256, 0, s>>>(r64, c.dnorm, r32, N);
+            k_scaled_to_float<<<scale_grid(N), 256, 0, s>>>(r64, c.dnorm, r32, N);
             EVAP_CHECK_LAUNCH("to32");
             EVAP_CUDA(cudaMemsetAsync(d32, 0, N * sizeof(float), s));
             int its = 0;
@@ -683,7 +711,7 @@ int solve_gmres(evap_mesh* h, const double* f, double* x, int mixed, int m, doub
             used += its;
             // the refinement scale |r| is needed on the device again (the inner solve reused the scalar slot)
             if ((rc = norm2_dev<double>(c, r64, c.dnorm))) return rc;
-            k_refine<<<G, 256, 0, s>>>(x, d32, c.dnorm, N);
+            k_refine<<<scale_grid(N), 256, 0, s>>>(x, d32, c.dnorm, N);
             EVAP_CHECK_LAUNCH("refine");
         }
     }
@@ -735,7 +763,7 @@ __global__ void k_residual_inplace(const double* __restrict__ b, double* __restr
 }
 
 __global__ void k_scale_vec(double* __restrict__ v, const double* __restrict__ nrm2, int64_t N) {
-    const double inv = 1.0 / sqrt(*nrm2);
+    const double inv = block_scale<true>(nrm2);
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
         v[k] *= inv;
 }
@@ -754,12 +782,6 @@ __global__ void k_update_split(const double* __restrict__ Z, int64_t ld, const d
     }
 }
 
-// t = v + (double) w
-__global__ void k_add_float(const double* __restrict__ v, const float* __restrict__ w, double* __restrict__ t, int64_t N) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
-        t[k] = v[k] + (double)w[k];
-}
-
 struct SaddleSpace {
     double *V, *Z, *b, *t;  // outer basis [(m+1) ld], directions [m ld], right-hand side [ld], velocity scratch [3 N_u]
     float *V32, *w32, *z32, *r32, *d32;  // inner FP32 workspace
@@ -770,28 +792,23 @@ static int saddle_precond(Ctx& inner, SaddleSpace& sp, const double* v, double* 
     evap_mesh* h = inner.h;
     cudaStream_t s = inner.s;
     const int64_t Nu3 = 3 * h->m.Nu, Np = h->m.Np;
-    const int G = blocks_for(Nu3, 256);
     int rc = schur_apply(h, v + Nu3, z + Nu3, SADDLE_SCHUR_CG, s);
     if (rc) return rc;
     // t = v_u + B^T z_p, the gradient in FP32 (it enters the FP32 velocity solve)
-    if ((rc = launch_to_float(z + Nu3, sp.z32, Np, s))) return rc;
-    EVAP_CUDA(cudaMemsetAsync(sp.w32, 0, Nu3 * sizeof(float), s));
-    if ((rc = launch_pressure_gradient<float>(h, sp.z32, 1.0f, sp.w32, s))) return rc;
-    k_add_float<<<G, 256, 0, s>>>(v, sp.w32, sp.t, Nu3);
-    EVAP_CHECK_LAUNCH("saddle_add_grad");
-    // velocity block: FP32 GMRES on t / |t| from zero, then z_u = |t| d
-    if ((rc = norm2_dev<double>(inner, sp.t, inner.dnorm))) return rc;
-    k_scaled_to_float<<<G, 256, 0, s>>>(sp.t, inner.dnorm, sp.r32, Nu3);
+    if ((rc = launch_to_float(z + Nu3, sp.z32, Np, s))) return rc;  // (27 reads per node: converted once)
+    if ((rc = launch_add_gradient(h, sp.z32, v, sp.t, s))) return rc;
+    // velocity block: FP32 GMRES on t / |t| from zero, one cycle, then z_u = |t| d
+    double* const tnorm = inner.dnorm + 1;  // (the solve overwrites dnorm[0])
+    if ((rc = norm2_dev<double>(inner, sp.t, tnorm))) return rc;
+    k_scaled_to_float<<<scale_grid(Nu3), 256, 0, s>>>(sp.t, tnorm, sp.r32, Nu3);
     EVAP_CHECK_LAUNCH("saddle_to32");
     EVAP_CUDA(cudaMemsetAsync(sp.d32, 0, Nu3 * sizeof(float), s));
     int its = 0;
     double res = 0.0;
     if ((rc = gmres<float>(inner, SADDLE_INNER_M, sp.r32, sp.d32, true, h->diag32, sp.V32, sp.w32, sp.z32,
-                           SADDLE_INNER_TOL, SADDLE_INNER_M, &its, &res)))
+                           SADDLE_INNER_TOL, SADDLE_INNER_M, &its, &res, true)))
         return rc;
-    if ((rc = norm2_dev<double>(inner, sp.t, inner.dnorm))) return rc;
-    EVAP_CUDA(cudaMemsetAsync(z, 0, Nu3 * sizeof(double), s));
-    k_refine<<<G, 256, 0, s>>>(z, sp.d32, inner.dnorm, Nu3);
+    k_scaled_to_double<<<scale_grid(Nu3), 256, 0, s>>>(z, sp.d32, tnorm, Nu3);
     EVAP_CHECK_LAUNCH("saddle_velocity");
     return EVAP_OK;
 }
@@ -896,7 +913,7 @@ int solve_saddle(evap_mesh* h, const double* f, double* x, double* p, int m, dou
         if ((rc = fetch(c, c.dnorm, 1, c.hcol))) return rc;
         beta = std::sqrt(c.hcol[0]);
         if (beta <= target || used >= max_iter || !(beta > 0.0)) break;
-        k_scale_vec<<<G, 256, 0, s>>>(sp.V, c.dnorm, N);
+        k_scale_vec<<<scale_grid(N), 256, 0, s>>>(sp.V, c.dnorm, N);
         EVAP_CHECK_LAUNCH("saddle_scale");
         std::fill(gv.begin(), gv.end(), 0.0);
         gv[0] = beta;
@@ -916,7 +933,7 @@ int solve_saddle(evap_mesh* h, const double* f, double* x, double* p, int m, dou
             EVAP_CUDA(cudaStreamSynchronize(s));
             for (int i = 0; i < nv; ++i) col[i] = c.hcol[i];
             double after = c.hcol[m + 2];
-            if (after < REORTH64 * c.hcol[nv]) {
+            if (after < REORTH_SADDLE * c.hcol[nv]) {
                 if ((rc = cgs_pass<double>(c, sp.V, Wn, nv, c.dcol + (m + 2), false))) return rc;
                 EVAP_CUDA(cudaMemcpyAsync(c.hcol, c.dcol + (m + 2), (size_t)nv * sizeof(double),
                                           cudaMemcpyDeviceToHost, s));
@@ -928,7 +945,7 @@ int solve_saddle(evap_mesh* h, const double* f, double* x, double* p, int m, dou
             const double hn = std::sqrt(after);
             col[j + 1] = hn;
             if (hn > 0.0) {
-                k_scale_vec<<<G, 256, 0, s>>>(Wn, c.dnorm, N);
+                k_scale_vec<<<scale_grid(N), 256, 0, s>>>(Wn, c.dnorm, N);
                 EVAP_CHECK_LAUNCH("saddle_scale");
             }
             for (int i = 0; i < j; ++i) {

@@ -1,6 +1,6 @@
 // Velocity-pressure coupling of Eq. (weakNavierStokes) with the Q1 pressure of Sec. 2.5 (k_p = 1), FP64:
-//   pressure term of the momentum row   y_(c,i) += s sum_q W p_h(x_q) d_c N_i(x_q)      (s = -1: -(div v, p); the
-//                                       saddle-point apply folds it into the momentum kernel's stress flux)
+//   pressure gradient of the preconditioner   t = v + B^T p   (the saddle-point apply folds its pressure term -(div v, p)
+//                                       into the momentum kernel's stress flux)
 //   continuity right-hand side         g_j = sum_q W N1_j v_dil                           (Eq. continuity, evaporDil)
 //   saddle-point apply                 [y; y_p] = [A x - B^T p; B x]
 // with B the divergence row of the momentum apply (velocity Gauss rule, Dirichlet entries of x read as 0) and
@@ -9,87 +9,74 @@
 
 namespace evap {
 
-// B^T p, scaled by s, added to y: one thread per velocity quadrature point, CB cells per block.  The pressure is
-// interpolated at the point from the cell's 8 Q1 nodes; the test with d_c N_i is the transpose of the momentum
-// apply's gradient (collocation derivative at the Gauss points along c, then S^T along z, y, x), so B^T here is
-// the exact transpose of the divergence row.
-template <typename T, int P, int CB>
-__global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
-    k_pressure_gradient(MeshArgs<T> m, Basis<T> bas, const T* __restrict__ p, T s, T* __restrict__ y) {
-    constexpr int Q = P + 1, NQ = Q * Q * Q;
-    __shared__ T sS[Q][Q], sDc[Q][Q], sN1[Q][2];
-    __shared__ T val[CB][NQ];
-    __shared__ T buf[2][CB][3][NQ];
-    const int tid = threadIdx.x;
-    const int lc = tid / NQ, t = tid % NQ;
-    const int64_t cell = (int64_t)blockIdx.x * CB + lc;
-    const bool active = cell < m.ncell;
-    if (tid < Q * Q) {
-        sS[tid / Q][tid % Q] = bas.S[tid / Q][tid % Q];
-        sDc[tid / Q][tid % Q] = bas.Dc[tid / Q][tid % Q] * m.inv_h;
+// t = v + B^T p with the gradient in FP32.  B_c[j][v] = prod_d F^c_d[j_d][v_d] is a tensor product of 1D integrals (as in
+// schur.cu: g1 = the integral of N1_J l_V' along c, a1 = that of N1_J l_V along the other two, both exact with the
+// velocity Gauss rule), and a velocity node meets at most 3 pressure nodes per direction.  So one thread per velocity node
+// sums its 3 x 3 x 3 neighbours separably (x, then y, then z) and adds v: no scatter, no intermediate vector.  Measured at
+// 64^3 Q2 (us): 63; a quadrature kernel with its scatter, memset and addition took 109 + 4 + 28.
+// The 1D row of velocity node V: its first pressure node I0 and the factors of I0, I0 + 1, I0 + 2 (0 where there is none).
+__device__ __forceinline__ int gradient_row(const float (&a1)[2][MAXQ], const float (&g1)[2][MAXQ], int P, int n, int V,
+                                            float (&a)[3], float (&g)[3]) {
+    const int e = V / P, b = V - e * P;  // cell and local node; b = 0: a vertex, shared with cell e - 1
+    a[0] = a[1] = a[2] = g[0] = g[1] = g[2] = 0.f;
+    if (b != 0) {  // inside cell e: pressure nodes e, e + 1
+        a[0] = a1[0][b]; a[1] = a1[1][b];
+        g[0] = g1[0][b]; g[1] = g1[1][b];
+        return e;
     }
-    if (tid < 2 * Q) sN1[tid / 2][tid % 2] = bas.N1[tid / 2][tid % 2];
-    __syncthreads();
-    const int a = t % Q, b = (t / Q) % Q, c = t / (Q * Q);
-    const int n = m.n;
-    int cx = 0, cy = 0, cz = 0;
-    if (active) {
-        cx = (int)(cell % n);
-        cy = (int)((cell / n) % n);
-        cz = (int)(cell / ((int64_t)n * n));
-        const int64_t m1 = n + 1;
-        T pq = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int ja = j & 1, jb = (j >> 1) & 1, jc = j >> 2;
-            pq += sN1[a][ja] * sN1[b][jb] * sN1[c][jc] * p[(cx + ja) + m1 * ((cy + jb) + m1 * (cz + jc))];
-        }
-        val[lc][t] = s * bas.w[a] * bas.w[b] * bas.w[c] * m.vol_w * pq;
+    // vertex e: node e - 1 and e from cell e - 1 (local node P), e and e + 1 from cell e (local node 0)
+    if (e > 0) {
+        a[0] = a1[0][P]; a[1] = a1[1][P];
+        g[0] = g1[0][P]; g[1] = g1[1][P];
     }
-    __syncthreads();
-    if (active) {
-        T d0 = 0, d1 = 0, d2 = 0;
-#pragma unroll
-        for (int r = 0; r < Q; ++r) {
-            d0 += sDc[r][a] * val[lc][r + Q * (b + Q * c)];
-            d1 += sDc[r][b] * val[lc][a + Q * (r + Q * c)];
-            d2 += sDc[r][c] * val[lc][a + Q * (b + Q * r)];
-        }
-        buf[0][lc][0][t] = d0;
-        buf[0][lc][1][t] = d1;
-        buf[0][lc][2][t] = d2;
+    if (e < n) {
+        a[1] += a1[0][0]; a[2] = a1[1][0];
+        g[1] += g1[0][0]; g[2] = g1[1][0];
     }
-    __syncthreads();
-    if (active)
+    return e - 1;
+}
+struct GradientTables {
+    float a[2][MAXQ], g[2][MAXQ];  // a[j][b] = h sum_q w_q N1_j l_b, g[j][b] = sum_q w_q N1_j l_b'
+};
+__global__ void __launch_bounds__(128) k_add_gradient(int n, int P, int M, int64_t Nu, unsigned faces, GradientTables tab,
+                                                      const float* __restrict__ p, const double* __restrict__ v,
+                                                      double* __restrict__ t) {
+    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.y, z = blockIdx.z;
+    if (x >= M || y >= M) return;
+    const int64_t node = x + (int64_t)M * (y + (int64_t)M * z);
+    float acc[3] = {0.f, 0.f, 0.f};
+    if (!constrained_node(x, y, z, M, faces)) {
+        float ax[3], gx[3], ay[3], gy[3], az[3], gz[3];
+        const int ix = gradient_row(tab.a, tab.g, P, n, x, ax, gx), iy = gradient_row(tab.a, tab.g, P, n, y, ay, gy),
+                  iz = gradient_row(tab.a, tab.g, P, n, z, az, gz);
+        const int m1 = n + 1;
 #pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            T v = 0;
+        for (int kz = 0; kz < 3; ++kz) {
+            if (az[kz] == 0.f && gz[kz] == 0.f) continue;
+            float r0 = 0.f, r1 = 0.f, r2 = 0.f;
 #pragma unroll
-            for (int q = 0; q < Q; ++q) v += sS[q][c] * buf[0][lc][f][a + Q * (b + Q * q)];
-            buf[1][lc][f][t] = v;
+            for (int ky = 0; ky < 3; ++ky) {
+                if (ay[ky] == 0.f && gy[ky] == 0.f) continue;
+                const float* row = p + ix + (int64_t)m1 * ((iy + ky) + (int64_t)m1 * (iz + kz));
+                float sa = 0.f, sg = 0.f;
+#pragma unroll
+                for (int kx = 0; kx < 3; ++kx) {
+                    if (ax[kx] == 0.f && gx[kx] == 0.f) continue;  // (also keeps the reads inside the lattice)
+                    const float q = row[kx];
+                    sa = fmaf(ax[kx], q, sa);
+                    sg = fmaf(gx[kx], q, sg);
+                }
+                r0 = fmaf(ay[ky], sg, r0);
+                r1 = fmaf(gy[ky], sa, r1);
+                r2 = fmaf(ay[ky], sa, r2);
+            }
+            acc[0] = fmaf(az[kz], r0, acc[0]);
+            acc[1] = fmaf(az[kz], r1, acc[1]);
+            acc[2] = fmaf(gz[kz], r2, acc[2]);
         }
-    __syncthreads();
-    if (active)
-#pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            T v = 0;
-#pragma unroll
-            for (int q = 0; q < Q; ++q) v += sS[q][b] * buf[1][lc][f][a + Q * (q + Q * c)];
-            buf[0][lc][f][t] = v;
-        }
-    __syncthreads();
-    if (!active) return;
-    const int M = m.M;
-    const int gx = P * cx + a, gy = P * cy + b, gz = P * cz + c;
-    if (constrained_node(gx, gy, gz, M, m.faces)) return;
-    const int64_t gidx = gx + (int64_t)M * (gy + (int64_t)M * gz);
-#pragma unroll
-    for (int f = 0; f < 3; ++f) {
-        T v = 0;
-#pragma unroll
-        for (int q = 0; q < Q; ++q) v += sS[q][a] * buf[0][lc][f][q + Q * (b + Q * c)];
-        atomicAdd(&y[f * m.Nu + gidx], v);
     }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) t[c * Nu + node] = v[c * Nu + node] + (double)acc[c];
 }
 
 // g_j += sum_q N1_j(x_q) (W v_dil)_q over the cell's velocity Gauss points, from the cached coefficient slot 18.
@@ -114,105 +101,6 @@ __global__ void __launch_bounds__(128) k_continuity_rhs(MeshArgs<double> m, Basi
 #pragma unroll
     for (int j = 0; j < 8; ++j)
         atomicAdd(&g[(cx + (j & 1)) + m1 * ((cy + ((j >> 1) & 1)) + m1 * (cz + (j >> 2)))], out[j]);
-}
-
-// y_p += B D^(-1) x (D = diag when given, else the identity): the divergence row of the momentum apply without its
-// source, sum_q W N1_j (div x)(x_q); values at the points by S sweeps (x, y, z), the divergence by the collocation
-// derivative, the Q1 test by three sweeps of N1.
-template <typename T, int P, int CB>
-__global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
-    k_divergence(MeshArgs<T> m, Basis<T> bas, const T* __restrict__ x, const T* __restrict__ diag,
-                 T* __restrict__ yp) {
-    constexpr int Q = P + 1, NQ = Q * Q * Q;
-    __shared__ T sS[Q][Q], sDc[Q][Q], sN1[Q][2];
-    __shared__ T buf[2][3][CB][NQ];
-    __shared__ T rbuf[CB][NQ], q1a[CB][2 * Q * Q], q1b[CB][4 * Q];
-    const int tid = threadIdx.x;
-    const int lc = tid / NQ, t = tid % NQ;
-    const int64_t cell = (int64_t)blockIdx.x * CB + lc;
-    const bool active = cell < m.ncell;
-    if (tid < Q * Q) {
-        sS[tid / Q][tid % Q] = bas.S[tid / Q][tid % Q];
-        sDc[tid / Q][tid % Q] = bas.Dc[tid / Q][tid % Q] * m.inv_h;
-    }
-    if (tid < 2 * Q) sN1[tid / 2][tid % 2] = bas.N1[tid / 2][tid % 2];
-    const int a = t % Q, b = (t / Q) % Q, c = t / (Q * Q);
-    const int n = m.n, M = m.M;
-    int cx = 0, cy = 0, cz = 0;
-    if (active) {
-        cx = (int)(cell % n);
-        cy = (int)((cell / n) % n);
-        cz = (int)(cell / ((int64_t)n * n));
-        const int gx = P * cx + a, gy = P * cy + b, gz = P * cz + c;
-        const int64_t gidx = gx + (int64_t)M * (gy + (int64_t)M * gz);
-        const bool cons = constrained_node(gx, gy, gz, M, m.faces);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int64_t i = k * m.Nu + gidx;
-            buf[0][k][lc][t] = cons ? T(0) : (diag ? x[i] / diag[i] : x[i]);
-        }
-    }
-    __syncthreads();
-    if (active)
-#pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            T v = 0;
-#pragma unroll
-            for (int k = 0; k < Q; ++k) v += sS[a][k] * buf[0][f][lc][k + Q * (b + Q * c)];
-            buf[1][f][lc][t] = v;
-        }
-    __syncthreads();
-    if (active)
-#pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            T v = 0;
-#pragma unroll
-            for (int k = 0; k < Q; ++k) v += sS[b][k] * buf[1][f][lc][a + Q * (k + Q * c)];
-            buf[0][f][lc][t] = v;
-        }
-    __syncthreads();
-    if (active)
-#pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            T v = 0;
-#pragma unroll
-            for (int k = 0; k < Q; ++k) v += sS[c][k] * buf[0][f][lc][a + Q * (b + Q * k)];
-            buf[1][f][lc][t] = v;
-        }
-    __syncthreads();
-    if (active) {
-        T tr = 0;
-#pragma unroll
-        for (int r = 0; r < Q; ++r)
-            tr += sDc[a][r] * buf[1][0][lc][r + Q * (b + Q * c)] + sDc[b][r] * buf[1][1][lc][a + Q * (r + Q * c)] +
-                  sDc[c][r] * buf[1][2][lc][a + Q * (b + Q * r)];
-        rbuf[lc][t] = bas.w[a] * bas.w[b] * bas.w[c] * m.vol_w * tr;
-    }
-    __syncthreads();
-    if (active && t < 2 * Q * Q) {  // x-sweep: [jx][qy][qz]
-        const int jx = t & 1, qy = (t >> 1) % Q, qz = (t >> 1) / Q;
-        T v = 0;
-#pragma unroll
-        for (int q = 0; q < Q; ++q) v += sN1[q][jx] * rbuf[lc][q + Q * (qy + Q * qz)];
-        q1a[lc][t] = v;
-    }
-    __syncthreads();
-    if (active && t < 4 * Q) {  // y-sweep: [jx][jy][qz]
-        const int jx = t & 1, jy = (t >> 1) & 1, qz = t >> 2;
-        T v = 0;
-#pragma unroll
-        for (int q = 0; q < Q; ++q) v += sN1[q][jy] * q1a[lc][jx + 2 * (q + Q * qz)];
-        q1b[lc][t] = v;
-    }
-    __syncthreads();
-    if (active && t < 8) {  // z-sweep: Q1 node (jx, jy, jz)
-        const int jx = t & 1, jy = (t >> 1) & 1, jz = t >> 2;
-        T v = 0;
-#pragma unroll
-        for (int q = 0; q < Q; ++q) v += sN1[q][jz] * q1b[lc][jx + 2 * (jy + 2 * q)];
-        const int64_t m1 = n + 1;
-        atomicAdd(&yp[(cx + jx) + m1 * ((cy + jy) + m1 * (cz + jz))], v);
-    }
 }
 
 // f += sum_q W rho c_m N_i (u_c + g_c / c_m) at the velocity Gauss points (the BDF1 inertia load of the old velocity
@@ -323,37 +211,25 @@ __global__ void k_add_vec(double* __restrict__ y, const double* __restrict__ g, 
         y[i] += g[i];
 }
 
-template <typename T>
-int launch_pressure_gradient(evap_mesh* h, const T* p, T s, T* y, cudaStream_t st) {
-    const MeshArgs<T> m = mesh_args<T>(h);
-    const Basis<T> b = cast_basis<T>(h->b);
-    if (m.P == 2) {
-        constexpr int CB = 8;
-        k_pressure_gradient<T, 2, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 27, 0, st>>>(m, b, p, s, y);
-    } else {
-        constexpr int CB = 4;
-        k_pressure_gradient<T, 3, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 64, 0, st>>>(m, b, p, s, y);
-    }
-    EVAP_CHECK_LAUNCH("pressure_gradient");
+int launch_add_gradient(evap_mesh* h, const float* p, const double* v, double* t, cudaStream_t st) {
+    const MeshArgs<double>& m = h->m;
+    const Basis<double>& b = h->b;
+    GradientTables tab{};
+    for (int j = 0; j < 2; ++j)
+        for (int k = 0; k <= m.P; ++k) {
+            double sa = 0.0, sg = 0.0;
+            for (int q = 0; q < b.Q; ++q) {
+                sa += b.w[q] * b.N1[q][j] * b.S[q][k];
+                sg += b.w[q] * b.N1[q][j] * b.D[q][k];
+            }
+            tab.a[j][k] = (float)(m.h * sa);
+            tab.g[j][k] = (float)sg;
+        }
+    const dim3 grid((unsigned)((m.M + 31) / 32), (unsigned)((m.M + 3) / 4), (unsigned)m.M);
+    k_add_gradient<<<grid, dim3(32, 4), 0, st>>>(m.n, m.P, m.M, m.Nu, m.faces, tab, p, v, t);
+    EVAP_CHECK_LAUNCH("add_gradient");
     return EVAP_OK;
 }
-template int launch_pressure_gradient<float>(evap_mesh*, const float*, float, float*, cudaStream_t);
-
-template <typename T>
-int launch_divergence(evap_mesh* h, const T* x, const T* diag, T* yp, cudaStream_t st) {
-    const MeshArgs<T> m = mesh_args<T>(h);
-    const Basis<T> b = cast_basis<T>(h->b);
-    if (m.P == 2) {
-        constexpr int CB = 8;
-        k_divergence<T, 2, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 27, 0, st>>>(m, b, x, diag, yp);
-    } else {
-        constexpr int CB = 4;
-        k_divergence<T, 3, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 64, 0, st>>>(m, b, x, diag, yp);
-    }
-    EVAP_CHECK_LAUNCH("divergence");
-    return EVAP_OK;
-}
-template int launch_divergence<float>(evap_mesh*, const float*, const float*, float*, cudaStream_t);
 
 // z = S~^(-1) r, S~ = B diag(A)^(-1) B^T (a SIMPLE-type approximation of the Schur complement B A^(-1) B^T: it keeps
 // the discrete B, so the pressure nodes of open faces are treated like every other node): at most cg_iters iterations
