@@ -135,15 +135,12 @@ struct evap_mesh {
     double* table = nullptr;
     float* table32 = nullptr;
     float2* adj_table = nullptr;  // [table_cap][ADJ_K][nq] pairs for the adjoint
-    // quadrature-point coefficients of the FP64 momentum operator, all cells [ncell][QC_K][nq]
-    double* qc = nullptr;
-    // the same coefficients as double-float pairs (hi, lo) [ncell][QC_K][nq] for the double-float FP64 apply
+    // quadrature-point coefficients of the momentum operator, all cells, as double-float pairs (hi, lo) [ncell][QC_K][nq]
     float* qcdf = nullptr;
     int64_t qcdf_len = 0;  // floats
-    // FP32 copy of the u0 coefficients (slots 1..12 of qc) in the 32-cell block layout of the FP32 apply
+    // FP32 copy of the u0 coefficients (slots 1..12 of qcdf) in the 32-cell block layout of the FP32 apply
     float* qc32 = nullptr;
     int64_t qc32_len = 0;
-    int64_t qc_len = 0;
     // transport velocity
     double* ugamma = nullptr;
     float* ugamma32 = nullptr;

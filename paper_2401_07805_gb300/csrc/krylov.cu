@@ -11,17 +11,17 @@
 #include <cmath>
 #include <vector>
 
-#include "evap_internal.cuh"
+#include "df_lines.cuh"
 
 namespace evap {
 
 // ------------------------------------------------------------------------------------------- Jacobi diagonal
 // diag_(i,c) = sum_q [ W rho c_m N_i^2 + N_i (W rho u0 . grad N_i) + N_i^2 newton W rho d_c u0_c
 //                      + 2 W mu ( (|grad N_i|^2 + (d_c N_i)^2)/2 - (z n)_c d_c N_i ((z n) . grad N_i) ) ]
-// in FP32 from the quadrature-point cache of set_fields (k_qp_coeffs); one thread per (cell, local node).
+// in FP32 from the high parts of the quadrature-point cache of set_fields (k_qp_coeffs); one thread per (cell, local node).
 template <int P, int CB>
 __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
-    k_diagonal(MeshArgs<float> m, Basis<float> bas, const double* __restrict__ qc,
+    k_diagonal(MeshArgs<float> m, Basis<float> bas, float dscale, const float2* __restrict__ qc,
                float* __restrict__ diag, int colour) {
     constexpr int Q = P + 1, NQ = Q * Q * Q;
     __shared__ float sS[Q][Q], sD[Q][Q];
@@ -32,14 +32,14 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
     const int64_t cell = cx + (int64_t)m.n * (cy + (int64_t)m.n * cz);
     if (tid < Q * Q) {
         sS[tid / Q][tid % Q] = bas.S[tid / Q][tid % Q];
-        sD[tid / Q][tid % Q] = bas.D[tid / Q][tid % Q];
+        sD[tid / Q][tid % Q] = bas.D[tid / Q][tid % Q] * dscale;
     }
     const int a = t % Q, b = (t / Q) % Q, c = t / (Q * Q);
     if (active) {
-        const double* qp = qc + cell * QC_K * NQ + t;
+        const float2* qp = qc + cell * QC_K * NQ + t;
         constexpr int slot[11] = {0, 1, 2, 3, 4, 8, 12, 13, 14, 15, 16};
 #pragma unroll
-        for (int k = 0; k < 11; ++k) qd[lc][k][t] = (float)qp[slot[k] * NQ];
+        for (int k = 0; k < 11; ++k) qd[lc][k][t] = qp[slot[k] * NQ].x;
     }
     __syncthreads();
     if (!active) return;
@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
         const int qa = q % Q, qb = (q / Q) % Q, qcz = q / (Q * Q);
         const float sa = sS[qa][a], sb = sS[qb][b], sc = sS[qcz][c];
         const float N = sa * sb * sc;
-        const float g[3] = {sD[qa][a] * sb * sc * m.inv_h, sa * sD[qb][b] * sc * m.inv_h, sa * sb * sD[qcz][c] * m.inv_h};
+        const float g[3] = {sD[qa][a] * sb * sc, sa * sD[qb][b] * sc, sa * sb * sD[qcz][c]};
         const float conv = qd[lc][1][q] * g[0] + qd[lc][2][q] * g[1] + qd[lc][3][q] * g[2];
         const float gg = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
         const float ng = qd[lc][8][q] * g[0] + qd[lc][9][q] * g[1] + qd[lc][10][q] * g[2];
@@ -82,15 +82,16 @@ __global__ void k_diag_finish(int M, int64_t Nu, unsigned faces, float* d32, dou
 // of the deterministic mode.
 static int diagonal_passes(evap_mesh* h, const MeshArgs<float>& m, const Basis<float>& b, float* acc, cudaStream_t s) {
     const int c0 = h->deterministic ? 0 : -1, c1 = h->deterministic ? 8 : 0;
+    const float dscale = (float)(h->m.inv_h / df_kappa(h->m));  // gradients in units of kappa, as the cached slots expect
     for (int colour = c0; colour < std::max(c1, c0 + 1); ++colour) {
         const int64_t cells = colour_cells(m.n, colour);
         if (cells == 0) continue;
         if (m.P == 2) {
             constexpr int CB = 8;
-            k_diagonal<2, CB><<<(unsigned)((cells + CB - 1) / CB), CB * 27, 0, s>>>(m, b, h->qc, acc, colour);
+            k_diagonal<2, CB><<<(unsigned)((cells + CB - 1) / CB), CB * 27, 0, s>>>(m, b, dscale, (const float2*)h->qcdf, acc, colour);
         } else {
             constexpr int CB = 4;
-            k_diagonal<3, CB><<<(unsigned)((cells + CB - 1) / CB), CB * 64, 0, s>>>(m, b, h->qc, acc, colour);
+            k_diagonal<3, CB><<<(unsigned)((cells + CB - 1) / CB), CB * 64, 0, s>>>(m, b, dscale, (const float2*)h->qcdf, acc, colour);
         }
         EVAP_CHECK_LAUNCH("diagonal");
     }

@@ -3,9 +3,7 @@
 //   k_momentum_init   y = x on the Dirichlet DoFs, 0 elsewhere (the scatter of the applies adds the free rows)
 //   k_qp_coeffs       the quadrature-point coefficients of the operator (W rho c_m, W rho u0, W rho grad u0, 2 W mu,
 //                     z n, W, W v_dil), evaluated once per set_fields in double-float arithmetic and stored as
-//                     double-float pairs (the FP64-accurate apply of momentum_df.cu and the adjoint), in FP64 (Jacobi
-//                     diagonal, continuity right-hand side, mass load) and, for the u0 terms, in FP32 (the FP32
-//                     apply of momentum32.cu): on GB300 the
+//                     double-float pairs and, for the u0 terms, in FP32 (the FP32 apply of momentum32.cu): on GB300 the
 //                     arithmetic, not HBM, bounds these operators, and the material law and the u0 interpolation
 //                     would otherwise be recomputed by every apply
 //   launch_momentum   dispatch: FP64 -> double-float kernel, FP32 -> line kernel; the lifting variant (all columns)
@@ -37,138 +35,172 @@ __global__ void __launch_bounds__(256) k_momentum_init(int M, int64_t Nu, unsign
     }
 }
 
-// Quadrature-point coefficients of the FP64 momentum operator, evaluated once per set_fields from u0 and the
-// material-law table (layout [cell][QC_K][nq]):
-//   0: W rho c_m   1..3: W rho u0_b   4..12: newton W rho d_d u0_c (index 4 + 3c + d)   13: 2 W mu
+// Quadrature-point coefficients of the momentum operator, evaluated once per set_fields from u0 and the material-law table,
+// as double-float pairs (layout [cell][QC_K][nq]):
+//   0: W rho c_m   1..3: kappa W rho u0_b   4..12: newton W rho d_d u0_c (index 4 + 3c + d)   13: kappa^2 2 W mu
 //   14..16: z n_b (correction gate times normal)   17: W   18: W v_dil
-// W = w_qx w_qy w_qz h^3.  One thread per quadrature point, CB cells per block (u0 interpolated by sum factorization).
-// Slots 1..12 are also stored in FP32 for the FP32 apply (slots 1..3 divided by h: that kernel takes reference
-// gradients), in its 32-cell block layout
+// W = w_qx w_qy w_qz h^3, kappa = DSCALE / h the factor between a gradient and the derivative sweeps (df_lines.cuh).  The
+// FP64-accurate apply and the adjoint read the pairs as they stand; the Jacobi diagonal, the mass load and the continuity
+// right-hand side read the few slots they need.  Slots 1..12 are also stored in FP32 for the FP32 apply (there W rho u0 / h:
+// that kernel takes reference gradients), in its 32-cell block layout
 // qc32[((blk * QC32_K + k) * NQ + pt) * 32 + lane], cell 32 blk + lane (lexicographic).
-// The interpolation of u0 and every product run in double-float arithmetic (dfloat.cuh) on the FP32 pipe: the FP64
-// pipe keeps the conversions (u0 in, the FP64 copy of each coefficient out) and the few scalar factors.  The
-// double-float results are the pairs of the apply's cache as they stand; the FP64 copy is their sum (within 2^-48).
+// u0 is interpolated by lines (df_lines.cuh).  The weights and, outside table cells, W rho and 2 W mu take the same NQ
+// values in every cell: tabulated on the host, so that the FP64 pipe converts u0 and the table cells' entries only.  A
+// block takes CB cells of one 32-cell block, and writes their FP32 entries through shared memory in runs of CB floats.
+// Measured at 64^3 Q2 (us): 1374 -> 372 (point-wise dot products, an FP64 copy of every coefficient beside the pairs, 1.1
+// GB, and scattered FP32 stores before); the writes alone take 210 at the HBM rate.
+template <int NQ>
+struct QpTables {
+    float2 w[NQ], wr[2][NQ], wm[2][NQ];  // W; W rho and kappa^2 2 W mu of gas (0) and liquid (1)
+};
 template <int P, int CB>
 __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
-    k_qp_coeffs(MeshArgs<double> m, Basis<double> bas, DfBasis dfb, dfl cm_df, dfl invh_df, dfl kap, dfl kap2,
-                const int8_t* __restrict__ code, const int32_t* __restrict__ tindex, const double* __restrict__ table,
-                const double* __restrict__ u0, double* __restrict__ qc, float2* __restrict__ qcdf,
+    k_qp_coeffs(MeshArgs<double> m, Basis<double> bas, QpTables<(P + 1) * (P + 1) * (P + 1)> tabs, dfl cm_df, dfl kap,
+                dfl kap2, dfl ik, const int8_t* __restrict__ code, const int32_t* __restrict__ tindex,
+                const double* __restrict__ table, const double* __restrict__ u0, float2* __restrict__ qcdf,
                 float* __restrict__ qc32) {
-    constexpr int Q = P + 1, NQ = Q * Q * Q;
-    __shared__ dfl sS[Q][Q], sDc[Q][Q];
-    __shared__ dfl buf[2][CB][3][NQ];
+    constexpr int Q = P + 1, NQ = Q * Q * Q, NL = Q * Q, TASKS = 3 * NL;
+    static_assert(32 % CB == 0, "a block's cells lie in one 32-cell block");
+    using Ln = DfLine<Q>;
+    __shared__ dfl buf[CB][12][NQ];  // slots: 0..2 U, 3 + 3 k + d the derivatives (in units of kappa)
+    __shared__ float2 sw[NQ], swr[2][NQ], swm[2][NQ];
     const int tid = threadIdx.x;
     const int lc = tid / NQ, t = tid % NQ;
-    const int64_t cell = (int64_t)blockIdx.x * CB + lc;
-    const bool active = cell < m.ncell;
-    if (tid < Q * Q) {
-        sS[tid / Q][tid % Q] = dfb.S[tid / Q][tid % Q];
-        sDc[tid / Q][tid % Q] = dfb.Dc[tid / Q][tid % Q];  // physical: Dc / h
-    }
-    const int a = t % Q, b = (t / Q) % Q, c = t / (Q * Q);
-    const int n = m.n, M = m.M;
-    if (active) {
-        const int cx = (int)(cell % n), cy = (int)((cell / n) % n), cz = (int)(cell / ((int64_t)n * n));
-        const int64_t gidx = (P * cx + a) + (int64_t)M * ((P * cy + b) + (int64_t)M * (P * cz + c));
+    const unsigned cell0 = blockIdx.x * CB;
+    int cx, cy, cz;
+    const bool active = colour_cell32(cell0 + lc, m.n, -1, cx, cy, cz);
+    for (int i = tid; i < NQ; i += CB * NQ) {
+        sw[i] = tabs.w[i];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) buf[0][lc][k][t] = df_from_double(u0[k * m.Nu + gidx]);
-    }
-    __syncthreads();
-    if (active) {
-        dfl Sa[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Sa[k] = sS[a][k];
-#pragma unroll
-        for (int f = 0; f < 3; ++f) buf[1][lc][f][t] = df_dot<Q>(Sa, &buf[0][lc][f][Q * (b + Q * c)], 1);
-    }
-    __syncthreads();
-    if (active) {
-        dfl Sb[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Sb[k] = sS[b][k];
-#pragma unroll
-        for (int f = 0; f < 3; ++f) buf[0][lc][f][t] = df_dot<Q>(Sb, &buf[1][lc][f][a + Q * Q * c], Q);
-    }
-    __syncthreads();
-    if (active) {
-        dfl Sc[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) Sc[k] = sS[c][k];
-#pragma unroll
-        for (int f = 0; f < 3; ++f) buf[1][lc][f][t] = df_dot<Q>(Sc, &buf[0][lc][f][a + Q * b], Q * Q);
-    }
-    __syncthreads();
-    if (!active) return;
-    dfl U[3], GU[3][3];
-    {
-        dfl Da[Q], Db[Q], Dz[Q];
-#pragma unroll
-        for (int k = 0; k < Q; ++k) {
-            Da[k] = sDc[a][k];
-            Db[k] = sDc[b][k];
-            Dz[k] = sDc[c][k];
+        for (int k = 0; k < 2; ++k) {
+            swr[k][i] = tabs.wr[k][i];
+            swm[k][i] = tabs.wm[k][i];
         }
+    }
+    const int M = m.M;
+    const int64_t zst = (int64_t)M * M;
+    for (int k0 = t; k0 < TASKS; k0 += NQ) {
+        const int f = k0 / NL, l = k0 % NL;
+        const double* src = u0 + f * m.Nu + (P * cx + l % Q) + (int64_t)M * (P * cy + l / Q) + zst * (P * cz);
+        dfl u[Q], v[Q];
+#pragma unroll
+        for (int k = 0; k < Q; ++k) u[k] = df_from_double(src[k * zst]);
+        Ln::val(u, v);
+        st_line<Q, 2>(buf[lc][3 + f], l, v);
+    }
+    __syncthreads();
+    for (int k0 = t; k0 < TASKS; k0 += NQ) {
+        const int f = k0 / NL, l = k0 % NL;
+        dfl u[Q], v[Q];
+        ld_line<Q, 1>(buf[lc][3 + f], l, u);
+        Ln::val(u, v);
+        st_line<Q, 1>(buf[lc][6 + f], l, v);
+    }
+    __syncthreads();
+    for (int k0 = t; k0 < TASKS; k0 += NQ) {
+        const int f = k0 / NL, l = k0 % NL;
+        dfl u[Q], v[Q];
+        ld_line<Q, 0>(buf[lc][6 + f], l, u);
+        Ln::val(u, v);
+        st_line<Q, 0>(buf[lc][f], l, v);
+    }
+    __syncthreads();
+    for (int k0 = t; k0 < TASKS; k0 += NQ) {
+        const int f = k0 / NL, l = k0 % NL;
+        dfl u[Q], v[Q];
+        ld_line<Q, 0>(buf[lc][f], l, u);
+        Ln::der(u, v);
+        st_line<Q, 0>(buf[lc][3 + 3 * f], l, v);
+        ld_line<Q, 1>(buf[lc][f], l, u);
+        Ln::der(u, v);
+        st_line<Q, 1>(buf[lc][4 + 3 * f], l, v);
+        ld_line<Q, 2>(buf[lc][f], l, u);
+        Ln::der(u, v);
+        st_line<Q, 2>(buf[lc][5 + 3 * f], l, v);
+    }
+    __syncthreads();
+    const unsigned cell = cell0 + lc;
+    float f32[QC32_K];
+    {
+        const dfl W = ld_df(&sw[t]);
+        dfl wr, wm, nz[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, wv{0.f, 0.f};
+        const int8_t cc = active ? code[cell] : (int8_t)CELL_GAS;
+        if (cc == CELL_TABLE) {
+            const double* tb = table + (int64_t)tindex[cell] * TAB_K * NQ + t;
+            const double Wd = bas.w[t % Q] * bas.w[(t / Q) % Q] * bas.w[t / NL] * m.vol_w;
+            wr = df_from_double(Wd * tb[0]);
+            wm = df_mul(df_from_double(2.0 * Wd * tb[NQ]), kap2);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) nz[d] = df_from_double(tb[(2 + d) * NQ]);
+            wv = df_from_double(Wd * tb[5 * NQ]);
+        } else {
+            const int liq = cc == CELL_LIQUID ? 1 : 0;
+            wr = ld_df(&swr[liq][t]);
+            wm = ld_df(&swm[liq][t]);
+        }
+        const dfl wk = df_mul(wr, kap);
+        float2* dst = qcdf + (int64_t)cell * QC_K * NQ + t;
+        auto put = [&](int k, dfl v) {
+            if (active) dst[k * NQ] = make_float2(v.hi, v.lo);
+        };
+        put(0, df_mul(wr, cm_df));
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            U[k] = buf[1][lc][k][t];
-            GU[k][0] = df_dot<Q>(Da, &buf[1][lc][k][Q * (b + Q * c)], 1);
-            GU[k][1] = df_dot<Q>(Db, &buf[1][lc][k][a + Q * Q * c], Q);
-            GU[k][2] = df_dot<Q>(Dz, &buf[1][lc][k][a + Q * b], Q * Q);
+            const dfl v = df_mul(wk, buf[lc][k][t]);
+            put(1 + k, v);
+            f32[k] = df_mul(v, ik).hi;
+        }
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const dfl v = m.newton ? df_mul(wk, df_norm(buf[lc][3 + k][t])) : dfl{0.f, 0.f};
+            put(4 + k, v);
+            f32[3 + k] = v.hi;
+        }
+        put(13, wm);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) put(14 + d, nz[d]);
+        put(17, W);
+        put(18, wv);
+    }
+    __syncthreads();
+    float* const st = reinterpret_cast<float*>(buf);  // [k][point][cell]
+#pragma unroll
+    for (int k = 0; k < QC32_K; ++k) st[(k * NQ + t) * CB + lc] = f32[k];
+    __syncthreads();
+    float* const dst32 = qc32 + (int64_t)(cell0 >> 5) * QC32_K * NQ * 32 + (cell0 & 31u);
+    const int live = min(CB, (int)(m.ncell - (int64_t)cell0));
+    for (int i = tid; i < QC32_K * NQ * CB; i += CB * NQ)
+        if (i % CB < live) dst32[(int64_t)(i / CB) * 32 + i % CB] = st[i];
+}
+
+template <int P, int CB>
+static void run_qp_coeffs(evap_mesh* h, cudaStream_t s) {
+    constexpr int Q = P + 1, NQ = Q * Q * Q;
+    const MeshArgs<double>& m = h->m;
+    const double kd = df_kappa(m);
+    const dfl kap2 = df_from_double(kd * kd);
+    QpTables<NQ> tabs;
+    auto pair = [](double v) {
+        const dfl d = df_from_double(v);
+        return make_float2(d.hi, d.lo);
+    };
+    for (int q = 0; q < NQ; ++q) {
+        const double W = h->b.w[q % Q] * h->b.w[(q / Q) % Q] * h->b.w[q / (Q * Q)] * m.vol_w;
+        tabs.w[q] = pair(W);
+        for (int k = 0; k < 2; ++k) {
+            tabs.wr[k][q] = pair(W * (k ? m.rho_H1 : m.rho_H0));
+            tabs.wm[k][q] = pair(kd * kd * 2.0 * W * (k ? m.mu_H1 : m.mu_H0));
         }
     }
-    double rho, mu, nz[3], vd;
-    const int8_t cc = code[cell];
-    const bool tab = cc == CELL_TABLE;
-    if (tab) {
-        const double* tb = table + (int64_t)tindex[cell] * TAB_K * NQ + t;
-        rho = tb[0]; mu = tb[NQ]; nz[0] = tb[2 * NQ]; nz[1] = tb[3 * NQ]; nz[2] = tb[4 * NQ]; vd = tb[5 * NQ];
-    } else {
-        const bool liq = cc == CELL_LIQUID;
-        rho = liq ? m.rho_H1 : m.rho_H0;
-        mu = liq ? m.mu_H1 : m.mu_H0;
-        nz[0] = nz[1] = nz[2] = 0.0;
-        vd = 0.0;
-    }
-    const double W = bas.w[a] * bas.w[b] * bas.w[c] * m.vol_w;
-    const dfl wr = df_from_double(W * rho);
-    dfl v[QC_K];
-    v[0] = df_mul(wr, cm_df);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) v[1 + k] = df_mul(wr, U[k]);
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) v[4 + 3 * k + d] = m.newton ? df_mul(wr, GU[k][d]) : dfl{0.f, 0.f};
-    v[13] = df_from_double(2.0 * W * mu);
-    const dfl z0{0.f, 0.f};
-    v[14] = tab ? df_from_double(nz[0]) : z0;
-    v[15] = tab ? df_from_double(nz[1]) : z0;
-    v[16] = tab ? df_from_double(nz[2]) : z0;
-    v[17] = df_from_double(W);
-    v[18] = tab ? df_from_double(W * vd) : z0;
-    const int64_t base = cell * QC_K * NQ + t;
-#pragma unroll
-    for (int k = 0; k < QC_K; ++k) {
-        qc[base + (int64_t)k * NQ] = df_to_double(v[k]);
-        const dfl w = k >= 1 && k <= 3 ? df_mul(v[k], kap) : (k == 13 ? df_mul(v[k], kap2) : v[k]);
-        qcdf[base + (int64_t)k * NQ] = make_float2(w.hi, w.lo);
-    }
-    float* dst = qc32 + ((cell >> 5) * QC32_K * NQ + t) * 32 + (cell & 31);
-#pragma unroll
-    for (int k = 0; k < QC32_K; ++k) dst[(int64_t)k * NQ * 32] = k < 3 ? df_mul(v[1 + k], invh_df).hi : v[1 + k].hi;
+    k_qp_coeffs<P, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * NQ, 0, s>>>(
+        m, h->b, tabs, df_from_double(m.c_mass), df_from_double(kd), kap2, df_from_double(m.inv_h / kd), h->cell_code,
+        h->table_index, h->table, h->u, (float2*)h->qcdf, h->qc32);
 }
 
 int launch_qp_coeffs(evap_mesh* h, cudaStream_t s) {
     const MeshArgs<double>& m = h->m;
     const int nq = h->b.Q * h->b.Q * h->b.Q;
     const int64_t need = m.ncell * QC_K * nq;
-    if (h->qc_len < need) {
-        if (h->qc) cudaFree(h->qc);
-        h->qc = nullptr;
-        h->qc_len = 0;
-        EVAP_CUDA(cudaMalloc(&h->qc, need * sizeof(double)));
-        h->qc_len = need;
-    }
     if (h->qcdf_len < 2 * need) {
         if (h->qcdf) cudaFree(h->qcdf);
         h->qcdf = nullptr;
@@ -184,19 +216,10 @@ int launch_qp_coeffs(evap_mesh* h, cudaStream_t s) {
         EVAP_CUDA(cudaMalloc(&h->qc32, need32 * sizeof(float)));
         h->qc32_len = need32;
     }
-    const DfBasis dfb = make_df_basis(h->b, m.inv_h);
-    const dfl cm = df_from_double(m.c_mass), ih = df_from_double(m.inv_h);
-    const double kd = df_kappa(m);
-    const dfl kap = df_from_double(kd), kap2 = df_from_double(kd * kd);
-    if (m.P == 2) {
-        constexpr int CB = 8;
-        k_qp_coeffs<2, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 27, 0, s>>>(
-            m, h->b, dfb, cm, ih, kap, kap2, h->cell_code, h->table_index, h->table, h->u, h->qc, (float2*)h->qcdf, h->qc32);
-    } else {
-        constexpr int CB = 4;
-        k_qp_coeffs<3, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 64, 0, s>>>(
-            m, h->b, dfb, cm, ih, kap, kap2, h->cell_code, h->table_index, h->table, h->u, h->qc, (float2*)h->qcdf, h->qc32);
-    }
+    if (m.P == 2)
+        run_qp_coeffs<2, 8>(h, s);
+    else
+        run_qp_coeffs<3, 4>(h, s);
     EVAP_CHECK_LAUNCH("qp_coeffs");
     return EVAP_OK;
 }

@@ -5,6 +5,7 @@
 //   saddle-point apply                 [y; y_p] = [A x - B^T p; B x]
 // with B the divergence row of the momentum apply (velocity Gauss rule, Dirichlet entries of x read as 0) and
 // Dirichlet-constrained velocity rows left to the momentum apply (identity), so B^T p vanishes there.
+#include "dfloat.cuh"
 #include "physics.cuh"
 
 namespace evap {
@@ -82,17 +83,17 @@ __global__ void __launch_bounds__(128) k_add_gradient(int n, int P, int M, int64
 // g_j += sum_q N1_j(x_q) (W v_dil)_q over the cell's velocity Gauss points, from the cached coefficient slot 18.
 template <int P>
 __global__ void __launch_bounds__(128) k_continuity_rhs(MeshArgs<double> m, Basis<double> bas,
-                                                        const double* __restrict__ qc, double* __restrict__ g) {
+                                                        const float2* __restrict__ qc, double* __restrict__ g) {
     constexpr int Q = P + 1, NQ = Q * Q * Q;
     const int64_t cell = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (cell >= m.ncell) return;
     const int n = m.n;
     const int cx = (int)(cell % n), cy = (int)((cell / n) % n), cz = (int)(cell / ((int64_t)n * n));
-    const double* v = qc + cell * QC_K * NQ + 18 * NQ;
+    const float2* v = qc + cell * QC_K * NQ + 18 * NQ;
     double out[8] = {};
     for (int t = 0; t < NQ; ++t) {
         const int a = t % Q, b = (t / Q) % Q, c = t / (Q * Q);
-        const double vt = v[t];
+        const double vt = df_to_double(ld_df(v + t));
 #pragma unroll
         for (int j = 0; j < 8; ++j)
             out[j] += bas.N1[a][j & 1] * bas.N1[b][(j >> 1) & 1] * bas.N1[c][j >> 2] * vt;
@@ -108,7 +109,7 @@ __global__ void __launch_bounds__(128) k_continuity_rhs(MeshArgs<double> m, Basi
 // constrained rows of f are left untouched (zero).
 template <int P, int CB>
 __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
-    k_mass_load(MeshArgs<double> m, Basis<double> bas, const double* __restrict__ qc, const double* __restrict__ u,
+    k_mass_load(MeshArgs<double> m, Basis<double> bas, const float2* __restrict__ qc, const double* __restrict__ u,
                 double g0, double g1, double g2, double* __restrict__ f) {
     constexpr int Q = P + 1, NQ = Q * Q * Q;
     __shared__ double sS[Q][Q];
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
         }
     __syncthreads();
     if (active) {
-        const double cf0 = qc[cell * QC_K * NQ + t];  // W rho c_m
+        const double cf0 = df_to_double(ld_df(qc + cell * QC_K * NQ + t));  // W rho c_m
         const double gc[3] = {g0 / m.c_mass, g1 / m.c_mass, g2 / m.c_mass};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -195,11 +196,11 @@ int launch_mass_load(evap_mesh* h, const double* u, const double g[3], double* f
     EVAP_CUDA(cudaMemsetAsync(f, 0, 3 * m.Nu * sizeof(double), st));
     if (m.P == 2) {
         constexpr int CB = 8;
-        k_mass_load<2, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 27, 0, st>>>(m, h->b, h->qc, u, g[0], g[1],
+        k_mass_load<2, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 27, 0, st>>>(m, h->b, (const float2*)h->qcdf, u, g[0], g[1],
                                                                                    g[2], f);
     } else {
         constexpr int CB = 4;
-        k_mass_load<3, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 64, 0, st>>>(m, h->b, h->qc, u, g[0], g[1],
+        k_mass_load<3, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 64, 0, st>>>(m, h->b, (const float2*)h->qcdf, u, g[0], g[1],
                                                                                    g[2], f);
     }
     EVAP_CHECK_LAUNCH("mass_load");
@@ -250,9 +251,9 @@ int continuity_rhs(evap_mesh* h, const double** g, cudaStream_t st) {
         EVAP_CUDA(cudaMemsetAsync(h->cont_rhs, 0, m.Np * sizeof(double), st));
         const unsigned grid = (unsigned)blocks_for(m.ncell, 128, 1LL << 40);
         if (m.P == 2)
-            k_continuity_rhs<2><<<grid, 128, 0, st>>>(m, h->b, h->qc, h->cont_rhs);
+            k_continuity_rhs<2><<<grid, 128, 0, st>>>(m, h->b, (const float2*)h->qcdf, h->cont_rhs);
         else
-            k_continuity_rhs<3><<<grid, 128, 0, st>>>(m, h->b, h->qc, h->cont_rhs);
+            k_continuity_rhs<3><<<grid, 128, 0, st>>>(m, h->b, (const float2*)h->qcdf, h->cont_rhs);
         EVAP_CHECK_LAUNCH("continuity_rhs");
         h->cont_valid = true;
     }

@@ -83,14 +83,33 @@ __global__ void k_classify(MeshArgs<double> m, Basis<double> b, const double* __
     const int n = m.n;
     const int cx = (int)(cell % n), cy = (int)((cell / n) % n), cz = (int)(cell / ((int64_t)n * n));
     bool all_liq = true, all_gas = true;
-    for (int qz = 0; qz < b.Q; ++qz)
-        for (int qy = 0; qy < b.Q; ++qy)
-            for (int qx = 0; qx < b.Q; ++qx) {
-                double v, g[3];
-                ls_at(phi, m, cx, cy, cz, b.t[qx], b.t[qy], b.t[qz], v, g);
-                all_liq = all_liq && (v >= PHI_BAND);
-                all_gas = all_gas && (v <= -PHI_BAND);
-            }
+    // the interpolant lies between the cell's nodal values: away from the zone's edges these decide (most cells)
+    constexpr double EDGE = PHI_BAND + 1e-12;  // more than the rounding of an interpolated value
+    bool liq = true, gas = true;
+    {
+        const int k = m.nsub, ml = m.nl + 1;
+        const double* f = phi + k * cx + (int64_t)ml * (k * cy + (int64_t)ml * (k * cz));
+        for (int c = 0; c <= k; ++c)
+            for (int bb = 0; bb <= k; ++bb)
+                for (int a = 0; a <= k; ++a) {
+                    const double v = f[a + ml * (bb + (int64_t)ml * c)];
+                    liq = liq && v >= EDGE;
+                    gas = gas && v <= -EDGE;
+                }
+    }
+    if (liq || gas) {
+        all_liq = liq;
+        all_gas = gas;
+    } else {
+        for (int qz = 0; qz < b.Q && (all_liq || all_gas); ++qz)
+            for (int qy = 0; qy < b.Q; ++qy)
+                for (int qx = 0; qx < b.Q && (all_liq || all_gas); ++qx) {
+                    double v, g[3];
+                    ls_at(phi, m, cx, cy, cz, b.t[qx], b.t[qy], b.t[qz], v, g);
+                    all_liq = all_liq && (v >= PHI_BAND);
+                    all_gas = all_gas && (v <= -PHI_BAND);
+                }
+    }
     const bool everywhere = m.stress != 0 && m.corr_zone != 0;
     int8_t c = (!everywhere && all_liq) ? CELL_LIQUID : ((!everywhere && all_gas) ? CELL_GAS : CELL_TABLE);
     code[cell] = c;
@@ -99,58 +118,103 @@ __global__ void k_classify(MeshArgs<double> m, Basis<double> b, const double* __
 
 // Table entries at one quadrature point of a table cell: rho, mu, z n (z = correction gate), v_dil (Eq. evaporDil
 // with the sign of App. A, dilation_coefficient), delta.
+//
+// The FP64 pipe bounds it: one location and one set of weights for phi, its gradient and mdot, the logarithm, sine and
+// cosine shared by the table and the adjoint's factors, one reciprocal for the normal.  The density jump multiplies the
+// rounding of phi and H by up to the density ratio, so these keep their order of operations.  Measured at 64^3 (31.7 k
+// table cells): 728 -> 486 us (an interpolation per field and every function evaluated twice before).
 __global__ void k_fill_table(MeshArgs<double> m, Basis<double> b, const double* __restrict__ phi,
                              const double* __restrict__ mdot, const int8_t* __restrict__ code,
                              const int32_t* __restrict__ tindex, double* table, float* table32, float2* adj) {
-    const int nq = b.Q * b.Q * b.Q;
+    const unsigned nq = b.Q * b.Q * b.Q;
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t cell = gid / nq;
+    const unsigned cell = (unsigned)(gid / nq);
     if (cell >= m.ncell || code[cell] != CELL_TABLE) return;
-    const int q = (int)(gid % nq);
-    const int qx = q % b.Q, qy = (q / b.Q) % b.Q, qz = q / (b.Q * b.Q);
-    const int n = m.n;
-    const int cx = (int)(cell % n), cy = (int)((cell / n) % n), cz = (int)(cell / ((int64_t)n * n));
-    double ph, g[3], md, gm[3];
-    ls_at(phi, m, cx, cy, cz, b.t[qx], b.t[qy], b.t[qz], ph, g);
-    ls_at(mdot, m, cx, cy, cz, b.t[qx], b.t[qy], b.t[qz], md, gm);
-    const Material mat = material(ph, g[0], g[1], g[2], m);
-    const double z = correction_on(m, mat.zone) ? 1.0 : 0.0;
-    const double vals[TAB_K] = {mat.rho, mat.mu, z * mat.n[0], z * mat.n[1], z * mat.n[2],
-                                md * dilation_coefficient(m) * mat.delta, mat.delta};
-    const int64_t base = (int64_t)tindex[cell] * TAB_K * nq + q;
+    const unsigned q = (unsigned)(gid - (int64_t)cell * nq);
+    const unsigned Q = b.Q, qx = q % Q, qy = (q / Q) % Q, qz = q / (Q * Q);
+    const unsigned n = m.n, row = cell / n;
+    int ci[3] = {(int)(cell - row * n), (int)(row % n), (int)(row / n)};
+    double loc[3] = {b.t[qx], b.t[qy], b.t[qz]};
+    double ih = m.inv_h;
+    if (m.nsub > 1) {  // the level-set cell holding the point (the upper one on a face)
 #pragma unroll
-    for (int k = 0; k < TAB_K; ++k) {
-        table[base + (int64_t)k * nq] = vals[k];
-        table32[base + (int64_t)k * nq] = (float)vals[k];
+        for (int a = 0; a < 3; ++a) {
+            const double s = loc[a] * m.nsub;
+            int c = (int)floor(s);
+            c = c < 0 ? 0 : (c > m.nsub - 1 ? m.nsub - 1 : c);
+            ci[a] = m.nsub * ci[a] + c;
+            loc[a] = s - c;
+        }
+        ih *= m.nsub;
     }
-    // adjoint factors: H'(d) d'(phi) and its phi-derivative (H''(d) d'(phi)^2 + H'(d) d''(phi)) in the zone
-    double dHdd = 0.0, d2 = 0.0;
-    if (mat.zone) {
+    const int64_t m1 = m.nl + 1, base = ci[0] + m1 * (ci[1] + m1 * ci[2]);
+    // the same weighted sums over the 8 nodes as ls_at, with their products formed once
+    double ph = 0.0, g[3] = {0.0, 0.0, 0.0}, md = 0.0;
+    {
+        const double wx[2] = {1.0 - loc[0], loc[0]}, wy[2] = {1.0 - loc[1], loc[1]}, wz[2] = {1.0 - loc[2], loc[2]};
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+                for (int a = 0; a < 2; ++a) {
+                    const int64_t r = base + a + m1 * (bb + m1 * c);
+                    const double v = phi[r], w = wx[a] * wy[bb] * wz[c];
+                    ph += w * v;
+                    md += w * mdot[r];
+                    g[0] += (a ? wy[bb] : -wy[bb]) * wz[c] * v;
+                    g[1] += (bb ? wx[a] : -wx[a]) * wz[c] * v;
+                    g[2] += wx[a] * wy[bb] * (c ? v : -v);
+                }
+        g[0] *= ih;
+        g[1] *= ih;
+        g[2] *= ih;
+    }
+    // material law (Eqs. heaviside, rhoEff, muEff, normal_vector, delta) and
+    // the derivatives of H: H'(d) d'(phi) and H''(d) d'(phi)^2 + H'(d) d''(phi)
+    const bool zone = fabs(ph) < PHI_BAND;
+    double H = ph >= PHI_BAND ? 1.0 : 0.0, dHdd = 0.0, d2 = 0.0;
+    if (zone) {
+        // (H in this very order: the reciprocal density multiplies its rounding by the density ratio)
         const double d = m.eps * log((1.0 + ph) / (1.0 - ph));
         double sn, cs;
         sincos(PI * d / (3.0 * m.eps), &sn, &cs);
-        const double dH = (1.0 + cs) / (6.0 * m.eps), d2H = -PI * sn / (18.0 * m.eps * m.eps);
-        const double om = 1.0 - ph * ph;
-        const double dd = 2.0 * m.eps / om, d2d = 4.0 * m.eps * ph / (om * om);
-        dHdd = dH * dd;
-        d2 = d2H * dd * dd + dH * d2d;
+        H = 0.5 + d / (6.0 * m.eps) + sn / (2.0 * PI);
+        const double io = 1.0 / (1.0 - ph * ph);  // d'(phi) = 2 eps io, d''(phi) = 4 eps phi io^2
+        const double h1 = (1.0 + cs) * (1.0 / 6.0), h2 = sn * (-PI / 18.0);  // eps H'(d), eps^2 H''(d)
+        dHdd = 2.0 * h1 * io;
+        d2 = 4.0 * (io * io) * (h2 + h1 * ph);
     }
+    const double irl = 1.0 / m.rho_l, irg = 1.0 / m.rho_g;
+    const double irho = H / m.rho_l + (1.0 - H) / m.rho_g, rho = 1.0 / irho;
+    const double mu = H * m.mu_l + (1.0 - H) * m.mu_g;
     const double gn = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
-    const double kdil = dilation_coefficient(m);
+    const bool dir = gn * m.h > GRAD_TINY;
+    const double ign = dir ? 1.0 / gn : 0.0;
+    const double nv[3] = {dir ? g[0] * ign : 0.0, dir ? g[1] * ign : 0.0, dir ? g[2] * ign : 0.0};
+    const double z = correction_on(m, zone) ? 1.0 : 0.0, kdil = irg - irl;  // dilation_coefficient
+    const double delta = zone ? dHdd * gn : 0.0;
+    const double vals[TAB_K] = {rho, mu, z * nv[0], z * nv[1], z * nv[2], md * kdil * delta, delta};
+    const int64_t tb = (int64_t)tindex[cell] * TAB_K * nq + q;
+#pragma unroll
+    for (int k = 0; k < TAB_K; ++k) {
+        table[tb + (int64_t)k * nq] = vals[k];
+        table32[tb + (int64_t)k * nq] = (float)vals[k];
+    }
     double av[ADJ_K];
-    av[ADJ_CRHO] = -mat.rho * mat.rho * (1.0 / m.rho_l - 1.0 / m.rho_g) * dHdd;
+    av[ADJ_CRHO] = -rho * rho * (irl - irg) * dHdd;
     av[ADJ_CMU] = (m.mu_l - m.mu_g) * dHdd;
-    av[ADJ_N + 0] = mat.n[0];
-    av[ADJ_N + 1] = mat.n[1];
-    av[ADJ_N + 2] = mat.n[2];
+    av[ADJ_N + 0] = nv[0];
+    av[ADJ_N + 1] = nv[1];
+    av[ADJ_N + 2] = nv[2];
     av[ADJ_ZG] = z;
-    av[ADJ_IGN] = gn * m.h > GRAD_TINY ? 1.0 / gn : 0.0;
-    av[ADJ_KD1] = kdil * mat.delta;
+    av[ADJ_IGN] = ign;
+    av[ADJ_KD1] = kdil * delta;
     av[ADJ_KD2] = md * kdil * d2 * gn;
     av[ADJ_KD3] = md * kdil * dHdd;
-    av[ADJ_IRHO] = 1.0 / mat.rho;
-    av[ADJ_RHO] = mat.rho;
-    av[ADJ_ZONE] = mat.zone ? 1.0 : 0.0;
+    av[ADJ_IRHO] = irho;
+    av[ADJ_RHO] = rho;
+    av[ADJ_ZONE] = zone ? 1.0 : 0.0;
     const int64_t abase = (int64_t)tindex[cell] * ADJ_K * nq + q;
 #pragma unroll
     for (int k = 0; k < ADJ_K; ++k) {
