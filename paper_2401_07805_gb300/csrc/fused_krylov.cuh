@@ -136,7 +136,7 @@ __device__ __forceinline__ void grid_sum_df(const float2* part, float2* sh, dfl 
 // mirrored interior rows, and the operator is a sum of their tensor products.  So the neighbours of one kind are added
 // first: 23 additions and 4 multiplications per node.
 struct HelmholtzStencil {
-    static constexpr int SMEM = 0;
+    static constexpr int SMEM = 0, MIN_BLOCKS = 0;
     int n;
     dfl c[4];
     __device__ __forceinline__ void load(float2*) const {}
@@ -200,7 +200,7 @@ inline HelmholtzStencil helmholtz_op(int n, double h, double c) {
 // the lattice.  Those products are formed all the same, with whatever the vector's memory holds there: it has
 // stencil_guard(n) zero entries in front, and every entry read is finite.
 struct NodeStencil {
-    static constexpr int SMEM = 0;
+    static constexpr int SMEM = 0, MIN_BLOCKS = 1;  // (registers for all 54 loads of a row: without it 64 and 1.07 to 1.2 times the time)
     int n;
     int64_t N;
     const float2* C;
@@ -275,7 +275,7 @@ struct CgScalars {
 // preconditioner; FP32 changes only the iteration count).  part holds 3 gridDim.x pairs.  out[0] = updates,
 // out[1] = |r|, out[2] = |r0| (block 0).
 template <class Op>
-__global__ void __launch_bounds__(FK_THREADS) k_cg_fused(Op op, int64_t N, const double* __restrict__ b, double* x,
+__global__ void __launch_bounds__(FK_THREADS, Op::MIN_BLOCKS) k_cg_fused(Op op, int64_t N, const double* __restrict__ b, double* x,
                                                          float2* xd,
                                                          float* dinv, float2* r, float2* u, float2* p, float2* sv,
                                                          float2* w, double rtol, double atol, int max_iter,
@@ -730,9 +730,12 @@ int fused_space(evap_mesh* h, int nvec, FusedSpace& f);
 // the launch's result words (iterations, |r|, |r0|) and its barrier's error word, after one synchronization
 int fused_result(evap_mesh* h, const FusedSpace& f, cudaStream_t s, double res[3]);
 
-// Grid of a single-launch solver: as many blocks as can be co-resident, at most 2 per SM and `cap` in all.
+// Grid of a single-launch solver over N entries: as many blocks as can be co-resident, at most 2 per SM and `cap` in all,
+// and no more than have a thread per entry (an iteration on a small lattice is its grid barriers and partial sums: 8.2 us
+// at 24^3 with 152 blocks).  The kernels' registers leave one block per SM; capped to two, a CG iteration took 1.03 to 1.9
+// times as long.
 template <class K>
-inline int fused_grid(K kernel, size_t smem, int cap, int& G) {
+inline int fused_grid(K kernel, size_t smem, int cap, int64_t N, int& G) {
     int dev = 0, sms = 0, per_sm = 0;
     EVAP_CUDA(cudaGetDevice(&dev));
     EVAP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -743,6 +746,8 @@ inline int fused_grid(K kernel, size_t smem, int cap, int& G) {
         set_error("single-launch solver: no block of " + std::to_string(FK_THREADS) + " threads fits on an SM");
         return EVAP_ECUDA;
     }
+    const int64_t need = (N + FK_THREADS - 1) / FK_THREADS;
+    if (G > need) G = (int)need;
     return EVAP_OK;
 }
 

@@ -348,7 +348,7 @@ static int cg_solve_fused(evap_mesh* h, Op op, const double* b, double* x, doubl
     int rc = fused_space(h, 6, f), G = 0;
     if (rc) return rc;
     const size_t smem = Op::SMEM * sizeof(float2);
-    if ((rc = fused_grid(k_cg_fused<Op>, smem, FK_MAX_BLOCKS, G))) return rc;
+    if ((rc = fused_grid(k_cg_fused<Op>, smem, FK_MAX_BLOCKS, N, G))) return rc;
     EVAP_CUDA(cudaMemsetAsync(f.gb, 0, sizeof(GridBarrier), s));
     double* xx = x;
     float2 *xd = f.vec, *r = f.vec + N, *u = f.vec + 2 * N, *p = f.vec + 3 * N, *sv = f.vec + 4 * N, *w = f.vec + 5 * N;
@@ -380,7 +380,7 @@ static int gmres_solve_fused(evap_mesh* h, Op op, int m, const double* b, double
     int rc = fused_space(h, m + 3, f), G = 0;
     if (rc) return rc;
     const size_t smem = Op::SMEM * sizeof(float2);
-    if ((rc = fused_grid(k_gmres_fused<Op>, smem, FK_MAX_BLOCKS, G))) return rc;
+    if ((rc = fused_grid(k_gmres_fused<Op>, smem, FK_MAX_BLOCKS, N, G))) return rc;
     EVAP_CUDA(cudaMemsetAsync(f.gb, 0, sizeof(GridBarrier), s));
     double* xx = x;
     float2 *xd = f.vec, *z = f.vec + N, *V = f.vec + 2 * N;

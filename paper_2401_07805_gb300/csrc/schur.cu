@@ -237,7 +237,7 @@ int schur_solve(evap_mesh* h, const double* r, double* z, double rtol, int max_i
     FusedSpace f;
     if ((rc = fused_space(h, 3, f))) return rc;  // 3 pair vectors = 6 float vectors of N_phi >= N_p entries
     int G = 0;
-    if ((rc = fused_grid(k_cg_fused32<SchurStencil>, 0, FK_MAX_BLOCKS, G))) return rc;
+    if ((rc = fused_grid(k_cg_fused32<SchurStencil>, 0, FK_MAX_BLOCKS, N, G))) return rc;
     EVAP_CUDA(cudaMemsetAsync(f.gb, 0, sizeof(GridBarrier), s));
     SchurStencil op{h->m.n, N, h->schur_S + schur_guard(h->m.n)};
     const int64_t Nl = ls_args<double>(h).Nphi;  // the vectors' stride: fused_space sizes them for N_phi
