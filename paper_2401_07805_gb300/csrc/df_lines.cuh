@@ -33,7 +33,8 @@ __device__ __forceinline__ dfl df_half(dfl a) { return {0.5f * a.hi, 0.5f * a.lo
 // Which sums are normalized: results stored for the next sweep (df_addo) and sums multiplied next (df_addi); sums that are
 // added further are not.  Measured at 64^3 Q2 (us per apply, error against 64 bits; 1.12e-14 with Q-term dot products):
 // both 552, 1.10e-14; only the multiplied ones 540, 1.14e-14; only the stored ones 540, 1.11e-14 (5.25e-15 at 8^3, 5.21e-15
-// before); none 529, 1.17e-14.  Both are, so that no case loses accuracy.
+// before); none 529, 1.17e-14.  For Q = 3 both are, so that no case loses accuracy; for Q = 4 the stored ones (45^3 Q3: 576
+// -> 544 us, 3.74e-14 -> 3.75e-14; 3.79e-14 with dot products).
 __device__ __forceinline__ dfl df_addo(dfl a, dfl b) { return df_add(a, b); }
 __device__ __forceinline__ dfl df_addi(dfl a, dfl b) { return df_add(a, b); }
 
@@ -106,15 +107,15 @@ struct DfLine<4> {
     }
     static __device__ __forceinline__ void val(const dfl u[4], dfl y[4]) {
         const dfl e0 = df_addl(u[0], u[3]), e1 = df_addl(u[1], u[2]);
-        const dfl o0 = df_addi(u[0], df_neg(u[3])), o1 = df_addi(u[1], df_neg(u[2]));
-        const dfl f = df_addi(e0, df_neg(e1));
+        const dfl o0 = df_addl(u[0], df_neg(u[3])), o1 = df_addl(u[1], df_neg(u[2]));
+        const dfl f = df_addl(e0, df_neg(e1));
         val_pair<0>(df_half(e1), f, o0, o1, y);
         val_pair<1>(df_half(e1), f, o0, o1, y);
     }
     template <bool FINAL>
     static __device__ __forceinline__ void valT(const dfl t[4], dfl o[4]) {
-        const dfl s0 = df_addi(t[0], t[3]), s1 = df_addi(t[1], t[2]);
-        const dfl d0 = df_addi(t[0], df_neg(t[3])), d1 = df_addi(t[1], df_neg(t[2]));
+        const dfl s0 = df_addl(t[0], t[3]), s1 = df_addl(t[1], t[2]);
+        const dfl d0 = df_addl(t[0], df_neg(t[3])), d1 = df_addl(t[1], df_neg(t[2]));
         constexpr double a0 = al(0), a1 = al(1), g0 = ga(0), g1 = ga(1), e0 = de(0), e1 = de(1);
         const dfl ev = dot2(EVAP_DFK(a0), s0, EVAP_DFK(a1), s1);               // even result of the outer pair
         const dfl ei = df_addl(df_half(df_addl(s0, s1)), df_neg(ev));           // and of the inner one
@@ -125,8 +126,8 @@ struct DfLine<4> {
         o[2] = FINAL ? df_addl(ei, df_neg(oi)) : df_addo(ei, df_neg(oi));
     }
     static __device__ __forceinline__ void der(const dfl y[4], dfl d[4]) {
-        const dfl o0 = df_addi(y[0], df_neg(y[3])), o1 = df_addi(y[1], df_neg(y[2]));
-        const dfl f = df_addi(df_addl(y[0], y[3]), df_neg(df_addl(y[1], y[2])));
+        const dfl o0 = df_addl(y[0], df_neg(y[3])), o1 = df_addl(y[1], df_neg(y[2]));
+        const dfl f = df_addl(df_addl(y[0], y[3]), df_neg(df_addl(y[1], y[2])));
         constexpr double h0 = eta(0), h1 = eta(1), a0 = xa(0), a1 = xa(1), b0 = xb(0), b1 = xb(1);
         const dfl v0 = df_mul(EVAP_DFK(h0), f), v1 = df_mul(EVAP_DFK(h1), f);
         const dfl w0 = dot2(EVAP_DFK(a0), o0, EVAP_DFK(b0), o1), w1 = dot2(EVAP_DFK(a1), o0, EVAP_DFK(b1), o1);
@@ -136,8 +137,8 @@ struct DfLine<4> {
         d[2] = df_addl(w1, df_neg(v1));
     }
     static __device__ __forceinline__ void derT(const dfl t[4], dfl o[4]) {
-        const dfl s0 = df_addi(t[0], t[3]), s1 = df_addi(t[1], t[2]);  // act on the odd part
-        const dfl d0 = df_addi(t[0], df_neg(t[3])), d1 = df_addi(t[1], df_neg(t[2]));
+        const dfl s0 = df_addl(t[0], t[3]), s1 = df_addl(t[1], t[2]);  // act on the odd part
+        const dfl d0 = df_addl(t[0], df_neg(t[3])), d1 = df_addl(t[1], df_neg(t[2]));
         constexpr double h0 = eta(0), h1 = eta(1), a0 = xa(0), a1 = xa(1), b0 = xb(0), b1 = xb(1);
         const dfl ev = dot2(EVAP_DFK(h0), d0, EVAP_DFK(h1), d1);  // even result, + on the outer and - on the inner pair
         const dfl oo = dot2(EVAP_DFK(a0), s0, EVAP_DFK(a1), s1), oi = dot2(EVAP_DFK(b0), s0, EVAP_DFK(b1), s1);
