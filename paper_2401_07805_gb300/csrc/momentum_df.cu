@@ -51,7 +51,7 @@ __device__ __forceinline__ constexpr int t_slot(int k, int l) {
 // Cells per block and blocks per SM (a register cap).  Measured at 64^3 Q2 with the divergence row (us per apply; one
 // point per thread with Q-term dot products: 673): CB 1 / 28 blocks 503 (a block is one warp, so that the barriers of
 // the sweeps cost nothing); 2 / 16 526; 4 / 8 510; 5 / 6 552; 7 / 4 592; 8 / 4 581; 13 / 2 757.  Q3 at 45^3 (701
-// before): 2 and 4 cells 576.  ncu at 64^3, CB 4: 1842 warp instructions per cell (1064 FADD, 194 FMUL and FFMA, 142
+// before): 2 and 4 cells 544, 1 cell 579.  ncu at 64^3, CB 4: 1842 warp instructions per cell (1064 FADD, 194 FMUL and FFMA, 142
 // shared accesses), issue 77 % active, FP64 pipe 59 % (conversions).
 #ifndef EVAP_DF_CB2
 #define EVAP_DF_CB2 1
@@ -75,14 +75,11 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
     using Ln = DfLine<Q>;
     __shared__ dfl sN1[Q][2];
     __shared__ dfl q1a[CB][2 * Q * Q], q1b[CB][4 * Q];
-    // the pressure at the cell's corners, then interpolated along x and y (z: by the point's thread), in double-float
-    // arithmetic: 14 FP64 operations and a conversion per point had made the FP64 pipe the bound (672 -> 531 us at 64^3)
-    __shared__ dfl p0[PRES ? CB : 1][8], px[PRES ? CB : 1][4 * Q], py[PRES ? CB : 1][2 * Q * Q];
-    auto lerp = [&](dfl u, dfl v, int q) -> dfl {  // at Gauss point q, in double-float arithmetic
-        dfl r = u;
-        df_fma(r, sN1[q][1], df_add(v, df_neg(u)));
-        return df_norm(r);
-    };
+    // the pressure at the cell's corners, then interpolated along x and y (z: by the point's thread), in FP64: 2 FP64
+    // operations per sweep instead of 14 per point (672 -> 562 us at 64^3; in double-float arithmetic 531, but with the
+    // error of a pure pressure term 6.6e-15 -> 7.4e-15 against 64 bits)
+    __shared__ double p0[PRES ? CB : 1][8], px[PRES ? CB : 1][4 * Q], py[PRES ? CB : 1][2 * Q * Q];
+    auto lerp = [&](double u, double v, int q) -> double { return fma(bas.t[q], v - u, u); };  // at Gauss point q
     extern __shared__ float2 smem_df[];
     dfl* const sb = reinterpret_cast<dfl*>(smem_df);  // [cell][slot][point]
     constexpr int CELL = (DF_SLOTS + QC_K) * NQ;
@@ -137,7 +134,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         int ex, ey, ez;
         colour_cell32(cell0 + c2, n, DET ? colour : -1, ex, ey, ez);
         const int64_t m1 = n + 1;
-        p0[c2][o] = df_from_double(pin[(ex + (o & 1)) + m1 * ((ey + ((o >> 1) & 1)) + m1 * (ez + (o >> 2)))]);
+        p0[c2][o] = pin[(ex + (o & 1)) + m1 * ((ey + ((o >> 1) & 1)) + m1 * (ez + (o >> 2)))];
     }
     __syncthreads();
     if (PRES && tid < CB * 4 * Q) {  // [qx][jb][jc]
@@ -207,7 +204,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         const dfl sm = corr ? df_mul(c13, tr) : dfl{0.f, 0.f};
         const dfl rw = PRES || yp ? df_mul(q[17 * NQ], kap) : dfl{0.f, 0.f};  // kappa W
         dfl wp{0.f, 0.f};
-        if constexpr (PRES) wp = df_mul(rw, lerp(py[lc][t % NL], py[lc][t % NL + NL], t / NL));
+        if constexpr (PRES) wp = df_mul(rw, df_from_double(lerp(py[lc][t % NL], py[lc][t % NL + NL], t / NL)));
 #pragma unroll
         for (int k = 0; k < 3; ++k)
 #pragma unroll
