@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(256) k_adjoint_init(int M, int64_t Nu, int64_t
 // its own point's values and gradients with them.  Only the threads of table cells run the interface-zone work and the
 // level-set sweeps.  At most 48 KB of shared memory per block, so no launch needs a function attribute.
 // Measured at 48^3 Q2 (us; one point per thread with Q-term dot products 775 to 800): cells per block / blocks per SM 4 / 5
-// 632 (96 registers); 7 / 3 631; 2 / 10 651; 4 / 6 655; 1 / 20 669; 5 / 4 671; 3 / 7 673; 4 / 4 684.
+// 582 (96 registers); 4 / 4 595; 2 / 10 603; 3 / 6 612; 1 / 20 637.  ncu: issue 59 %, FP64 pipe 63 % (conversions).
 // Normalization as in the forward apply: the gradients at the points, the value sensitivities that start the test sums
 // and the last transposed sweep (converted to FP64 next) are left unnormalized.
 #ifndef EVAP_ADJ_CB2
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
               const float2* __restrict__ qcd, const double* __restrict__ w,
               const double* __restrict__ wp, const double* __restrict__ x, double* gx, double* gu, double* gphi,
               double* gm, int colour) {
-    constexpr int Q = P + 1, NQ = Q * Q * Q, NL = Q * Q, TASKS = 6 * NL;
+    constexpr int Q = P + 1, NQ = Q * Q * Q, NL = Q * Q;
     using Ln = DfLine<Q>;
     static_assert(K * Q * Q <= NQ && K * K * K <= NQ, "one thread per entry of each level-set test sweep");
     __shared__ double sNL[Q][K], sDL[Q][K];
@@ -118,54 +118,61 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         sNL[tid / K][tid % K] = bas.NL[tid / K][tid % K];
         sDL[tid / K][tid % K] = bas.DL[tid / K][tid % K];
     }
-    const int a = t % Q, b = (t / Q) % Q, c = t / (Q * Q);
     const int n = m.n, M = m.M;
     const int64_t m1 = n + 1;     // pressure nodes per axis (w_p)
     const int64_t ml = m.nl + 1;  // level-set nodes per axis
     const bool tcell = code[cell] == CELL_TABLE;
-    // z-line l of a cell: offset of its first node in a component, and which of its nodes are constrained (bit k)
+    // this thread's lines: line l of the fields f0, f0 + Q, ...; its z-line's offset in a component, and which of its nodes
+    // are constrained (bit k)
+    const int f0 = t / NL, l = t % NL;
     const int64_t zst = (int64_t)M * M;
-    auto zline = [&](int l, unsigned& cons) -> int64_t {
+    int64_t zoff;
+    unsigned zcons;
+    {
         const int gxi = P * cx + l % Q, gyi = P * cy + l / Q, gz0 = P * cz;
         const unsigned fc = m.faces;
-        cons = ((fc & 1u) && gxi == 0) || ((fc & 2u) && gxi == M - 1) || ((fc & 4u) && gyi == 0) ||
-                       ((fc & 8u) && gyi == M - 1)
-                   ? (1u << Q) - 1u
-                   : 0u;
-        if ((fc & 16u) && gz0 == 0) cons |= 1u;
-        if ((fc & 32u) && gz0 + P == M - 1) cons |= 1u << P;
-        return gxi + (int64_t)M * gyi + zst * gz0;
-    };
+        zcons = ((fc & 1u) && gxi == 0) || ((fc & 2u) && gxi == M - 1) || ((fc & 4u) && gyi == 0) ||
+                        ((fc & 8u) && gyi == M - 1)
+                    ? (1u << Q) - 1u
+                    : 0u;
+        if ((fc & 16u) && gz0 == 0) zcons |= 1u;
+        if ((fc & 32u) && gz0 + P == M - 1) zcons |= 1u << P;
+        zoff = gxi + (int64_t)M * gyi + zst * gz0;
+    }
+    // w_p interpolated to the points along x, y (z: by the point's thread), in FP64: 2 operations per sweep, not 14 per point
+    __shared__ double p0[CB][8], px[CB][4 * Q], py[CB][2 * Q * Q];
+    auto lerp = [&](double u, double v, int q) -> double { return fma(bas.t[q], v - u, u); };  // at Gauss point q
+    if (wp && t < 8) p0[lc][t] = wp[(cx + (t & 1)) + m1 * ((cy + ((t >> 1) & 1)) + m1 * (cz + (t >> 2)))];
     // values at the points: the lines along z (from memory), y and x, then the derivatives along the three directions
-    for (int k0 = t; k0 < TASKS; k0 += NQ) {
-        const int f = k0 / NL, l = k0 % NL;
-        unsigned cons;
-        const double* src = (f < 3 ? x : w) + (f < 3 ? f : f - 3) * m.Nu + zline(l, cons);
+    for (int f = f0; f < 6; f += Q) {
+        const double* src = (f < 3 ? x : w) + (f < 3 ? f : f - 3) * m.Nu + zoff;
         dfl u[Q], v[Q];
 #pragma unroll
-        for (int k = 0; k < Q; ++k) u[k] = (cons >> k) & 1u ? dfl{0.f, 0.f} : df_from_double(src[k * zst]);
+        for (int k = 0; k < Q; ++k) u[k] = (zcons >> k) & 1u ? dfl{0.f, 0.f} : df_from_double(src[k * zst]);
         Ln::val(u, v);
         st_line<Q, 2>(cb + (6 + f) * NQ, l, v);
     }
     __syncthreads();
-    for (int k0 = t; k0 < TASKS; k0 += NQ) {
-        const int f = k0 / NL, l = k0 % NL;
+    for (int f = f0; f < 6; f += Q) {
         dfl u[Q], v[Q];
         ld_line<Q, 1>(cb + (6 + f) * NQ, l, u);
         Ln::val(u, v);
         st_line<Q, 1>(cb + (12 + f) * NQ, l, v);
     }
+    if (wp && t < 4 * Q) px[lc][t] = lerp(p0[lc][2 * (t / Q)], p0[lc][2 * (t / Q) + 1], t % Q);  // [qx][jb][jc]
     __syncthreads();
-    for (int k0 = t; k0 < TASKS; k0 += NQ) {
-        const int f = k0 / NL, l = k0 % NL;
+    for (int f = f0; f < 6; f += Q) {
         dfl u[Q], v[Q];
         ld_line<Q, 0>(cb + (12 + f) * NQ, l, u);
         Ln::val(u, v);
         st_line<Q, 0>(cb + f * NQ, l, v);
     }
+    if (wp && t < 2 * NL) {  // [qx][qy][jc]
+        const int q = t % Q, r = (t / Q) % Q, jc = t / NL;
+        py[lc][t] = lerp(px[lc][q + Q * (2 * jc)], px[lc][q + Q * (2 * jc + 1)], r);
+    }
     __syncthreads();
-    for (int k0 = t; k0 < TASKS; k0 += NQ) {
-        const int f = k0 / NL, l = k0 % NL;
+    for (int f = f0; f < 6; f += Q) {
         dfl u[Q], v[Q];
         ld_line<Q, 0>(cb + f * NQ, l, u);
         Ln::der(u, v);
@@ -194,27 +201,12 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         const float2* ap = tcell ? adjt + (int64_t)tindex[cell] * ADJ_K * NQ + t : nullptr;
         const dfl rho = tcell ? ld_df(ap + ADJ_RHO * NQ) : (code[cell] == CELL_LIQUID ? rho_liq : rho_gas);
         const dfl wr = df_mul(Wk, rho);
-        // w_p (pressure space, Q1 on the cell) at the point
-        double pi = 0;
-        if (wp) {  // trilinear interpolation by successive linear interpolation (14 FP64 operations, not 40)
-            const double tx = bas.t[a], ty = bas.t[b], tz = bas.t[c];
-            const double* w0 = wp + cx + m1 * (cy + m1 * cz);
-            double e[2][2];
-#pragma unroll
-            for (int jc = 0; jc < 2; ++jc)
-#pragma unroll
-                for (int jb = 0; jb < 2; ++jb) {
-                    const double* r = w0 + m1 * (jb + m1 * jc);
-                    e[jc][jb] = fma(tx, r[1] - r[0], r[0]);
-                }
-            const double f0 = fma(ty, e[0][1] - e[0][0], e[0][0]), f1 = fma(ty, e[1][1] - e[1][0], e[1][0]);
-            pi = fma(tz, f1 - f0, f0);
-        }
         // the phi / mdot sensitivities and the normal are needed only in the interface zone (or with the correction
         // applied everywhere), which lies in table cells; elsewhere H is 0 or 1 and its derivatives vanish
         const bool full = tcell && (ap[ADJ_ZONE * NQ].x != 0.f || (m.stress != 0 && m.corr_zone != 0));
         const dfl wm = qp[13 * NQ];
-        const dfl pid = df_from_double(pi), Wkpi = df_mul(Wk, pid);
+        const dfl pid = wp ? df_from_double(lerp(py[lc][t % NL], py[lc][t % NL + NL], t / NL)) : dfl{0.f, 0.f};  // w_p here
+        const dfl Wkpi = df_mul(Wk, pid);
         dfl corr{0.f, 0.f};
         if (full) {  // material-law sensitivities (interface-zone points only), double-float arithmetic
             const dfl nv[3] = {ld_df(ap + (ADJ_N + 0) * NQ), ld_df(ap + (ADJ_N + 1) * NQ), ld_df(ap + (ADJ_N + 2) * NQ)};
@@ -347,9 +339,8 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
     }
     __syncthreads();
     // test with gradients: the lines along y and z into the coefficients' slots (u0: only with the Newton term)
-    const int gtasks = m.newton ? TASKS : TASKS / 2;
-    for (int k0 = t; k0 < gtasks; k0 += NQ) {
-        const int f = k0 / NL, l = k0 % NL;
+    const int gfields = m.newton ? 6 : 3;
+    for (int f = f0; f < gfields; f += Q) {
         dfl u[Q], v[Q];
         ld_line<Q, 1>(cb + (7 + 3 * f) * NQ, l, u);
         Ln::derT(u, v);
@@ -374,8 +365,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         }
     }
     __syncthreads();
-    for (int k0 = t; k0 < TASKS; k0 += NQ) {  // x: values + the three tests, and their value sweep
-        const int f = k0 / NL, l = k0 % NL;
+    for (int f = f0; f < 6; f += Q) {  // x: values + the three tests, and their value sweep
         dfl u[Q], v[Q], s[Q];
         ld_line<Q, 0>(cb + f * NQ, l, s);
         if (f < 3 || m.newton) {
@@ -418,8 +408,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         if (gphi) acc_add(&gphi[nd], r[0] + m.inv_h * (r[1] + r[2] + r[3]), plain);
         if (gm) acc_add(&gm[nd], r[4], plain);
     }
-    for (int k0 = t; k0 < TASKS; k0 += NQ) {
-        const int f = k0 / NL, l = k0 % NL;
+    for (int f = f0; f < 6; f += Q) {
         dfl u[Q], v[Q];
         ld_line<Q, 1>(cb + f * NQ, l, u);
         Ln::template valT<false>(u, v);
@@ -427,13 +416,11 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
     }
     __syncthreads();
     if (!active) return;
-    for (int k0 = t; k0 < TASKS; k0 += NQ) {  // z, and the scatter
-        const int f = k0 / NL, l = k0 % NL;
+    for (int f = f0; f < 6; f += Q) {  // z, and the scatter
         double* const out = f < 3 ? gx : gu;
         if (!out) continue;
-        unsigned cons;
-        double* dst = out + (f < 3 ? f : f - 3) * m.Nu + zline(l, cons);
-        if (f >= 3) cons = 0u;
+        double* dst = out + (f < 3 ? f : f - 3) * m.Nu + zoff;
+        const unsigned cons = f < 3 ? zcons : 0u;
         dfl u[Q], v[Q];
         ld_line<Q, 2>(cb + f * NQ, l, u);
         Ln::template valT<true>(u, v);
