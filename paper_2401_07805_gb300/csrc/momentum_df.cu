@@ -49,10 +49,10 @@ __device__ __forceinline__ constexpr int t_slot(int k, int l) {
 }
 
 // Cells per block and blocks per SM (a register cap).  Measured at 64^3 Q2 with the divergence row (us per apply; one
-// point per thread with Q-term dot products: 673): CB 1 / 28 blocks 503 (a block is one warp, so that the barriers of
-// the sweeps cost nothing); 2 / 16 526; 4 / 8 510; 5 / 6 552; 7 / 4 592; 8 / 4 581; 13 / 2 757.  Q3 at 45^3 (701
-// before): 2 and 4 cells 544, 1 cell 579.  ncu at 64^3, CB 4: 1842 warp instructions per cell (1064 FADD, 194 FMUL and FFMA, 142
-// shared accesses), issue 77 % active, FP64 pipe 59 % (conversions).
+// point per thread with Q-term dot products: 673): CB 1 / 28 blocks 503 (a block is one warp), 495 with the sweeps
+// ordered by warp barriers (128^3: 3610 -> 3518); 2 / 16 526; 4 / 8 510; 5 / 6 552; 7 / 4 592; 8 / 4 581; 13 / 2 757.
+// Q3 at 45^3 (701 before): 2 and 4 cells 544, 1 cell 579.  ncu at 64^3, CB 4: 1842 warp instructions per cell (1064 FADD,
+// 194 FMUL and FFMA, 142 shared accesses), issue 77 % active, FP64 pipe 59 % (conversions).
 #ifndef EVAP_DF_CB2
 #define EVAP_DF_CB2 1
 #endif
@@ -73,6 +73,10 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
                   double* __restrict__ y, double* __restrict__ yp, const double* __restrict__ pin, int colour) {
     constexpr int Q = P + 1, NQ = Q * Q * Q, NL = Q * Q, TASKS = 3 * NL;
     using Ln = DfLine<Q>;
+    auto sync = [] {  // a block of one warp needs no block barrier
+        if (CB * NQ <= 32) __syncwarp();
+        else __syncthreads();
+    };
     __shared__ dfl sN1[Q][2];
     __shared__ dfl q1a[CB][2 * Q * Q], q1b[CB][4 * Q];
     // the pressure at the cell's corners, then interpolated along x and y (z: by the point's thread), in FP64: 2 FP64
@@ -136,7 +140,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         const int64_t m1 = n + 1;
         p0[c2][o] = pin[(ex + (o & 1)) + m1 * ((ey + ((o >> 1) & 1)) + m1 * (ez + (o >> 2)))];
     }
-    __syncthreads();
+    sync();
     if (PRES && tid < CB * 4 * Q) {  // [qx][jb][jc]
         const int c2 = tid / (4 * Q), o = tid % (4 * Q), q = o % Q, r = o / Q;
         px[c2][o] = lerp(p0[c2][2 * r], p0[c2][2 * r + 1], q);
@@ -147,7 +151,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         Ln::val(u, v);
         st_line<Q, 1>(lb + (6 + f) * NQ, l, v);
     }
-    __syncthreads();
+    sync();
     if (PRES && tid < CB * 2 * Q * Q) {  // [qx][qy][jc]
         const int c2 = tid / (2 * Q * Q), o = tid % (2 * Q * Q), q = o % Q, r = (o / Q) % Q, jc = o / (Q * Q);
         py[c2][o] = lerp(px[c2][q + Q * (2 * jc)], px[c2][q + Q * (2 * jc + 1)], r);
@@ -158,7 +162,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         Ln::val(u, v);
         st_line<Q, 0>(lb + f * NQ, l, v);
     }
-    __syncthreads();
+    sync();
     if (line) {
         dfl u[Q], v[Q];
         ld_line<Q, 0>(lb + f * NQ, l, u);
@@ -171,7 +175,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         Ln::der(u, v);
         st_line<Q, 2>(lb + (5 + 3 * f) * NQ, l, v);
     }
-    __syncthreads();
+    sync();
     // quadrature-point fluxes from the cached coefficients; a thread reads and overwrites its own point's entries only
     {
         dfl X[3], G[3][3];
@@ -227,7 +231,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
             cb[9 * NQ + t] = df_norm(r);
         }
     }
-    __syncthreads();
+    sync();
     // test with gradients: the lines along y and z into the coefficients' slots
     if (line) {
         dfl u[Q], v[Q];
@@ -247,7 +251,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         for (int qq = 1; qq < Q; ++qq) df_fma(s, sN1[qq][o & 1], r[qq]);
         q1a[c2][o] = df_norm(s);
     }
-    __syncthreads();
+    sync();
     if (line) {  // x: F + the three tests, and its value sweep
         dfl u[Q], v[Q], w[Q];
         ld_line<Q, 0>(lb + t_slot(f, 0) * NQ, l, u);
@@ -269,7 +273,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         for (int qq = 1; qq < Q; ++qq) df_fma(s, sN1[qq][jy], q1a[c2][jx + 2 * (qq + Q * qz)]);
         q1b[c2][o] = df_norm(s);
     }
-    __syncthreads();
+    sync();
     if (line) {
         dfl u[Q], v[Q];
         ld_line<Q, 1>(lb + f * NQ, l, u);
@@ -287,7 +291,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
             acc_add(&yp[(ex + jx) + m1 * ((ey + jy) + m1 * (ez + jz))], df_to_double(df_norm(s)), plain);
         }
     }
-    __syncthreads();
+    sync();
     if (line && lact) {  // z, and the scatter of the line's free nodes
         dfl u[Q], v[Q];
         ld_line<Q, 2>(lb + f * NQ, l, u);
