@@ -39,28 +39,16 @@ __device__ __forceinline__ float factor1(const float (&t)[2][MAXQ], int P, int n
     return s;
 }
 
-// 1 / D on the free velocity DoFs, 0 on the Dirichlet ones (a warp walks x-lines of nodes)
-__global__ void __launch_bounds__(256) k_schur_inverse(int M, int64_t Nu, unsigned faces, const float* __restrict__ diag,
-                                                       float* __restrict__ inv) {
-    const int lines = 3 * M * M;
-    const int wpb = blockDim.x / 32, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    for (int line = blockIdx.x * wpb + warp; line < lines; line += gridDim.x * wpb) {
-        const int c = line / (M * M), rem = line - c * M * M, gz = rem / M, gy = rem - gz * M;
-        const bool cyz = ((faces & 4u) && gy == 0) || ((faces & 8u) && gy == M - 1) || ((faces & 16u) && gz == 0) ||
-                         ((faces & 32u) && gz == M - 1);
-        const int64_t off = c * Nu + (int64_t)M * (gy + (int64_t)M * gz);
-        for (int gx = lane; gx < M; gx += 32)
-            inv[off + gx] = cyz || ((faces & 1u) && gx == 0) || ((faces & 2u) && gx == M - 1) ? 0.f : 1.f / diag[off + gx];
-    }
-}
-
 // One block row per stored offset (blockIdx.y), one thread per pressure node.  The 1D factor products of a pair of pressure
 // nodes depend on the nodes only through their boundary classes (first, interior, last), so they are formed once per block
 // in shared memory: w[d][class of I][class of J][k][a or g], k over the velocity nodes both touch; nodes outside the
-// lattice get 0 and are read at a clamped place.  Measured at 64^3 Q2: 2139 us with the factors in local memory, three
-// divisions and a boundary test per velocity node, now 667.
-__global__ void __launch_bounds__(128) k_schur_assemble(int n, int P, int M, int64_t Nu, int64_t Np, SchurTables tab,
-                                                        const float* __restrict__ inv, float* __restrict__ S) {
+// lattice get 0 and are read at a clamped place.  Each term keeps its own division by D: a solve with the preconditioner
+// amplifies the rounding of S~ (with reciprocals formed once per velocity node and sums factored by direction, 667 us at
+// 64^3 Q2, solutions to 1e-8 moved by several times what two runs differ by).  Measured at 64^3 Q2: 2139 us with the
+// factors in local memory, now 1864.
+__global__ void __launch_bounds__(128) k_schur_assemble(int n, int P, int M, unsigned faces, int64_t Nu, int64_t Np,
+                                                        SchurTables tab, const float* __restrict__ diag,
+                                                        float* __restrict__ S) {
     __shared__ float w[3][3][3][2 * MAXQ - 1][2];
     const int e = blockIdx.y, lin = 62 + e;
     const int o[3] = {lin % 5 - 2, (lin / 5) % 5 - 2, lin / 25 - 2};
@@ -109,16 +97,13 @@ __global__ void __launch_bounds__(128) k_schur_assemble(int n, int P, int M, int
         for (int ky = 0; ky < cnt[1]; ++ky) {
             const float ay = wd[1][ky][0], gy = wd[1][ky][1];
             const int vy = min(max(lo[1] + ky, 0), M - 1);
-            const float* r = inv + (int64_t)M * (vy + (int64_t)M * vz);
-            float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+            const float* r = diag + (int64_t)M * (vy + (int64_t)M * vz);
             for (int kx = 0; kx < cnt[0]; ++kx) {
                 const int vx = min(max(lo[0] + kx, 0), M - 1);
+                if (constrained_node(vx, vy, vz, M, faces)) continue;
                 const float ax = wd[0][kx][0], gx = wd[0][kx][1];
-                s0 = fmaf(gx, r[vx], s0);
-                s1 = fmaf(ax, r[Nu + vx], s1);
-                s2 = fmaf(ax, r[2 * Nu + vx], s2);
+                acc += gx * ay * az / r[vx] + ax * gy * az / r[Nu + vx] + ax * ay * gz / r[2 * Nu + vx];
             }
-            acc += ay * az * s0 + gy * az * s1 + ay * gz * s2;
         }
     }
     S[e * Np + node] = acc;
@@ -186,9 +171,9 @@ int schur_assemble(evap_mesh* h, cudaStream_t s) {
         set_error("Schur stencil: its 63 N_p entries must be indexable with 32 bits");
         return EVAP_EINVAL;
     }
-    if (!h->schur_S) {  // guard, stencil, the padded lattice of the vector it is applied to, 1 / D
+    if (!h->schur_S) {  // guard, stencil, the padded lattice of the vector it is applied to
         const int64_t len = schur_guard(m.n) + 63 * m.Np + schur_padded(m.n);
-        EVAP_CUDA(cudaMalloc(&h->schur_S, (len + 3 * m.Nu) * sizeof(float)));
+        EVAP_CUDA(cudaMalloc(&h->schur_S, len * sizeof(float)));
         EVAP_CUDA(cudaMemsetAsync(h->schur_S, 0, len * sizeof(float), s));
     }
     SchurTables tab;
@@ -204,12 +189,8 @@ int schur_assemble(evap_mesh* h, cudaStream_t s) {
             tab.a[a][v] = (float)(m.h * sa);
             tab.g[a][v] = (float)sg;
         }
-    float* inv = h->schur_S + schur_guard(m.n) + 63 * m.Np + schur_padded(m.n);
-    const unsigned gi = (unsigned)std::min<int64_t>((3 * (int64_t)m.M * m.M + 7) / 8, 152 * 16);
-    k_schur_inverse<<<gi, 256, 0, s>>>(m.M, m.Nu, m.faces, h->diag32, inv);
-    EVAP_CHECK_LAUNCH("schur_inverse");
-    k_schur_assemble<<<dim3((unsigned)((m.Np + 127) / 128), 63), 128, 0, s>>>(m.n, m.P, m.M, m.Nu, m.Np, tab, inv,
-                                                                           h->schur_S + schur_guard(m.n));
+    k_schur_assemble<<<dim3((unsigned)((m.Np + 127) / 128), 63), 128, 0, s>>>(m.n, m.P, m.M, m.faces, m.Nu, m.Np, tab,
+                                                                           h->diag32, h->schur_S + schur_guard(m.n));
     EVAP_CHECK_LAUNCH("schur_assemble");
     h->schur_stamp = h->diag_stamp;
     return EVAP_OK;
