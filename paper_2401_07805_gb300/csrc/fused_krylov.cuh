@@ -726,7 +726,7 @@ struct FusedSpace {
     GridBarrier* gb;
     double* out;
 };
-int fused_space(evap_mesh* h, int nvec, FusedSpace& f);
+int fused_space(evap_mesh* h, int nvec, FusedSpace& f, cudaStream_t s);
 // the launch's result words (iterations, |r|, |r0|) and its barrier's error word, after one synchronization
 int fused_result(evap_mesh* h, const FusedSpace& f, cudaStream_t s, double res[3]);
 

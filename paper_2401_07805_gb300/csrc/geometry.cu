@@ -249,14 +249,15 @@ __global__ void __launch_bounds__(CG_THREADS) k_diff_norm(const double* __restri
     if (cg_finish2(cg_block_sum(s), 0.0, part, ticket, tot) && threadIdx.x == 0) *out = tot[0];
 }
 
-// Workspace: r, z, p, q [N_phi] + partials + scalars + ticket (allocated once per mesh).
-static int geo_workspace(evap_mesh* h) {
+// Workspace: r, z, p, q [N_phi] + partials + scalars + ticket (allocated once per mesh).  Cleared on the stream of the call
+// that uses it first: the legacy default stream does not order work before that of a non-blocking stream.
+static int geo_workspace(evap_mesh* h, cudaStream_t s) {
     if (h->geo_ws) return EVAP_OK;
     const int64_t Np = h->m.Nphi;
     const size_t vec = ((size_t)Np * sizeof(double) + 255) & ~(size_t)255;
     const size_t bytes = 10 * vec + (2 * CG_BLOCKS + 8) * sizeof(double) + 256;
     EVAP_CUDA(cudaMalloc(&h->geo_ws, bytes));
-    EVAP_CUDA(cudaMemset(h->geo_ws, 0, bytes));
+    EVAP_CUDA(cudaMemsetAsync(h->geo_ws, 0, bytes, s));
     if (!h->geo_host) EVAP_CUDA(cudaMallocHost(&h->geo_host, 8 * sizeof(double)));
     return EVAP_OK;
 }
@@ -289,7 +290,7 @@ static CgSpace cg_space(evap_mesh* h) {
 // Workspace of the single-launch solvers (FusedSpace, fused_krylov.cuh), grown on demand.
 static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-int fused_space(evap_mesh* h, int nvec, FusedSpace& f) {
+int fused_space(evap_mesh* h, int nvec, FusedSpace& f, cudaStream_t s) {
     if (!h->geo_host) EVAP_CUDA(cudaMallocHost(&h->geo_host, 8 * sizeof(double)));  // the result words' mirror
     const MeshArgs<double> lm = ls_args<double>(h);
     const int64_t N = lm.Nphi;
@@ -303,8 +304,9 @@ int fused_space(evap_mesh* h, int nvec, FusedSpace& f) {
         h->geo_kry = nullptr;
         h->geo_kry_bytes = 0;
         EVAP_CUDA(cudaMalloc(&h->geo_kry, need));
+        // the guard (read by boundary rows, written by nobody), on the stream of the solve that reads it
+        EVAP_CUDA(cudaMemsetAsync(h->geo_kry, 0, gbytes, s));
         h->geo_kry_bytes = need;
-        EVAP_CUDA(cudaMemset(h->geo_kry, 0, gbytes));  // the guard: read by boundary rows, written by nobody
     }
     char* base = (char*)h->geo_kry;
     const size_t vcap = h->geo_kry_bytes - dbytes - pbytes - tail;  // the vectors keep whatever room they had
@@ -345,7 +347,7 @@ static int cg_solve_fused(evap_mesh* h, Op op, const double* b, double* x, doubl
         return EVAP_EINVAL;
     }
     FusedSpace f;
-    int rc = fused_space(h, 6, f), G = 0;
+    int rc = fused_space(h, 6, f, s), G = 0;
     if (rc) return rc;
     const size_t smem = Op::SMEM * sizeof(float2);
     if ((rc = fused_grid(k_cg_fused<Op>, smem, FK_MAX_BLOCKS, N, G))) return rc;
@@ -377,7 +379,7 @@ static int gmres_solve_fused(evap_mesh* h, Op op, int m, const double* b, double
         return EVAP_EINVAL;
     }
     FusedSpace f;
-    int rc = fused_space(h, m + 3, f), G = 0;
+    int rc = fused_space(h, m + 3, f, s), G = 0;
     if (rc) return rc;
     const size_t smem = Op::SMEM * sizeof(float2);
     if ((rc = fused_grid(k_gmres_fused<Op>, smem, FK_MAX_BLOCKS, N, G))) return rc;
@@ -412,7 +414,7 @@ int geo_helmholtz(evap_mesh* h, double c, int ncomp, const double* x, double* y,
 
 int geo_projected_normal(evap_mesh* h, double* n, int* iters, double* relres, cudaStream_t s) {
     const MeshArgs<double> lm = ls_args<double>(h);  // the level-set mesh
-    int rc = geo_workspace(h);
+    int rc = geo_workspace(h, s);
     if (rc) return rc;
     CgSpace w = cg_space(h);
     const int64_t Np = lm.Nphi;
@@ -435,7 +437,7 @@ int geo_projected_normal(evap_mesh* h, double* n, int* iters, double* relres, cu
 
 int geo_curvature(evap_mesh* h, const double* nf, double* kappa, int* iters, double* relres, cudaStream_t s) {
     const MeshArgs<double> lm = ls_args<double>(h);  // the level-set mesh
-    int rc = geo_workspace(h);
+    int rc = geo_workspace(h, s);
     if (rc) return rc;
     CgSpace w = cg_space(h);
     const int64_t Np = lm.Nphi;
@@ -522,7 +524,7 @@ static int geo_elem_reserve(evap_mesh* h, int64_t need) {
 // `steps` pseudo-time steps of the reinitialization with the frozen normal of the level-set operators.
 int geo_reinitialize(evap_mesh* h, double* psi, int steps, int* iters, double* last_change, cudaStream_t s) {
     const MeshArgs<double> lm = ls_args<double>(h);  // the level-set mesh
-    int rc = geo_workspace(h);
+    int rc = geo_workspace(h, s);
     if (rc) return rc;
     CgSpace w = cg_space(h);
     const int64_t Np = lm.Nphi;
@@ -680,7 +682,7 @@ constexpr double ADVECT_REORTH = 1e-2;  // second Gram-Schmidt pass where the fi
 int geo_advect_levelset(evap_mesh* h, double* phi, int max_iters, double tol, int* fp_iters, int* lin_iters,
                         double* last_change, cudaStream_t s) {
     const MeshArgs<double> lm = ls_args<double>(h);  // the level-set mesh
-    int rc = geo_workspace(h);
+    int rc = geo_workspace(h, s);
     if (rc) return rc;
     CgSpace w = cg_space(h);
     const int64_t Np = lm.Nphi;

@@ -267,7 +267,7 @@ static void factor_band(const std::vector<double>& Mg, int M, int P, int lo, int
 }
 
 // Factors of the three axes (FP64 and FP32 copies, then the 1D mass diagonal in FP64): they depend on the mesh
-// and its Dirichlet faces only, so they are built and uploaded once per mesh (a synchronous copy).  Sigma follows
+// and its Dirichlet faces only, so they are built and uploaded once per mesh (on the stream, waited for).  Sigma follows
 // the Jacobi diagonal: the FP32 scale after every new diagonal, the FP64 one only when an FP64 solve asks for it;
 // both are enqueued on the stream without a host synchronization.
 int tensor_prec_setup(evap_mesh* h, bool fp64, cudaStream_t s) {
@@ -295,8 +295,9 @@ int tensor_prec_setup(evap_mesh* h, bool fp64, cudaStream_t s) {
         EVAP_CUDA(cudaMalloc(&h->tp_fac, bytes));
         std::vector<float> f32(all.begin(), all.begin() + nf);
         double* fac64 = (double*)h->tp_fac;
-        EVAP_CUDA(cudaMemcpy(fac64, all.data(), all.size() * sizeof(double), cudaMemcpyHostToDevice));
-        EVAP_CUDA(cudaMemcpy(fac64 + nf + M, f32.data(), nf * sizeof(float), cudaMemcpyHostToDevice));
+        EVAP_CUDA(cudaMemcpyAsync(fac64, all.data(), all.size() * sizeof(double), cudaMemcpyHostToDevice, s));
+        EVAP_CUDA(cudaMemcpyAsync(fac64 + nf + M, f32.data(), nf * sizeof(float), cudaMemcpyHostToDevice, s));
+        EVAP_CUDA(cudaStreamSynchronize(s));  // the host copies end here
         h->tp_nf = (int64_t)nf;
     }
     const double* md = (const double*)h->tp_fac + h->tp_nf;

@@ -216,7 +216,7 @@ int schur_solve(evap_mesh* h, const double* r, double* z, double rtol, int max_i
     if (rc) return rc;
     int64_t N = h->m.Np;
     FusedSpace f;
-    if ((rc = fused_space(h, 3, f))) return rc;  // 3 pair vectors = 6 float vectors of N_phi >= N_p entries
+    if ((rc = fused_space(h, 3, f, s))) return rc;  // 3 pair vectors = 6 float vectors of N_phi >= N_p entries
     int G = 0;
     if ((rc = fused_grid(k_cg_fused32<SchurStencil>, 0, FK_MAX_BLOCKS, N, G))) return rc;
     EVAP_CUDA(cudaMemsetAsync(f.gb, 0, sizeof(GridBarrier), s));
