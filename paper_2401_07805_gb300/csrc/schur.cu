@@ -151,14 +151,33 @@ struct SchurStencil {
 inline int64_t schur_guard(int n) { return 2 * ((int64_t)(n + 1) * (n + 1) + (n + 1) + 1); }
 inline int64_t schur_padded(int n) { return (int64_t)(n + 5) * (n + 5) * (n + 5); }
 
-// x (FP64) onto the padded lattice in FP32; y = S~ x (FP64 out), one thread per pressure node.
-__global__ void k_schur_pad(SchurStencil op, const double* __restrict__ x, float* __restrict__ xp) {
+// y = S~ x (x, y FP64, products and sums in FP32), one thread per pressure node, neighbours outside the lattice left out.
+// An apply writes nothing but y, so that applies on several streams can share a handle (the padded lattice behind the
+// stencil belongs to the CG); the sums are those of row(), whose extra products are zeros.
+__global__ void __launch_bounds__(256) k_schur_apply(SchurStencil op, const double* __restrict__ x,
+                                                     double* __restrict__ y) {
     const int64_t node = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (node < op.Np) xp[op.pos(node)] = (float)x[node];
-}
-__global__ void k_schur_apply(SchurStencil op, const float* __restrict__ xp, double* __restrict__ y) {
-    const int64_t node = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (node < op.Np) y[node] = (double)op.row(node, xp, nullptr);
+    if (node >= op.Np) return;
+    const int n = op.n, m1 = n + 1, m2 = m1 * m1;
+    const unsigned nd = (unsigned)node, t = nd / (unsigned)m1;
+    const int i = (int)(nd - t * (unsigned)m1), k = (int)(t / (unsigned)m1), j = (int)t - k * m1;
+    const float* c = op.S + node;
+    float acc = 0.f;
+#pragma unroll
+    for (int dz = -2; dz <= 2; ++dz)
+#pragma unroll
+        for (int dy = -2; dy <= 2; ++dy) {
+            const bool in = (unsigned)(k + dz) <= (unsigned)n && (unsigned)(j + dy) <= (unsigned)n;
+            const int nb = m1 * dy + m2 * dz;
+#pragma unroll
+            for (int dx = -2; dx <= 2; ++dx)
+                if (in && (unsigned)(i + dx) <= (unsigned)n) {
+                    const int lin = 25 * (dz + 2) + 5 * (dy + 2) + (dx + 2);
+                    const float cf = lin >= 62 ? c[(lin - 62) * op.Np] : c[(62 - lin) * op.Np + (nb + dx)];
+                    acc = fmaf(cf, (float)x[node + nb + dx], acc);
+                }
+        }
+    y[node] = (double)acc;
 }
 
 // Assembles S~ for the mesh's current Jacobi diagonal of A (launch_diagonal), once per diagonal.
@@ -171,7 +190,7 @@ int schur_assemble(evap_mesh* h, cudaStream_t s) {
         set_error("Schur stencil: its 63 N_p entries must be indexable with 32 bits");
         return EVAP_EINVAL;
     }
-    if (!h->schur_S) {  // guard, stencil, the padded lattice of the vector it is applied to
+    if (!h->schur_S) {  // guard, stencil, the padded lattice of the CG's vector
         const int64_t len = schur_guard(m.n) + 63 * m.Np + schur_padded(m.n);
         EVAP_CUDA(cudaMalloc(&h->schur_S, len * sizeof(float)));
         EVAP_CUDA(cudaMemsetAsync(h->schur_S, 0, len * sizeof(float), s));
@@ -200,11 +219,7 @@ int launch_schur_apply(evap_mesh* h, const double* x, double* y, cudaStream_t s)
     int rc = schur_assemble(h, s);
     if (rc) return rc;
     const SchurStencil op{h->m.n, h->m.Np, h->schur_S + schur_guard(h->m.n)};
-    float* xp = h->schur_S + schur_guard(h->m.n) + 63 * h->m.Np;  // its halo stays zero
-    const unsigned grid = (unsigned)((h->m.Np + 255) / 256);
-    k_schur_pad<<<grid, 256, 0, s>>>(op, x, xp);
-    EVAP_CHECK_LAUNCH("schur_pad");
-    k_schur_apply<<<grid, 256, 0, s>>>(op, xp, y);
+    k_schur_apply<<<(unsigned)((h->m.Np + 255) / 256), 256, 0, s>>>(op, x, y);
     EVAP_CHECK_LAUNCH("schur_apply");
     return EVAP_OK;
 }

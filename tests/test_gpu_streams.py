@@ -49,3 +49,22 @@ def test_first_solve_on_a_side_stream(name, n):
     side.synchronize()
     got = got.cpu().numpy()
     assert rel(got, want) <= bar
+
+
+@pytest.mark.parametrize("n,p", [(3, 2), (20, 2), (9, 3)])
+def test_schur_applies_on_two_streams(n, p):
+    """Applies of one handle on two streams at a time: each its own vector's product, bit for bit."""
+    op = make_op(workloads.random_workload(n, p, 80 + n, geom="sphere", dirichlet_faces=0x1F))
+    g = torch.Generator(device="cuda").manual_seed(n)
+    xs = [torch.rand(op.n_p, generator=g, device="cuda", dtype=torch.float64) for _ in range(2)]
+    want = [op.apply_schur(x) for x in xs]
+    streams = [torch.cuda.Stream() for _ in xs]
+    torch.cuda.synchronize()
+    got = [[], []]
+    for _ in range(50):
+        for k, st in enumerate(streams):
+            with torch.cuda.stream(st):
+                got[k].append(op.apply_schur(xs[k]))
+    torch.cuda.synchronize()
+    for k in range(2):
+        assert all(torch.equal(y, want[k]) for y in got[k])
