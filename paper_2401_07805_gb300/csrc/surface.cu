@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
     const int n = m.n;
     int cx = 0, cy = 0, cz = 0;
     // delta vanishes in cells without a point of the interface zone: their contribution is zero unless the caller's
-    // fields are not finite there
+    // factor or fields are not finite there (the factor is tested in its product with the curvature)
     bool active = cell < m.ncell;
     if (active) {
         cx = (int)(cell % n);
@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
         bool need = code[cell] == CELL_TABLE;
         for (int j = t; j < K * K * K && !need; j += NQ) {
             const int64_t node = (ns * cx + j % K) + (int64_t)ml * ((ns * cy + (j / K) % K) + (int64_t)ml * (ns * cz + j / (K * K)));
-            need = !(isfinite(kappa[node]) && isfinite(nf[node]) && isfinite(nf[m.Nphi + node]) &&
+            need = !(isfinite(alpha_crho * kappa[node]) && isfinite(nf[node]) && isfinite(nf[m.Nphi + node]) &&
                      isfinite(nf[2 * m.Nphi + node]));
         }
         active = need;
