@@ -87,7 +87,7 @@ constexpr size_t adj_smem() {
 
 template <int P, int CB, int K, int MINB>
 __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
-    k_adjoint(MeshArgs<double> m, Basis<double> bas, dfl rho_liq, dfl rho_gas, dfl kap,
+    k_adjoint(MeshArgs<double> m, Basis<double> bas, dfl rho_liq, dfl rho_gas,
               const int8_t* __restrict__ code, const int32_t* __restrict__ tindex, const float2* __restrict__ adjt,
               const float2* __restrict__ qcd, const double* __restrict__ w,
               const double* __restrict__ wp, const double* __restrict__ x, double* gx, double* gu, double* gphi,
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         auto OmG = [pt](int k, int d) { return pt[(15 + 3 * k + d) * NQ]; };
         cp_async_wait_all();
         const dfl* qp = cb + ADJ_SLOTS * NQ + t;
-        const dfl W = qp[14 * NQ], Wk = df_mul(W, kap);
+        const dfl Wk = qp[14 * NQ];  // kappa W
         // this point's entries of the adjoint table (table cells only; k_fill_table)
         const float2* ap = tcell ? adjt + (int64_t)tindex[cell] * ADJ_K * NQ + t : nullptr;
         const dfl rho = tcell ? ld_df(ap + ADJ_RHO * NQ) : (code[cell] == CELL_LIQUID ? rho_liq : rho_gas);
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
                 for (int l = k + 1; l < 3; ++l)
                     df_fma(smu, df_add(OmG(k, l), OmG(l, k)), df_scale2(df_add(G(k, l), G(l, k)), 0.5f));
             if (zg) df_fma(smu, df_neg(tr), nOn);
-            const dfl dL_dmu = df_mul(df_mul(df_scale2(Wk, 2.0f), kap), df_norm(smu));
+            const dfl dL_dmu = df_mul(df_scale2(Wk, 2.0f), df_norm(smu));  // (/ kappa)
             // dL/dn = -2 W mu z tr(G) (OmG + OmG^T) n; its part normal to n drops out (dn/dgrad phi)
             dfl dLdn[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
             if (zg) {
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
                 dgv[i] = df_mul(df_norm(u), ign);
             }
             if (wp) {  // through v_dil = mdot c_1 delta (Eq. evaporDil), dL/dv_dil = -W pi
-                const dfl dLdv = df_neg(df_mul(W, pid));
+                const dfl dLdv = df_neg(Wkpi);  // (times kappa)
                 dm = df_to_double(df_mul(dLdv, ld_df(ap + ADJ_KD1 * NQ)));
                 df_fma(dp, dLdv, ld_df(ap + ADJ_KD2 * NQ));
                 const dfl k3 = df_mul(dLdv, ld_df(ap + ADJ_KD3 * NQ));
@@ -436,7 +436,6 @@ int launch_adjoint(evap_mesh* h, const double* w, const double* wp, const double
     const unsigned gi = (unsigned)std::min<int64_t>((3 * (int64_t)m.M * m.M + 7) / 8, 152 * 16);
     k_adjoint_init<<<gi, 256, 0, s>>>(m.M, m.Nu, m.Nphi, m.faces, w, gx, gu, gphi, gm);
     EVAP_CHECK_LAUNCH("adjoint_init");
-    const dfl kap = df_from_double(df_kappa(m));
     const float2* qcd = reinterpret_cast<const float2*>(h->qcdf);
     const dfl rho_liq = df_from_double(m.rho_H1), rho_gas = df_from_double(m.rho_H0);  // rho outside table cells
     const int c0 = h->deterministic ? 0 : -1, c1 = h->deterministic ? 8 : 0;  // colour passes, or one atomic pass
@@ -444,7 +443,7 @@ int launch_adjoint(evap_mesh* h, const double* w, const double* wp, const double
         for (int colour = c0; colour < std::max(c1, c0 + 1); ++colour) {
             const int64_t cells = colour_cells(m.n, colour);
             if (cells == 0) continue;
-            kern<<<(unsigned)((cells + CB - 1) / CB), threads, dyn, s>>>(m, h->b, rho_liq, rho_gas, kap, h->cell_code,
+            kern<<<(unsigned)((cells + CB - 1) / CB), threads, dyn, s>>>(m, h->b, rho_liq, rho_gas, h->cell_code,
                                                                        h->table_index, h->adj_table, qcd, w, wp, x,
                                                                        gx, gu, gphi, gm, colour);
             EVAP_CHECK_LAUNCH("adjoint");

@@ -30,11 +30,13 @@ __device__ __forceinline__ dfl df_addl(dfl a, dfl b) {
 __device__ __forceinline__ dfl df_twice(dfl a) { return {a.hi + a.hi, a.lo + a.lo}; }
 __device__ __forceinline__ dfl df_half(dfl a) { return {0.5f * a.hi, 0.5f * a.lo}; }
 
-// Which sums are normalized: results stored for the next sweep (df_addo) and sums multiplied next (df_addi); sums that are
-// added further are not.  Measured at 64^3 Q2 (us per apply, error against 64 bits; 1.12e-14 with Q-term dot products):
-// both 552, 1.10e-14; only the multiplied ones 540, 1.14e-14; only the stored ones 540, 1.11e-14 (5.25e-15 at 8^3, 5.21e-15
-// before); none 529, 1.17e-14.  For Q = 3 both are, so that no case loses accuracy; for Q = 4 the stored ones (45^3 Q3: 576
-// -> 544 us, 3.74e-14 -> 3.75e-14; 3.79e-14 with dot products).
+// Which sums are normalized, Q = 3: results stored for the next sweep (df_addo), sums multiplied next (df_addi), the even part
+// that both outer values share, and the gradients; the sums of the transposes that are added further are not.  Errors
+// against 64 bits relative to Q-term dot products, geometric means over 59 to 89 drawn cases (velocity rows / divergence row
+// / adjoint g_x / g_u0): 0.98 / 1.02 / 1.00 / 1.01 with the even part and the gradients left unnormalized, 0.98 / 0.98 / 0.99
+// / 0.96 with them normalized (48^3 Q2 apply 218 -> 220 us).  At 64^3 Q2 (us per apply): both of df_addo and df_addi 552,
+// one of them 540, none 529 with an error larger than the dot products'.  Q = 4 normalizes the stored results only (45^3 Q3:
+// 576 -> 544 us; 0.91 / 0.99 / 0.90 / 0.93).
 __device__ __forceinline__ dfl df_addo(dfl a, dfl b) { return df_add(a, b); }
 __device__ __forceinline__ dfl df_addi(dfl a, dfl b) { return df_add(a, b); }
 
@@ -48,7 +50,7 @@ struct DfLine<3> {
     static __device__ __forceinline__ void val(const dfl u[3], dfl y[3]) {
         const dfl dm = df_addi(u[2], df_neg(u[0]));
         const dfl C = df_addi(df_addl(u[0], u[2]), df_neg(df_twice(u[1])));
-        const dfl base = df_addl(u[1], df_mul(C, EVAP_DFK(0.3)));
+        const dfl base = df_add(u[1], df_mul(C, EVAP_DFK(0.3)));
         const dfl m = df_mul(dm, EVAP_DFK(TAU));
         y[0] = df_addo(base, df_neg(m));
         y[1] = u[1];
@@ -66,9 +68,9 @@ struct DfLine<3> {
     static __device__ __forceinline__ void der(const dfl y[3], dfl d[3]) {
         const dfl A = df_addl(y[1], df_neg(y[0])), B = df_addl(y[2], df_neg(y[1]));
         const dfl D = df_addl(A, df_neg(B));
-        d[0] = df_addl(D, df_twice(A));
-        d[1] = df_addl(A, B);
-        d[2] = df_addl(df_twice(B), df_neg(D));
+        d[0] = df_add(D, df_twice(A));
+        d[1] = df_add(A, B);
+        d[2] = df_add(df_twice(B), df_neg(D));
     }
     static __device__ __forceinline__ void derT(const dfl t[3], dfl o[3]) {
         const dfl a = df_addl(t[0], df_neg(t[2]));

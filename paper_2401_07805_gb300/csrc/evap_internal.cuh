@@ -210,13 +210,13 @@ struct evap_mesh {
 // normal_vector, delta, evaporDil): see adjoint.cu.
 enum AdjSlot : int {
     ADJ_CRHO = 0,  // (drho/dH) H'(d) d'(phi) in the zone, else 0
-    ADJ_CMU,       // (dmu/dH) H'(d) d'(phi) in the zone, else 0
+    ADJ_CMU,       // kappa (dmu/dH) H'(d) d'(phi) in the zone, else 0 (kappa: df_lines.cuh)
     ADJ_N,         // 3 slots: the unit normal (0 where |grad phi| h <= GRAD_TINY)
     ADJ_ZG = ADJ_N + 3,  // correction gate z (1 or 0)
     ADJ_IGN,       // 1 / |grad phi| (0 where the normal is 0)
-    ADJ_KD1,       // c_1 delta (the v_dil factor of mdot)
-    ADJ_KD2,       // mdot c_1 (H''(d) d'(phi)^2 + H'(d) d''(phi)) |grad phi|
-    ADJ_KD3,       // mdot c_1 H'(d) d'(phi)
+    ADJ_KD1,       // c_1 delta / kappa (the v_dil factor of mdot)
+    ADJ_KD2,       // mdot c_1 (H''(d) d'(phi)^2 + H'(d) d''(phi)) |grad phi| / kappa
+    ADJ_KD3,       // mdot c_1 H'(d) d'(phi) / kappa
     ADJ_IRHO,      // 1 / rho
     ADJ_RHO,       // rho
     ADJ_ZONE,      // 1 in the zone |phi| < tanh(3/2), else 0

@@ -38,12 +38,14 @@ __global__ void __launch_bounds__(256) k_momentum_init(int M, int64_t Nu, unsign
 // Quadrature-point coefficients of the momentum operator, evaluated once per set_fields from u0 and the material-law table,
 // as double-float pairs (layout [cell][QC_K][nq]):
 //   0: W rho c_m   1..3: kappa W rho u0_b   4..12: newton W rho d_d u0_c (index 4 + 3c + d)   13: kappa^2 2 W mu
-//   14..16: z n_b (correction gate times normal)   17: W   18: W v_dil
+//   14..16: z n_b (correction gate times normal)   17: kappa W   18: W v_dil
 // W = w_qx w_qy w_qz h^3, kappa = DSCALE / h the factor between a gradient and the derivative sweeps (df_lines.cuh).  The
 // FP64-accurate apply and the adjoint read the pairs as they stand; the Jacobi diagonal, the mass load and the continuity
 // right-hand side read the few slots they need.  Slots 1..12 are also stored in FP32 for the FP32 apply (there W rho u0 / h:
 // that kernel takes reference gradients), in its 32-cell block layout
 // qc32[((blk * QC32_K + k) * NQ + pt) * 32 + lane], cell 32 blk + lane (lexicographic).
+// Every factor that does not depend on u0 is formed in FP64 and rounded once to a pair (a power of kappa applied to a pair
+// would round it twice: the divergence row at Q2 then had 1.03 times the error against 64 bits).
 // u0 is interpolated by lines (df_lines.cuh).  The weights and, outside table cells, W rho and 2 W mu take the same NQ
 // values in every cell: tabulated on the host, so that the FP64 pipe converts u0 and the table cells' entries only.  A
 // block takes CB cells of one 32-cell block, and writes their FP32 entries through shared memory in runs of CB floats.
@@ -51,29 +53,30 @@ __global__ void __launch_bounds__(256) k_momentum_init(int M, int64_t Nu, unsign
 // GB, and scattered FP32 stores before); the writes alone take 210 at the HBM rate.
 template <int NQ>
 struct QpTables {
-    float2 w[NQ], wr[2][NQ], wm[2][NQ];  // W; W rho and kappa^2 2 W mu of gas (0) and liquid (1)
+    float2 wk[NQ], wr[2][NQ], wkr[2][NQ], wm[2][NQ];  // kappa W; W rho, kappa W rho and kappa^2 2 W mu of gas (0), liquid (1)
 };
 template <int P, int CB>
 __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
-    k_qp_coeffs(MeshArgs<double> m, Basis<double> bas, QpTables<(P + 1) * (P + 1) * (P + 1)> tabs, dfl cm_df, dfl kap,
-                dfl kap2, dfl ik, const int8_t* __restrict__ code, const int32_t* __restrict__ tindex,
+    k_qp_coeffs(MeshArgs<double> m, Basis<double> bas, QpTables<(P + 1) * (P + 1) * (P + 1)> tabs, dfl cm_df,
+                double kappa, double kappa2, dfl ik, const int8_t* __restrict__ code, const int32_t* __restrict__ tindex,
                 const double* __restrict__ table, const double* __restrict__ u0, float2* __restrict__ qcdf,
                 float* __restrict__ qc32) {
     constexpr int Q = P + 1, NQ = Q * Q * Q, NL = Q * Q, TASKS = 3 * NL;
     static_assert(32 % CB == 0, "a block's cells lie in one 32-cell block");
     using Ln = DfLine<Q>;
     __shared__ dfl buf[CB][12][NQ];  // slots: 0..2 U, 3 + 3 k + d the derivatives (in units of kappa)
-    __shared__ float2 sw[NQ], swr[2][NQ], swm[2][NQ];
+    __shared__ float2 swk[NQ], swr[2][NQ], swkr[2][NQ], swm[2][NQ];
     const int tid = threadIdx.x;
     const int lc = tid / NQ, t = tid % NQ;
     const unsigned cell0 = blockIdx.x * CB;
     int cx, cy, cz;
     const bool active = colour_cell32(cell0 + lc, m.n, -1, cx, cy, cz);
     for (int i = tid; i < NQ; i += CB * NQ) {
-        sw[i] = tabs.w[i];
+        swk[i] = tabs.wk[i];
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             swr[k][i] = tabs.wr[k][i];
+            swkr[k][i] = tabs.wkr[k][i];
             swm[k][i] = tabs.wm[k][i];
         }
     }
@@ -122,23 +125,24 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
     const unsigned cell = cell0 + lc;
     float f32[QC32_K];
     {
-        const dfl W = ld_df(&sw[t]);
-        dfl wr, wm, nz[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, wv{0.f, 0.f};
+        dfl wr, wk, wm, nz[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, wv{0.f, 0.f};
         const int8_t cc = active ? code[cell] : (int8_t)CELL_GAS;
         if (cc == CELL_TABLE) {
             const double* tb = table + (int64_t)tindex[cell] * TAB_K * NQ + t;
             const double Wd = bas.w[t % Q] * bas.w[(t / Q) % Q] * bas.w[t / NL] * m.vol_w;
-            wr = df_from_double(Wd * tb[0]);
-            wm = df_mul(df_from_double(2.0 * Wd * tb[NQ]), kap2);
+            const double wrd = Wd * tb[0];
+            wr = df_from_double(wrd);
+            wk = df_from_double(kappa * wrd);
+            wm = df_from_double(kappa2 * (2.0 * Wd * tb[NQ]));
 #pragma unroll
             for (int d = 0; d < 3; ++d) nz[d] = df_from_double(tb[(2 + d) * NQ]);
             wv = df_from_double(Wd * tb[5 * NQ]);
         } else {
             const int liq = cc == CELL_LIQUID ? 1 : 0;
             wr = ld_df(&swr[liq][t]);
+            wk = ld_df(&swkr[liq][t]);
             wm = ld_df(&swm[liq][t]);
         }
-        const dfl wk = df_mul(wr, kap);
         float2* dst = qcdf + (int64_t)cell * QC_K * NQ + t;
         auto put = [&](int k, dfl v) {
             if (active) dst[k * NQ] = make_float2(v.hi, v.lo);
@@ -159,7 +163,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
         put(13, wm);
 #pragma unroll
         for (int d = 0; d < 3; ++d) put(14 + d, nz[d]);
-        put(17, W);
+        put(17, ld_df(&swk[t]));
         put(18, wv);
     }
     __syncthreads();
@@ -178,7 +182,6 @@ static void run_qp_coeffs(evap_mesh* h, cudaStream_t s) {
     constexpr int Q = P + 1, NQ = Q * Q * Q;
     const MeshArgs<double>& m = h->m;
     const double kd = df_kappa(m);
-    const dfl kap2 = df_from_double(kd * kd);
     QpTables<NQ> tabs;
     auto pair = [](double v) {
         const dfl d = df_from_double(v);
@@ -186,15 +189,17 @@ static void run_qp_coeffs(evap_mesh* h, cudaStream_t s) {
     };
     for (int q = 0; q < NQ; ++q) {
         const double W = h->b.w[q % Q] * h->b.w[(q / Q) % Q] * h->b.w[q / (Q * Q)] * m.vol_w;
-        tabs.w[q] = pair(W);
+        tabs.wk[q] = pair(kd * W);
         for (int k = 0; k < 2; ++k) {
-            tabs.wr[k][q] = pair(W * (k ? m.rho_H1 : m.rho_H0));
+            const double wr = W * (k ? m.rho_H1 : m.rho_H0);
+            tabs.wr[k][q] = pair(wr);
+            tabs.wkr[k][q] = pair(kd * wr);
             tabs.wm[k][q] = pair(kd * kd * 2.0 * W * (k ? m.mu_H1 : m.mu_H0));
         }
     }
     k_qp_coeffs<P, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * NQ, 0, s>>>(
-        m, h->b, tabs, df_from_double(m.c_mass), df_from_double(kd), kap2, df_from_double(m.inv_h / kd), h->cell_code,
-        h->table_index, h->table, h->u, (float2*)h->qcdf, h->qc32);
+        m, h->b, tabs, df_from_double(m.c_mass), kd, kd * kd, df_from_double(m.inv_h / kd), h->cell_code, h->table_index,
+        h->table, h->u, (float2*)h->qcdf, h->qc32);
 }
 
 int launch_qp_coeffs(evap_mesh* h, cudaStream_t s) {

@@ -24,8 +24,8 @@
 // What bounds it: FP32 issue (the additions of the error-free transformations).
 //
 // The quadrature-point coefficients are the pairs of k_qp_coeffs (qcdf, [cell][QC_K][nq] float2), 8 bytes per
-// coefficient as in FP64, with the factor kappa = DSCALE / h of the derivative in the slots that multiply one (1..3)
-// and kappa^2 in the viscous one (13).  Each thread copies its point's coefficients into shared memory with
+// coefficient as in FP64, with the factor kappa = DSCALE / h of the derivative in the slots that multiply one (1..3,
+// 17) and kappa^2 in the viscous one (13).  Each thread copies its point's coefficients into shared memory with
 // cp.async at the start, so that their HBM latency is hidden behind the interpolation sweeps.  The correction term is
 // skipped at points where its gate z n is zero (outside the interface zone), and the Newton terms on Picard meshes.
 #include <algorithm>
@@ -68,8 +68,7 @@ __device__ __forceinline__ constexpr int t_slot(int k, int l) {
 
 template <int P, int CB, bool PRES, int MINB, bool DET>
 __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
-    k_momentum_df(MeshArgs<double> m, DfBasis bas, dfl kap, const float2* __restrict__ qc,
-                  const double* __restrict__ x,
+    k_momentum_df(MeshArgs<double> m, DfBasis bas, const float2* __restrict__ qc, const double* __restrict__ x,
                   double* __restrict__ y, double* __restrict__ yp, const double* __restrict__ pin, int colour) {
     constexpr int Q = P + 1, NQ = Q * Q * Q, NL = Q * Q, TASKS = 3 * NL;
     using Ln = DfLine<Q>;
@@ -206,7 +205,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
         const dfl nz[3] = {q[14 * NQ], q[15 * NQ], q[16 * NQ]};
         const bool corr = (nz[0].hi != 0.f) || (nz[1].hi != 0.f) || (nz[2].hi != 0.f);
         const dfl sm = corr ? df_mul(c13, tr) : dfl{0.f, 0.f};
-        const dfl rw = PRES || yp ? df_mul(q[17 * NQ], kap) : dfl{0.f, 0.f};  // kappa W
+        const dfl rw = q[17 * NQ];  // kappa W
         dfl wp{0.f, 0.f};
         if constexpr (PRES) wp = df_mul(rw, df_from_double(lerp(py[lc][t % NL], py[lc][t % NL + NL], t / NL)));
 #pragma unroll
@@ -321,7 +320,6 @@ DfBasis make_df_basis(const Basis<double>& b, double inv_h) {
 int launch_momentum_df(evap_mesh* h, const MeshArgs<double>& m, const double* x, double* y, double* yp,
                        const double* p, cudaStream_t s) {
     const DfBasis b = make_df_basis(h->b, m.inv_h);
-    const dfl kap = df_from_double(df_kappa(m));
     const float2* qc = reinterpret_cast<const float2*>(h->qcdf);
     const int c0 = h->deterministic ? 0 : -1, c1 = h->deterministic ? 8 : 0;  // colour passes, or one atomic pass
     // at most 48 KB of shared memory per block, so no launch needs a function attribute
@@ -330,7 +328,7 @@ int launch_momentum_df(evap_mesh* h, const MeshArgs<double>& m, const double* x,
             const int64_t cells = colour_cells(m.n, colour);
             if (cells == 0) continue;
             const unsigned grid = (unsigned)((cells + CB - 1) / CB);
-            kern<<<grid, threads, dyn, s>>>(m, b, kap, qc, x, y, yp, p, colour);
+            kern<<<grid, threads, dyn, s>>>(m, b, qc, x, y, yp, p, colour);
             EVAP_CHECK_LAUNCH("momentum_df");
         }
         return EVAP_OK;

@@ -2,7 +2,7 @@
 // the level-set transport velocity with closest-point projection (App. C).
 #include <cmath>
 
-#include "dfloat.cuh"
+#include "df_lines.cuh"
 #include "physics.cuh"
 
 namespace evap {
@@ -125,7 +125,8 @@ __global__ void k_classify(MeshArgs<double> m, Basis<double> b, const double* __
 // table cells): 728 -> 486 us (an interpolation per field and every function evaluated twice before).
 __global__ void k_fill_table(MeshArgs<double> m, Basis<double> b, const double* __restrict__ phi,
                              const double* __restrict__ mdot, const int8_t* __restrict__ code,
-                             const int32_t* __restrict__ tindex, double* table, float* table32, float2* adj) {
+                             const int32_t* __restrict__ tindex, double kdmu, double kdk, double* table,
+                             float* table32, float2* adj) {
     const unsigned nq = b.Q * b.Q * b.Q;
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const unsigned cell = (unsigned)(gid / nq);
@@ -201,17 +202,18 @@ __global__ void k_fill_table(MeshArgs<double> m, Basis<double> b, const double* 
         table[tb + (int64_t)k * nq] = vals[k];
         table32[tb + (int64_t)k * nq] = (float)vals[k];
     }
+    // (the adjoint's weight is kappa W: kdmu = kappa (mu_l - mu_g), kdk = kdil / kappa)
     double av[ADJ_K];
     av[ADJ_CRHO] = -rho * rho * (irl - irg) * dHdd;
-    av[ADJ_CMU] = (m.mu_l - m.mu_g) * dHdd;
+    av[ADJ_CMU] = kdmu * dHdd;
     av[ADJ_N + 0] = nv[0];
     av[ADJ_N + 1] = nv[1];
     av[ADJ_N + 2] = nv[2];
     av[ADJ_ZG] = z;
     av[ADJ_IGN] = ign;
-    av[ADJ_KD1] = kdil * delta;
-    av[ADJ_KD2] = md * kdil * d2 * gn;
-    av[ADJ_KD3] = md * kdil * dHdd;
+    av[ADJ_KD1] = kdk * delta;
+    av[ADJ_KD2] = md * kdk * d2 * gn;
+    av[ADJ_KD3] = md * kdk * dHdd;
     av[ADJ_IRHO] = irho;
     av[ADJ_RHO] = rho;
     av[ADJ_ZONE] = zone ? 1.0 : 0.0;
@@ -251,8 +253,10 @@ int launch_setup_coefficients(evap_mesh* h, cudaStream_t s) {
     }
     if (count > 0) {
         const int64_t total = m.ncell * nq;
+        const double kdil = 1.0 / m.rho_g - 1.0 / m.rho_l;
         k_fill_table<<<blocks_for(total, 256, 1LL << 40), 256, 0, s>>>(m, h->b, h->phi, h->mdot, h->cell_code,
-                                                                       h->table_index, h->table, h->table32,
+                                                                       h->table_index, df_kappa(m) * (m.mu_l - m.mu_g),
+                                                                       kdil / df_kappa(m), h->table, h->table32,
                                                                        h->adj_table);
         EVAP_CHECK_LAUNCH("fill_table");
     }
