@@ -1,5 +1,5 @@
 """The accuracy of the momentum apply against FP64, as the geometric mean over a fixed set of small cases: coefficients rounded
-once to a pair, line sums normalized before they are multiplied or added twice.
+once to a pair, line sums normalized before they are multiplied or added twice, FP32 sums of values and tests paired.
 
 Bars: the means of the kernels that formed every product and sum point by point with Q-term dot products (2 % more: the
 means' repeatability is a few tenths of a per cent, from the order of the atomic adds).
@@ -27,7 +27,8 @@ def mean_errors(p, prec):
     return np.exp(np.log(np.array(e)).mean(0))
 
 
-BARS = {(2, 64): (5.447e-15, 5.549e-15), (3, 64): (8.696e-15, 1.0628e-14)}
+BARS = {(2, 64): (5.447e-15, 5.549e-15), (3, 64): (8.696e-15, 1.0628e-14), (2, 32): (1.447e-7, 1.96e-7),
+        (3, 32): (1.3507e-7, 1.535e-7)}
 
 
 @pytest.mark.parametrize("p,prec", sorted(BARS))
