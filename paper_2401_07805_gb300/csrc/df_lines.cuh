@@ -1,11 +1,11 @@
 // Sweeps of the double-float operators along one line of Q = P + 1 points, in double-float arithmetic (dfloat.cuh).
 //
-// Support points (Gauss-Lobatto) and quadrature points (Gauss-Legendre) are symmetric about 1/2, so a line's even and
-// odd parts are transformed apart (the even-odd decomposition of tensor-product elements), and for Q = 3 the
-// interpolation of a quadratic c(t) = c_1 + (t - 1/2) dm + 2 (t - 1/2)^2 C with dm = c_2 - c_0, C = c_0 - 2 c_1 + c_2
-// needs only two multiplications: by tau = sqrt(3/20), the distance of the outer Gauss points from 1/2, and by
-// 2 tau^2 = 3/10.  FP32 instructions per line of 3 results: 80 (values), 60 (derivatives), against 93 for three
-// 3-term dot products each (df_dot), with a third of their shared-memory loads, since one thread forms a whole line.
+// Support points (Gauss-Lobatto) and quadrature points (Gauss-Legendre) are symmetric about 1/2.  Q = 3: the middle points
+// coincide, the outer values are three-term dot products, and the transposed sweep takes the even and the odd part of the
+// outer points with three multiplications (3/10, 4/10 and tau = sqrt(3/20), the distance of the outer Gauss points from
+// 1/2).  Q = 4: even and odd parts are transformed apart (the even-odd decomposition of tensor-product elements).  FP32
+// instructions per line of 3 results: 62 (values), 61 (derivatives), against 93 for three 3-term dot products, with a
+// third of their shared-memory loads, since one thread forms a whole line.
 //
 //   val   y_q = sum_a S[q][a] u_a           valT  o_a = sum_q S[q][a] f_q
 //   der   d_q = sum_r D[q][r] y_r           derT  o_r = sum_q D[q][r] t_q,   D = (collocation derivative) / DSCALE:
@@ -30,13 +30,14 @@ __device__ __forceinline__ dfl df_addl(dfl a, dfl b) {
 __device__ __forceinline__ dfl df_twice(dfl a) { return {a.hi + a.hi, a.lo + a.lo}; }
 __device__ __forceinline__ dfl df_half(dfl a) { return {0.5f * a.hi, 0.5f * a.lo}; }
 
-// Which sums are normalized, Q = 3: results stored for the next sweep (df_addo), sums multiplied next (df_addi), the even part
-// that both outer values share, and the gradients; the sums of the transposes that are added further are not.  Errors
-// against 64 bits relative to Q-term dot products, geometric means over 59 to 89 drawn cases (velocity rows / divergence row
-// / adjoint g_x / g_u0): 0.98 / 1.02 / 1.00 / 1.01 with the even part and the gradients left unnormalized, 0.98 / 0.98 / 0.99
-// / 0.96 with them normalized (48^3 Q2 apply 218 -> 220 us).  At 64^3 Q2 (us per apply): both of df_addo and df_addi 552,
-// one of them 540, none 529 with an error larger than the dot products'.  Q = 4 normalizes the stored results only (45^3 Q3:
-// 576 -> 544 us; 0.91 / 0.99 / 0.90 / 0.93).
+// Which sums are normalized: results stored for the next sweep (df_addo) and, for Q = 3, sums multiplied next (df_addi) and the
+// gradients; sums that are added further are not.  Errors against 64 bits relative to point-wise dot products, geometric
+// means (velocity rows / divergence row / adjoint g_x / g_u0 / g_phi over 100 to 2242 drawn Q2 cases; pressure term alone, 34):
+//   outer values as u_1 + 3/10 C -+ tau dm with C = u_0 - 2 u_1 + u_2, the transposed middle as s + f_1 - 2 (3/10 s),
+//     even part and gradients unnormalized    0.98 / 1.02 / 1.00 / 1.00 / 1.05 / 1.12   (48^3 Q2 apply 218 us, adjoint 561)
+//   this arrangement                          0.90 / 0.91 / 0.82 / 0.81 / 1.004 +- 0.005 / 0.77   (216 us, 549)
+// 64^3 Q2 apply with the first arrangement (us): both of df_addo and df_addi normalized 552, one of them 540, none 529.
+// Q = 4 normalizes the stored results only (45^3 Q3: 576 -> 544 us; 0.89 / 0.97 / 0.88 / 0.90 / 0.98 / 0.99).
 __device__ __forceinline__ dfl df_addo(dfl a, dfl b) { return df_add(a, b); }
 __device__ __forceinline__ dfl df_addi(dfl a, dfl b) { return df_add(a, b); }
 
@@ -47,22 +48,25 @@ template <>
 struct DfLine<3> {
     static constexpr double TAU = 0.5 * 0.7745966692414833770358531;  // sqrt(3/5) / 2
     static constexpr double DSCALE = 1.0 / (2.0 * TAU);
+    static __device__ __forceinline__ dfl dot3(const dfl u[3], dfl c0, dfl c1, dfl c2) {
+        dfl s = df_prod(c0, u[0]);
+        df_fma(s, c1, u[1]);
+        df_fma(s, c2, u[2]);
+        return df_norm(s);
+    }
     static __device__ __forceinline__ void val(const dfl u[3], dfl y[3]) {
-        const dfl dm = df_addi(u[2], df_neg(u[0]));
-        const dfl C = df_addi(df_addl(u[0], u[2]), df_neg(df_twice(u[1])));
-        const dfl base = df_add(u[1], df_mul(C, EVAP_DFK(0.3)));
-        const dfl m = df_mul(dm, EVAP_DFK(TAU));
-        y[0] = df_addo(base, df_neg(m));
+        constexpr double a0 = 0.3 + TAU, a2 = 0.3 - TAU;
+        y[0] = dot3(u, EVAP_DFK(a0), EVAP_DFK(0.4), EVAP_DFK(a2));
         y[1] = u[1];
-        y[2] = df_addo(base, m);
+        y[2] = dot3(u, EVAP_DFK(a2), EVAP_DFK(0.4), EVAP_DFK(a0));
     }
     template <bool FINAL>  // FINAL: the results are converted next
     static __device__ __forceinline__ void valT(const dfl f[3], dfl o[3]) {
         const dfl s = df_addi(f[0], f[2]), d = df_addi(f[0], df_neg(f[2]));
         const dfl p = df_mul(s, EVAP_DFK(0.3)), r = df_mul(d, EVAP_DFK(TAU));
-        const dfl s1 = df_addl(s, f[1]), p2 = df_neg(df_twice(p));
+        const dfl p2 = df_mul(s, EVAP_DFK(0.4));  // (not s - 2 p: that doubles the rounding of p)
         o[0] = FINAL ? df_addl(p, r) : df_addo(p, r);
-        o[1] = FINAL ? df_addl(s1, p2) : df_addo(s1, p2);
+        o[1] = FINAL ? df_addl(f[1], p2) : df_addo(f[1], p2);
         o[2] = FINAL ? df_addl(p, df_neg(r)) : df_addo(p, df_neg(r));
     }
     static __device__ __forceinline__ void der(const dfl y[3], dfl d[3]) {

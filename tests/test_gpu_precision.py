@@ -1,14 +1,16 @@
-"""The accuracy of the momentum apply against FP64, as the geometric mean over a fixed set of small cases: coefficients rounded
-once to a pair, line sums normalized before they are multiplied or added twice, FP32 sums of values and tests paired.
+"""The accuracy of the momentum applies and the adjoint against FP64, as the geometric mean over a fixed set of small cases:
+coefficients rounded once to a pair, line sums normalized before they are multiplied or added twice, FP32 sums of values and
+tests paired.
 
 Bars: the means of the kernels that formed every product and sum point by point with Q-term dot products (2 % more: the
 means' repeatability is a few tenths of a per cent, from the order of the atomic adds).
 """
 import numpy as np
 import pytest
+import torch
 
 import workloads
-from oracle import momentum
+from oracle import adjoint, momentum
 from test_gpu_parity import cuda, make_op, rel
 
 pytestmark = pytest.mark.gpu
@@ -36,3 +38,42 @@ def test_mean_error(p, prec):
     got, bar = mean_errors(p, prec), BARS[p, prec]
     print(f"mean errors Q{p} FP{prec}: {got[0]:.3e} {got[1]:.3e}")
     assert got[0] <= 1.02 * bar[0] and got[1] <= 1.02 * bar[1]
+
+
+def mean_pressure_error(p):
+    """Of the pressure term alone: the velocity rows of the velocity-pressure apply at x = 0, and the oracle's -B^T p."""
+    e = []
+    for k in range(12):
+        wl = workloads.random_workload(3 + k % 3, p, 600 + k, geom="sphere", dirichlet_faces=0x1F)
+        op = make_op(wl)
+        pr = np.random.default_rng(k).uniform(-1, 1, op.n_p)
+        y, _ = op.apply_saddle(torch.zeros(3 * op.n_u, dtype=torch.float64, device="cuda"), cuda(pr))
+        B, _ = momentum.divergence(momentum.Problem.from_workload(wl))
+        e.append(rel(y, -(B.T @ pr)))
+    return np.exp(np.log(e).mean())
+
+
+def mean_adjoint_errors(p):
+    """Of g_x, g_u0 and g_phi."""
+    e = []
+    for k in range(60):
+        wl = workloads.random_workload(4, p, 700 + k, geom=("sphere", "deformed", "slab")[k % 3])
+        pb = momentum.Problem.from_workload(wl)
+        rng = np.random.default_rng(k)
+        w, wp = rng.uniform(-1, 1, wl.x.shape), rng.uniform(-1, 1, 5 ** 3)
+        g = make_op(wl).apply_adjoint(cuda(w), cuda(wl.x), cuda(wp))
+        gu, gphi, _ = adjoint.param_gradients(pb, wl.x, w, wp)
+        e.append((rel(g["x"], adjoint.grad_x(pb, w, wp)), rel(g["u0"], gu), rel(g["phi"], gphi)))
+    return np.exp(np.log(np.array(e)).mean(0))
+
+
+def test_mean_error_of_the_pressure_term():
+    got = mean_pressure_error(2)
+    print(f"mean error, pressure term: {got:.3e}")
+    assert got <= 1.02 * 5.484e-15
+
+
+def test_mean_errors_of_the_adjoint():
+    got = mean_adjoint_errors(2)
+    print("mean errors, adjoint:", got)
+    assert (got <= 1.02 * np.array([4.702e-15, 8.542e-15, 4.686e-15])).all()
