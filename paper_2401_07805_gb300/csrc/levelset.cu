@@ -16,7 +16,7 @@
 namespace evap {
 
 template <typename T, int MODE, bool DET>
-__global__ void __launch_bounds__(128) k_levelset(MeshArgs<T> m, const T* __restrict__ phi,
+__global__ void __launch_bounds__(128) k_levelset(MeshArgs<T> m, T wm, T wd, const T* __restrict__ phi,
                                                   const T* __restrict__ nf, const T* __restrict__ ug,
                                                   const T* __restrict__ x, T* __restrict__ y, int colour) {
     int cx, cy, cz;
@@ -64,7 +64,6 @@ __global__ void __launch_bounds__(128) k_levelset(MeshArgs<T> m, const T* __rest
     } else {
         T nv[8][3], F[8], G0[8], G1[8], G2[8];  // G: flux tested with the reference gradients (physical flux / h)
         frozen_normals<T>(nf != nullptr, uv, pv, nv);
-        const T wm = W / m.dtau, wd = MODE == EVAP_REINIT ? W * m.eps * ih * ih : W * T(0.5) * ih;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const int qx = q & 1, qy = (q >> 1) & 1, qz = q >> 2;
@@ -218,6 +217,12 @@ __global__ void __launch_bounds__(128) k_levelset_advect_sf(MeshArgs<double> m, 
 template <typename T>
 int launch_levelset(evap_mesh* h, int mode, const T* x, T* y, cudaStream_t s) {
     const MeshArgs<T> m = ls_args<T>(h);  // Q1 on the level-set mesh
+    // factors of the mass and the flux term of the reinitialization operators, formed in FP64 and rounded once: a rounded
+    // factor is wrong by the same amount at every point
+    const MeshArgs<double> md = ls_args<double>(h);
+    const double Wd = 0.125 * md.vol_w;
+    const T wm = (T)(Wd / md.dtau);
+    const T wd = (T)(mode == EVAP_REINIT ? Wd * md.eps * md.inv_h * md.inv_h : Wd * 0.5 * md.inv_h);
     const bool dbl = sizeof(T) == 8;
     const T* phi = dbl ? (const T*)h->phi : (const T*)h->phi32;
     const T* ug = dbl ? (const T*)h->ugamma : (const T*)h->ugamma32;
@@ -244,11 +249,11 @@ int launch_levelset(evap_mesh* h, int mode, const T* x, T* y, cudaStream_t s) {
             }
             if (done) {
             } else if (mode == EVAP_ADVECT) {
-                k_levelset<T, EVAP_ADVECT, DET><<<grid, threads, 0, s>>>(m, phi, nullptr, ug, x, y, colour);
+                k_levelset<T, EVAP_ADVECT, DET><<<grid, threads, 0, s>>>(m, wm, wd, phi, nullptr, ug, x, y, colour);
             } else if (mode == EVAP_REINIT) {
-                k_levelset<T, EVAP_REINIT, DET><<<grid, threads, 0, s>>>(m, phi, nf, ug, x, y, colour);
+                k_levelset<T, EVAP_REINIT, DET><<<grid, threads, 0, s>>>(m, wm, wd, phi, nf, ug, x, y, colour);
             } else {
-                k_levelset<T, EVAP_REINIT_RHS, DET><<<grid, threads, 0, s>>>(m, phi, nf, ug, x, y, colour);
+                k_levelset<T, EVAP_REINIT_RHS, DET><<<grid, threads, 0, s>>>(m, wm, wd, phi, nf, ug, x, y, colour);
             }
             EVAP_CHECK_LAUNCH("levelset");
         }

@@ -10,7 +10,7 @@ import pytest
 import torch
 
 import workloads
-from oracle import adjoint, momentum
+from oracle import adjoint, fe, levelset, momentum
 from test_gpu_parity import cuda, make_op, rel
 
 pytestmark = pytest.mark.gpu
@@ -77,3 +77,25 @@ def test_mean_errors_of_the_adjoint():
     got = mean_adjoint_errors(2)
     print("mean errors, adjoint:", got)
     assert (got <= 1.02 * np.array([4.702e-15, 8.542e-15, 4.686e-15])).all()
+
+
+def mean_levelset_errors():
+    """Of the FP32 level-set operators: reinitialization, its explicit side, advection."""
+    e = []
+    for k in range(40):
+        n = 3 + k % 6
+        wl = workloads.random_workload(n, 2, 800 + k, geom=("sphere", "deformed", "slab")[k % 3])
+        op, mesh, rng = make_op(wl), fe.Mesh(n, 2, 1.0), np.random.default_rng(k)
+        ug = rng.uniform(-1, 1, 3 * mesh.n_phi)
+        op.set_transport_velocity(cuda(ug))
+        x = rng.uniform(-1, 1, mesh.n_phi).astype(np.float32)
+        e.append([rel(op.apply_levelset(cuda(x), mode=m, prec=32).double(),
+                      levelset.apply(mesh, m, x.astype(np.float64), wl.phi, ug, wl.params))
+                  for m in ("reinit", "reinit_rhs", "advect")])
+    return np.exp(np.log(np.array(e)).mean(0))
+
+
+def test_mean_errors_of_the_fp32_levelset_operators():
+    got = mean_levelset_errors()
+    print("mean errors, FP32 level set:", got)
+    assert (got <= 1.02 * np.array([6.87e-8, 7.05e-8, 8.04e-8])).all()
