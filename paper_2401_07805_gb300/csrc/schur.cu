@@ -113,7 +113,8 @@ __global__ void __launch_bounds__(128) k_schur_assemble(int n, int P, int M, uns
 // on every side (pos), so the 125 products need no bounds tests and a node's loads are in flight together: the
 // coefficients of neighbours outside the lattice, read from a wrapped node's entry, meet a zero.  (With a tested path for
 // the nodes near the boundary, most warps of 32 consecutive nodes took both paths: 53 us per CG iteration at 64^3, now 27.)
-// Entries are indexed with 32 bits (63 N_p < 2^32, checked on the host); in front of S lie schur_guard(n) zeros.
+// Nodes of the padded lattice are numbered with 32 bits ((1024 + 5)^3 at most), entries of S with 64; in front of S lie
+// schur_guard(n) zeros.
 struct SchurStencil {
     static constexpr int SMEM = 0;
     int n;
@@ -186,10 +187,6 @@ int schur_assemble(evap_mesh* h, cudaStream_t s) {
     if (rc) return rc;
     if (h->schur_S && h->schur_stamp == h->diag_stamp) return EVAP_OK;
     const MeshArgs<double>& m = h->m;
-    if (63 * m.Np >= (int64_t)1 << 32) {
-        set_error("Schur stencil: its 63 N_p entries must be indexable with 32 bits");
-        return EVAP_EINVAL;
-    }
     if (!h->schur_S) {  // guard, stencil, the padded lattice of the CG's vector
         const int64_t len = schur_guard(m.n) + 63 * m.Np + schur_padded(m.n);
         EVAP_CUDA(cudaMalloc(&h->schur_S, len * sizeof(float)));
