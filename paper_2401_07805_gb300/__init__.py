@@ -138,13 +138,20 @@ def _check(rc: int, where: str, allow=()):
 
 
 # A small apply (8^3 cells, 11 us on the GPU) is bound by the host's work per call, so pointers and the stream are passed as
-# plain integers (the argument types convert them) and the stream comes without building a Stream object.
+# plain integers (the argument types convert them) and the stream comes without building a Stream object, by two functions that
+# torch keeps for compiled code; without them (another build of torch) from the public Stream object, about 1 us more.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _ptr(t: torch.Tensor | None):
     return None if t is None else t.data_ptr()
 
 
 def _stream():
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if _raw_stream is None or _current_device is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream  # (initializes CUDA, or says why it cannot be)
+    return _raw_stream(_current_device())
 
 
 def make_params(n: int, L: float = 1.0, **over) -> EvapParams:
