@@ -9,6 +9,8 @@
 // skipped (one cell in eight is not, on four drops at 64^3), delta and rho come from the material-law table: 3156 us at
 // 64^3 Q2 when every cell evaluated its interpolants and the material law, now 270.
 #include <cmath>
+#include <cstring>
+#include <limits>
 
 #include "physics.cuh"
 
@@ -18,7 +20,7 @@ template <int P, int CB>
 __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
     k_surface_tension(MeshArgs<double> m, Basis<double> bas, const int8_t* __restrict__ code,
                       const int32_t* __restrict__ tindex, const double* __restrict__ table,
-                      const double* __restrict__ nf, const double* __restrict__ kappa, double alpha_crho,
+                      const double* __restrict__ nf, const double* __restrict__ kappa, unsigned kappa_hi, double alpha_crho,
                       double* __restrict__ out) {
     constexpr int Q = P + 1, NQ = Q * Q * Q;
     __shared__ double sS[Q][Q];
@@ -30,7 +32,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
     const int n = m.n;
     int cx = 0, cy = 0, cz = 0;
     // delta vanishes in cells without a point of the interface zone: their contribution is zero unless the caller's
-    // factor or fields are not finite there (the factor is tested in its product with the curvature)
+    // factor or fields are not finite there, or the product of factor and curvature may not be (kappa_hi: launch)
     bool active = cell < m.ncell;
     if (active) {
         cx = (int)(cell % n);
@@ -40,7 +42,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1))
         bool need = code[cell] == CELL_TABLE;
         for (int j = t; j < K * K * K && !need; j += NQ) {
             const int64_t node = (ns * cx + j % K) + (int64_t)ml * ((ns * cy + (j / K) % K) + (int64_t)ml * (ns * cz + j / (K * K)));
-            need = !(isfinite(alpha_crho * kappa[node]) && isfinite(nf[node]) && isfinite(nf[m.Nphi + node]) &&
+            need = !(((unsigned)__double2hiint(kappa[node]) & 0x7fffffffu) < kappa_hi && isfinite(nf[node]) && isfinite(nf[m.Nphi + node]) &&
                      isfinite(nf[2 * m.Nphi + node]));
         }
         active = need;
@@ -130,15 +132,25 @@ int launch_surface_tension(evap_mesh* h, const double* nf, const double* kappa, 
     const MeshArgs<double>& m = h->m;
     const double rl = m.rho_l, rg = m.rho_g;
     const double crho = (rg - rl) / (rl * rg * std::log(rg / rl));
+    // high word from which on a curvature is not finite or its product with the factor may overflow; 0, every curvature, for
+    // a factor that is not finite
+    const double fac = std::fabs(alpha * crho);
+    unsigned kappa_hi = 0;
+    if (std::isfinite(fac)) {
+        const double most = fac > 1.0 ? std::numeric_limits<double>::max() / fac : std::numeric_limits<double>::infinity();
+        uint64_t bits;
+        std::memcpy(&bits, &most, sizeof(bits));
+        kappa_hi = (unsigned)(bits >> 32);
+    }
     EVAP_CUDA(cudaMemsetAsync(out, 0, 3 * m.Nu * sizeof(double), s));
     if (m.P == 2) {
         constexpr int CB = 8;
         k_surface_tension<2, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 27, 0, s>>>(m, h->b, h->cell_code, h->table_index, h->table, nf, kappa,
-                                                                                        alpha * crho, out);
+                                                                                        kappa_hi, alpha * crho, out);
     } else {
         constexpr int CB = 4;
         k_surface_tension<3, CB><<<(unsigned)((m.ncell + CB - 1) / CB), CB * 64, 0, s>>>(m, h->b, h->cell_code, h->table_index, h->table, nf, kappa,
-                                                                                        alpha * crho, out);
+                                                                                        kappa_hi, alpha * crho, out);
     }
     EVAP_CHECK_LAUNCH("surface_tension");
     return EVAP_OK;
