@@ -23,14 +23,6 @@ int cuda_fail(const char* what, cudaError_t e) {
     return e == cudaErrorMemoryAllocation ? EVAP_ENOMEM : EVAP_ECUDA;
 }
 
-// 2-point Gauss-Legendre rule on [0, 1] (Q1 level-set operators).
-static void gauss_rule2(double* t, double* w) {
-    constexpr double r = 0.5773502691896257645091488;  // 1 / sqrt 3
-    t[0] = 0.5 * (1.0 - r);
-    t[1] = 0.5 * (1.0 + r);
-    w[0] = w[1] = 0.5;
-}
-
 template <int P>
 static void copy_ct_basis(Basis<double>& b) {
     constexpr CtBasis<P> c = make_ct_basis<P>();
@@ -56,7 +48,6 @@ void host_basis(int P, Basis<double>& b, int nsub) {
         copy_ct_basis<2>(b);
     else
         copy_ct_basis<3>(b);
-    gauss_rule2(b.g2t, b.g2w);
     for (int q = 0; q < b.Q; ++q) {  // level-set hats of the n_sub times subdivided interval
         const double s = nsub * b.t[q];
         const int k = std::min(std::max((int)std::floor(s), 0), nsub - 1);
@@ -88,10 +79,6 @@ Basis<T> cast_basis(const Basis<double>& b) {
             o.NL[i][j] = (T)b.NL[i][j];
             o.DL[i][j] = (T)b.DL[i][j];
         }
-    }
-    for (int i = 0; i < 2; ++i) {
-        o.g2t[i] = (T)b.g2t[i];
-        o.g2w[i] = (T)b.g2w[i];
     }
     return o;
 }

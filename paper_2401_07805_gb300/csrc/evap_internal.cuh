@@ -24,7 +24,6 @@ struct Basis {
     T w[MAXQ];         // Gauss weights on [0, 1]
     T t[MAXQ];         // Gauss points on [0, 1]
     T N1[MAXQ][2];     // Q1 shape values (1 - t_q, t_q) (pressure space)
-    T g2t[2], g2w[2];  // 2-point Gauss rule of the Q1 operators
     // level-set space on one velocity cell (Q1 on the n_sub sub-intervals per direction, Sec. 2.5): the n_sub + 1
     // piecewise-linear hats at the Gauss points, NL[q][a], and their reference derivatives DL[q][a] (d/dt; divide by
     // h for physical units); a Gauss point on a sub-interval boundary takes the upper sub-interval's slopes
@@ -48,16 +47,9 @@ struct MeshArgs {
 
 enum CellCode : int8_t { CELL_GAS = 0, CELL_LIQUID = 1, CELL_TABLE = 2 };
 constexpr int TAB_K = 7;  // table entries per quadrature point: rho, mu, z n_x, z n_y, z n_z, v_dil, delta
+constexpr int TAB32_K = 6;  // of which the FP32 copy holds the first
 constexpr int QC_K = 19;  // cached momentum coefficients per quadrature point (see k_qp_coeffs)
 constexpr int QC32_K = 12;  // of which the u0 terms, in FP32 for the FP32 apply (slots 1..12)
-
-template <typename T>
-struct Coeffs {            // quadrature-point coefficients of the momentum operator
-    const int8_t* cell_code;
-    const int32_t* table_index;
-    const T* table;        // [ntable][TAB_K][nq]
-    const T* u0;           // [3 N_u]
-};
 
 // Deterministic accumulation (evap_set_deterministic): the cells are taken in 8 passes, one per parity class
 // colour = px + 2 py + 4 pz (cx = px, cy = py, cz = pz mod 2).  Two cells of one class differ by at least 2 in some
@@ -329,7 +321,6 @@ int solve_saddle(evap_mesh* h, const double* f, double* x, double* p, int restar
 template <typename T>
 int launch_fill(T* p, int64_t n, T v, cudaStream_t s);
 int launch_to_float(const double* a, float* b, int64_t n, cudaStream_t s);
-int launch_to_double(const float* a, double* b, int64_t n, cudaStream_t s);
 
 inline int blocks_for(int64_t n, int threads, int64_t cap = 152 * 64) {
     int64_t b = (n + threads - 1) / threads;

@@ -136,11 +136,10 @@ __device__ __forceinline__ void grid_sum_df(const float2* part, float2* sh, dfl 
 // mirrored interior rows, and the operator is a sum of their tensor products.  So the neighbours of one kind are added
 // first: 23 additions and 4 multiplications per node.
 struct HelmholtzStencil {
-    static constexpr int SMEM = 0, MIN_BLOCKS = 0;
+    static constexpr int MIN_BLOCKS = 0;
     int n;
     dfl c[4];
-    __device__ __forceinline__ void load(float2*) const {}
-    __device__ __forceinline__ dfl row(int64_t node, const float2* x, const float2*) const {
+    __device__ __forceinline__ dfl row(int64_t node, const float2* x) const {
         const unsigned m1 = (unsigned)n + 1u, nd = (unsigned)node;
         const unsigned t = nd / m1, i = nd - t * m1, k = t / m1, j = t - k * m1;
         const int sy = (int)m1, sz = (int)(m1 * m1);
@@ -176,7 +175,7 @@ struct HelmholtzStencil {
     }
     // the diagonal entry to FP32, for the Jacobi scaling (n = 1 adds the mirrored neighbours to it, but any positive
     // diagonal is a valid preconditioner)
-    __device__ __forceinline__ float diag(int64_t node, const float2*) const {
+    __device__ __forceinline__ float diag(int64_t node) const {
         const unsigned m1 = (unsigned)n + 1u, nd = (unsigned)node;
         const unsigned t = nd / m1, i = nd - t * m1, k = t / m1, j = t - k * m1;
         return c[0].hi * scale(i, j, k);
@@ -200,12 +199,11 @@ inline HelmholtzStencil helmholtz_op(int n, double h, double c) {
 // the lattice.  Those products are formed all the same, with whatever the vector's memory holds there: it has
 // stencil_guard(n) zero entries in front, and every entry read is finite.
 struct NodeStencil {
-    static constexpr int SMEM = 0, MIN_BLOCKS = 1;  // (registers for all 54 loads of a row: without it 64 and 1.07 to 1.2 times the time)
+    static constexpr int MIN_BLOCKS = 1;  // (registers for all 54 loads of a row: without it 64 and 1.07 to 1.2 times the time)
     int n;
     int64_t N;
     const float2* C;
-    __device__ __forceinline__ void load(float2*) const {}
-    __device__ __forceinline__ dfl row(int64_t node, const float2* x, const float2*) const {
+    __device__ __forceinline__ dfl row(int64_t node, const float2* x) const {
         const unsigned m1 = (unsigned)n + 1u;
         const float2* c = C + node;
         const float2* p = x + node;
@@ -226,7 +224,7 @@ struct NodeStencil {
             }
         return df_norm(acc);
     }
-    __device__ __forceinline__ float diag(int64_t node, const float2*) const { return C[13 * N + node].x; }
+    __device__ __forceinline__ float diag(int64_t node) const { return C[13 * N + node].x; }
 };
 // entries a row may read before the first or after the last of its vector
 inline int64_t stencil_guard(int n) { return (int64_t)(n + 1) * (n + 1) + (n + 1) + 1; }
@@ -280,19 +278,16 @@ __global__ void __launch_bounds__(FK_THREADS, Op::MIN_BLOCKS) k_cg_fused(Op op, 
                                                          float* dinv, float2* r, float2* u, float2* p, float2* sv,
                                                          float2* w, double rtol, double atol, int max_iter,
                                                          float2* part, GridBarrier* gb, double* out) {
-    extern __shared__ float2 op_sm[];  // Op::SMEM pairs staged by op.load
     __shared__ float2 sh[3 * FK_WARPS + 3];
     __shared__ double s_r0;
     __shared__ dfl s_alpha, s_beta;
     __shared__ int s_go;
     unsigned long long bar = 0;
     const int64_t i0 = blockIdx.x * (int64_t)FK_THREADS + threadIdx.x, stride = (int64_t)gridDim.x * FK_THREADS;
-    op.load(op_sm);
-    __syncthreads();
     const dfl zero{0.f, 0.f};
     for (int64_t i = i0; i < N; i += stride) {
         const dfl ri = df_from_double(b[i]);
-        const float di = 1.0f / op.diag(i, op_sm);
+        const float di = 1.0f / op.diag(i);
         st_df(xd + i, zero);
         st_df(r + i, ri);
         st_df(u + i, df_norm(dfl{ri.hi * di, __fmaf_rn(ri.hi, di, -ri.hi * di) + ri.lo * di}));
@@ -307,7 +302,7 @@ __global__ void __launch_bounds__(FK_THREADS, Op::MIN_BLOCKS) k_cg_fused(Op op, 
     for (;;) {
         dfl acc[3] = {zero, zero, zero};  // (r, u), (w, u), (r, r)
         for (int64_t i = i0; i < N; i += stride) {
-            const dfl wi = op.row(i, u, op_sm), ui = ld_df(u + i), ri = ld_df(r + i);
+            const dfl wi = op.row(i, u), ui = ld_df(u + i), ri = ld_df(r + i);
             st_df(w + i, wi);
             df_fma(acc[0], ri, ui);
             df_fma(acc[1], wi, ui);
@@ -382,7 +377,6 @@ __global__ void __launch_bounds__(FK_THREADS) k_gmres_fused(Op op, int64_t N, in
                                                             float* dinv, float2* z, float2* V, double rtol, double atol,
                                                             int max_iter, double reorth, float2* part, GridBarrier* gb,
                                                             double* out) {
-    extern __shared__ float2 op_sm[];
     __shared__ float2 sh[(GM_MAX + 2) * FK_WARPS];
     __shared__ dfl s_h[GM_MAX + 2];
     __shared__ double H[(GM_MAX + 1) * GM_MAX], cs[GM_MAX], sn[GM_MAX], g[GM_MAX + 1];
@@ -393,8 +387,6 @@ __global__ void __launch_bounds__(FK_THREADS) k_gmres_fused(Op op, int64_t N, in
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t i0 = blockIdx.x * (int64_t)FK_THREADS + threadIdx.x, stride = (int64_t)gridDim.x * FK_THREADS;
     const dfl zero{0.f, 0.f};
-    op.load(op_sm);
-    __syncthreads();
     // per-warp sums of K values (sh[k FK_WARPS + warp]) written as block partials part[k G + b]: warp q reduces values
     // q, q + FK_WARPS, ... by a shuffle tree
     auto partials = [&](int K) {
@@ -434,7 +426,7 @@ __global__ void __launch_bounds__(FK_THREADS) k_gmres_fused(Op op, int64_t N, in
     {
         dfl bb = zero;
         for (int64_t i = i0; i < N; i += stride) {
-            dinv[i] = 1.0f / op.diag(i, op_sm);
+            dinv[i] = 1.0f / op.diag(i);
             st_df(xd + i, df_from_double(x[i]));
             st_df(z + i, zero);  // (read behind xd with zero coefficients before it is written)
             const dfl bi = df_from_double(b[i]);
@@ -455,7 +447,7 @@ __global__ void __launch_bounds__(FK_THREADS) k_gmres_fused(Op op, int64_t N, in
         {
             dfl rr = zero;
             for (int64_t i = i0; i < N; i += stride) {
-                const dfl ri = df_sub(df_from_double(b[i]), op.row(i, xd, op_sm));
+                const dfl ri = df_sub(df_from_double(b[i]), op.row(i, xd));
                 st_df(V + i, ri);
                 df_fma(rr, ri, ri);
             }
@@ -489,7 +481,7 @@ __global__ void __launch_bounds__(FK_THREADS) k_gmres_fused(Op op, int64_t N, in
         int j = 0;
         for (; j < m; ++j) {
             float2* W = V + (int64_t)(j + 1) * N;
-            for (int64_t i = i0; i < N; i += stride) st_df(W + i, op.row(i, z, op_sm));
+            for (int64_t i = i0; i < N; i += stride) st_df(W + i, op.row(i, z));
             ++used;
             dots(W, j + 1, true);  // h_k = (w, v_k), k <= j, and |w|^2 at index j + 1
             if (!grid_barrier(gb, bar)) return;
@@ -626,7 +618,6 @@ __global__ void __launch_bounds__(FK_THREADS) k_cg_fused32(Op op, int64_t N, con
                                                            float* xs, float* dinv, float* r, float* u, float* p,
                                                            float* sv, float* w, double rtol, double atol, int max_iter,
                                                            float* part, GridBarrier* gb, double* out) {
-    extern __shared__ float op_sm32[];
     __shared__ float sh[3 * FK_WARPS];
     __shared__ double s_r0;
     __shared__ float s_alpha, s_beta;
@@ -634,10 +625,8 @@ __global__ void __launch_bounds__(FK_THREADS) k_cg_fused32(Op op, int64_t N, con
     unsigned long long bar = 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t i0 = blockIdx.x * (int64_t)FK_THREADS + threadIdx.x, stride = (int64_t)gridDim.x * FK_THREADS;
-    op.load(op_sm32);
-    __syncthreads();
     for (int64_t i = i0; i < N; i += stride) {
-        const float ri = (float)b[i], di = 1.0f / op.diag(i, op_sm32);
+        const float ri = (float)b[i], di = 1.0f / op.diag(i);
         xs[i] = 0.f;
         r[i] = ri;
         u[op.pos(i)] = ri * di;
@@ -652,7 +641,7 @@ __global__ void __launch_bounds__(FK_THREADS) k_cg_fused32(Op op, int64_t N, con
     for (;;) {
         float acc[3] = {0.f, 0.f, 0.f};  // (r, u), (w, u), (r, r)
         for (int64_t i = i0; i < N; i += stride) {
-            const float wi = op.row(i, u, op_sm32), ui = u[op.pos(i)], ri = r[i];
+            const float wi = op.row(i, u), ui = u[op.pos(i)], ri = r[i];
             w[i] = wi;
             acc[0] = fmaf(ri, ui, acc[0]);
             acc[1] = fmaf(wi, ui, acc[1]);
@@ -735,11 +724,11 @@ int fused_result(evap_mesh* h, const FusedSpace& f, cudaStream_t s, double res[3
 // at 24^3 with 152 blocks).  The kernels' registers leave one block per SM; capped to two, a CG iteration took 1.03 to 1.9
 // times as long.
 template <class K>
-inline int fused_grid(K kernel, size_t smem, int cap, int64_t N, int& G) {
+inline int fused_grid(K kernel, int cap, int64_t N, int& G) {
     int dev = 0, sms = 0, per_sm = 0;
     EVAP_CUDA(cudaGetDevice(&dev));
     EVAP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    EVAP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, FK_THREADS, smem));
+    EVAP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, FK_THREADS, 0));
     G = per_sm < 2 ? per_sm * sms : 2 * sms;
     if (G > cap) G = cap;
     if (G < 1) {

@@ -349,8 +349,7 @@ static int cg_solve_fused(evap_mesh* h, Op op, const double* b, double* x, doubl
     FusedSpace f;
     int rc = fused_space(h, 6, f, s), G = 0;
     if (rc) return rc;
-    const size_t smem = Op::SMEM * sizeof(float2);
-    if ((rc = fused_grid(k_cg_fused<Op>, smem, FK_MAX_BLOCKS, N, G))) return rc;
+    if ((rc = fused_grid(k_cg_fused<Op>, FK_MAX_BLOCKS, N, G))) return rc;
     EVAP_CUDA(cudaMemsetAsync(f.gb, 0, sizeof(GridBarrier), s));
     double* xx = x;
     float2 *xd = f.vec, *r = f.vec + N, *u = f.vec + 2 * N, *p = f.vec + 3 * N, *sv = f.vec + 4 * N, *w = f.vec + 5 * N;
@@ -359,7 +358,7 @@ static int cg_solve_fused(evap_mesh* h, Op op, const double* b, double* x, doubl
     GridBarrier* gb = f.gb;
     double* out = f.out;
     void* args[] = {&op, &N, &b, &xx, &xd, &dinv, &r, &u, &p, &sv, &w, &rtol, &atol, &max_iter, &part, &gb, &out};
-    EVAP_CUDA(cudaLaunchCooperativeKernel((const void*)k_cg_fused<Op>, dim3(G), dim3(FK_THREADS), args, smem, s));
+    EVAP_CUDA(cudaLaunchCooperativeKernel((const void*)k_cg_fused<Op>, dim3(G), dim3(FK_THREADS), args, 0, s));
     EVAP_CHECK_LAUNCH("cg_fused");
     double res[3];
     if ((rc = fused_result(h, f, s, res))) return rc;
@@ -381,8 +380,7 @@ static int gmres_solve_fused(evap_mesh* h, Op op, int m, const double* b, double
     FusedSpace f;
     int rc = fused_space(h, m + 3, f, s), G = 0;
     if (rc) return rc;
-    const size_t smem = Op::SMEM * sizeof(float2);
-    if ((rc = fused_grid(k_gmres_fused<Op>, smem, FK_MAX_BLOCKS, N, G))) return rc;
+    if ((rc = fused_grid(k_gmres_fused<Op>, FK_MAX_BLOCKS, N, G))) return rc;
     EVAP_CUDA(cudaMemsetAsync(f.gb, 0, sizeof(GridBarrier), s));
     double* xx = x;
     float2 *xd = f.vec, *z = f.vec + N, *V = f.vec + 2 * N;
@@ -391,7 +389,7 @@ static int gmres_solve_fused(evap_mesh* h, Op op, int m, const double* b, double
     GridBarrier* gb = f.gb;
     double* out = f.out;
     void* args[] = {&op, &N, &m, &b, &xx, &xd, &dinv, &z, &V, &rtol, &atol, &max_iter, &reorth, &part, &gb, &out};
-    EVAP_CUDA(cudaLaunchCooperativeKernel((const void*)k_gmres_fused<Op>, dim3(G), dim3(FK_THREADS), args, smem, s));
+    EVAP_CUDA(cudaLaunchCooperativeKernel((const void*)k_gmres_fused<Op>, dim3(G), dim3(FK_THREADS), args, 0, s));
     EVAP_CHECK_LAUNCH("gmres_fused");
     double res[3];
     if ((rc = fused_result(h, f, s, res))) return rc;

@@ -10,7 +10,7 @@
 // version), sum-factorized (k_levelset_advect_sf); the reinitialization operators stay in FP64.
 #include <type_traits>
 
-#include "dfloat.cuh"
+#include "df_lines.cuh"
 #include "q1_points.cuh"
 
 namespace evap {
@@ -86,8 +86,6 @@ __global__ void __launch_bounds__(128) k_levelset(MeshArgs<T> m, T wm, T wd, con
 // the testing with the shape functions as three 1D sweeps of the 2 x 2 matrix N[q][j] (N_0 = 1 - t, N_1 = t at the
 // Gauss points t), the reference gradient of x as differences along its own direction interpolated along the other
 // two: 132 two-term double-float dot products per cell in place of the direct sums' 8 x 7 eight-term ones.
-constexpr float dfc_hi(double v) { return (float)v; }
-constexpr float dfc_lo(double v) { return (float)(v - (double)(float)v); }
 __device__ __forceinline__ dfl dot2(dfl c0, dfl v0, dfl c1, dfl v1) {
     dfl s = df_prod(c0, v0);
     df_fma(s, c1, v1);
@@ -107,8 +105,7 @@ __global__ void __launch_bounds__(128) k_levelset_advect_sf(MeshArgs<double> m, 
     }
     constexpr double t0 = g2_point(0), t1 = g2_point(1);
     // N[q][j]: shape function j (0: 1 - t, 1: t) at Gauss point q
-    const dfl N[2][2] = {{{dfc_hi(1.0 - t0), dfc_lo(1.0 - t0)}, {dfc_hi(t0), dfc_lo(t0)}},
-                         {{dfc_hi(1.0 - t1), dfc_lo(1.0 - t1)}, {dfc_hi(t1), dfc_lo(t1)}}};
+    const dfl N[2][2] = {{EVAP_DFK(1.0 - t0), EVAP_DFK(t0)}, {EVAP_DFK(1.0 - t1), EVAP_DFK(t1)}};
     const int n = m.n;
     const int64_t m1 = n + 1;
     int64_t node[8];  // j = ja + 2 jb + 4 jc
@@ -237,19 +234,15 @@ int launch_levelset(evap_mesh* h, int mode, const T* x, T* y, cudaStream_t s) {
             const int64_t cells = colour_cells(m.n, colour);
             if (cells == 0) continue;
             const unsigned grid = (unsigned)((cells + threads - 1) / threads);
-            bool done = false;
-            if constexpr (sizeof(T) == 8) {
-                if (mode == EVAP_ADVECT) {  // FP64-accurate advection in double-float arithmetic
+            if (mode == EVAP_ADVECT) {
+                if constexpr (sizeof(T) == 8) {  // FP64-accurate advection in double-float arithmetic
                     const dfl W = df_from_double(0.125 * (double)m.vol_w);  // 2-point Gauss weights 1/2 per direction
                     const dfl thdt_ih = df_from_double((double)m.theta * (double)m.dt * (double)m.inv_h);
                     k_levelset_advect_sf<DET><<<grid, threads, 0, s>>>(m, W, thdt_ih, (const float2*)h->ugammadf,
                                                                        (const double*)x, (double*)y, colour);
-                    done = true;
+                } else {
+                    k_levelset<T, EVAP_ADVECT, DET><<<grid, threads, 0, s>>>(m, wm, wd, phi, nullptr, ug, x, y, colour);
                 }
-            }
-            if (done) {
-            } else if (mode == EVAP_ADVECT) {
-                k_levelset<T, EVAP_ADVECT, DET><<<grid, threads, 0, s>>>(m, wm, wd, phi, nullptr, ug, x, y, colour);
             } else if (mode == EVAP_REINIT) {
                 k_levelset<T, EVAP_REINIT, DET><<<grid, threads, 0, s>>>(m, wm, wd, phi, nf, ug, x, y, colour);
             } else {

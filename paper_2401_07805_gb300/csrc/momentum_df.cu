@@ -66,9 +66,15 @@ __device__ __forceinline__ constexpr int t_slot(int k, int l) {
 #define EVAP_DF_MINB3 4
 #endif
 
+// The pressure space at the 1D Gauss points: shape values as pairs, and the points in FP64.
+struct Q1Basis {
+    dfl N1[MAXQ][2];
+    double t[MAXQ];
+};
+
 template <int P, int CB, bool PRES, int MINB, bool DET>
 __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
-    k_momentum_df(MeshArgs<double> m, DfBasis bas, const float2* __restrict__ qc, const double* __restrict__ x,
+    k_momentum_df(MeshArgs<double> m, const __grid_constant__ Q1Basis bas, const float2* __restrict__ qc, const double* __restrict__ x,
                   double* __restrict__ y, double* __restrict__ yp, const double* __restrict__ pin, int colour) {
     constexpr int Q = P + 1, NQ = Q * Q * Q, NL = Q * Q, TASKS = 3 * NL;
     using Ln = DfLine<Q>;
@@ -301,25 +307,15 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
     }
 }
 
-DfBasis make_df_basis(const Basis<double>& b, double inv_h) {
-    DfBasis d{};
-    for (int q = 0; q < b.Q; ++q) {
-        for (int k = 0; k < b.Q; ++k) {
-            d.S[q][k] = df_from_double(b.S[q][k]);
-            d.Dc[q][k] = df_from_double(b.Dc[q][k] * inv_h);
-        }
-        d.N1[q][0] = df_from_double(b.N1[q][0]);
-        d.N1[q][1] = df_from_double(b.N1[q][1]);
-        d.t[q] = b.t[q];
-    }
-    return d;
-}
-
 // y = A x (+ y_p = B x - g, + the pressure term when p is given); the init kernel has written y = x on the Dirichlet
 // DoFs (faces of m) and zeros elsewhere.
 int launch_momentum_df(evap_mesh* h, const MeshArgs<double>& m, const double* x, double* y, double* yp,
                        const double* p, cudaStream_t s) {
-    const DfBasis b = make_df_basis(h->b, m.inv_h);
+    Q1Basis b{};
+    for (int q = 0; q < h->b.Q; ++q) {
+        b.t[q] = h->b.t[q];
+        for (int j = 0; j < 2; ++j) b.N1[q][j] = df_from_double(h->b.N1[q][j]);
+    }
     const float2* qc = reinterpret_cast<const float2*>(h->qcdf);
     const int c0 = h->deterministic ? 0 : -1, c1 = h->deterministic ? 8 : 0;  // colour passes, or one atomic pass
     // at most 48 KB of shared memory per block, so no launch needs a function attribute

@@ -65,7 +65,7 @@ constexpr double NODAL_NORMAL_TINY = 1e-4;
 // printed Eq. (evaporDil) has the bracket reversed with respect to the paper's 1D solution (App. A,
 // Eq. stefan_diffuse_velocity: div u = mdot (1/rho_g - 1/rho_l) delta) and to the c_1 of the variant-1 derivation;
 // the latter is taken, so evaporation (mdot > 0, rho_g < rho_l) expands the volume.
-__device__ __forceinline__ double dilation_coefficient(const MeshArgs<double>& m) {
+inline double dilation_coefficient(const MeshArgs<double>& m) {
     return 1.0 / m.rho_g - 1.0 / m.rho_l;
 }
 
@@ -120,6 +120,27 @@ __device__ __forceinline__ void ls_at(const double* __restrict__ f, const MeshAr
 // Whether the corrected-strain term is active at a point (Sec. 2.4.2; zone gate or everywhere).
 __device__ __forceinline__ bool correction_on(const MeshArgs<double>& m, bool zone) {
     return m.stress != 0 && (m.corr_zone != 0 || zone);
+}
+
+// 1D integrals of a Q1 pressure shape function N1_j and a velocity shape function l_k on a cell, exact with the velocity Gauss
+// rule: a[j][k] = h sum_q w_q N1_j l_k, g[j][k] = sum_q w_q N1_j l_k' (their products are the divergence row B).
+struct CouplingTables {
+    float a[2][MAXQ], g[2][MAXQ];
+};
+inline CouplingTables coupling_tables(const evap_mesh* h) {
+    const Basis<double>& b = h->b;
+    CouplingTables t{};
+    for (int j = 0; j < 2; ++j)
+        for (int k = 0; k <= h->m.P; ++k) {
+            double sa = 0.0, sg = 0.0;
+            for (int q = 0; q < b.Q; ++q) {
+                sa += b.w[q] * b.N1[q][j] * b.S[q][k];
+                sg += b.w[q] * b.N1[q][j] * b.D[q][k];
+            }
+            t.a[j][k] = (float)(h->m.h * sa);
+            t.g[j][k] = (float)sg;
+        }
+    return t;
 }
 
 }  // namespace evap

@@ -36,10 +36,7 @@ __device__ __forceinline__ int gradient_row(const float (&a1)[2][MAXQ], const fl
     }
     return e - 1;
 }
-struct GradientTables {
-    float a[2][MAXQ], g[2][MAXQ];  // a[j][b] = h sum_q w_q N1_j l_b, g[j][b] = sum_q w_q N1_j l_b'
-};
-__global__ void __launch_bounds__(128) k_add_gradient(int n, int P, int M, int64_t Nu, unsigned faces, GradientTables tab,
+__global__ void __launch_bounds__(128) k_add_gradient(int n, int P, int M, int64_t Nu, unsigned faces, CouplingTables tab,
                                                       const float* __restrict__ p, const double* __restrict__ v,
                                                       double* __restrict__ t) {
     const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.y, z = blockIdx.z;
@@ -214,18 +211,7 @@ __global__ void k_add_vec(double* __restrict__ y, const double* __restrict__ g, 
 
 int launch_add_gradient(evap_mesh* h, const float* p, const double* v, double* t, cudaStream_t st) {
     const MeshArgs<double>& m = h->m;
-    const Basis<double>& b = h->b;
-    GradientTables tab{};
-    for (int j = 0; j < 2; ++j)
-        for (int k = 0; k <= m.P; ++k) {
-            double sa = 0.0, sg = 0.0;
-            for (int q = 0; q < b.Q; ++q) {
-                sa += b.w[q] * b.N1[q][j] * b.S[q][k];
-                sg += b.w[q] * b.N1[q][j] * b.D[q][k];
-            }
-            tab.a[j][k] = (float)(m.h * sa);
-            tab.g[j][k] = (float)sg;
-        }
+    const CouplingTables tab = coupling_tables(h);
     const dim3 grid((unsigned)((m.M + 31) / 32), (unsigned)((m.M + 3) / 4), (unsigned)m.M);
     k_add_gradient<<<grid, dim3(32, 4), 0, st>>>(m.n, m.P, m.M, m.Nu, m.faces, tab, p, v, t);
     EVAP_CHECK_LAUNCH("add_gradient");

@@ -15,17 +15,11 @@
 // With the stencil, the Schur CG of every preconditioner application is one cooperative launch in FP32
 // (k_cg_fused32) instead of, per iteration, a matrix-free gradient and divergence over the whole velocity mesh.
 #include <algorithm>
-#include <cstring>
 
 #include "fused_krylov.cuh"
 #include "physics.cuh"
 
 namespace evap {
-
-struct SchurTables {
-    float a[2][MAXQ];  // a[a][b] = h sum_q w_q N1_a(t_q) l_b(t_q)
-    float g[2][MAXQ];  // g[a][b] =   sum_q w_q N1_a(t_q) l_b'(t_q)
-};
 
 // 1D assembled factor of pressure node I (0..n) and velocity node V (0..P n): the cells e in {I - 1, I} that hold both
 __device__ __forceinline__ float factor1(const float (&t)[2][MAXQ], int P, int n, int I, int V) {
@@ -47,7 +41,7 @@ __device__ __forceinline__ float factor1(const float (&t)[2][MAXQ], int P, int n
 // 64^3 Q2, solutions to 1e-8 moved by several times what two runs differ by).  Measured at 64^3 Q2: 2139 us with the
 // factors in local memory, now 1864.
 __global__ void __launch_bounds__(128) k_schur_assemble(int n, int P, int M, unsigned faces, int64_t Nu, int64_t Np,
-                                                        SchurTables tab, const float* __restrict__ diag,
+                                                        CouplingTables tab, const float* __restrict__ diag,
                                                         float* __restrict__ S) {
     __shared__ float w[3][3][3][2 * MAXQ - 1][2];
     const int e = blockIdx.y, lin = 62 + e;
@@ -116,17 +110,15 @@ __global__ void __launch_bounds__(128) k_schur_assemble(int n, int P, int M, uns
 // Nodes of the padded lattice are numbered with 32 bits ((1024 + 5)^3 at most), entries of S with 64; in front of S lie
 // schur_guard(n) zeros.
 struct SchurStencil {
-    static constexpr int SMEM = 0;
     int n;
     int64_t Np;
     const float* S;
-    __device__ __forceinline__ void load(float*) const {}
     __device__ __forceinline__ unsigned pos(int64_t node) const {
         const unsigned m1 = (unsigned)n + 1u, mp = m1 + 4u, nd = (unsigned)node;
         const unsigned t = nd / m1, i = nd - t * m1, k = t / m1, j = t - k * m1;
         return (i + 2u) + mp * ((j + 2u) + mp * (k + 2u));
     }
-    __device__ __forceinline__ float row(int64_t node, const float* x, const float*) const {
+    __device__ __forceinline__ float row(int64_t node, const float* x) const {
         const int m1 = n + 1, m2 = m1 * m1, mp = m1 + 4;
         const float* p = x + pos(node);
         const float* c = S + node;
@@ -147,7 +139,7 @@ struct SchurStencil {
             }
         return acc;
     }
-    __device__ __forceinline__ float diag(int64_t node, const float*) const { return S[node]; }
+    __device__ __forceinline__ float diag(int64_t node) const { return S[node]; }
 };
 inline int64_t schur_guard(int n) { return 2 * ((int64_t)(n + 1) * (n + 1) + (n + 1) + 1); }
 inline int64_t schur_padded(int n) { return (int64_t)(n + 5) * (n + 5) * (n + 5); }
@@ -192,19 +184,7 @@ int schur_assemble(evap_mesh* h, cudaStream_t s) {
         EVAP_CUDA(cudaMalloc(&h->schur_S, len * sizeof(float)));
         EVAP_CUDA(cudaMemsetAsync(h->schur_S, 0, len * sizeof(float), s));
     }
-    SchurTables tab;
-    std::memset(&tab, 0, sizeof(tab));
-    const Basis<double>& b = h->b;
-    for (int a = 0; a < 2; ++a)
-        for (int v = 0; v <= m.P; ++v) {
-            double sa = 0.0, sg = 0.0;
-            for (int q = 0; q < b.Q; ++q) {
-                sa += b.w[q] * b.N1[q][a] * b.S[q][v];
-                sg += b.w[q] * b.N1[q][a] * b.D[q][v];
-            }
-            tab.a[a][v] = (float)(m.h * sa);
-            tab.g[a][v] = (float)sg;
-        }
+    const CouplingTables tab = coupling_tables(h);
     k_schur_assemble<<<dim3((unsigned)((m.Np + 127) / 128), 63), 128, 0, s>>>(m.n, m.P, m.M, m.faces, m.Nu, m.Np, tab,
                                                                            h->diag32, h->schur_S + schur_guard(m.n));
     EVAP_CHECK_LAUNCH("schur_assemble");
@@ -230,7 +210,7 @@ int schur_solve(evap_mesh* h, const double* r, double* z, double rtol, int max_i
     FusedSpace f;
     if ((rc = fused_space(h, 3, f, s))) return rc;  // 3 pair vectors = 6 float vectors of N_phi >= N_p entries
     int G = 0;
-    if ((rc = fused_grid(k_cg_fused32<SchurStencil>, 0, FK_MAX_BLOCKS, N, G))) return rc;
+    if ((rc = fused_grid(k_cg_fused32<SchurStencil>, FK_MAX_BLOCKS, N, G))) return rc;
     EVAP_CUDA(cudaMemsetAsync(f.gb, 0, sizeof(GridBarrier), s));
     SchurStencil op{h->m.n, N, h->schur_S + schur_guard(h->m.n)};
     const int64_t Nl = ls_args<double>(h).Nphi;  // the vectors' stride: fused_space sizes them for N_phi

@@ -33,11 +33,6 @@ int launch_to_float(const double* a, float* b, int64_t n, cudaStream_t s) {
     return EVAP_OK;
 }
 
-__global__ void k_to_double(const float* __restrict__ a, double* __restrict__ b, int64_t n) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        b[i] = (double)a[i];
-}
-
 // b = (float)a and c = (hi, lo) of a
 __global__ void k_to_float_df(const double* __restrict__ a, float* __restrict__ b, float2* __restrict__ c, int64_t n) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -52,12 +47,6 @@ int refresh_ugamma_copies(evap_mesh* h, cudaStream_t s) {
     const int64_t n = 3 * h->m.Nphi;
     k_to_float_df<<<blocks_for(n, 256), 256, 0, s>>>(h->ugamma, h->ugamma32, (float2*)h->ugammadf, n);
     EVAP_CHECK_LAUNCH("ugamma_copies");
-    return EVAP_OK;
-}
-
-int launch_to_double(const float* a, double* b, int64_t n, cudaStream_t s) {
-    k_to_double<<<blocks_for(n, 256), 256, 0, s>>>(a, b, n);
-    EVAP_CHECK_LAUNCH("to_double");
     return EVAP_OK;
 }
 
@@ -117,7 +106,7 @@ __global__ void k_classify(MeshArgs<double> m, Basis<double> b, const double* __
 }
 
 // Table entries at one quadrature point of a table cell: rho, mu, z n (z = correction gate), v_dil (Eq. evaporDil
-// with the sign of App. A, dilation_coefficient), delta.
+// with the sign of App. A), delta.
 //
 // The FP64 pipe bounds it: one location and one set of weights for phi, its gradient and mdot, the logarithm, sine and
 // cosine shared by the table and the adjoint's factors, one reciprocal for the normal.  The density jump multiplies the
@@ -193,15 +182,15 @@ __global__ void k_fill_table(MeshArgs<double> m, Basis<double> b, const double* 
     const bool dir = gn * m.h > GRAD_TINY;
     const double ign = dir ? 1.0 / gn : 0.0;
     const double nv[3] = {dir ? g[0] * ign : 0.0, dir ? g[1] * ign : 0.0, dir ? g[2] * ign : 0.0};
-    const double z = correction_on(m, zone) ? 1.0 : 0.0, kdil = irg - irl;  // dilation_coefficient
+    const double z = correction_on(m, zone) ? 1.0 : 0.0, kdil = irg - irl;  // c_1
     const double delta = zone ? dHdd * gn : 0.0;
     const double vals[TAB_K] = {rho, mu, z * nv[0], z * nv[1], z * nv[2], md * kdil * delta, delta};
     const int64_t tb = (int64_t)tindex[cell] * TAB_K * nq + q;
 #pragma unroll
-    for (int k = 0; k < TAB_K; ++k) {
-        table[tb + (int64_t)k * nq] = vals[k];
-        table32[tb + (int64_t)k * nq] = (float)vals[k];
-    }
+    for (int k = 0; k < TAB_K; ++k) table[tb + (int64_t)k * nq] = vals[k];
+    const int64_t tb32 = (int64_t)tindex[cell] * TAB32_K * nq + q;
+#pragma unroll
+    for (int k = 0; k < TAB32_K; ++k) table32[tb32 + (int64_t)k * nq] = (float)vals[k];
     // (the adjoint's weight is kappa W: kdmu = kappa (mu_l - mu_g), kdk = kdil / kappa)
     double av[ADJ_K];
     av[ADJ_CRHO] = -rho * rho * (irl - irg) * dHdd;
@@ -247,13 +236,13 @@ int launch_setup_coefficients(evap_mesh* h, cudaStream_t s) {
         h->table_cap = 0;
         const int64_t cap = count + count / 8 + 16;
         EVAP_CUDA(cudaMalloc(&h->table, cap * TAB_K * nq * sizeof(double)));
-        EVAP_CUDA(cudaMalloc(&h->table32, cap * TAB_K * nq * sizeof(float)));
+        EVAP_CUDA(cudaMalloc(&h->table32, cap * TAB32_K * nq * sizeof(float)));
         EVAP_CUDA(cudaMalloc(&h->adj_table, cap * ADJ_K * nq * sizeof(float2)));
         h->table_cap = cap;
     }
     if (count > 0) {
         const int64_t total = m.ncell * nq;
-        const double kdil = 1.0 / m.rho_g - 1.0 / m.rho_l;
+        const double kdil = dilation_coefficient(m);
         k_fill_table<<<blocks_for(total, 256, 1LL << 40), 256, 0, s>>>(m, h->b, h->phi, h->mdot, h->cell_code,
                                                                        h->table_index, df_kappa(m) * (m.mu_l - m.mu_g),
                                                                        kdil / df_kappa(m), h->table, h->table32,
