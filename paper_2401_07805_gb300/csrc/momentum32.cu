@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1), MINB)
                 Line32<Q>::val(u, gz[f]);
             }
             const int8_t cc = code[cell];
-            const float* tb = cc == CELL_TABLE ? table + (int64_t)tindex[cell] * TAB32_K * NQ : nullptr;
+            const float* tb = cc == CELL_TABLE ? table + (int64_t)tindex[cell] * TAB_K * NQ : nullptr;
             const float wyz = B.wf[qy] * B.wf[qz];
             float Pd[2] = {0.f, 0.f};
 #pragma unroll

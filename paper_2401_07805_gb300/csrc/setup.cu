@@ -187,10 +187,10 @@ __global__ void k_fill_table(MeshArgs<double> m, Basis<double> b, const double* 
     const double vals[TAB_K] = {rho, mu, z * nv[0], z * nv[1], z * nv[2], md * kdil * delta, delta};
     const int64_t tb = (int64_t)tindex[cell] * TAB_K * nq + q;
 #pragma unroll
-    for (int k = 0; k < TAB_K; ++k) table[tb + (int64_t)k * nq] = vals[k];
-    const int64_t tb32 = (int64_t)tindex[cell] * TAB32_K * nq + q;
-#pragma unroll
-    for (int k = 0; k < TAB32_K; ++k) table32[tb32 + (int64_t)k * nq] = (float)vals[k];
+    for (int k = 0; k < TAB_K; ++k) {
+        table[tb + (int64_t)k * nq] = vals[k];
+        table32[tb + (int64_t)k * nq] = (float)vals[k];
+    }
     // (the adjoint's weight is kappa W: kdmu = kappa (mu_l - mu_g), kdk = kdil / kappa)
     double av[ADJ_K];
     av[ADJ_CRHO] = -rho * rho * (irl - irg) * dHdd;
@@ -236,7 +236,7 @@ int launch_setup_coefficients(evap_mesh* h, cudaStream_t s) {
         h->table_cap = 0;
         const int64_t cap = count + count / 8 + 16;
         EVAP_CUDA(cudaMalloc(&h->table, cap * TAB_K * nq * sizeof(double)));
-        EVAP_CUDA(cudaMalloc(&h->table32, cap * TAB32_K * nq * sizeof(float)));
+        EVAP_CUDA(cudaMalloc(&h->table32, cap * TAB_K * nq * sizeof(float)));
         EVAP_CUDA(cudaMalloc(&h->adj_table, cap * ADJ_K * nq * sizeof(float2)));
         h->table_cap = cap;
     }
