@@ -28,7 +28,10 @@
  *             evap_set_fields copies its inputs into library-owned device memory.  Output arrays must not alias
  *             inputs.
  *   Streams:  `stream` is a cudaStream_t passed as void* (NULL = legacy default stream).  All work of a call is
- *             enqueued on that stream and the call returns without synchronizing, except where stated.
+ *             enqueued on that stream and the call returns without synchronizing, except where stated.  Applies
+ *             (evap_apply_*) write nothing but their results, so several streams may run them on one handle at a time
+ *             (evap_apply_schur once its stencil is assembled, and not with evap_set_checks on); every other call uses
+ *             the handle's own arrays: one at a time.
  *   Errors:   every function returns EVAP_OK (0) or a negative status; evap_status_string() names it and
  *             evap_last_error() returns the message of the most recent failure in the calling host thread.
  *             Arguments are validated before any work is enqueued; on EVAP_EINVAL nothing was enqueued.

@@ -59,10 +59,12 @@ __global__ void __launch_bounds__(256) k_adjoint_init(int M, int64_t Nu, int64_t
 // w, two rounds over a cell's Q^3 threads) and the sensitivities by one thread per quadrature point, which overwrites
 // its own point's values and gradients with them.  Only the threads of table cells run the interface-zone work and the
 // level-set sweeps.  At most 48 KB of shared memory per block, so no launch needs a function attribute.
-// Measured at 48^3 Q2 (us; one point per thread with Q-term dot products 775 to 800): cells per block / blocks per SM 4 / 5
-// 582 (96 registers); 4 / 4 595; 2 / 10 603; 3 / 6 612; 1 / 20 637.  ncu: issue 59 %, FP64 pipe 63 % (conversions).
-// Normalization as in the forward apply: the gradients at the points, the value sensitivities that start the test sums
-// and the last transposed sweep (converted to FP64 next) are left unnormalized.
+// Measured at 48^3 Q2 (us; one point per thread with Q-term dot products 779): cells per block / blocks per SM 4 / 5 550 (96
+// registers); 2 / 10 564; 4 / 4 586; 3 / 6 589.  On a subdivided level set (n_sub = 2; 947 before): 4 / 5 599; 4 / 4 and 3 / 6 591;
+// 2 / 10 605.  Q3 at 32^3 (859 before; one cell, more exceed 48 KB): 1, 4, 6 and 8 blocks per SM 519, 9 543.  ncu at 64^3: issue
+// 59 %, FP64 pipe 61 % (conversions).
+// Normalization as in the forward apply: the value sensitivities that start the test sums and the last transposed sweep (converted
+// to FP64 next) are left unnormalized.
 #ifndef EVAP_ADJ_CB2
 #define EVAP_ADJ_CB2 4
 #endif

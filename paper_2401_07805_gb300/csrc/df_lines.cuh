@@ -32,12 +32,13 @@ __device__ __forceinline__ dfl df_half(dfl a) { return {0.5f * a.hi, 0.5f * a.lo
 
 // Which sums are normalized: results stored for the next sweep (df_addo) and, for Q = 3, sums multiplied next (df_addi) and the
 // gradients; sums that are added further are not.  Errors against 64 bits relative to point-wise dot products, geometric
-// means (velocity rows / divergence row / adjoint g_x / g_u0 / g_phi over 100 to 2242 drawn Q2 cases; pressure term alone, 34):
+// means (velocity rows / divergence row / adjoint g_x / g_u0 / g_phi over 100 to 2242 drawn Q2 cases, g_phi 1.004 +- 0.005; pressure
+// term alone, 34):
 //   outer values as u_1 + 3/10 C -+ tau dm with C = u_0 - 2 u_1 + u_2, the transposed middle as s + f_1 - 2 (3/10 s),
-//     even part and gradients unnormalized    0.98 / 1.02 / 1.00 / 1.00 / 1.05 / 1.12   (48^3 Q2 apply 218 us, adjoint 561)
-//   this arrangement                          0.90 / 0.91 / 0.82 / 0.81 / 1.004 +- 0.005 / 0.77   (216 us, 549)
+//     even part and gradients unnormalized    0.98 / 1.03 / 0.99 / 1.00 / 1.05 / 1.12          (48^3 Q2 apply 218 us, adjoint 561)
+//   this arrangement                          0.92 / 0.91 / 0.90 / 0.89 / 1.00 / 0.77          (216 us, 550)
 // 64^3 Q2 apply with the first arrangement (us): both of df_addo and df_addi normalized 552, one of them 540, none 529.
-// Q = 4 normalizes the stored results only (45^3 Q3: 576 -> 544 us; 0.89 / 0.97 / 0.88 / 0.90 / 0.98 / 0.99).
+// Q = 4 normalizes the stored results only (45^3 Q3: 576 -> 544 us; 0.91 / 0.97 / 0.92 / 0.92 / 0.95 / 0.99).
 __device__ __forceinline__ dfl df_addo(dfl a, dfl b) { return df_add(a, b); }
 __device__ __forceinline__ dfl df_addi(dfl a, dfl b) { return df_add(a, b); }
 

@@ -7,7 +7,7 @@
 // the whole solve is one cooperative launch: each block owns a fixed share of the nodes for all iterations, the grid
 // meets at a barrier wherever a step reads other blocks' entries (the operator reads neighbours; a scalar product
 // needs every block's partial), and the vectors are double-float pairs (dfloat.cuh) so that the iteration runs on the
-// FP32 pipe; FP64 only converts the inputs and the result and forms the scalars.
+// FP32 pipe; FP64 only converts the inputs and the result and forms the GMRES scalars (those of the CG are double-float pairs too).
 //
 // Scalar products are summed from per-block partials by every block in the same order, so all blocks take the same
 // scalars and the same stopping decision and a solve is bitwise reproducible.  The barrier's wait is bounded: a block
@@ -127,7 +127,7 @@ __device__ __forceinline__ void grid_sum_df(const float2* part, float2* sh, dfl 
 // The operators as 27-point stencils on the Q1 node lattice (n + 1 nodes per direction), x as pairs: row `node` is
 // sum_s C_s(node) x(node + o_s) over the offsets o_s = (dx, dy, dz) in {-1, 0, 1}^3, s = 9 (dz + 1) + 3 (dy + 1) +
 // (dx + 1).  Neither operator branches on the lattice boundary, so that a node's 27 loads are in flight together (with a
-// test per neighbour the CG took 18.5 and 24 us per iteration at 64^3 for the two operators, now 15 and 19).  Node indices fit 32 bits
+// test per neighbour the CG took 18.5 and 24 us per iteration at 64^3 for the two operators, 15 and 19 without).  Node indices fit 32 bits
 // (checked on the host).
 
 // (M + c K) for one field: constant coefficients, 4 distinct ones (by the number of nonzero components of the offset: 0
@@ -229,7 +229,8 @@ struct NodeStencil {
 // entries a row may read before the first or after the last of its vector
 inline int64_t stencil_guard(int n) { return (int64_t)(n + 1) * (n + 1) + (n + 1) + 1; }
 
-// a / b (relative error ~2^-46): three quotient terms by the reciprocal of b.hi, each from the exact remainder's pair
+// a / b (relative error ~2^-46): long division by three quotient terms, each from the remainder of the last (the scheme of Hida, Li
+// and Bailey, ARITH-15, 2001), with the reciprocal of b.hi
 __device__ __forceinline__ dfl df_div(dfl a, dfl b) {
     if (fabsf(b.hi) < 0x1p-100f) {  // keep the reciprocal finite
         a = df_scale2(a, 0x1p60f);
@@ -247,7 +248,9 @@ __device__ __forceinline__ dfl df_div(dfl a, dfl b) {
 
 // The scalars of a Chronopoulos-Gear iteration from its three sums, in double-float arithmetic by one thread: on the FP64
 // pipe (64 cycles per instruction of a lone warp) the divisions and the square root took ~2 us of every iteration (CG at
-// 64^3: 15 -> 13 us, 19 -> 17 us per iteration for the two stencils).
+// 64^3: 15 -> 13 us, 19 -> 17 us per iteration for the two stencils).  Against the solvers with FP64 scalars the
+// solutions' errors to 64 bits are 0.98, 0.98 and 0.997 times as large (normal, curvature, reinitialized field; geometric means over 99
+// to 111 drawn level sets), the iteration counts of 60 reinitializations the same but for one more in two.
 struct CgScalars {
     dfl gamma_old{1.f, 0.f}, alpha_old{1.f, 0.f};
     // beta and alpha of the iteration (first: beta = 0)
@@ -605,7 +608,7 @@ __global__ void __launch_bounds__(FK_THREADS) k_gmres_fused(Op op, int64_t N, in
 // ------------------------------------------------------------------------------------- FP32 conjugate gradients
 // The same Chronopoulos-Gear CG in FP32 for operators whose solve only has to be approximate (the Schur solve inside
 // the velocity-pressure preconditioner): vectors and coefficients in FP32, the scalar products summed in FP32 in a
-// fixed order (warp shuffle trees, then the blocks' partials), the scalars formed in FP64 by thread 0.  Op::row
+// fixed order (warp shuffle trees, then the blocks' partials), the scalars formed in double-float arithmetic by thread 0.  Op::row
 // returns float.  b and x are FP64 (converted once in and out).  Same out[] convention as k_cg_fused.
 __device__ __forceinline__ float warp_sum_f(float v) {
 #pragma unroll
@@ -706,7 +709,7 @@ __global__ void __launch_bounds__(FK_THREADS) k_cg_fused32(Op op, int64_t N, con
 
 // ------------------------------------------------------------------------------------------ host-side workspace
 // Workspace of the single-launch solvers, kept with the mesh (geometry.cu): stencil_guard zero pairs, nvec pair vectors of
-// N_phi entries (or, read as floats, 2 nvec float vectors), an FP32 vector, (GM_MAX + 2) CG_BLOCKS partial pairs, the
+// N_phi entries (or, read as floats, 2 nvec float vectors), an FP32 vector, (GM_MAX + 2) FK_MAX_BLOCKS partial pairs, the
 // barrier and 4 result words.
 struct FusedSpace {
     float2* vec;  // vector k at vec + k N

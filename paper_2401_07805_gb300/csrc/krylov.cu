@@ -404,8 +404,9 @@ constexpr double REORTH64 = 0.5;
 constexpr double REORTH32 = 1e-2;
 // The velocity-pressure solve: its preconditioned operator is close to the identity, so the DGKS test fired on almost
 // every step as well, and on GB300 a second pass over the FP64 basis costs as much as the operator (FP64-pipe bound).
-// With 1e-2 in place of 1/2 the solves and steps at 20^3 to 64^3 kept their application counts to within one in 28; the
-// true residual decides as before.  A step at 64^3: 105 -> 92 ms.
+// With 1e-2 in place of 1/2 the application counts of 360 solves were the same in 354, one fewer in 3 and one or two more in 3
+// (6^3 to 56^3, Q2 and Q3, density ratios 1e3 and 1e4, restart 30 to 255, relative residuals 1e-8 to 1e-13, 10 to 41
+// applications); the true residual decides as before.  A step at 64^3: 105 -> 92 ms.
 constexpr double REORTH_SADDLE = 1e-2;
 // the operator of a solve (the momentum system; the level-set solves run in fused_krylov.cuh)
 enum { OP_MOMENTUM = 0 };
@@ -480,7 +481,7 @@ static int set_scale(Ctx& c, int i, double sc) {
 // (the first residual is b, no apply).  The Krylov basis is kept unnormalized (v_i = sc_i V_i): the operator writes
 // A z straight into the next basis slot and the scales enter the Gram-Schmidt coefficients, so no vector pass is
 // spent on normalization.  one_cycle: a single cycle without the check of its true residual (an inexact solve inside a
-// flexible method, which would only discard it).  Classical Gram-Schmidt with a second pass only under REORTH64 / REORTH32.  Stops when the
+// flexible method, which would only discard it; the outer counts are the same with the check).  Classical Gram-Schmidt with a second pass only under REORTH64 / REORTH32.  Stops when the
 // Arnoldi residual estimate is <= tol_abs (then the true residual is recomputed) or after maxit applications.
 template <typename T>
 static int gmres(Ctx& c, int m, const T* b, T* x, bool x_zero, const T* diag, T* V, T* w, T* z, double tol_abs,

@@ -2,7 +2,7 @@
 // y_p = B x - g (Eq. continuity with the dilation rate of Eq. evaporDil): the pieces shared by its implementations.
 //   k_momentum_init   y = x on the Dirichlet DoFs, 0 elsewhere (the scatter of the applies adds the free rows)
 //   k_qp_coeffs       the quadrature-point coefficients of the operator (W rho c_m, W rho u0, W rho grad u0, 2 W mu,
-//                     z n, W, W v_dil), evaluated once per set_fields in double-float arithmetic and stored as
+//                     z n, W, W v_dil, some with powers of kappa), evaluated once per set_fields and stored as
 //                     double-float pairs and, for the u0 terms, in FP32 (the FP32 apply of momentum32.cu): on GB300 the
 //                     arithmetic, not HBM, bounds these operators, and the material law and the u0 interpolation
 //                     would otherwise be recomputed by every apply
@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(256) k_momentum_init(int M, int64_t Nu, unsign
 //   14..16: z n_b (correction gate times normal)   17: kappa W   18: W v_dil
 // W = w_qx w_qy w_qz h^3, kappa = DSCALE / h the factor between a gradient and the derivative sweeps (df_lines.cuh).  The
 // FP64-accurate apply and the adjoint read the pairs as they stand; the Jacobi diagonal, the mass load and the continuity
-// right-hand side read the few slots they need.  Slots 1..12 are also stored in FP32 for the FP32 apply (there W rho u0 / h:
+// right-hand side read the few slots they need (the two FP64 loads thus take their factors to ~48 bits, as every consumer).  Slots 1..12 are also stored in FP32 for the FP32 apply (there W rho u0 / h:
 // that kernel takes reference gradients), in its 32-cell block layout
 // qc32[((blk * QC32_K + k) * NQ + pt) * 32 + lane], cell 32 blk + lane (lexicographic).
 // Every factor that does not depend on u0 is formed in FP64 and rounded once to a pair (a power of kappa applied to a pair

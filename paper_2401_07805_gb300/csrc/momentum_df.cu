@@ -17,7 +17,7 @@
 //
 // Layout: CB cells per block with Q^3 threads each.  In a sweep a thread owns one line of Q points of one component
 // (Q^2 lines x 3 components: every thread for Q = 3, 48 of 64 for Q = 4) and forms its Q results in registers with the
-// even-odd line transforms of df_lines.cuh, so a sweep costs Q shared loads and Q stores per thread; the fluxes are
+// line transforms of df_lines.cuh, so a sweep costs Q shared loads and Q stores per thread; the fluxes are
 // formed by one thread per quadrature point.  The first sweep (z) gathers its lines from memory and the last one (z)
 // scatters its own, both as rows of x-consecutive nodes.  The lines of the test along y and z overlay the coefficient
 // slots, which the fluxes have read by then.
@@ -50,9 +50,10 @@ __device__ __forceinline__ constexpr int t_slot(int k, int l) {
 
 // Cells per block and blocks per SM (a register cap).  Measured at 64^3 Q2 with the divergence row (us per apply; one
 // point per thread with Q-term dot products: 673): CB 1 / 28 blocks 503 (a block is one warp), 495 with the sweeps
-// ordered by warp barriers (128^3: 3610 -> 3518); 2 / 16 526; 4 / 8 510; 5 / 6 552; 7 / 4 592; 8 / 4 581; 13 / 2 757.
-// Q3 at 45^3 (701 before): 2 and 4 cells 544, 1 cell 579.  ncu at 64^3, CB 4: 1842 warp instructions per cell (1064 FADD,
-// 194 FMUL and FFMA, 142 shared accesses), issue 77 % active, FP64 pipe 59 % (conversions).
+// ordered by warp barriers (128^3: 3610 -> 3518), 489 with three-term dots (3499); 2 / 16 526; 4 / 8 510; 5 / 6 552; 7 / 4 592; 8 / 4
+// 581; 13 / 2 757 (these with 503).
+// Q3 at 45^3 (701 before): 2 and 4 cells 544, 1 cell 579.  ncu at 64^3: 1843 warp instructions per cell, issue 82 % active, FP64
+// pipe 68 % (conversions).
 #ifndef EVAP_DF_CB2
 #define EVAP_DF_CB2 1
 #endif
@@ -85,8 +86,8 @@ __global__ void __launch_bounds__(CB*(P + 1) * (P + 1) * (P + 1), MINB)
     __shared__ dfl sN1[Q][2];
     __shared__ dfl q1a[CB][2 * Q * Q], q1b[CB][4 * Q];
     // the pressure at the cell's corners, then interpolated along x and y (z: by the point's thread), in FP64: 2 FP64
-    // operations per sweep instead of 14 per point (672 -> 562 us at 64^3; in double-float arithmetic 531, but with the
-    // error of a pure pressure term 6.6e-15 -> 7.4e-15 against 64 bits)
+    // operations per sweep instead of 14 per point (672 -> 562 us at 64^3, the call with its initialization 608, 584 with the line
+    // transforms as they are; the pressure interpolated in double-float arithmetic 531, but with a larger error of the pressure term)
     __shared__ double p0[PRES ? CB : 1][8], px[PRES ? CB : 1][4 * Q], py[PRES ? CB : 1][2 * Q * Q];
     auto lerp = [&](double u, double v, int q) -> double { return fma(bas.t[q], v - u, u); };  // at Gauss point q
     extern __shared__ float2 smem_df[];
